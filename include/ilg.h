@@ -44,7 +44,7 @@ typedef enum {
   ILG_E_OOM = 2,      /* device allocation failed */
   ILG_E_OVERFLOW = 3, /* some occupation would exceed 65535; state rolled back */
   ILG_E_CUDA = 4,     /* CUDA runtime error */
-  ILG_E_TIMEOUT = 5,  /* a bounded device wait gave up */
+  ILG_E_TIMEOUT = 5,  /* a bounded device wait gave up (a context's state is then lost) */
   ILG_E_STATE = 6     /* call out of order (e.g. step before init/set_state) */
 } ilg_status;
 
@@ -143,7 +143,8 @@ ilg_status ilg_set_temporal_blocking(ilg_ctx* ctx, uint32_t depth);
  * for later ilg_step calls:
  *   candidate 0  row-tiled step, 8 nodes per thread (16-byte vectors), 3 blocks per SM
  *   candidate 1  row-tiled step, 4 nodes per thread (8-byte vectors), 3 blocks per SM
- *   candidate 2  node-parallel step, one node per thread
+ *   candidate 2  node-parallel step, one node per thread; D1Q3 and D2Q5: up to 4096
+ *                steps per launch (the default on lattices of at most 8192 nodes per SM)
  *   candidate 3, 4  temporal blocking of depth 2, 4 (D2Q5; the remainder of a call
  *                takes the fastest single-step candidate)
  *   candidate 5  8-node vectors in warp segments: each warp walks 8192 nodes of a row,
@@ -155,7 +156,7 @@ ilg_status ilg_set_temporal_blocking(ilg_ctx* ctx, uint32_t depth);
  *                compile-time plane order, the fast collision branch-free, the
  *                values crossing a segment's ends written by the warp that computes
  *                them (no node computed twice); one block of 384 threads per SM
- *                (the default where it applies)
+ *                (the default where it applies, on larger lattices)
  *   candidate 7  as 6 with 4-node vectors (rows a multiple of 4), 640 threads per SM
  *                (the default where 6 does not apply and 7 does)
  *   D2Q9 lattices: candidate 2 (node-parallel, two nodes of a row per thread where

@@ -28,7 +28,8 @@ struct ilg_ctx {
   uint64_t t = 0;
   bool has_state = false;
   uint32_t* d_tables = nullptr;            // thinning table, rest table
-  unsigned long long* d_fail = nullptr;    // first failing step, ~0 if none
+  unsigned long long* d_fail = nullptr;    // [0] first failing step, ~0 if none; [1], [2] the
+                                           // words of a several-step launch (launch_step_run)
   unsigned long long* d_col = nullptr;     // Lx
   unsigned long long* d_row = nullptr;     // Ly
   unsigned long long* d_mass = nullptr;
@@ -39,11 +40,13 @@ struct ilg_ctx {
   uint32_t general = 0;                    // too many nodes would fail the fast collision: general at once
   int kernel_choice = -1;                  // single-step kernel chosen by ilg_autotune (-1: default)
   double omega_star = 0;
-  unsigned long long* h_word = nullptr;    // pinned 8-byte readback
+  unsigned long long* h_word = nullptr;    // pinned readback, kFailWords words
   std::string err;
 };
 
 namespace {
+
+constexpr size_t kFailWords = 3;
 
 thread_local std::string g_create_error;
 
@@ -210,11 +213,11 @@ ilg_status ilg_create(const ilg_params* params, void* stream, ilg_ctx** out) {
   static_assert(kBlockWords == kDevBlockWords && kBlockWords9 == kDevBlockWords9, "table block layout");
   const size_t block_words = c->Q == 9 ? kBlockWords9 : kBlockWords;
   if ((e = dev_alloc(&c->d_tables, sizeof(uint32_t) * block_words)) != cudaSuccess) return bail(e, "cudaMalloc tables");
-  if ((e = dev_alloc(&c->d_fail, sizeof(unsigned long long))) != cudaSuccess) return bail(e, "cudaMalloc flag");
+  if ((e = dev_alloc(&c->d_fail, sizeof(unsigned long long) * kFailWords)) != cudaSuccess) return bail(e, "cudaMalloc flag");
   if ((e = dev_alloc(&c->d_col, sizeof(unsigned long long) * c->p.Lx)) != cudaSuccess) return bail(e, "cudaMalloc sums");
   if ((e = dev_alloc(&c->d_row, sizeof(unsigned long long) * c->p.Ly)) != cudaSuccess) return bail(e, "cudaMalloc sums");
   if ((e = dev_alloc(&c->d_mass, sizeof(unsigned long long))) != cudaSuccess) return bail(e, "cudaMalloc mass");
-  if ((e = cudaMallocHost(&c->h_word, sizeof(unsigned long long))) != cudaSuccess) return bail(e, "cudaMallocHost");
+  if ((e = cudaMallocHost(&c->h_word, sizeof(unsigned long long) * kFailWords)) != cudaSuccess) return bail(e, "cudaMallocHost");
 
   std::vector<uint32_t> tables(block_words, 0u);
   build_table_block(c->Q, c->p.sampler, c->P_omega, c->P_rest, c->P_axis, tables.data());
@@ -225,6 +228,7 @@ ilg_status ilg_create(const ilg_params* params, void* stream, ilg_ctx** out) {
   e = cudaMemcpyAsync(c->d_tables, tables.data(), sizeof(uint32_t) * tables.size(), cudaMemcpyHostToDevice, c->stream);
   if (e != cudaSuccess) return bail(e, "copy tables");
   e = cudaMemsetAsync(c->d_fail, 0xFF, sizeof(unsigned long long), c->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->d_fail + 1, 0, 2 * sizeof(unsigned long long), c->stream);
   if (e != cudaSuccess) return bail(e, "reset flag");
   e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return bail(e, "cudaStreamSynchronize");
@@ -378,12 +382,20 @@ bool kernel_applies(const ilg_ctx* c, const StepArgs& a, int kind) {
 // resident warps of the row-tiled kernels (3 blocks of 8 warps per SM)
 uint64_t vec_warps(const ilg_ctx* c) { return uint64_t(c->sms) * 3 * 8; }
 
+// D1Q3 and D2Q5 lattices of at most this many nodes per SM run node-parallel, several
+// steps per launch: there a launch, its table staging and its idle warps per step cost
+// the staged warp kernel more than its cheaper collision saves (D2Q5, 10 per velocity,
+// us per step node-parallel / staged warp: 64^2 2.3 / 24.7, 512^2 5.8 / 22.7, 1024^2
+// 15.3 / 22.7, 1448^2 27.5 / 24.9, 2048^2 50 / 37)
+constexpr uint64_t kRunNodesPerSm = 8192;
+
 // the kernel a step runs: the tuned one while it applies to the current state, else
-// the default: the shared-memory-staged warp kernel with 8-node, else 4-node vectors
-// where the rows and probabilities allow; else 8-node row tiles where the rows allow;
-// node-parallel otherwise
+// the default: node-parallel on small lattices; the shared-memory-staged warp kernel
+// with 8-node, else 4-node vectors where the rows and probabilities allow; else 8-node
+// row tiles where the rows allow; node-parallel otherwise
 int pick_kernel(const ilg_ctx* c, const StepArgs& a) {
   if (c->kernel_choice >= 0 && kernel_applies(c, a, c->kernel_choice)) return c->kernel_choice;
+  if (c->Q != 9 && c->nodes <= kRunNodesPerSm * uint64_t(c->sms)) return kKernelNode;
   if (kernel_applies(c, a, kKernelWarp8)) return kKernelWarp8;
   if (kernel_applies(c, a, kKernelWarp4)) return kKernelWarp4;
   if (!kernel_applies(c, a, kKernelVec8)) return kKernelNode;
@@ -415,8 +427,36 @@ cudaError_t launch_single(const ilg_ctx* c, int kind, const StepArgs& a, const u
     return launch_step_warp(c->Q, shape, a, in, out, uint32_t(t), fail_word,
                             int(step_warp_grid(c->Q, c->p.Lx, Ly, uint32_t(c->sms), shape)), c->stream);
   }
-  return launch_step(c->Q, a, in, out, uint32_t(t), fail_word,
-                     step_grid(c, step_kernel_blocks_per_sm(), step_kernel_threads()), c->stream);
+  return launch_step_run(c->Q, a, const_cast<uint16_t*>(in), out, uint32_t(t), 1, fail_word, fail_word + 1,
+                         uint32_t(c->sms), c->stream);
+}
+
+// T single steps from step t (the state in bufs[cur], the steps alternate the buffers);
+// the node-parallel kernel takes them in few launches of several steps each
+cudaError_t launch_singles(const ilg_ctx* c, int kind, const StepArgs& a, uint16_t* const* bufs, int cur, uint64_t t,
+                           uint32_t T, unsigned long long* fail_word) {
+  constexpr uint32_t kRunSteps = 4096;  // per launch
+  bool run = kind == kKernelNode && c->Q != 9;
+  for (uint32_t k = 0; k < T;) {
+    const uint32_t n = run ? std::min(T - k, kRunSteps) : 1;
+    cudaError_t e;
+    if (n > 1) {
+      e = launch_step_run(c->Q, a, bufs[cur], bufs[cur ^ 1], uint32_t(t + k), n, fail_word, fail_word + 1,
+                          uint32_t(c->sms), c->stream);
+      if (e == cudaErrorCooperativeLaunchTooLarge) {
+        // the device cannot hold all blocks at once (SMs reserved elsewhere): step by step
+        cudaGetLastError();
+        run = false;
+        continue;
+      }
+    } else {
+      e = launch_single(c, kind, a, bufs[cur], bufs[cur ^ 1], t + k, fail_word);
+    }
+    if (e != cudaSuccess) return e;
+    k += n;
+    cur ^= int(n & 1u);
+  }
+  return cudaSuccess;
 }
 
 int tb_grid(const ilg_ctx* c, uint32_t depth) {
@@ -439,9 +479,8 @@ ilg_status ilg_step(ilg_ctx* c, uint32_t T) {
   const int kind = pick_kernel(c, a);
   const int cur0 = c->cur;
   const uint64_t t0 = c->t;
-  // launches: blocks of tb_depth steps (temporal blocking), then single steps;
-  // launch_t[k] is the step a launch starts from, its input is buffer cur0 ^ (k & 1)
-  std::vector<uint64_t> launch_t;
+  // blocks of tb_depth steps (temporal blocking), then single steps; a block or step k
+  // reads buffer cur0 ^ (k & 1)
   int cur = cur0;
   uint64_t t = t0;
   const uint32_t tb = c->tb_depth;
@@ -451,26 +490,35 @@ ilg_status ilg_step(ilg_ctx* c, uint32_t T) {
       cudaError_t e = launch_step_tb(a, c->buf[cur], c->buf[cur ^ 1], uint32_t(t), tb, tb_tile(tb), c->d_fail, tgrid,
                                      c->stream);
       if (e != cudaSuccess) return cuda_fail(c, e, "temporal blocking kernel");
-      launch_t.push_back(t);
       t += tb;
       cur ^= 1;
     }
   }
-  while (t < t0 + T) {
-    cudaError_t e = launch_single(c, kind, a, c->buf[cur], c->buf[cur ^ 1], t, c->d_fail);
+  const uint64_t t_single = t;  // single steps from here
+  const uint64_t blocks = tb >= 2 ? (t - t0) / tb : 0;
+  if (const uint32_t n = uint32_t(t0 + T - t)) {
+    const cudaError_t e = launch_singles(c, kind, a, c->buf, cur, t, n, c->d_fail);
     if (e != cudaSuccess) return cuda_fail(c, e, "step kernel");
-    launch_t.push_back(t);
-    t += 1;
-    cur ^= 1;
+    cur ^= int(n & 1u);
   }
-  ILG_CUDA(c, cudaMemcpyAsync(c->h_word, c->d_fail, sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream),
+  ILG_CUDA(c, cudaMemcpyAsync(c->h_word, c->d_fail, sizeof(unsigned long long) * kFailWords, cudaMemcpyDeviceToHost,
+                              c->stream),
            "read overflow word");
   ILG_CUDA(c, cudaStreamSynchronize(c->stream), "step");
-  const unsigned long long f = *c->h_word;
+  const unsigned long long f = c->h_word[0];
+  if (c->h_word[2] != 0) {
+    // a bounded wait between the blocks of a several-step launch gave up: the buffers
+    // hold parts of different steps
+    c->has_state = false;
+    ILG_CUDA(c, cudaMemsetAsync(c->d_fail, 0xFF, sizeof(unsigned long long), c->stream), "reset flag");
+    ILG_CUDA(c, cudaMemsetAsync(c->d_fail + 1, 0, 2 * sizeof(unsigned long long), c->stream), "reset flag");
+    ILG_CUDA(c, cudaStreamSynchronize(c->stream), "reset flag");
+    return fail(c, ILG_E_TIMEOUT, "a wait between the blocks of a several-step launch gave up: the state is lost");
+  }
   if (f != ~0ull) {
-    // the launch that started at step f failed: its input buffer still holds the state at f
-    size_t k = 0;
-    while (k < launch_t.size() && launch_t[k] != f) ++k;
+    // the block or step that started at step f failed: its input buffer still holds the
+    // state at f
+    const uint64_t k = f < t_single ? (f - t0) / tb : blocks + (f - t_single);
     c->cur = cur0 ^ int(k & 1u);
     c->t = f;
     ILG_CUDA(c, cudaMemsetAsync(c->d_fail, 0xFF, sizeof(unsigned long long), c->stream), "reset flag");
@@ -515,7 +563,7 @@ ilg_status ilg_autotune(ilg_ctx* c, uint32_t trial_steps, ilg_tuning* out) {
   };
   cudaError_t e = dev_alloc(&s[0], bytes);
   if (e == cudaSuccess) e = dev_alloc(&s[1], bytes);
-  if (e == cudaSuccess) e = dev_alloc(&fw, sizeof(unsigned long long));
+  if (e == cudaSuccess) e = dev_alloc(&fw, sizeof(unsigned long long) * kFailWords);
   if (e == cudaSuccess) e = cudaEventCreate(&e0);
   if (e == cudaSuccess) e = cudaEventCreate(&e1);
   if (e == cudaSuccess) e = cudaMemcpyAsync(s[0], c->buf[c->cur], bytes, cudaMemcpyDeviceToDevice, c->stream);
@@ -534,18 +582,26 @@ ilg_status ilg_autotune(ilg_ctx* c, uint32_t trial_steps, ilg_tuning* out) {
     const uint32_t launches = std::max<uint32_t>(1, trial_steps / depth);
     uint64_t t = c->t;
     int cur = 0;
-    auto one = [&]() -> cudaError_t {
-      cudaError_t r = depth > 1 ? launch_step_tb(a, s[cur], s[cur ^ 1], uint32_t(t), depth, tb_tile(depth), fw, tb_grid(c, depth),
-                                                 c->stream)
-                                : launch_single(c, cand, a, s[cur], s[cur ^ 1], t, fw);
-      t += depth;
-      cur ^= 1;
+    auto some = [&](uint32_t n) -> cudaError_t {  // n launches of `depth` steps
+      cudaError_t r = cudaSuccess;
+      if (depth == 1) {
+        r = launch_singles(c, cand, a, s, cur, t, n, fw);
+        cur ^= int(n & 1u);
+      } else {
+        for (uint32_t k = 0; k < n && r == cudaSuccess; ++k) {
+          r = launch_step_tb(a, s[cur], s[cur ^ 1], uint32_t(t) + k * depth, depth, tb_tile(depth), fw, tb_grid(c, depth),
+                             c->stream);
+          cur ^= 1;
+        }
+      }
+      t += uint64_t(n) * depth;
       return r;
     };
     cudaError_t r = cudaMemsetAsync(fw, 0xFF, sizeof(unsigned long long), c->stream);
-    if (r == cudaSuccess) r = one();  // warm-up launch
+    if (r == cudaSuccess) r = cudaMemsetAsync(fw + 1, 0, 2 * sizeof(unsigned long long), c->stream);
+    if (r == cudaSuccess) r = some(1);  // warm-up launch
     if (r == cudaSuccess) r = cudaEventRecord(e0, c->stream);
-    for (uint32_t k = 0; k < launches && r == cudaSuccess; ++k) r = one();
+    if (r == cudaSuccess) r = some(launches);
     if (r == cudaSuccess) r = cudaEventRecord(e1, c->stream);
     if (r == cudaSuccess) r = cudaMemcpyAsync(c->h_word, fw, sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream);
     if (r == cudaSuccess) r = cudaStreamSynchronize(c->stream);

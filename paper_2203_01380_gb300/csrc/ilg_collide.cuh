@@ -1,0 +1,233 @@
+// The collision of one node per lane by a whole warp (D1Q3, D2Q5; any occupations):
+// the node-parallel kernels' collision, where many nodes need more random words than
+// the eight slot words.
+//
+// What bounds it: the ALU pipe (two cycles per warp instruction and sub-partition),
+// then the wide products of Philox on the FMA-heavy pipe.  Per-lane loops over chunks
+// and groups spend most of their issue slots on divergence and on branches per lane,
+// so here every loop runs as often as the warp's neediest lane asks (a vote), and a
+// lane that is done draws from row 0 of the table or masks its bits away: the same
+// result without a branch.  The words beyond the slot words wait in a ring of K words
+// per lane in shared memory (lane-interleaved, so no access conflicts), filled one
+// Philox block at a time by all lanes together when one of them runs short.
+#pragma once
+
+#include <cstdint>
+
+#include "ilg_device.cuh"
+
+namespace ilg {
+
+constexpr unsigned kFullWarp = 0xFFFFFFFFu;
+
+// What is the same for every node of a launch (or of a lattice and step) in the first
+// three Philox rounds (see StepKeys), and the two words an extension block's own part
+// of them starts from.
+struct WordKeys {
+  StepKeys<2> slot;
+  uint32_t ext_c;  // round 2's x2 of extension block 0, without the block index
+  uint32_t ext_e;  // round 3's x0 without the block's product
+};
+
+__device__ __forceinline__ WordKeys word_keys(const StepArgs& a, uint32_t t) {
+  constexpr uint32_t M0 = 0xD2511F53u, M1 = 0xCD9E8D57u;
+  WordKeys k;
+  k.slot = step_keys<2>(a, t);
+  k.ext_c = uint32_t((uint64_t(M0) * t) >> 32) ^ kDevTagExt ^ a.rk[1];
+  k.ext_e = uint32_t(uint64_t(M1) * a.replica) ^ a.rk[2];
+  return k;
+}
+
+// Rounds 4..10 of a block whose words after round 3 are c.
+__device__ __forceinline__ uint4 philox_tail(uint4 c, const uint32_t (&rk)[20]) {
+#pragma unroll
+  for (int r = 3; r < 10; ++r) {
+    const uint64_t p0 = uint64_t(0xD2511F53u) * c.x;
+    const uint64_t p1 = uint64_t(0xCD9E8D57u) * c.z;
+    c = make_uint4(uint32_t(p1 >> 32) ^ c.y ^ rk[2 * r], uint32_t(p1), uint32_t(p0 >> 32) ^ c.w ^ rk[2 * r + 1],
+                   uint32_t(p0));
+  }
+  return c;
+}
+
+// The words of one node and step.  S: bytes between a lane's consecutive words in the
+// ring (4 x the threads that share it), K: words per lane (a power of two).
+template <uint32_t S, uint32_t K>
+struct NodeWords {
+  static_assert((K & (K - 1)) == 0 && (S & (S - 1)) == 0 && K >= 8, "a ring of whole blocks");
+  static constexpr uint32_t kWrap = S * K - 1;
+  unsigned char* ring;     // shared memory
+  uint32_t rd, wr;         // byte positions of the next word to take and to write (unwrapped)
+  uint32_t r2h, r2l, p1l;  // the node's part of rounds 1-3
+  uint32_t blk;            // next extension block
+
+  __device__ __forceinline__ void begin(const WordKeys& k, unsigned char* ring_, uint32_t lane_off, uint32_t node) {
+    const uint64_t P1 = uint64_t(0xD2511F53u) * (node ^ k.slot.A);
+    const uint64_t R2 = uint64_t(0xCD9E8D57u) * (uint32_t(P1 >> 32) ^ k.slot.G);
+    r2h = uint32_t(R2 >> 32);
+    r2l = uint32_t(R2);
+    p1l = uint32_t(P1);
+    ring = ring_;
+    rd = wr = lane_off;
+    blk = 0;
+  }
+  __device__ __forceinline__ uint4 slot(const WordKeys& k, const uint32_t (&rk)[20], int b) const {
+    return philox_tail(make_uint4(r2h ^ k.slot.H[b], r2l, p1l ^ k.slot.I[b], k.slot.J[b]), rk);
+  }
+  // the next extension block into the ring
+  __device__ __forceinline__ void fill(const WordKeys& k, const uint32_t (&rk)[20]) {
+    const uint64_t R1 = uint64_t(0xCD9E8D57u) * (k.ext_c ^ blk);
+    const uint64_t P2 = uint64_t(0xD2511F53u) * (uint32_t(R1 >> 32) ^ k.ext_e);
+    const uint4 b = philox_tail(make_uint4(r2h ^ uint32_t(R1) ^ rk[4], r2l, p1l ^ uint32_t(P2 >> 32) ^ rk[5], uint32_t(P2)), rk);
+    uint32_t* p = reinterpret_cast<uint32_t*>(ring + (wr & kWrap));  // whole blocks: the four words do not wrap
+    p[0] = b.x;
+    p[S / 4] = b.y;
+    p[2 * (S / 4)] = b.z;
+    p[3 * (S / 4)] = b.w;
+    wr += 4 * S;
+    blk += 1;
+  }
+  // every lane has at least `bytes` of words afterwards (bytes <= (K - 4) S, a multiple of
+  // S); lanes with room fill together
+  __device__ __forceinline__ void ensure(const WordKeys& k, const uint32_t (&rk)[20], uint32_t bytes) {
+    while (__any_sync(kFullWarp, wr - rd < bytes)) {
+      if (wr - rd <= (K - 4) * S) fill(k, rk);
+    }
+  }
+  // the word `ahead` places after the next one
+  __device__ __forceinline__ uint32_t peek(uint32_t ahead = 0) const {
+    return *reinterpret_cast<const uint32_t*>(ring + ((rd + ahead * S) & kWrap));
+  }
+};
+
+// Binomial(x, P) beyond its first chunk: chunks of 63 trials, each with the lane's next
+// extension word, two per pass; left = x - 63 (negative or zero: none).  A lane that is
+// done draws from row 0: nothing.
+template <uint32_t S, uint32_t K, class Tab>
+__device__ __forceinline__ uint32_t more_chunks(NodeWords<S, K>& e, const WordKeys& k, const uint32_t (&rk)[20],
+                                                const Tab& A, int32_t left) {
+  uint32_t r = 0;
+  while (__any_sync(kFullWarp, left > 0)) {
+    e.ensure(k, rk, left > int32_t(kDevNmax) ? 2 * S : (left > 0 ? S : 0u));
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      r += A(uint32_t(__vimin_s32_relu(left, int32_t(kDevNmax))), e.peek());
+      if (left > 0) e.rd += S;
+      left -= int32_t(kDevNmax);
+    }
+  }
+  return r;
+}
+
+// The collision of one node per lane (m: its occupations after the flip, all zero for a
+// lane without a node); all 32 lanes call it together.  The same words and results as
+// collide().  ring: the block's ring of K words per thread in shared memory, lane_off:
+// 4 x the thread's index.
+template <int Q, uint32_t S, uint32_t K, class Tab>
+__device__ __forceinline__ void collide_warp(const StepArgs& a, const WordKeys& k, const Tab& to, const Tab& tr,
+                                             unsigned char* ring, uint32_t lane_off, uint32_t node,
+                                             const uint32_t (&m)[Q], uint32_t (&out)[Q]) {
+  static_assert(Q == 3 || Q == 5, "D1Q3 and D2Q5");
+  constexpr int32_t kN = int32_t(kDevNmax);
+  NodeWords<S, K> e;
+  e.begin(k, ring, lane_off, node);
+  uint32_t W[8];
+#pragma unroll
+  for (int b = 0; b < 2; ++b) {
+    const uint4 v = e.slot(k, a.rk, b);
+    W[4 * b] = v.x;
+    W[4 * b + 1] = v.y;
+    W[4 * b + 2] = v.z;
+    W[4 * b + 3] = v.w;
+  }
+
+  // thinning
+  uint32_t r[Q], removed = 0;
+  if (a.omega_mode == kTable) {
+    uint32_t most = m[0];
+#pragma unroll
+    for (int i = 1; i < Q; ++i) most = max(most, m[i]);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) r[i] = to(min(m[i], kDevNmax), W[i]);
+    if (__any_sync(kFullWarp, most > uint32_t(kN))) {
+      if (!__any_sync(kFullWarp, most > uint32_t(2 * kN))) {
+        // one more chunk at most: no loop
+        uint32_t need = 0;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) need += m[i] > uint32_t(kN) ? S : 0u;
+        e.ensure(k, a.rk, need);
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+          r[i] += to(uint32_t(max(int32_t(m[i]) - kN, 0)), e.peek());
+          if (m[i] > uint32_t(kN)) e.rd += S;
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < Q; ++i) r[i] += more_chunks(e, k, a.rk, to, int32_t(m[i]) - kN);
+      }
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < Q; ++i) r[i] = a.omega_mode == kAlways ? m[i] : 0u;
+  }
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    out[i] = m[i] - r[i];
+    removed += r[i];
+  }
+
+  // share sent to rest
+  uint32_t to_rest;
+  if (a.rest_mode == kTable) {
+    to_rest = tr(min(removed, kDevNmax), W[Q]);
+    to_rest += more_chunks(e, k, a.rk, tr, int32_t(removed) - kN);
+  } else {
+    to_rest = a.rest_mode == kAlways ? removed : 0u;
+  }
+  out[0] += to_rest;
+
+  // directions of the moving particles, 32 at a time (a mask of no bits once a lane is done)
+  const uint32_t moving = removed - to_rest;
+  int32_t left = int32_t(moving);
+  uint32_t mask = __funnelshift_lc(kFullWarp, 0u, uint32_t(left));
+  left = max(left - 32, 0);
+  constexpr uint32_t kWords = Q == 3 ? 1 : 2;               // per group
+  constexpr int32_t kPass = Q == 3 ? 8 : 4;                 // groups whose words are asked for at once
+  auto ask = [&](int32_t l) { return min(uint32_t(l + 31) >> 5, uint32_t(kPass)) * (kWords * S); };
+  if constexpr (Q == 3) {
+    uint32_t minus = __popc(W[Q + 1] & mask);
+    while (__any_sync(kFullWarp, left > 0)) {
+      e.ensure(k, a.rk, ask(left));
+      for (int u = 0; u < kPass && __any_sync(kFullWarp, left > 0); ++u) {
+        mask = __funnelshift_lc(kFullWarp, 0u, uint32_t(left));
+        minus += __popc(e.peek() & mask);
+        if (left > 0) e.rd += S;
+        left = max(left - 32, 0);
+      }
+    }
+    out[1] += moving - minus;
+    out[2] += minus;
+  } else {
+    uint32_t A = W[Q + 1] & mask, B = W[Q + 2] & mask;
+    uint32_t ny = __popc(A), nmy = __popc(A & B), nmx = __popc(B & ~A);
+    while (__any_sync(kFullWarp, left > 0)) {
+      e.ensure(k, a.rk, ask(left));
+      for (int u = 0; u < kPass && __any_sync(kFullWarp, left > 0); ++u) {
+        mask = __funnelshift_lc(kFullWarp, 0u, uint32_t(left));
+        A = e.peek() & mask;
+        B = e.peek(1) & mask;
+        ny += __popc(A);
+        nmy += __popc(A & B);
+        nmx += __popc(B & ~A);
+        if (left > 0) e.rd += 2 * S;
+        left = max(left - 32, 0);
+      }
+    }
+    out[1] += moving - ny - nmx;
+    out[2] += nmx;
+    out[3] += ny - nmy;
+    out[4] += nmy;
+  }
+}
+
+}  // namespace ilg

@@ -3,116 +3,195 @@
 // projections of the observables, and a Philox probe.
 #include <cuda_runtime.h>
 
-#include <type_traits>
+#include <algorithm>
 
+#include "ilg_collide.cuh"
 #include "ilg_device.cuh"
 #include "ilg_launch.h"
 
 namespace ilg {
 
 // --------------------------------------------------------------------------
-// step: one thread per node, any extent.  Loads the Q occupations of its node,
-// flips, collides and scatters n'_i to the neighbour x + v_i (periodic).
-// The lattice's two alias tables (packed one word per column, or as {threshold,
-// alias} pairs) are staged in shared memory once per block, beside 20 extension
-// words per thread for the general collision.  A block returns without work when an
-// earlier launch recorded an overflow.
+// steps, node-parallel: any extent, any occupations.  Each lane loads the Q occupations
+// of its node, flips, collides with its warp (collide_warp) and scatters n'_i to the neighbour
+// x + v_i (periodic).  One launch takes T steps: the alias tables are staged in shared
+// memory once, and a barrier of all blocks (a cooperative launch) separates the steps,
+// instead of a launch, a staging pass and an idle tail per step.
+// Bound: integer issue (72 % of it, ~720 warp instructions per 32 nodes at 50 per
+// velocity and omega* = 0.5) on large lattices; the barrier and the latency of one node
+// (about 2 us a step) on small ones.  One block of 1024 threads per SM holds the tables
+// once, in the 64-bit form whose draw takes two instructions fewer than the packed one
+// (29.1 against 31.0 us per step for two blocks of 512, 33 with packed tables).  Us per
+// step against one launch per step with a collision that loops per lane: 1024^2 at 50 per
+// velocity 28.6 / 37.3 (omega* 0.5), 19.8 / 26.8 (0.1); 1501 x 777 at 100 per velocity
+// 55 / 66; 1024^2 at 200 per velocity, omega* = 1, 93 / 241; 96 x 40 2.2 / 18.7.
 // --------------------------------------------------------------------------
-constexpr int kStepThreads = 256;
-constexpr int kStepBlocksPerSm = 4;
-// packed tables (32 KB, one word per column) leave room for four blocks per SM; the
-// pair form (64 KB) saves two instructions per draw
-constexpr bool kStepPairTables = false;
-using StepTab = std::conditional_t<kStepPairTables, Alias8, Alias4>;
-constexpr uint32_t kStepTableWords = kStepPairTables ? kDevStagedWords : kDevTableWords4;
+constexpr uint32_t kStepRing = 16;  // extension words per lane
 
-template <int Q>
-__global__ void __launch_bounds__(kStepThreads, kStepBlocksPerSm) step_kernel(StepArgs a, const uint16_t* __restrict__ in,
-                                                      uint16_t* __restrict__ out, uint32_t t,
-                                                      unsigned long long* __restrict__ fail) {
+// Barrier of all blocks of a cooperative launch: word = arrivals (low half) and, once a
+// step overflowed, a mark (high half).  Returns the word, or ~0 when the wait gave up
+// (bounded: the kernel then returns and the host reports it).
+constexpr unsigned long long kRunMark = 1ull << 32;
+constexpr uint32_t kRunPolls = 1u << 23;  // seconds; a step's blocks differ by far less
+
+__device__ __forceinline__ unsigned long long run_barrier(unsigned long long* word, uint32_t target) {
+  __threadfence();
+  atomicAdd(word, 1ull);
+  unsigned long long v = 0;
+  for (uint32_t k = 0; k < kRunPolls; ++k) {
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(word) : "memory");
+    if (uint32_t(v) >= target) return v;
+  }
+  return ~0ull;
+}
+
+// sync[0]: the barrier word, sync[1]: set to 1 when a wait gave up
+template <int Q, int THREADS, int MINB>
+__global__ void __launch_bounds__(THREADS, MINB)
+    step_run_kernel(const __grid_constant__ StepArgs a, uint16_t* buf0, uint16_t* buf1, uint32_t t0, uint32_t T,
+                    unsigned long long* fail, unsigned long long* sync) {
   extern __shared__ uint4 smem4[];
-  __shared__ int skip;
+  __shared__ int stop;
   uint32_t* s = reinterpret_cast<uint32_t*>(smem4);
-  uint32_t* xb = s + kStepTableWords + threadIdx.x;  // this thread's extension words
-  if (threadIdx.x == 0) skip = (*reinterpret_cast<volatile unsigned long long*>(fail) != ~0ull);
-  if constexpr (kStepPairTables) {
-    // the block's first words: the pair tables, or the particle sampler's boundaries
+  if (threadIdx.x == 0) stop = (*reinterpret_cast<volatile unsigned long long*>(fail) != ~0ull);
+  {
+    // the block's first words: the two alias tables, or the particle sampler's boundaries
     const uint4* g4 = reinterpret_cast<const uint4*>(a.tables);
-    for (uint32_t i = threadIdx.x; i < kDevStagedWords / 4; i += blockDim.x) smem4[i] = g4[i];
-  } else {
-    stage_tables4(a.tables, s, a.particle != 0);
+#pragma unroll 8
+    for (uint32_t i = threadIdx.x; i < kDevStagedWords / 4; i += THREADS) smem4[i] = g4[i];
   }
   __syncthreads();
-  if (skip) return;
+  if (stop) return;
+  unsigned char* const ring = reinterpret_cast<unsigned char*>(smem4) + 4 * kDevStagedWords;
+  const Alias8 to = Alias8::of(s, 0), tr = Alias8::of(s, 1);
 
   const uint32_t nodes = a.Lx * a.Ly;
   const size_t plane = nodes;
-  bool bad = false;
-  // (x, y) of the node, advanced by the grid stride (stride_y rows and stride_x
-  // nodes) with a carry instead of a division per node
-  const uint32_t stride = gridDim.x * blockDim.x;
+  const uint32_t stride = gridDim.x * THREADS;
   const uint32_t stride_y = stride / a.Lx, stride_x = stride - stride_y * a.Lx;
-  uint32_t node = blockIdx.x * blockDim.x + threadIdx.x;
-  uint32_t y = node / a.Lx, x = node - y * a.Lx;
-  const StepKeys<2> keys = step_keys<2>(a, t);  // the launch-wide Philox rounds of the slot blocks
-  for (; node < nodes; node += stride) {
-    uint32_t n[Q], m[Q], post[Q];
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t base0 = blockIdx.x * THREADS + (threadIdx.x - lane);  // the warp's first node
+  const uint32_t y0 = (base0 + lane) / a.Lx, x0 = base0 + lane - y0 * a.Lx;
+  for (uint32_t step = 0;; ++step) {
+    const uint32_t t = t0 + step;
+    const uint16_t* const in = (step & 1) ? buf1 : buf0;
+    uint16_t* const out = (step & 1) ? buf0 : buf1;
+    bool bad = false;
+    // (x, y) of the lane's node, advanced by the grid stride (stride_y rows and stride_x
+    // nodes) with a carry instead of a division per node
+    uint32_t base = base0, x = x0, y = y0;
+    const WordKeys keys = word_keys(a, t);  // the launch-wide Philox rounds
+    while (base < nodes) {
+      const uint32_t node = base + lane;
+      const bool active = node < nodes && node >= base;
+      uint32_t m[Q], post[Q];
+      // (through L2 only: another SM wrote these lines in the step before)
 #pragma unroll
-    for (int i = 0; i < Q; ++i) n[i] = in[i * plane + node];
-    if constexpr (Q == 3) {
-      m[0] = n[0];
-      m[1] = a.flip ? n[2] : n[1];
-      m[2] = a.flip ? n[1] : n[2];
-    } else {
-      m[0] = n[0];
-      m[1] = a.flip ? n[2] : n[1];
-      m[2] = a.flip ? n[1] : n[2];
-      m[3] = a.flip ? n[4] : n[3];
-      m[4] = a.flip ? n[3] : n[4];
-    }
-    if (a.general || !collide_try_fast<Q, StepTab>(a, s, node, t, m, post, &keys)) {
-      collide_general<Q, kExtWords, kStepThreads, StepTab, true>(a, s, node, t, m, post, xb, &keys);
+      for (int i = 0; i < Q; ++i) m[i] = active ? __ldcg(in + (i * plane + node)) : 0u;
+      if (a.flip) {
+        uint32_t v = m[1];
+        m[1] = m[2];
+        m[2] = v;
+        if constexpr (Q == 5) {
+          v = m[3];
+          m[3] = m[4];
+          m[4] = v;
+        }
+      }
+      if (a.particle) collide_particle<Q>(a, s, node, t, m, post);
+      else collide_warp<Q, 4 * THREADS, kStepRing>(a, keys, to, tr, ring, 4 * threadIdx.x, node, m, post);
+      if (active) {
+        uint32_t high = 0;
 #pragma unroll
-      for (int i = 0; i < Q; ++i) bad |= post[i] > 65535u;
+        for (int i = 0; i < Q; ++i) high |= post[i];
+        bad |= high > 65535u;
+        uint16_t* const o = out + node;  // row y starts at node - x
+        o[0] = uint16_t(post[0]);
+        (o + plane)[x + 1 == a.Lx ? -int64_t(x) : 1] = uint16_t(post[1]);
+        (o + 2 * plane)[x == 0 ? int64_t(a.Lx) - 1 : -1] = uint16_t(post[2]);
+        if constexpr (Q == 5) {
+          const uint32_t yp = y + 1 == a.Ly ? 0 : y + 1;
+          const uint32_t ym = y == 0 ? a.Ly - 1 : y - 1;
+          out[3 * plane + size_t(yp) * a.Lx + x] = uint16_t(post[3]);
+          out[4 * plane + size_t(ym) * a.Lx + x] = uint16_t(post[4]);
+        }
+      }
+      x += stride_x;
+      y += stride_y;
+      if (x >= a.Lx) {
+        x -= a.Lx;
+        y += 1;
+      }
+      if (nodes - base <= stride) break;  // (base + stride may pass 2^32)
+      base += stride;
     }
-    const uint32_t xp = x + 1 == a.Lx ? 0 : x + 1;
-    const uint32_t xm = x == 0 ? a.Lx - 1 : x - 1;
-    const size_t row = size_t(y) * a.Lx;
-    out[node] = uint16_t(post[0]);
-    out[plane + row + xp] = uint16_t(post[1]);
-    out[2 * plane + row + xm] = uint16_t(post[2]);
-    if constexpr (Q == 5) {
-      const uint32_t yp = y + 1 == a.Ly ? 0 : y + 1;
-      const uint32_t ym = y == 0 ? a.Ly - 1 : y - 1;
-      out[3 * plane + size_t(yp) * a.Lx + x] = uint16_t(post[3]);
-      out[4 * plane + size_t(ym) * a.Lx + x] = uint16_t(post[4]);
+    if (bad) {
+      atomicMin(fail, static_cast<unsigned long long>(t));
+      __threadfence();
+      atomicOr(sync, kRunMark);
     }
-    x += stride_x;
-    y += stride_y;
-    if (x >= a.Lx) {
-      x -= a.Lx;
-      y += 1;
+    if (step + 1 == T) break;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      const unsigned long long v = run_barrier(sync, (step + 1) * gridDim.x);
+      if (v == ~0ull) {
+        atomicExch(sync + 1, 1ull);
+        stop = 1;
+      } else if (v >= kRunMark) {
+        // a step overflowed: this one, or already the next one (a faster block's)
+        stop = *reinterpret_cast<volatile unsigned long long*>(fail) <= t;
+      }
     }
+    __syncthreads();
+    if (stop) break;
   }
-  if (bad) atomicMin(fail, static_cast<unsigned long long>(t));
 }
 
-constexpr size_t kStepSmem = sizeof(uint32_t) * (kStepTableWords + kExtWords * kStepThreads);
+constexpr size_t run_smem(int threads) { return sizeof(uint32_t) * (kDevStagedWords + size_t(kStepRing) * threads); }
+
+// Shapes: one block per SM of as few threads (128, 512, 1024) as give every node a lane of
+// its own; 1024 beyond that.
+struct RunShape {
+  const void* fn;
+  int threads;
+};
+
+template <int THREADS>
+static const void* run_fn(int Q) {
+  return Q == 3 ? reinterpret_cast<const void*>(step_run_kernel<3, THREADS, 1>)
+                : reinterpret_cast<const void*>(step_run_kernel<5, THREADS, 1>);
+}
+
+static RunShape run_shape(int Q, uint64_t nodes, uint32_t sms) {
+  if (nodes <= uint64_t(sms) * 128) return {run_fn<128>(Q), 128};
+  if (nodes <= uint64_t(sms) * 512) return {run_fn<512>(Q), 512};
+  return {run_fn<1024>(Q), 1024};
+}
 
 cudaError_t prepare_step_kernels() {
-  cudaError_t e = cudaFuncSetAttribute(step_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kStepSmem));
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(step_kernel<5>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kStepSmem));
+  cudaError_t e = cudaSuccess;
+  auto set = [&](const void* f, int threads) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(run_smem(threads)));
+  };
+  for (int Q : {3, 5}) {
+    set(run_fn<128>(Q), 128);
+    set(run_fn<512>(Q), 512);
+    set(run_fn<1024>(Q), 1024);
+  }
+  return e;
 }
 
-uint32_t step_kernel_threads() { return kStepThreads; }
-uint32_t step_kernel_blocks_per_sm() { return kStepBlocksPerSm; }
-
-cudaError_t launch_step(int Q, const StepArgs& a, const uint16_t* in, uint16_t* out, uint32_t t,
-                        unsigned long long* fail, int grid, cudaStream_t s) {
-  if (Q == 3) step_kernel<3><<<grid, kStepThreads, kStepSmem, s>>>(a, in, out, t, fail);
-  else step_kernel<5><<<grid, kStepThreads, kStepSmem, s>>>(a, in, out, t, fail);
-  return cudaGetLastError();
+cudaError_t launch_step_run(int Q, const StepArgs& a, uint16_t* buf0, uint16_t* buf1, uint32_t t, uint32_t T,
+                            unsigned long long* fail, unsigned long long* sync, uint32_t sms, cudaStream_t s) {
+  const uint64_t nodes = uint64_t(a.Lx) * a.Ly;
+  const RunShape r = run_shape(Q, nodes, sms);
+  const dim3 grid(uint32_t(std::min<uint64_t>((nodes + r.threads - 1) / r.threads, sms)));
+  StepArgs args = a;
+  void* p[] = {&args, &buf0, &buf1, &t, &T, &fail, &sync};
+  if (T == 1) return cudaLaunchKernel(r.fn, grid, dim3(r.threads), p, run_smem(r.threads), s);
+  const cudaError_t e = cudaMemsetAsync(sync, 0, sizeof(unsigned long long), s);
+  if (e != cudaSuccess) return e;
+  return cudaLaunchCooperativeKernel(r.fn, grid, dim3(r.threads), p, run_smem(r.threads), s);
 }
 
 // --------------------------------------------------------------------------

@@ -23,10 +23,11 @@ struct InitArgs {
 };
 
 cudaError_t prepare_step_kernels();  // opt in to the table block's shared memory
-uint32_t step_kernel_threads();       // block shape of the node-parallel step
-uint32_t step_kernel_blocks_per_sm();
-cudaError_t launch_step(int Q, const StepArgs& a, const uint16_t* in, uint16_t* out, uint32_t t,
-                        unsigned long long* fail, int grid, cudaStream_t s);
+// T node-parallel steps from step t in one launch (buf0 holds the state; the steps
+// alternate the buffers).  sync: two words, zeroed sync[1] on entry; sync[1] becomes 1 if
+// a wait between blocks gave up
+cudaError_t launch_step_run(int Q, const StepArgs& a, uint16_t* buf0, uint16_t* buf1, uint32_t t, uint32_t T,
+                            unsigned long long* fail, unsigned long long* sync, uint32_t sms, cudaStream_t s);
 cudaError_t prepare_step_vec_kernels();
 uint32_t step_vec_width();  // nodes per thread of the default row-tiled step (rows must be a multiple)
 uint32_t step_vec_blocks_per_sm(int npt);
