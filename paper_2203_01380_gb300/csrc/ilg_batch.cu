@@ -7,7 +7,10 @@
 // block ran it or on the other replicas of the batch.
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "ilg_batch.h"
+#include "ilg_collide.cuh"
 #include "ilg_device.cuh"
 
 namespace ilg {
@@ -51,18 +54,10 @@ __device__ double block_dot2(double s, double c, double* red) {
   return r;  // valid in thread 0
 }
 
-// Exact 128-bit integer accumulator of products of int64 values.
+// A 128-bit integer as the record holds it.
 struct I128 {
   unsigned long long lo = 0;
   long long hi = 0;
-  __device__ __forceinline__ void add(unsigned long long l, long long h) {
-    const unsigned long long n = lo + l;
-    hi += h + (n < lo ? 1 : 0);
-    lo = n;
-  }
-  __device__ __forceinline__ void add_product(long long a, long long b) {
-    add((unsigned long long)(a * b), __mul64hi(a, b));
-  }
 };
 
 // v * 2^-62 rounded once to double (round to nearest even).
@@ -95,235 +90,356 @@ __device__ __forceinline__ longlong2 trig_fixed(uint32_t r, uint32_t L) {
   return make_longlong2(__double2ll_rn(ldexp(cs, 62)), __double2ll_rn(ldexp(sn, 62)));
 }
 
-// Complex amplitude of axis mode m of a ring held in shared memory (buf, planes
-// Lmax apart): with D(x) = L N(x) - M and r = (m x) mod L,
+// Complex amplitude of axis mode m of a ring: with D(x) = L N(x) - M and r = (m x) mod L,
 //   re = sum_x cos(2 pi r / L) D(x) / L,  im = sum_x sin(2 pi r / L) D(x) / L.
-// The trigonometric values enter as 2^-62 fixed-point integers (from trig, indexed
-// by x, when given) and the sums are exact in 128-bit integers, so they do not
-// depend on the summation order.  ring_partials: every warp reduces its nodes and
-// its lane 0 stores (re.lo, re.hi, im.lo, im.hi) at red[4 warp ..]; no barrier.
-template <int THREADS>
-__device__ void ring_partials(const uint16_t* buf, uint32_t L, uint32_t Lmax, uint64_t mass, uint32_t m,
-                              const longlong2* trig, unsigned long long* red) {
-  I128 ac, as;
-  for (uint32_t x = threadIdx.x; x < L; x += THREADS) {
-    const long long N = (long long)buf[x] + buf[Lmax + x] + buf[2 * Lmax + x];
-    const long long D = (long long)L * N - (long long)mass;
-    const longlong2 cs = trig ? trig[x] : trig_fixed(uint32_t((uint64_t(m) * x) % L), L);
-    ac.add_product(cs.x, D);
-    as.add_product(cs.y, D);
+// The trigonometric values enter as 2^-62 fixed-point integers and the sums are exact, so
+// they do not depend on the summation order.  A step adds only
+//   sum_x c(x) N(x),  c = c1 2^32 + c0:  N c0 < 2^50 and |N c1| < 2^48 per node, below 2^63
+// over a ring (four wide multiply-adds per node, against two 64 x 64 -> 128 products);
+// the factor L and the M sum_x c(x) term, the same for every step, join when a state's
+// sums are written out (write_sums).
+struct ModeSums {
+  long long v[4];  // cos low, cos high, sin low, sin high
+  __device__ __forceinline__ void clear() { v[0] = v[1] = v[2] = v[3] = 0; }
+  __device__ __forceinline__ void add(const longlong2& cs, uint32_t N) {
+    v[0] += (long long)(uint64_t(uint32_t(cs.x)) * N);
+    v[1] += (long long)(int32_t(cs.x >> 32)) * (long long)(int32_t(N));
+    v[2] += (long long)(uint64_t(uint32_t(cs.y)) * N);
+    v[3] += (long long)(int32_t(cs.y >> 32)) * (long long)(int32_t(N));
   }
+  // Sums over the warp: lane 8 k returns the sum of v[k] (k = 0..3).  The first two
+  // exchanges halve the values a lane keeps: 6 exchanges instead of 20.
+  __device__ __forceinline__ long long warp_sum(uint32_t lane) const {
+    const bool hi = (lane & 16) != 0;
+    long long a = hi ? v[2] : v[0], b = hi ? v[3] : v[1];
+    a += __shfl_xor_sync(kFullWarp, hi ? v[0] : v[2], 16);
+    b += __shfl_xor_sync(kFullWarp, hi ? v[1] : v[3], 16);
+    const bool odd = (lane & 8) != 0;
+    long long c = odd ? b : a;
+    c += __shfl_xor_sync(kFullWarp, odd ? a : b, 8);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long cl = __shfl_down_sync(0xFFFFFFFFu, ac.lo, o);
-    const long long ch = __shfl_down_sync(0xFFFFFFFFu, ac.hi, o);
-    const unsigned long long sl = __shfl_down_sync(0xFFFFFFFFu, as.lo, o);
-    const long long sh = __shfl_down_sync(0xFFFFFFFFu, as.hi, o);
-    ac.add(cl, ch);
-    as.add(sl, sh);
+    for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(kFullWarp, c, o);
+    return c;
   }
-  if ((threadIdx.x & 31) == 0) {
-    const int w = threadIdx.x >> 5;
-    red[4 * w + 0] = ac.lo;
-    red[4 * w + 1] = (unsigned long long)ac.hi;
-    red[4 * w + 2] = as.lo;
-    red[4 * w + 3] = (unsigned long long)as.hi;
+};
+
+// One thread: out[0..3] = the 128-bit sums (L 2^62 re, L 2^62 im) of a state as (lo, hi)
+// pairs, from the warps' partials red[4 warp + k] and the ring's c[k] = sum_x of the
+// parts of its trigonometric values.
+__device__ void write_sums(const long long* red, uint32_t warps, const long long* c, uint32_t L, uint64_t mass,
+                           long long* out) {
+  long long v[4] = {0, 0, 0, 0};
+  for (uint32_t w = 0; w < warps; ++w)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] += red[4 * w + k];
+#pragma unroll
+  for (int k = 0; k < 4; k += 2) {
+    const __int128 S = (__int128(v[k + 1]) << 32) + v[k];
+    const __int128 C = (__int128(c[k + 1]) << 32) + c[k];
+    const __int128 r = S * __int128(L) - C * __int128((long long)mass);
+    out[k] = (long long)(unsigned long long)r;
+    out[k + 1] = (long long)(r >> 64);
   }
 }
 
-// Sum of the warps' partials (one thread): the raw 128-bit sums of re and im
-// (times L 2^62) go to out[0..3].
-template <int THREADS>
-__device__ void ring_finalise(const unsigned long long* red, long long* out) {
-  I128 c, s;
-  for (int w = 0; w < THREADS / 32; ++w) {
-    c.add(red[4 * w + 0], (long long)red[4 * w + 1]);
-    s.add(red[4 * w + 2], (long long)red[4 * w + 3]);
-  }
-  out[0] = (long long)c.lo;
-  out[1] = c.hi;
-  out[2] = (long long)s.lo;
-  out[3] = s.hi;
+// What the slot and extension blocks of one step share (StepKeys, WordKeys) without the
+// words that depend on the ring alone, as two 16-byte shared loads.
+struct __align__(16) BatchStepKeys {
+  uint32_t G, H0, I0, J0, H1, I1, J1, ext_c;
+};
+
+// Lane j of a warp: the launch-wide words of step s0 + j (s0 a multiple of 32) of a ring
+// whose step counter is t0.
+__device__ __forceinline__ void make_step_keys(const StepArgs& a, uint32_t t0, uint32_t s0, BatchStepKeys (&keys)[2][32]) {
+  const uint32_t j = threadIdx.x & 31u;
+  const WordKeys k = word_keys(a, t0 + s0 + j);
+  keys[(s0 >> 5) & 1][j] = BatchStepKeys{k.slot.G,    k.slot.H[0], k.slot.I[0], k.slot.J[0],
+                                         k.slot.H[1], k.slot.I[1], k.slot.J[1], k.ext_c};
 }
 
+// Rings of a block: shared memory, the block's threads and how its words are kept.  Bound:
+// integer issue for long rings (see collide_warp), the latency of a step (its node's
+// Philox rounds, two dependent table draws and a barrier) for short ones.  A block holds
+// the alias tables in 64-bit form where one block per SM is resident (1024 threads; a
+// draw takes two instructions fewer), packed where several share an SM.  Measured
+// against per-lane loops and one 128-bit projection per node and step: 2048 rings of 64 to
+// 8192 nodes x 2000 steps 205 ms / 249 ms; 512 rings of 320 nodes x 2000 steps with
+// statistics 7.9 / 10.6 ms; one ring of 256 nodes with its records 1.45 / 2.0 us per step.
 template <int THREADS>
-__global__ void __launch_bounds__(THREADS, 1024 / THREADS) batch_d1q3_kernel(BatchArgs b, StepArgs common) {
+struct BatchShape {
+  static constexpr int kPerSm = 1024 / THREADS;
+  static constexpr bool kPairs = THREADS == 1024;
+  static constexpr uint32_t kTableWords = kPairs ? kDevStagedWords : kDevTableWords4;
+  static constexpr uint32_t kRing = kBatchExtWords;
+  // states whose partial sums are written out together: by one warp each, every kGroup
+  // steps, so that no step waits for one thread to add them up
+  static constexpr uint32_t kGroup = THREADS == 1024 ? 2 : (THREADS == 512 ? 4 : 8);
+};
+
+// The shared memory of a batch block beside its dynamic part.
+template <int THREADS>
+struct BatchShared {
+  static constexpr uint32_t kSlots = 2 * BatchShape<THREADS>::kGroup;
+  uint32_t task;
+  uint32_t fail;  // first step that would overflow
+  unsigned long long mass;
+  long long c[4];                                // sums of the mode's trigonometric values
+  long long red[kSlots][4 * (THREADS / 32)];     // partial sums of the last states
+  BatchStepKeys keys[2][32];                     // of 64 steps
+};
+
+// All steps of one ring that lies in src (3 planes of L; dst: the other buffer), by the
+// first `warps` warps of the block.  REC: the mode's sums at every state; STATES: every
+// state to b.states; TABLES: see collide_warp (and the binomial sampler).  Returns the
+// steps done; src is the buffer that holds the state.
+template <int THREADS, bool REC, bool STATES, bool TABLES, class Tab>
+__device__ __forceinline__ uint32_t run_ring(const BatchArgs& b, const StepArgs& a, const ReplicaDesc& d, uint32_t r,
+                                             const uint32_t* tables, const Tab& to, const Tab& tr, unsigned char* words,
+                                             BatchShared<THREADS>& sh, uint16_t*& src, uint16_t* dst, uint32_t warps) {
+  constexpr uint32_t S = 4 * THREADS;
+  constexpr uint32_t kGroup = BatchShape<THREADS>::kGroup, kSlots = BatchShared<THREADS>::kSlots;
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, threads = blockDim.x;
+  const uint32_t L = d.L, T = b.T;
+  const uint64_t mass = sh.mass;
+  // no occupation can pass 65535 while the whole ring holds no more than that
+  const bool safe = mass <= 65535ull;
+  const longlong2* trig = REC ? b.trig + d.state_off / 3 : nullptr;  // this ring's values
+  const auto bar = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(warps * 32) : "memory"); };
+  // the flip F_i(n) = n_{-i}: velocity i of the collision reads plane -i
+  const uint32_t p1 = d.flip ? 2 * L : L, p2 = d.flip ? L : 2 * L;
+  WordKeys k;
+  k.slot.A = uint32_t((uint64_t(0xCD9E8D57u) * a.replica) >> 32) ^ a.rk[0];
+  k.ext_e = uint32_t(uint64_t(0xCD9E8D57u) * a.replica) ^ a.rk[2];
+  uint32_t s = 0;
+  for (;; ++s) {
+    if (!REC && !STATES && s == T) break;
+    {
+      const uint4* q = reinterpret_cast<const uint4*>(&sh.keys[(s >> 5) & 1][s & 31]);
+      const uint4 k0 = q[0], k1 = q[1];
+      k.slot.G = k0.x;
+      k.slot.H[0] = k0.y;
+      k.slot.I[0] = k0.z;
+      k.slot.J[0] = k0.w;
+      k.slot.H[1] = k1.x;
+      k.slot.I[1] = k1.y;
+      k.slot.J[1] = k1.z;
+      k.ext_c = k1.w;
+    }
+    bool bad = false;
+    ModeSums ms;
+    if constexpr (REC) ms.clear();
+    for (uint32_t x0 = warp * 32; x0 < L; x0 += threads) {
+      const uint32_t x = x0 + lane;
+      const bool active = x < L;
+      uint32_t m[3], post[3];
+      m[0] = active ? src[x] : 0u;
+      m[1] = active ? src[p1 + x] : 0u;
+      m[2] = active ? src[p2 + x] : 0u;
+      if constexpr (REC) {
+        if (active) ms.add(trig[x], m[0] + m[1] + m[2]);
+      }
+      if constexpr (STATES) {
+        if (s > 0 && active) {
+          // the state after step s - 1, planes rest, +1, -1
+          uint16_t* rs = b.states + d.state_off * T + size_t(s - 1) * 3 * L + x;
+          rs[0] = uint16_t(m[0]);
+          rs[p1] = uint16_t(m[1]);
+          rs[p2] = uint16_t(m[2]);
+        }
+      }
+      if ((REC || STATES) && s == T) continue;
+      if (!TABLES && a.particle) collide_particle<3>(a, tables, x, d.t + s, m, post);
+      else collide_warp<3, S, BatchShape<THREADS>::kRing, TABLES>(a, k, to, tr, words, 4 * tid, x, m, post);
+      if (active) {
+        bad |= (post[0] | post[1] | post[2]) > 65535u;
+        dst[x] = uint16_t(post[0]);
+        dst[L + (x + 1 == L ? 0 : x + 1)] = uint16_t(post[1]);
+        dst[2 * L + (x == 0 ? L - 1 : x - 1)] = uint16_t(post[2]);
+      }
+    }
+    if constexpr (REC) {
+      // the partial sums of state s; kGroup states at a time are written out, one per
+      // warp, after the barrier that follows the last of them
+      const long long v = ms.warp_sum(lane);
+      if ((lane & 7) == 0) sh.red[s % kSlots][4 * warp + (lane >> 3)] = v;
+    }
+    if ((REC || STATES) && s == T) break;
+    if (bad) atomicMin(&sh.fail, s);
+    bar();
+    // (a faster warp may already have marked the next step)
+    if (!safe && *reinterpret_cast<volatile uint32_t*>(&sh.fail) <= s) break;  // src still holds the state
+    // the steps' launch-wide Philox words, over those of the 32 steps just done
+    if (warp == 0 && (s & 31) == 31) make_step_keys(a, d.t, s + 33, sh.keys);
+    uint16_t* tmp = src;
+    src = dst;
+    dst = tmp;
+    if (REC && (s % kGroup) == kGroup - 1) {
+      for (uint32_t g = warp; g < kGroup; g += warps)
+        if (lane == 0) {
+          const uint32_t st = s - (kGroup - 1) + g;
+          write_sums(sh.red[st % kSlots], warps, sh.c, L, mass, b.record + (size_t(r) * (T + 1) + st) * 4);
+        }
+    }
+  }
+  bar();
+  if constexpr (REC) {
+    // the states since the last group (s: the last state whose sums exist)
+    for (uint32_t st = s / kGroup * kGroup + warp; st <= s; st += warps)
+      if (lane == 0)
+        write_sums(sh.red[st % kSlots], warps, sh.c, L, mass, b.record + (size_t(r) * (T + 1) + st) * 4);
+  }
+  return s;
+}
+
+template <int THREADS, bool REC, bool STATES>
+__global__ void __launch_bounds__(THREADS, BatchShape<THREADS>::kPerSm)
+    batch_d1q3_kernel(const __grid_constant__ BatchArgs b, const __grid_constant__ StepArgs common) {
+  using Shape = BatchShape<THREADS>;
+  using Tab = std::conditional_t<Shape::kPairs, Alias8, Alias4>;
   extern __shared__ uint4 smem4[];
-  uint32_t* tables = reinterpret_cast<uint32_t*>(smem4);                     // kBatchTableWords words
-  uint32_t* xbuf = tables + kBatchTableWords;                                 // kBatchExtWords x THREADS
-  uint16_t* ring = reinterpret_cast<uint16_t*>(xbuf + kBatchExtWords * THREADS);  // 2 x 3 x Lmax
-  __shared__ uint32_t s_task;
-  __shared__ int s_fail;
-  __shared__ unsigned long long s_mass;
-  __shared__ unsigned long long s_red[2][4 * (THREADS / 32)];   // projection partials, by state parity
-  const int tid = threadIdx.x;
+  uint32_t* tables = reinterpret_cast<uint32_t*>(smem4);
+  unsigned char* const words = reinterpret_cast<unsigned char*>(tables + Shape::kTableWords);
+  uint16_t* ring = reinterpret_cast<uint16_t*>(words + Shape::kRing * 4 * THREADS);  // 2 x 3 x Lmax
+  __shared__ BatchShared<THREADS> sh;
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+  const uint32_t threads = blockDim.x;
 
   for (;;) {
     if (tid == 0) {
-      s_task = atomicAdd(b.counter, 1u);
-      s_fail = -1;
-      s_mass = 0ull;
+      sh.task = atomicAdd(b.counter, 1u);
+      sh.fail = ~0u;
+      sh.mass = 0ull;
+      sh.c[0] = sh.c[1] = sh.c[2] = sh.c[3] = 0;
     }
     __syncthreads();
-    const uint32_t task = s_task;
+    const uint32_t task = sh.task;
     if (task >= b.n) break;
     const uint32_t r = b.order[task];
     const ReplicaDesc d = b.desc[r];
     const uint32_t L = d.L;
     StepArgs a = common;
-    a.Lx = L;
-    a.Ly = 1;
-    a.flip = d.flip;
     a.omega_mode = d.omega_mode;
     a.rest_mode = d.rest_mode;
     a.replica = d.replica;
-    a.general = d.general;
     a.particle = d.particle;
 
-    // tables (the two alias tables packed one word per column; the particle
-    // sampler's boundaries as they are) and ring into shared memory
-    stage_tables4(b.tables + size_t(r) * kDevBlockWords, tables, a.particle != 0);
-    const uint16_t* gs = b.state + d.state_off;
-    uint16_t* buf0 = ring;
-    uint16_t* buf1 = ring + 3 * b.Lmax;
-    for (uint32_t i = tid; i < 3 * L; i += THREADS) buf0[(i / L) * b.Lmax + (i % L)] = gs[i];
+    // tables (the particle sampler's boundaries as they are) and ring into shared memory
+    if constexpr (Shape::kPairs) {
+      const uint4* g4 = reinterpret_cast<const uint4*>(b.tables + size_t(r) * kDevBlockWords);
+#pragma unroll 8
+      for (uint32_t i = tid; i < kDevStagedWords / 4; i += threads) smem4[i] = g4[i];
+    } else {
+      stage_tables4(b.tables + size_t(r) * kDevBlockWords, tables, a.particle != 0);
+    }
+    const Tab to = Tab::of(tables, 0), tr = Tab::of(tables, 1);
+    uint16_t* const gs = b.state + d.state_off;
+    unsigned long long part = 0;
+    for (uint32_t i = tid; i < 3 * L; i += threads) {
+      ring[i] = gs[i];
+      part += gs[i];
+    }
+    // the ring's mass, and the sums of the recorded mode's trigonometric values
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(kFullWarp, part, o);
+    if (lane == 0 && part) atomicAdd(&sh.mass, part);
+    if constexpr (REC) {
+      const longlong2* trig = b.trig + d.state_off / 3;
+      ModeSums ms;
+      ms.clear();
+      for (uint32_t x0 = warp * 32; x0 < L; x0 += threads)
+        if (x0 + lane < L) ms.add(trig[x0 + lane], 1u);
+      const long long v = ms.warp_sum(lane);
+      if ((lane & 7) == 0) atomicAdd(reinterpret_cast<unsigned long long*>(&sh.c[lane >> 3]), (unsigned long long)v);
+    }
+    if (warp == 0) {
+      make_step_keys(a, d.t, 0, sh.keys);
+      make_step_keys(a, d.t, 32, sh.keys);
+    }
     __syncthreads();
-
-    // mass and mode phases for the amplitude record (integers, exact)
-    uint64_t mass = 0;
-    const bool rec = b.record != nullptr;
-    const uint32_t mrec = rec ? uint32_t(((int64_t(b.record_mode) % int64_t(L)) + L) % L) : 0u;
-    const longlong2* trig = b.trig ? b.trig + d.state_off / 3 : nullptr;  // this ring's values
-    if (rec) {
-      unsigned long long part = 0;
-      for (uint32_t x = tid; x < L; x += THREADS)
-        part += (unsigned long long)buf0[x] + buf0[b.Lmax + x] + buf0[2 * b.Lmax + x];
-      if (part) atomicAdd(&s_mass, part);
-      __syncthreads();
-      mass = s_mass;
-      // partials of state 0 into slot 0 (finalised after the first step's barrier)
-      ring_partials<THREADS>(buf0, L, b.Lmax, mass, mrec, trig, s_red[0]);
-    }
-
-    uint16_t* src = buf0;
-    uint16_t* dst = buf1;
-    uint32_t steps_done = 0;
-    for (uint32_t s = 0; s < b.T; ++s) {
-      const uint32_t t = d.t + s;
-      bool bad = false;
-      for (uint32_t x = tid; x < L; x += THREADS) {
-        const uint32_t n[3] = {src[x], src[b.Lmax + x], src[2 * b.Lmax + x]};
-        uint32_t m[3], post[3];
-        m[0] = n[0];
-        m[1] = a.flip ? n[2] : n[1];
-        m[2] = a.flip ? n[1] : n[2];
-        if (a.general || !collide_try_fast<3, Alias4>(a, tables, x, t, m, post)) {
-          collide_general<3, kBatchExtWords, THREADS, Alias4>(a, tables, x, t, m, post, xbuf + tid);
-          bad |= post[0] > 65535u || post[1] > 65535u || post[2] > 65535u;
-        }
-        const uint32_t xp = x + 1 == L ? 0 : x + 1;
-        const uint32_t xm = x == 0 ? L - 1 : x - 1;
-        dst[x] = uint16_t(post[0]);
-        dst[b.Lmax + xp] = uint16_t(post[1]);
-        dst[2 * b.Lmax + xm] = uint16_t(post[2]);
+    const uint32_t warps = (min(L, threads) + 31) >> 5;  // the others have no node of this ring
+    if (warp < warps) {
+      uint16_t* src = ring;
+      const bool plain = !a.particle && a.omega_mode == kTable && a.rest_mode == kTable;
+      const uint32_t done =
+          plain ? run_ring<THREADS, REC, STATES, true>(b, a, d, r, tables, to, tr, words, sh, src, ring + 3 * L, warps)
+                : run_ring<THREADS, REC, STATES, false>(b, a, d, r, tables, to, tr, words, sh, src, ring + 3 * L, warps);
+      // ring back to global memory; the replica's step counter moves on
+      for (uint32_t i = tid; i < 3 * L; i += warps * 32) gs[i] = src[i];
+      if (tid == 0) {
+        b.desc[r].t = d.t + done;
+        if (sh.fail != ~0u) b.failed[r] = 1u;
       }
-      if (bad) atomicMax(&s_fail, 0);
-      __syncthreads();
-      if (s_fail >= 0) break;  // src still holds the state at step t: keep it
-      uint16_t* tmp = src;
-      src = dst;
-      dst = tmp;
-      steps_done = s + 1;
-      if (b.states) {
-        // the state after this step, planes rest, +1, -1 as the batch buffer holds them
-        uint16_t* rs = b.states + d.state_off * b.T + size_t(s) * 3 * L;
-        for (uint32_t i = tid; i < 3 * L; i += THREADS) {
-          const uint32_t pl = i >= 2 * L ? 2u : (i >= L ? 1u : 0u);
-          rs[i] = src[pl * b.Lmax + (i - pl * L)];
-        }
-      }
-      if (rec) {
-        // state s was reduced into slot s & 1 before this step's barrier: finalise
-        // it; then the warps reduce the new state s + 1 into the other slot
-        if (tid == 0) ring_finalise<THREADS>(s_red[s & 1], b.record + (size_t(r) * (b.T + 1) + s) * 4);
-        ring_partials<THREADS>(src, L, b.Lmax, mass, mrec, trig, s_red[(s + 1) & 1]);
-      }
-    }
-    if (rec && s_fail < 0) {
-      __syncthreads();
-      if (tid == 0) ring_finalise<THREADS>(s_red[b.T & 1], b.record + (size_t(r) * (b.T + 1) + b.T) * 4);
-    }
-    // ring back to global memory; the replica's step counter moves on
-    uint16_t* gd = b.state + d.state_off;
-    for (uint32_t i = tid; i < 3 * L; i += THREADS) gd[i] = src[(i / L) * b.Lmax + (i % L)];
-    if (tid == 0) {
-      b.desc[r].t = d.t + steps_done;
-      if (s_fail >= 0) b.failed[r] = 1u;
     }
     __syncthreads();
   }
 }
 
+// The instantiation for a shape and what it records.
+const void* batch_fn(int threads, bool rec, bool states) {
+  auto pick = [&](auto shape) {
+    constexpr int N = decltype(shape)::value;
+    if (rec) return states ? reinterpret_cast<const void*>(batch_d1q3_kernel<N, true, true>)
+                           : reinterpret_cast<const void*>(batch_d1q3_kernel<N, true, false>);
+    return states ? reinterpret_cast<const void*>(batch_d1q3_kernel<N, false, true>)
+                  : reinterpret_cast<const void*>(batch_d1q3_kernel<N, false, false>);
+  };
+  if (threads == 256) return pick(std::integral_constant<int, 256>{});
+  if (threads == 512) return pick(std::integral_constant<int, 512>{});
+  return pick(std::integral_constant<int, 1024>{});
+}
+
 }  // namespace
 
-// Default shape: batches whose rings all have at most kBatchSmallL nodes run on
-// 256-thread blocks, several per SM; others on 1024-thread blocks, or 512 where the
-// longest ring does not fit beside 1024 threads' buffers.  The autotuner
-// (ilg_batch_autotune) may pick 256, 512 or 1024 threads instead.
-constexpr int kBatchThreads = 1024;
-constexpr int kBatchSmallThreads = 256;
+// Default shape: 256-thread blocks, several per SM, for rings of at most kBatchSmallL nodes
+// where there are more rings than SMs (or the rings need no more threads); else one
+// 1024-thread block per SM.  The autotuner (ilg_batch_autotune) may pick 256, 512 or 1024
+// threads instead.
 constexpr uint32_t kBatchSmallL = 1024;
 
 size_t batch_smem_bytes(uint32_t Lmax, int threads) {
-  return sizeof(uint32_t) * (kBatchTableWords + size_t(kBatchExtWords) * threads) +
-         sizeof(uint16_t) * 2 * 3 * size_t(Lmax);
+  const uint32_t table = threads == 1024 ? BatchShape<1024>::kTableWords : BatchShape<256>::kTableWords;
+  return sizeof(uint32_t) * (table + size_t(kBatchExtWords) * threads) + sizeof(uint16_t) * 2 * 3 * size_t(Lmax);
 }
 
 // largest dynamic shared memory a shape may ask for (the 227 KB a block may opt into,
 // less room for the kernel's static shared memory)
-constexpr size_t kBatchSmemCap = 223 * 1024;
+constexpr size_t kBatchSmemCap = 220 * 1024;
 
 bool batch_shape_fits(uint32_t Lmax, int threads) { return batch_smem_bytes(Lmax, threads) <= kBatchSmemCap; }
 
-uint32_t batch_default_threads(uint32_t Lmax) {
-  if (Lmax <= kBatchSmallL) return kBatchSmallThreads;
-  return batch_shape_fits(Lmax, kBatchThreads) ? kBatchThreads : kBatchThreads / 2;
+uint32_t batch_default_threads(uint32_t Lmax, uint32_t n, uint32_t sms) {
+  return Lmax <= 256 || (Lmax <= kBatchSmallL && n > sms) ? 256 : 1024;
 }
 
-template <int THREADS>
-static cudaError_t batch_attr(uint32_t Lmax) {
-  return cudaFuncSetAttribute(batch_d1q3_kernel<THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              int(batch_smem_bytes(Lmax, THREADS)));
-}
-
+// The same limit for every batch of the process, whatever its rings' length.
 cudaError_t prepare_batch_kernel(uint32_t Lmax, int threads) {
   if (!batch_shape_fits(Lmax, threads)) return cudaErrorInvalidValue;
-  if (threads == 256) return batch_attr<256>(Lmax);
-  if (threads == 512) return batch_attr<512>(Lmax);
-  if (threads == 1024) return batch_attr<1024>(Lmax);
-  return cudaErrorInvalidValue;
+  for (bool rec : {false, true})
+    for (bool states : {false, true}) {
+      const cudaError_t e = cudaFuncSetAttribute(batch_fn(threads, rec, states), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 int(kBatchSmemCap));
+      if (e != cudaSuccess) return e;
+    }
+  return cudaSuccess;
 }
 
 // Persistent grid: as many blocks as fit on every SM (shared memory and registers
-// decide), at most one per ring.
-template <int THREADS>
-static cudaError_t launch_shape(const BatchArgs& b, const StepArgs& common, int sms, cudaStream_t s) {
-  const size_t smem = batch_smem_bytes(b.Lmax, THREADS);
+// decide), at most one per ring.  A block has as many of its shape's threads as the longest
+// ring keeps equally busy (320 nodes on the 256-thread shape: 160 threads, two nodes each).
+cudaError_t launch_batch(const BatchArgs& b, const StepArgs& common, int sms, cudaStream_t s, int shape) {
+  const size_t smem = batch_smem_bytes(b.Lmax, shape);
+  const uint32_t rounds = (b.Lmax + uint32_t(shape) - 1) / uint32_t(shape);
+  const int threads = int(((b.Lmax + rounds - 1) / rounds + 31) / 32 * 32);
+  const void* fn = batch_fn(shape, b.record != nullptr, b.states != nullptr);
   int per_sm = 1;
-  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_d1q3_kernel<THREADS>, THREADS, smem);
+  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) per_sm = 1;
   const uint32_t cap = uint32_t(per_sm) * uint32_t(sms);
-  const int grid = int(b.n < cap ? b.n : cap);
-  batch_d1q3_kernel<THREADS><<<grid, THREADS, smem, s>>>(b, common);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_batch(const BatchArgs& b, const StepArgs& common, int sms, cudaStream_t s, int threads) {
-  if (threads == 0) threads = int(batch_default_threads(b.Lmax));
-  if (threads == 256) return launch_shape<256>(b, common, sms, s);
-  if (threads == 512) return launch_shape<512>(b, common, sms, s);
-  return launch_shape<1024>(b, common, sms, s);
+  BatchArgs ba = b;
+  StepArgs ca = common;
+  void* p[] = {&ba, &ca};
+  return cudaLaunchKernel(fn, dim3(b.n < cap ? b.n : cap), dim3(threads), p, smem, s);
 }
 
 }  // namespace ilg

@@ -11,9 +11,7 @@
 namespace ilg {
 
 constexpr uint32_t kBatchMaxL = 10240;  // longest ring (the ring and its copy live in shared memory)
-constexpr int kBatchExtWords = 16;      // extension words per thread in shared memory
-// the ring's alias tables in shared memory, one word per column (Alias4)
-constexpr uint32_t kBatchTableWords = kDevTableWords4;
+constexpr int kBatchExtWords = 8;       // extension words per thread in shared memory
 
 struct ReplicaDesc {
   uint32_t L;           // ring length
@@ -22,8 +20,8 @@ struct ReplicaDesc {
   uint32_t rest_mode;
   uint32_t replica;     // replica word of the Philox counter
   uint32_t t;           // step counter (advanced by the kernel)
-  uint32_t general;     // 1: skip the fast path (high occupation or particle sampler)
   uint32_t particle;    // 1: particle sampler
+  uint32_t pad;
   uint64_t state_off;   // first of the replica's 3 L occupations in the batch buffer
 };
 
@@ -42,19 +40,18 @@ struct BatchArgs {
                            // (lo, hi) pairs of the recorded mode at the launch's start, then
                            // after every step; or NULL
   const longlong2* trig;   // fixed-point (cos, sin) of the recorded mode, ring r's values at
-                           // x + state_off / 3 (its nodes' place in the batch); or NULL
-                           // (computed per node and step)
+                           // x + state_off / 3 (its nodes' place in the batch); NULL
+                           // without a record
   uint16_t* states;        // state of every ring after every step, or NULL: ring r's
                            // T x 3 L_r occupations at T * state_off, step s at s * 3 L_r
 };
 
 size_t batch_smem_bytes(uint32_t Lmax, int threads);
 bool batch_shape_fits(uint32_t Lmax, int threads);
-// block shapes: 256, 512 or 1024 threads (ceil(L / threads) nodes per thread and step)
-uint32_t batch_default_threads(uint32_t Lmax);
+// block shapes: up to 256, 512 or 1024 threads (ceil(L / threads) nodes per thread and step)
+uint32_t batch_default_threads(uint32_t Lmax, uint32_t n, uint32_t sms);
 cudaError_t prepare_batch_kernel(uint32_t Lmax, int threads);
-// threads 0: the default shape for Lmax
-cudaError_t launch_batch(const BatchArgs& b, const StepArgs& common, int sms, cudaStream_t s, int threads = 0);
+cudaError_t launch_batch(const BatchArgs& b, const StepArgs& common, int sms, cudaStream_t s, int shape);
 cudaError_t launch_batch_obs(const ReplicaDesc* desc, const uint16_t* state, uint32_t n, int32_t mode,
                              unsigned long long* mass, double* amp, cudaStream_t s);
 cudaError_t launch_batch_amp(const ReplicaDesc* desc, const double* record, uint32_t n, uint32_t T, double* amp,

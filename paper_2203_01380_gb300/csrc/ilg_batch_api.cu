@@ -151,7 +151,6 @@ ilg_status ilg_batch_create(const ilg_params* params, uint32_t n, void* stream, 
     d.replica = q.replica;
     d.t = 0;
     d.particle = q.sampler == ILG_SAMPLER_PARTICLE ? 1u : 0u;
-    d.general = general_path(ILG_D1Q3, q.theta, omega_star, q.n0, q.Lx) | d.particle;
     d.state_off = b->total;
     b->total += 3 * size_t(q.Lx);
     b->Lmax = std::max(b->Lmax, q.Lx);
@@ -176,7 +175,7 @@ ilg_status ilg_batch_create(const ilg_params* params, uint32_t n, void* stream, 
       (e = cudaMemsetAsync(b->d_state, 0, sizeof(uint16_t) * b->total, b->stream)) != cudaSuccess ||
       (e = cudaStreamSynchronize(b->stream)) != cudaSuccess)
     return bail(e, "upload");
-  b->threads = int(batch_default_threads(b->Lmax));
+  b->threads = int(batch_default_threads(b->Lmax, n, uint32_t(b->sms)));
   if ((e = prepare_batch_kernel(b->Lmax, b->threads)) != cudaSuccess) return bail(e, "cudaFuncSetAttribute");
   round_keys(params[0].seed, b->common.rk);
   b->common.key0 = uint32_t(params[0].seed);
@@ -244,10 +243,6 @@ ilg_status ilg_batch_set_state(ilg_batch* b, uint32_t i, const uint16_t* host, s
   if (n != 3 * size_t(b->desc[i].L)) return bfail(b, ILG_E_INVALID, "state size must be 3 * L");
   if (t >= (uint64_t(1) << 32)) return bfail(b, ILG_E_INVALID, "t must be below 2^32");
   b->desc[i].t = uint32_t(t);
-  uint64_t mass = 0;
-  for (size_t k = 0; k < n; ++k) mass += host[k];
-  const double om = b->p[i].omega_eff > 1.0 ? 2.0 - b->p[i].omega_eff : b->p[i].omega_eff;
-  b->desc[i].general = general_path(ILG_D1Q3, b->p[i].theta, om, double(mass) / double(n), b->p[i].Lx) | b->desc[i].particle;
   BCUDA(b, cudaMemcpyAsync(b->d_state + b->desc[i].state_off, host, sizeof(uint16_t) * n, cudaMemcpyHostToDevice, b->stream),
         "copy state in");
   BCUDA(b, cudaMemcpyAsync(b->d_desc + i, &b->desc[i], sizeof(ReplicaDesc), cudaMemcpyHostToDevice, b->stream), "copy desc");

@@ -122,12 +122,15 @@ __device__ __forceinline__ uint32_t more_chunks(NodeWords<S, K>& e, const WordKe
 // The collision of one node per lane (m: its occupations after the flip, all zero for a
 // lane without a node); all 32 lanes call it together.  The same words and results as
 // collide().  ring: the block's ring of K words per thread in shared memory, lane_off:
-// 4 x the thread's index.
-template <int Q, uint32_t S, uint32_t K, class Tab>
+// 4 x the thread's index.  TABLES: both probabilities lie strictly between 0 and 1 and are
+// drawn through their tables (known outside the loop over nodes: the tests for the other
+// cases would be made for every node).
+template <int Q, uint32_t S, uint32_t K, bool TABLES, class Tab>
 __device__ __forceinline__ void collide_warp(const StepArgs& a, const WordKeys& k, const Tab& to, const Tab& tr,
                                              unsigned char* ring, uint32_t lane_off, uint32_t node,
                                              const uint32_t (&m)[Q], uint32_t (&out)[Q]) {
   static_assert(Q == 3 || Q == 5, "D1Q3 and D2Q5");
+  static_assert(K >= 4 + uint32_t(Q), "a word for each velocity beside the block being written");
   constexpr int32_t kN = int32_t(kDevNmax);
   NodeWords<S, K> e;
   e.begin(k, ring, lane_off, node);
@@ -143,7 +146,7 @@ __device__ __forceinline__ void collide_warp(const StepArgs& a, const WordKeys& 
 
   // thinning
   uint32_t r[Q], removed = 0;
-  if (a.omega_mode == kTable) {
+  if (TABLES || a.omega_mode == kTable) {
     uint32_t most = m[0];
 #pragma unroll
     for (int i = 1; i < Q; ++i) most = max(most, m[i]);
@@ -178,7 +181,7 @@ __device__ __forceinline__ void collide_warp(const StepArgs& a, const WordKeys& 
 
   // share sent to rest
   uint32_t to_rest;
-  if (a.rest_mode == kTable) {
+  if (TABLES || a.rest_mode == kTable) {
     to_rest = tr(min(removed, kDevNmax), W[Q]);
     to_rest += more_chunks(e, k, a.rk, tr, int32_t(removed) - kN);
   } else {
@@ -192,7 +195,8 @@ __device__ __forceinline__ void collide_warp(const StepArgs& a, const WordKeys& 
   uint32_t mask = __funnelshift_lc(kFullWarp, 0u, uint32_t(left));
   left = max(left - 32, 0);
   constexpr uint32_t kWords = Q == 3 ? 1 : 2;               // per group
-  constexpr int32_t kPass = Q == 3 ? 8 : 4;                 // groups whose words are asked for at once
+  // groups whose words are asked for at once
+  constexpr int32_t kPass = int32_t((K - 4 < 8 ? K - 4 : 8) / kWords);
   auto ask = [&](int32_t l) { return min(uint32_t(l + 31) >> 5, uint32_t(kPass)) * (kWords * S); };
   if constexpr (Q == 3) {
     uint32_t minus = __popc(W[Q + 1] & mask);

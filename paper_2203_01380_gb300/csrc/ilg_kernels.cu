@@ -45,9 +45,10 @@ __device__ __forceinline__ unsigned long long run_barrier(unsigned long long* wo
   return ~0ull;
 }
 
-// sync[0]: the barrier word, sync[1]: set to 1 when a wait gave up
-template <int Q, int THREADS, int MINB>
-__global__ void __launch_bounds__(THREADS, MINB)
+// sync[0]: the barrier word, sync[1]: set to 1 when a wait gave up.  TABLES: the binomial
+// sampler with both probabilities strictly between 0 and 1; false: anything else.
+template <int Q, int THREADS, bool TABLES>
+__global__ void __launch_bounds__(THREADS, 1)
     step_run_kernel(const __grid_constant__ StepArgs a, uint16_t* buf0, uint16_t* buf1, uint32_t t0, uint32_t T,
                     unsigned long long* fail, unsigned long long* sync) {
   extern __shared__ uint4 smem4[];
@@ -80,6 +81,10 @@ __global__ void __launch_bounds__(THREADS, MINB)
     // (x, y) of the lane's node, advanced by the grid stride (stride_y rows and stride_x
     // nodes) with a carry instead of a division per node
     uint32_t base = base0, x = x0, y = y0;
+    // the flip F_i(n) = n_{-i}: velocity i of the collision reads plane -i
+    const uint16_t* from[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) from[i] = in + (i == 0 || !a.flip ? i : (i & 1 ? i + 1 : i - 1)) * plane;
     const WordKeys keys = word_keys(a, t);  // the launch-wide Philox rounds
     while (base < nodes) {
       const uint32_t node = base + lane;
@@ -87,19 +92,9 @@ __global__ void __launch_bounds__(THREADS, MINB)
       uint32_t m[Q], post[Q];
       // (through L2 only: another SM wrote these lines in the step before)
 #pragma unroll
-      for (int i = 0; i < Q; ++i) m[i] = active ? __ldcg(in + (i * plane + node)) : 0u;
-      if (a.flip) {
-        uint32_t v = m[1];
-        m[1] = m[2];
-        m[2] = v;
-        if constexpr (Q == 5) {
-          v = m[3];
-          m[3] = m[4];
-          m[4] = v;
-        }
-      }
-      if (a.particle) collide_particle<Q>(a, s, node, t, m, post);
-      else collide_warp<Q, 4 * THREADS, kStepRing>(a, keys, to, tr, ring, 4 * threadIdx.x, node, m, post);
+      for (int i = 0; i < Q; ++i) m[i] = active ? __ldcg(from[i] + node) : 0u;
+      if (!TABLES && a.particle) collide_particle<Q>(a, s, node, t, m, post);
+      else collide_warp<Q, 4 * THREADS, kStepRing, TABLES>(a, keys, to, tr, ring, 4 * threadIdx.x, node, m, post);
       if (active) {
         uint32_t high = 0;
 #pragma unroll
@@ -157,15 +152,19 @@ struct RunShape {
 };
 
 template <int THREADS>
-static const void* run_fn(int Q) {
-  return Q == 3 ? reinterpret_cast<const void*>(step_run_kernel<3, THREADS, 1>)
-                : reinterpret_cast<const void*>(step_run_kernel<5, THREADS, 1>);
+static const void* run_fn(int Q, bool tables) {
+  if (Q == 3)
+    return tables ? reinterpret_cast<const void*>(step_run_kernel<3, THREADS, true>)
+                  : reinterpret_cast<const void*>(step_run_kernel<3, THREADS, false>);
+  return tables ? reinterpret_cast<const void*>(step_run_kernel<5, THREADS, true>)
+                : reinterpret_cast<const void*>(step_run_kernel<5, THREADS, false>);
 }
 
-static RunShape run_shape(int Q, uint64_t nodes, uint32_t sms) {
-  if (nodes <= uint64_t(sms) * 128) return {run_fn<128>(Q), 128};
-  if (nodes <= uint64_t(sms) * 512) return {run_fn<512>(Q), 512};
-  return {run_fn<1024>(Q), 1024};
+static RunShape run_shape(int Q, const StepArgs& a, uint64_t nodes, uint32_t sms) {
+  const bool tables = !a.particle && a.omega_mode == kTable && a.rest_mode == kTable;
+  if (nodes <= uint64_t(sms) * 128) return {run_fn<128>(Q, tables), 128};
+  if (nodes <= uint64_t(sms) * 512) return {run_fn<512>(Q, tables), 512};
+  return {run_fn<1024>(Q, tables), 1024};
 }
 
 cudaError_t prepare_step_kernels() {
@@ -173,18 +172,19 @@ cudaError_t prepare_step_kernels() {
   auto set = [&](const void* f, int threads) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(run_smem(threads)));
   };
-  for (int Q : {3, 5}) {
-    set(run_fn<128>(Q), 128);
-    set(run_fn<512>(Q), 512);
-    set(run_fn<1024>(Q), 1024);
-  }
+  for (int Q : {3, 5})
+    for (bool tables : {false, true}) {
+      set(run_fn<128>(Q, tables), 128);
+      set(run_fn<512>(Q, tables), 512);
+      set(run_fn<1024>(Q, tables), 1024);
+    }
   return e;
 }
 
 cudaError_t launch_step_run(int Q, const StepArgs& a, uint16_t* buf0, uint16_t* buf1, uint32_t t, uint32_t T,
                             unsigned long long* fail, unsigned long long* sync, uint32_t sms, cudaStream_t s) {
   const uint64_t nodes = uint64_t(a.Lx) * a.Ly;
-  const RunShape r = run_shape(Q, nodes, sms);
+  const RunShape r = run_shape(Q, a, nodes, sms);
   const dim3 grid(uint32_t(std::min<uint64_t>((nodes + r.threads - 1) / r.threads, sms)));
   StepArgs args = a;
   void* p[] = {&args, &buf0, &buf1, &t, &T, &fail, &sync};

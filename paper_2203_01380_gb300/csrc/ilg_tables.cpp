@@ -189,13 +189,10 @@ double poisson_tail(double lambda, int k) {
 // moving particles (D2Q9: 32 axis and 32 diagonal).  With Poisson occupations of the
 // given mean, removals and movers are thinned Poisson counts; the lattice goes straight
 // to the general collision when the expected share of nodes that fail the fast one is
-// above kGeneralShare, or, where sync_nodes nodes wait for one another every step (a
-// batched ring and its block barrier), when one of them is expected to fail in more
-// than about one step in three: trying the fast collision first then costs more than it
-// saves, since the warp or block that holds a failing node runs both collisions.
-uint32_t general_path(int lattice, double theta, double omega_star, double mean_occupation, uint32_t sync_nodes) {
+// above kGeneralShare: trying the fast collision first then costs more than it saves,
+// since the warp that holds a failing node runs both collisions.
+uint32_t general_path(int lattice, double theta, double omega_star, double mean_occupation) {
   constexpr double kGeneralShare = 0.02;
-  const double share = std::min(kGeneralShare, 0.3 / double(std::max<uint32_t>(sync_nodes, 1)));
   double w[9];
   weights(lattice, theta, w);
   const int Q = lattice == ILG_D1Q3 ? 3 : (lattice == ILG_D2Q9 ? 9 : 5);
@@ -207,7 +204,7 @@ uint32_t general_path(int lattice, double theta, double omega_star, double mean_
   } else {
     fail += poisson_tail(moving, 33);
   }
-  return fail > share ? 1u : 0u;
+  return fail > kGeneralShare ? 1u : 0u;
 }
 
 uint64_t quantise_probability(double p) {
