@@ -8,6 +8,7 @@
 #include "ilg_collide.cuh"
 #include "ilg_device.cuh"
 #include "ilg_launch.h"
+#include "ilg_sync.cuh"
 
 namespace ilg {
 
@@ -27,23 +28,6 @@ namespace ilg {
 // 55 / 66; 1024^2 at 200 per velocity, omega* = 1, 93 / 241; 96 x 40 2.2 / 18.7.
 // --------------------------------------------------------------------------
 constexpr uint32_t kStepRing = 16;  // extension words per lane
-
-// Barrier of all blocks of a cooperative launch: word = arrivals (low half) and, once a
-// step overflowed, a mark (high half).  Returns the word, or ~0 when the wait gave up
-// (bounded: the kernel then returns and the host reports it).
-constexpr unsigned long long kRunMark = 1ull << 32;
-constexpr uint32_t kRunPolls = 1u << 23;  // seconds; a step's blocks differ by far less
-
-__device__ __forceinline__ unsigned long long run_barrier(unsigned long long* word, uint32_t target) {
-  __threadfence();
-  atomicAdd(word, 1ull);
-  unsigned long long v = 0;
-  for (uint32_t k = 0; k < kRunPolls; ++k) {
-    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(word) : "memory");
-    if (uint32_t(v) >= target) return v;
-  }
-  return ~0ull;
-}
 
 // sync[0]: the barrier word, sync[1]: set to 1 when a wait gave up.  TABLES: the binomial
 // sampler with both probabilities strictly between 0 and 1; false: anything else.

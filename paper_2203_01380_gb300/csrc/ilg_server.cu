@@ -1,7 +1,7 @@
 // Serving loop (ilg_server_*): a worker thread admits D2Q5 lattice requests into a
 // preallocated device arena while memory and slots allow, keeps every admitted
 // lattice resident, and advances all of them together — one multi-lattice launch
-// per time step, a quantum of steps per round — so requests that arrive while
+// per round of a quantum of steps — so requests that arrive while
 // others run join the next round (continuous batching).  A finished request's
 // observables (and, if asked, its final state) are copied out, its memory goes back
 // to the arena, and waiting requests are admitted.  Every random number is keyed by
@@ -10,6 +10,7 @@
 
 #include <algorithm>
 #include <chrono>
+#include <cmath>
 #include <condition_variable>
 #include <cstring>
 #include <deque>
@@ -30,6 +31,7 @@ namespace {
 
 constexpr uint32_t kServerMaxSide = 32768;
 constexpr size_t kAlign = 256;
+constexpr uint32_t kRoundSteps = 4096;  // steps of one launch at most
 
 struct Request {
   uint64_t id;
@@ -44,7 +46,8 @@ struct Resident {
   size_t off_state = 0, state_bytes = 0;  // two buffers
   size_t off_tab = 0;
   uint32_t t = 0, remaining = 0, phase = 0;
-  uint32_t flip = 0, omega_mode = 0, rest_mode = 0, general = 0, particle = 0;
+  uint32_t flip = 0, omega_mode = 0, rest_mode = 0, particle = 0;
+  double cost = 0;  // of a run of nodes and step: estimated, then corrected by the rounds' block cycles
   double t_admit = 0;
   int status = ILG_OK;
 };
@@ -113,10 +116,10 @@ struct ilg_server {
   size_t arena_bytes = 0;
   Arena arena;
   LatDesc* d_lat = nullptr;
-  WorkItem* d_items = nullptr;
-  size_t items_cap = 0;
-  unsigned int* d_counters = nullptr;
-  uint32_t* d_fail = nullptr;
+  WorkShare* d_shares = nullptr;       // sms + max_slots (each cut adds one)
+  uint32_t* d_first = nullptr;         // sms + 1
+  // of a round: barrier word, block cycles, failing steps, a word for a wait that gave up
+  unsigned long long* d_round = nullptr;
   unsigned long long* d_col = nullptr;
   unsigned long long* d_row = nullptr;
   unsigned long long* d_mass = nullptr;
@@ -134,7 +137,7 @@ struct ilg_server {
   };
   std::vector<PendingInit> inits;
   cudaEvent_t round_ev = nullptr;   // end of a round's launches and its flag read-back
-  uint32_t* h_fail = nullptr;       // pinned: per-lattice overflow flags of a round
+  unsigned long long* h_round = nullptr;  // pinned: the same
 
   std::thread worker;
   std::mutex mu;
@@ -158,13 +161,13 @@ void free_server(ilg_server* s) {
   for (auto& pi : s->inits) cudaEventDestroy(pi.ev);
   s->inits.clear();
   if (s->round_ev) cudaEventDestroy(s->round_ev);
-  if (s->h_fail) cudaFreeHost(s->h_fail);
+  if (s->h_round) cudaFreeHost(s->h_round);
   if (s->init_stream) cudaStreamDestroy(s->init_stream);
   cudaFree(s->d_arena);
   cudaFree(s->d_lat);
-  cudaFree(s->d_items);
-  cudaFree(s->d_counters);
-  cudaFree(s->d_fail);
+  cudaFree(s->d_shares);
+  cudaFree(s->d_first);
+  cudaFree(s->d_round);
   cudaFree(s->d_col);
   cudaFree(s->d_row);
   cudaFree(s->d_mass);
@@ -174,6 +177,57 @@ void free_server(ilg_server* s) {
 }
 
 size_t state_bytes_of(const ilg_params& p) { return sizeof(uint16_t) * 5 * size_t(p.Lx) * p.Ly; }
+
+// Cost of a run of 32 nodes and step before a round has measured it: warp instructions of the
+// collision (a base, and what each further chunk of 63, group of 32 and extension block costs
+// the warp), from the counts that the neediest of 32 nodes has.  The particle sampler costs a
+// Philox block per four particles.
+double run_cost_estimate(const ilg_params& p, double omega_star, double w_rest) {
+  auto more = [](double mean, double per) { return std::max(0.0, std::ceil((mean + 2.2 * std::sqrt(mean)) / per) - 1.0); };
+  const double removed = omega_star * 5.0 * p.n0, moving = removed * (1.0 - w_rest);
+  if (p.sampler == ILG_SAMPLER_PARTICLE) return 200.0 + 5.0 * p.n0 / 4.0 * 100.0;
+  const double thin = 5.0 * more(p.n0, 63.0), rest = more(removed, 63.0), groups = more(moving, 32.0);
+  return 290.0 + 17.0 * thin + 25.0 * rest + 25.0 * groups + 45.0 * std::ceil((thin + rest + 2.0 * groups) / 4.0);
+}
+
+// A round's lattices laid end to end, their runs of 32 nodes weighted by cost (of a run and
+// step), cut into equal shares for at most `blocks` blocks; no more blocks than give each of
+// them a run for eight of its warps.  part[k]: share k's cost.
+void share_out(const std::vector<double>& run_cost, const std::vector<LatDesc>& lat, uint32_t blocks,
+               std::vector<WorkShare>* shares, std::vector<uint32_t>* first, std::vector<double>* part) {
+  constexpr uint64_t kRunsPerBlock = 8;
+  const uint32_t n = uint32_t(lat.size());
+  double total = 0;
+  uint64_t runs = 0;
+  auto runs_of = [&](uint32_t l) { return uint32_t((uint64_t(lat[l].Lx) * lat[l].Ly + kMultiRun - 1) / kMultiRun); };
+  for (uint32_t l = 0; l < n; ++l) {
+    total += run_cost[l] * runs_of(l);
+    runs += runs_of(l);
+  }
+  const uint32_t B = uint32_t(std::min<uint64_t>(blocks, std::max<uint64_t>(1, runs / kRunsPerBlock)));
+  shares->clear();
+  part->clear();
+  first->assign(1, 0);
+  uint32_t l = 0, r = 0;  // next run
+  double taken = 0;
+  for (uint32_t b = 0; b < B; ++b) {
+    const double goal = total * (b + 1) / B;
+    while (l < n && (b + 1 == B || goal - taken > 0.5 * run_cost[l])) {
+      const uint32_t left = runs_of(l) - r;
+      uint32_t take = left;
+      if (b + 1 < B) take = uint32_t(std::min<double>(left, std::max(1.0, std::floor((goal - taken) / run_cost[l] + 0.5))));
+      shares->push_back(WorkShare{l, r, r + take});
+      part->push_back(take * run_cost[l]);
+      taken += take * run_cost[l];
+      r += take;
+      if (r == runs_of(l)) {
+        ++l;
+        r = 0;
+      }
+    }
+    first->push_back(uint32_t(shares->size()));
+  }
+}
 
 // Admit one request: arena memory for two state buffers and its tables, Poisson
 // initial state.  Returns false (nothing changed) when the arena cannot hold it.
@@ -207,7 +261,7 @@ bool admit(ilg_server* s, const Request& rq, Resident* out, cudaError_t* cerr, s
   const uint64_t Po = quantise_probability(omega_star), Pr = quantise_probability(w[0]);
   r.flip = rq.p.omega_eff > 1.0 ? 1u : 0u;
   r.particle = rq.p.sampler == ILG_SAMPLER_PARTICLE ? 1u : 0u;
-  r.general = general_path(ILG_D2Q5, rq.p.theta, omega_star, rq.p.n0) | r.particle;
+  r.cost = run_cost_estimate(rq.p, omega_star, w[0]);
   r.omega_mode = mode_of(Po);
   r.rest_mode = mode_of(Pr);
   std::vector<uint32_t> tables(kBlockWords, 0u);
@@ -355,10 +409,16 @@ void admit_pending(ilg_server* s, cudaError_t& e) {
   }
 }
 
+// the barrier word, cycles per block, failing steps per lattice, the give-up word
+size_t round_bytes(int sms, size_t n) { return sizeof(unsigned long long) * (1 + size_t(sms)) + sizeof(uint32_t) * (n + 1); }
+
 void worker_main(ilg_server* s) {
   cudaError_t e = cudaSuccess;
+  bool gave_up = false;
   std::vector<LatDesc> lat;
-  std::vector<WorkItem> items;
+  std::vector<WorkShare> shares;
+  std::vector<uint32_t> first;
+  std::vector<double> cost, part;
   for (;;) {
     {
       std::unique_lock<std::mutex> lk(s->mu);
@@ -375,12 +435,13 @@ void worker_main(ilg_server* s) {
     admit_pending(s, e);
     double round_updates = 0;
     if (e != cudaSuccess) break;
-    // one round: up to `quantum` steps, each lattice taking min(quantum, remaining)
+    // one round: up to `quantum` steps (kRoundSteps at most: one launch), each lattice
+    // taking min(quantum, remaining)
     uint32_t q = 0;
     for (auto& r : s->resident)
-      if (r.status == ILG_OK) q = std::max(q, std::min(s->quantum, r.remaining));
+      if (r.status == ILG_OK) q = std::max(q, std::min(std::min(s->quantum, kRoundSteps), r.remaining));
     lat.clear();
-    items.clear();
+    cost.clear();
     std::vector<size_t> which;
     for (size_t k = 0; k < s->resident.size(); ++k) {
       Resident& r = s->resident[k];
@@ -395,41 +456,39 @@ void worker_main(ilg_server* s) {
       d.omega_mode = r.omega_mode;
       d.rest_mode = r.rest_mode;
       d.steps = std::min(q, r.remaining);
-      d.general = r.general;
       d.particle = r.particle;
       d.buf0 = reinterpret_cast<uint16_t*>(s->d_arena + r.off_state);
       d.buf1 = reinterpret_cast<uint16_t*>(s->d_arena + r.off_state + r.state_bytes);
       d.tables = reinterpret_cast<const uint32_t*>(s->d_arena + r.off_tab);
-      const uint32_t li = uint32_t(lat.size());
       lat.push_back(d);
       which.push_back(k);
-      const uint32_t nodes = d.Lx * d.Ly;
-      for (uint32_t n0 = 0; n0 < nodes; n0 += kItemNodes) items.push_back(WorkItem{li, n0, std::min(nodes, n0 + kItemNodes)});
+      cost.push_back(r.cost);
     }
     if (!lat.empty() && q > 0) {
-      if (items.size() > s->items_cap) {
-        cudaFree(s->d_items);
-        s->d_items = nullptr;
-        e = dev_alloc(&s->d_items, sizeof(WorkItem) * items.size() * 2);
-        if (e != cudaSuccess) break;
-        s->items_cap = items.size() * 2;
-      }
-      e = cudaMemcpyAsync(s->d_lat, lat.data(), sizeof(LatDesc) * lat.size(), cudaMemcpyHostToDevice, s->stream);
+      share_out(cost, lat, uint32_t(s->sms), &shares, &first, &part);
+      const size_t n = lat.size(), blocks = first.size() - 1;
+      unsigned long long* const d_cycles = s->d_round + 1;
+      uint32_t* const d_fail = reinterpret_cast<uint32_t*>(d_cycles + s->sms);
+      e = cudaMemcpyAsync(s->d_lat, lat.data(), sizeof(LatDesc) * n, cudaMemcpyHostToDevice, s->stream);
       if (e == cudaSuccess)
-        e = cudaMemcpyAsync(s->d_items, items.data(), sizeof(WorkItem) * items.size(), cudaMemcpyHostToDevice, s->stream);
-      if (e == cudaSuccess) e = cudaMemsetAsync(s->d_counters, 0, sizeof(unsigned int) * q, s->stream);
-      if (e == cudaSuccess) e = cudaMemsetAsync(s->d_fail, 0xFF, sizeof(uint32_t) * lat.size(), s->stream);
+        e = cudaMemcpyAsync(s->d_shares, shares.data(), sizeof(WorkShare) * shares.size(), cudaMemcpyHostToDevice, s->stream);
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(s->d_first, first.data(), sizeof(uint32_t) * first.size(), cudaMemcpyHostToDevice, s->stream);
+      if (e == cudaSuccess) e = cudaMemsetAsync(s->d_round, 0, sizeof(unsigned long long), s->stream);
+      if (e == cudaSuccess) e = cudaMemsetAsync(d_fail, 0xFF, sizeof(uint32_t) * n, s->stream);
+      if (e == cudaSuccess) e = cudaMemsetAsync(d_fail + n, 0, sizeof(uint32_t), s->stream);
       MultiArgs ma{};
       ma.lat = s->d_lat;
-      ma.items = s->d_items;
-      ma.n_items = uint32_t(items.size());
-      ma.counter = s->d_counters;
-      ma.fail = s->d_fail;
-      // persistent blocks: as many as are resident at once (3 per SM at this register count)
-      const int grid = int(std::min<size_t>(items.size(), size_t(s->sms) * kMultiBlocksPerSm));
-      for (uint32_t sub = 0; sub < q && e == cudaSuccess; ++sub) e = launch_multi_step(ma, s->common, sub, grid, s->stream);
+      ma.shares = s->d_shares;
+      ma.first = s->d_first;
+      ma.steps = q;
+      ma.sync = s->d_round;
+      ma.cycles = d_cycles;
+      ma.fail = d_fail;
+      ma.gave_up = d_fail + n;
+      if (e == cudaSuccess) e = launch_multi_round(ma, s->common, int(blocks), s->stream);
       if (e == cudaSuccess)
-        e = cudaMemcpyAsync(s->h_fail, s->d_fail, sizeof(uint32_t) * lat.size(), cudaMemcpyDeviceToHost, s->stream);
+        e = cudaMemcpyAsync(s->h_round, s->d_round, round_bytes(s->sms, n), cudaMemcpyDeviceToHost, s->stream);
       if (e == cudaSuccess) e = cudaEventRecord(s->round_ev, s->stream);
       // while the round runs, requests that arrive are admitted (their initial states
       // queued on the admission stream, for the next round)
@@ -444,7 +503,28 @@ void worker_main(ilg_server* s) {
         if (e == cudaSuccess) std::this_thread::sleep_for(std::chrono::microseconds(50));
       }
       if (e != cudaSuccess) break;
-      const uint32_t* fail = s->h_fail;
+      const uint32_t* fail = reinterpret_cast<const uint32_t*>(s->h_round + 1 + s->sms);
+      if (fail[n] != 0) {
+        gave_up = true;
+        break;
+      }
+      // a lattice costs more (less) than thought where its blocks were at work longer
+      // (shorter) than the average block: corrected by the ratio, weighted by their shares
+      std::vector<double> seen(n, 0.0), thought(n, 0.0);
+      double cycles = 0, all = 0;
+      for (size_t b = 0; b < blocks; ++b) {
+        double mine = 0;
+        for (uint32_t k = first[b]; k < first[b + 1]; ++k) mine += part[k];
+        cycles += double(s->h_round[1 + b]);
+        all += mine;
+        for (uint32_t k = first[b]; k < first[b + 1]; ++k) {
+          seen[shares[k].lattice] += part[k] * (double(s->h_round[1 + b]) / mine);
+          thought[shares[k].lattice] += part[k];
+        }
+      }
+      for (size_t j = 0; j < n; ++j)
+        if (lat[j].steps == q && cycles > 0 && thought[j] > 0 && fail[j] == 0xFFFFFFFFu)
+          s->resident[which[j]].cost *= std::min(2.0, std::max(0.5, seen[j] / thought[j] * (all / cycles)));
       for (size_t j = 0; j < which.size(); ++j) {
         Resident& r = s->resident[which[j]];
         const uint32_t done = fail[j] == 0xFFFFFFFFu ? lat[j].steps : fail[j];
@@ -479,10 +559,10 @@ void worker_main(ilg_server* s) {
       if (s->in_flight == 0) s->idle_cv.notify_all();
     }
   }
-  if (e != cudaSuccess) {
+  if (e != cudaSuccess || gave_up) {
     std::lock_guard<std::mutex> lk(s->mu);
-    s->fatal = ILG_E_CUDA;
-    s->err = std::string("server worker: ") + cudaGetErrorString(e);
+    s->fatal = gave_up ? ILG_E_TIMEOUT : ILG_E_CUDA;
+    s->err = std::string("server worker: ") + (gave_up ? "a wait between blocks gave up" : cudaGetErrorString(e));
     s->idle_cv.notify_all();
   }
 }
@@ -526,8 +606,10 @@ ilg_status ilg_server_create(uint64_t seed, uint64_t hbm_bytes, uint32_t max_slo
   s->arena_bytes = hbm_bytes;
   s->arena.reset(hbm_bytes);
   if ((e = dev_alloc(&s->d_lat, sizeof(LatDesc) * max_slots)) != cudaSuccess) return bail(e, "cudaMalloc");
-  if ((e = dev_alloc(&s->d_counters, sizeof(unsigned int) * quantum)) != cudaSuccess) return bail(e, "cudaMalloc");
-  if ((e = dev_alloc(&s->d_fail, sizeof(uint32_t) * max_slots)) != cudaSuccess) return bail(e, "cudaMalloc");
+  if ((e = prepare_multi_kernel()) != cudaSuccess) return bail(e, "cudaFuncSetAttribute");
+  if ((e = dev_alloc(&s->d_shares, sizeof(WorkShare) * (size_t(s->sms) + max_slots))) != cudaSuccess) return bail(e, "cudaMalloc");
+  if ((e = dev_alloc(&s->d_first, sizeof(uint32_t) * (size_t(s->sms) + 1))) != cudaSuccess) return bail(e, "cudaMalloc");
+  if ((e = dev_alloc(&s->d_round, round_bytes(s->sms, max_slots))) != cudaSuccess) return bail(e, "cudaMalloc");
   if ((e = dev_alloc(&s->d_col, sizeof(unsigned long long) * kServerMaxSide)) != cudaSuccess) return bail(e, "cudaMalloc");
   if ((e = dev_alloc(&s->d_row, sizeof(unsigned long long) * kServerMaxSide)) != cudaSuccess) return bail(e, "cudaMalloc");
   if ((e = dev_alloc(&s->d_mass, sizeof(unsigned long long))) != cudaSuccess) return bail(e, "cudaMalloc");
@@ -535,12 +617,11 @@ ilg_status ilg_server_create(uint64_t seed, uint64_t hbm_bytes, uint32_t max_slo
   if ((e = dev_alloc(&s->d_res, sizeof(double) * 4)) != cudaSuccess) return bail(e, "cudaMalloc");
   const int32_t mode1[2] = {1, 0};
   if ((e = cudaMemcpy(s->d_modes, mode1, sizeof(mode1), cudaMemcpyHostToDevice)) != cudaSuccess) return bail(e, "upload");
-  if ((e = prepare_multi_kernel()) != cudaSuccess) return bail(e, "cudaFuncSetAttribute");
   if ((e = cudaStreamCreateWithFlags(&s->init_stream, cudaStreamNonBlocking)) != cudaSuccess)
     return bail(e, "cudaStreamCreate");
   if ((e = cudaEventCreateWithFlags(&s->round_ev, cudaEventDisableTiming)) != cudaSuccess)
     return bail(e, "cudaEventCreate");
-  if ((e = cudaMallocHost(&s->h_fail, sizeof(uint32_t) * max_slots)) != cudaSuccess) return bail(e, "cudaMallocHost");
+  if ((e = cudaMallocHost(&s->h_round, round_bytes(s->sms, max_slots))) != cudaSuccess) return bail(e, "cudaMallocHost");
   round_keys(seed, s->common.rk);
   s->common.key0 = uint32_t(seed);
   s->common.key1 = uint32_t(seed >> 32);

@@ -1,0 +1,27 @@
+// Barrier between blocks of one cooperative launch that alternate two buffers step by step.
+#pragma once
+
+#include <cstdint>
+
+namespace ilg {
+
+// The barrier word counts arrivals in its low half; the high half is a mark that a step
+// overflowed.  Zero it before the launch.
+constexpr unsigned long long kRunMark = 1ull << 32;
+constexpr uint32_t kRunPolls = 1u << 23;  // seconds; the blocks of a step differ by far less
+
+// One thread per block, after the block's own barrier: arrive, and wait until `target`
+// arrivals.  Returns the word, or ~0 when the wait gave up (bounded: the kernel then
+// returns and the host reports it).
+__device__ __forceinline__ unsigned long long run_barrier(unsigned long long* word, uint32_t target) {
+  __threadfence();
+  atomicAdd(word, 1ull);
+  unsigned long long v = 0;
+  for (uint32_t k = 0; k < kRunPolls; ++k) {
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(word) : "memory");
+    if (uint32_t(v) >= target) return v;
+  }
+  return ~0ull;
+}
+
+}  // namespace ilg
