@@ -32,6 +32,7 @@ namespace {
 constexpr uint32_t kServerMaxSide = 32768;
 constexpr size_t kAlign = 256;
 constexpr uint32_t kRoundSteps = 4096;  // steps of one launch at most
+constexpr size_t kOutWords = 5;         // observables of a finished request: res[4], mass
 
 struct Request {
   uint64_t id;
@@ -122,9 +123,12 @@ struct ilg_server {
   unsigned long long* d_round = nullptr;
   unsigned long long* d_col = nullptr;
   unsigned long long* d_row = nullptr;
-  unsigned long long* d_mass = nullptr;
   int32_t* d_modes = nullptr;
-  double* d_res = nullptr;
+  // observables of the requests a round finished, kOutWords words each: res[4], mass
+  unsigned long long* d_out = nullptr;
+  unsigned long long* h_out = nullptr;    // pinned
+  cudaStream_t out_stream = nullptr;      // copies finished states out while the next round runs
+  cudaEvent_t out_ev = nullptr;           // the finished requests' observables are in h_out
   StepArgs common{};
   std::chrono::steady_clock::time_point t0;
   // admissions: a newcomer's tables and Poisson initial state are written on their own
@@ -170,9 +174,11 @@ void free_server(ilg_server* s) {
   cudaFree(s->d_round);
   cudaFree(s->d_col);
   cudaFree(s->d_row);
-  cudaFree(s->d_mass);
   cudaFree(s->d_modes);
-  cudaFree(s->d_res);
+  cudaFree(s->d_out);
+  if (s->h_out) cudaFreeHost(s->h_out);
+  if (s->out_ev) cudaEventDestroy(s->out_ev);
+  if (s->out_stream) cudaStreamDestroy(s->out_stream);
   if (s->own_stream) cudaStreamDestroy(s->stream);
 }
 
@@ -317,39 +323,75 @@ bool admit(ilg_server* s, const Request& rq, Resident* out, cudaError_t* cerr, s
   return true;
 }
 
-// Observables and (optionally) the final state of a finished request, then its
-// memory goes back to the arena.
-cudaError_t finish(ilg_server* s, Resident& r, ilg_result* res) {
-  std::memset(res, 0, sizeof(*res));
-  res->id = r.rq.id;
-  res->status = r.status;
-  res->t = r.t;
-  res->t_submit = r.rq.t_submit;
-  res->t_admit = r.t_admit;
+// A finished request holds a state to report.
+bool has_result(const Resident& r) { return r.state_bytes && (r.status == ILG_OK || r.status == ILG_E_OVERFLOW); }
+const uint16_t* state_of(const ilg_server* s, const Resident& r) {
+  return reinterpret_cast<const uint16_t*>(s->d_arena + r.off_state + (r.phase ? r.state_bytes : 0));
+}
+
+// Finished requests leave in two parts, so that neither their observables nor the copies of
+// their states to the caller's memory hold the next round back.  First their observables are
+// queued behind the round that finished them (a round's launch fills every SM, so after it
+// they would wait for the whole next round) ...
+cudaError_t queue_results(ilg_server* s, const std::vector<Resident>& out) {
   cudaError_t e = cudaSuccess;
-  if (r.status == ILG_OK || r.status == ILG_E_OVERFLOW) {
-    const uint16_t* st = reinterpret_cast<const uint16_t*>(s->d_arena + r.off_state + (r.phase ? r.state_bytes : 0));
+  for (size_t i = 0; i < out.size() && e == cudaSuccess; ++i) {
+    const Resident& r = out[i];
+    if (!has_result(r)) continue;
     const uint32_t Lx = r.rq.p.Lx, Ly = r.rq.p.Ly;
+    unsigned long long* const to = s->d_out + kOutWords * i;
     e = cudaMemsetAsync(s->d_col, 0, sizeof(unsigned long long) * Lx, s->stream);
-    if (e == cudaSuccess) e = launch_sums(5, st, Lx, Ly, s->d_col, s->d_row, 0, s->stream);
-    if (e == cudaSuccess) e = launch_project(s->d_col, s->d_row, Lx, Ly, s->d_modes, 1, s->d_res, s->d_mass, s->stream);
-    double h[4] = {0, 0, 0, 0};
-    unsigned long long M = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h, s->d_res, sizeof(h), cudaMemcpyDeviceToHost, s->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&M, s->d_mass, sizeof(M), cudaMemcpyDeviceToHost, s->stream);
-    if (e == cudaSuccess && r.rq.final_state)
-      e = cudaMemcpyAsync(r.rq.final_state, st, r.state_bytes, cudaMemcpyDeviceToHost, s->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-    res->mass = M;
-    res->amp = h[2];
-    res->Sk = h[3];
+    if (e == cudaSuccess) e = launch_sums(5, state_of(s, r), Lx, Ly, s->d_col, s->d_row, 0, s->stream);
+    if (e == cudaSuccess)
+      e = launch_project(s->d_col, s->d_row, Lx, Ly, s->d_modes, 1, reinterpret_cast<double*>(to), to + 4, s->stream);
   }
-  if (r.state_bytes) {
-    s->arena.release(r.off_state, 2 * r.state_bytes);
-    s->arena.release(r.off_tab, sizeof(uint32_t) * kBlockWords);
-  }
-  res->t_done = now_s(s->t0);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(s->h_out, s->d_out, sizeof(unsigned long long) * kOutWords * out.size(), cudaMemcpyDeviceToHost,
+                        s->stream);
+  if (e == cudaSuccess) e = cudaEventRecord(s->out_ev, s->stream);
   return e;
+}
+
+// ... then, with the next round already queued, the states are copied out on a stream of
+// their own (the round that wrote them has completed), the memory goes back to the arena and
+// the results to the result queue.
+cudaError_t deliver(ilg_server* s, std::vector<Resident>& out) {
+  if (out.empty()) return cudaSuccess;
+  cudaError_t e = cudaSuccess;
+  for (size_t i = 0; i < out.size() && e == cudaSuccess; ++i)
+    if (has_result(out[i]) && out[i].rq.final_state)
+      e = cudaMemcpyAsync(out[i].rq.final_state, state_of(s, out[i]), out[i].state_bytes, cudaMemcpyDeviceToHost,
+                          s->out_stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s->out_stream);
+  if (e == cudaSuccess) e = cudaEventSynchronize(s->out_ev);
+  if (e != cudaSuccess) return e;
+  std::vector<ilg_result> res(out.size());
+  for (size_t i = 0; i < out.size(); ++i) {
+    const Resident& r = out[i];
+    std::memset(&res[i], 0, sizeof(res[i]));
+    res[i].id = r.rq.id;
+    res[i].status = r.status;
+    res[i].t = r.t;
+    res[i].t_submit = r.rq.t_submit;
+    res[i].t_admit = r.t_admit;
+    if (has_result(r)) {
+      const unsigned long long* h = s->h_out + kOutWords * i;
+      std::memcpy(&res[i].amp, h + 2, sizeof(double));
+      std::memcpy(&res[i].Sk, h + 3, sizeof(double));
+      res[i].mass = h[4];
+    }
+    if (r.state_bytes) {
+      s->arena.release(r.off_state, 2 * r.state_bytes);
+      s->arena.release(r.off_tab, sizeof(uint32_t) * kBlockWords);
+    }
+    res[i].t_done = now_s(s->t0);
+  }
+  std::lock_guard<std::mutex> lk(s->mu);
+  s->done.insert(s->done.end(), res.begin(), res.end());
+  s->in_flight -= res.size();
+  if (s->in_flight == 0) s->idle_cv.notify_all();
+  out.clear();
+  return cudaSuccess;
 }
 
 // Initial states whose event has completed give their tables' arena memory back.
@@ -415,6 +457,7 @@ size_t round_bytes(int sms, size_t n) { return sizeof(unsigned long long) * (1 +
 void worker_main(ilg_server* s) {
   cudaError_t e = cudaSuccess;
   bool gave_up = false;
+  std::vector<Resident> out;  // finished in the last round, not yet delivered
   std::vector<LatDesc> lat;
   std::vector<WorkShare> shares;
   std::vector<uint32_t> first;
@@ -422,8 +465,8 @@ void worker_main(ilg_server* s) {
   for (;;) {
     {
       std::unique_lock<std::mutex> lk(s->mu);
-      s->cv.wait(lk, [&] { return s->stop || !s->pending.empty() || !s->resident.empty(); });
-      if (s->stop && s->resident.empty() && s->pending.empty()) break;
+      s->cv.wait(lk, [&] { return s->stop || !s->pending.empty() || !s->resident.empty() || !out.empty(); });
+      if (s->stop && s->resident.empty() && s->pending.empty() && out.empty()) break;
       if (s->stop) {
         // shutting down: drop what is queued
         s->in_flight -= s->pending.size();
@@ -433,6 +476,18 @@ void worker_main(ilg_server* s) {
     const double t_round = now_s(s->t0);
     NvtxRange nvtx("ilg_server round");
     admit_pending(s, e);
+    if (e == cudaSuccess && !out.empty()) {
+      // requests that wait for memory or a slot: what is finished goes first
+      bool waiting;
+      {
+        std::lock_guard<std::mutex> lk(s->mu);
+        waiting = !s->pending.empty();
+      }
+      if (waiting) {
+        e = deliver(s, out);
+        if (e == cudaSuccess) admit_pending(s, e);
+      }
+    }
     double round_updates = 0;
     if (e != cudaSuccess) break;
     // one round: up to `quantum` steps (kRoundSteps at most: one launch), each lattice
@@ -490,8 +545,11 @@ void worker_main(ilg_server* s) {
       if (e == cudaSuccess)
         e = cudaMemcpyAsync(s->h_round, s->d_round, round_bytes(s->sms, n), cudaMemcpyDeviceToHost, s->stream);
       if (e == cudaSuccess) e = cudaEventRecord(s->round_ev, s->stream);
-      // while the round runs, requests that arrive are admitted (their initial states
-      // queued on the admission stream, for the next round)
+      // while the round runs, the last round's finished requests are delivered, and requests
+      // that arrive are admitted (their initial states queued on the admission stream, for
+      // the next round); a short round is waited for awake (a sleep lasts 100 us and more)
+      if (e == cudaSuccess) e = deliver(s, out);
+      const double t_wait = now_s(s->t0);
       while (e == cudaSuccess) {
         const cudaError_t q_ = cudaEventQuery(s->round_ev);
         if (q_ == cudaSuccess) break;
@@ -500,7 +558,9 @@ void worker_main(ilg_server* s) {
           break;
         }
         admit_pending(s, e);
-        if (e == cudaSuccess) std::this_thread::sleep_for(std::chrono::microseconds(50));
+        if (e != cudaSuccess) break;
+        if (now_s(s->t0) - t_wait < 300e-6) std::this_thread::yield();
+        else std::this_thread::sleep_for(std::chrono::microseconds(50));
       }
       if (e != cudaSuccess) break;
       const uint32_t* fail = reinterpret_cast<const uint32_t*>(s->h_round + 1 + s->sms);
@@ -535,28 +595,17 @@ void worker_main(ilg_server* s) {
         if (fail[j] != 0xFFFFFFFFu) r.status = ILG_E_OVERFLOW;
       }
     }
-    // finished requests
-    std::vector<ilg_result> out;
-    std::vector<Resident> keep;
-    for (auto& r : s->resident) {
-      if (r.status == ILG_OK && r.remaining > 0) {
-        keep.push_back(r);
-        continue;
-      }
-      ilg_result res;
-      e = finish(s, r, &res);
-      if (e != cudaSuccess) break;
-      out.push_back(res);
-    }
+    if (e == cudaSuccess) e = deliver(s, out);  // (no round took place)
     if (e != cudaSuccess) break;
+    // finished requests
+    std::vector<Resident> keep;
+    for (auto& r : s->resident) (r.status == ILG_OK && r.remaining > 0 ? keep : out).push_back(r);
+    if (!out.empty() && (e = queue_results(s, out)) != cudaSuccess) break;
     {
       std::lock_guard<std::mutex> lk(s->mu);
       s->busy_s += now_s(s->t0) - t_round;
       s->node_updates += round_updates;
       s->resident.swap(keep);
-      for (auto& r : out) s->done.push_back(r);
-      s->in_flight -= out.size();
-      if (s->in_flight == 0) s->idle_cv.notify_all();
     }
   }
   if (e != cudaSuccess || gave_up) {
@@ -612,15 +661,19 @@ ilg_status ilg_server_create(uint64_t seed, uint64_t hbm_bytes, uint32_t max_slo
   if ((e = dev_alloc(&s->d_round, round_bytes(s->sms, max_slots))) != cudaSuccess) return bail(e, "cudaMalloc");
   if ((e = dev_alloc(&s->d_col, sizeof(unsigned long long) * kServerMaxSide)) != cudaSuccess) return bail(e, "cudaMalloc");
   if ((e = dev_alloc(&s->d_row, sizeof(unsigned long long) * kServerMaxSide)) != cudaSuccess) return bail(e, "cudaMalloc");
-  if ((e = dev_alloc(&s->d_mass, sizeof(unsigned long long))) != cudaSuccess) return bail(e, "cudaMalloc");
+  if ((e = dev_alloc(&s->d_out, sizeof(unsigned long long) * kOutWords * max_slots)) != cudaSuccess) return bail(e, "cudaMalloc");
   if ((e = dev_alloc(&s->d_modes, sizeof(int32_t) * 2)) != cudaSuccess) return bail(e, "cudaMalloc");
-  if ((e = dev_alloc(&s->d_res, sizeof(double) * 4)) != cudaSuccess) return bail(e, "cudaMalloc");
   const int32_t mode1[2] = {1, 0};
   if ((e = cudaMemcpy(s->d_modes, mode1, sizeof(mode1), cudaMemcpyHostToDevice)) != cudaSuccess) return bail(e, "upload");
   if ((e = cudaStreamCreateWithFlags(&s->init_stream, cudaStreamNonBlocking)) != cudaSuccess)
     return bail(e, "cudaStreamCreate");
-  if ((e = cudaEventCreateWithFlags(&s->round_ev, cudaEventDisableTiming)) != cudaSuccess)
+  if ((e = cudaStreamCreateWithFlags(&s->out_stream, cudaStreamNonBlocking)) != cudaSuccess)
+    return bail(e, "cudaStreamCreate");
+  if ((e = cudaEventCreateWithFlags(&s->round_ev, cudaEventDisableTiming)) != cudaSuccess ||
+      (e = cudaEventCreateWithFlags(&s->out_ev, cudaEventDisableTiming)) != cudaSuccess)
     return bail(e, "cudaEventCreate");
+  if ((e = cudaMallocHost(&s->h_out, sizeof(unsigned long long) * kOutWords * max_slots)) != cudaSuccess)
+    return bail(e, "cudaMallocHost");
   if ((e = cudaMallocHost(&s->h_round, round_bytes(s->sms, max_slots))) != cudaSuccess) return bail(e, "cudaMallocHost");
   round_keys(seed, s->common.rk);
   s->common.key0 = uint32_t(seed);
@@ -718,6 +771,7 @@ ilg_status ilg_server_destroy(ilg_server* s) {
   if (s->worker.joinable()) s->worker.join();
   cudaStreamSynchronize(s->stream);
   if (s->init_stream) cudaStreamSynchronize(s->init_stream);
+  if (s->out_stream) cudaStreamSynchronize(s->out_stream);
   free_server(s);
   delete s;
   return ILG_OK;
