@@ -380,7 +380,7 @@ ilg_status ilg_lb_observables(ilg_lb* lb, const int32_t* modes, uint32_t nmodes,
  *   stream           cudaStream_t the work runs on
  *   mass, re, im, amp, Sk   host outputs as in ilg_observables (each may be NULL)
  * The results equal those of ilg_observables on the same state.  Scratch lives in a
- * static device array of about 530 KB that every GPU which loads the library holds
+ * static device array of about 610 KB that every GPU which loads the library holds
  * until the process exits; nothing is allocated or freed.  The first call on a device
  * looks up that array's device address (with the device current) and caches it:
  * make that first call before any stream capture.  All calls share the one array and

@@ -30,11 +30,12 @@ struct ilg_ctx {
   uint32_t* d_tables = nullptr;            // thinning table, rest table
   unsigned long long* d_fail = nullptr;    // [0] first failing step, ~0 if none; [1], [2] the
                                            // words of a several-step launch (launch_step_run)
-  unsigned long long* d_col = nullptr;     // Lx
-  unsigned long long* d_row = nullptr;     // Ly
+  // sums of a state (mass | column sums, Lx | row sums, Ly) in one array, cleared at once
   unsigned long long* d_mass = nullptr;
-  int32_t* d_modes = nullptr;
-  double* d_res = nullptr;
+  unsigned long long* d_col = nullptr;
+  unsigned long long* d_row = nullptr;
+  unsigned long long* d_proj = nullptr;    // scratch of the projections
+  unsigned long long* h_obs = nullptr;     // pinned, written by the projections: mass, 4 per mode
   uint32_t mode_cap = 0;
   uint32_t tb_depth = 0;                   // temporal blocking: steps per launch (0: off)
   uint32_t general = 0;                    // too many nodes would fail the fast collision: general at once
@@ -149,11 +150,9 @@ void free_ctx(ilg_ctx* c) {
   cudaFree(c->buf[1]);
   cudaFree(c->d_tables);
   cudaFree(c->d_fail);
-  cudaFree(c->d_col);
-  cudaFree(c->d_row);
   cudaFree(c->d_mass);
-  cudaFree(c->d_modes);
-  cudaFree(c->d_res);
+  cudaFree(c->d_proj);
+  if (c->h_obs) cudaFreeHost(c->h_obs);
   if (c->h_word) cudaFreeHost(c->h_word);
 }
 
@@ -214,9 +213,12 @@ ilg_status ilg_create(const ilg_params* params, void* stream, ilg_ctx** out) {
   const size_t block_words = c->Q == 9 ? kBlockWords9 : kBlockWords;
   if ((e = dev_alloc(&c->d_tables, sizeof(uint32_t) * block_words)) != cudaSuccess) return bail(e, "cudaMalloc tables");
   if ((e = dev_alloc(&c->d_fail, sizeof(unsigned long long) * kFailWords)) != cudaSuccess) return bail(e, "cudaMalloc flag");
-  if ((e = dev_alloc(&c->d_col, sizeof(unsigned long long) * c->p.Lx)) != cudaSuccess) return bail(e, "cudaMalloc sums");
-  if ((e = dev_alloc(&c->d_row, sizeof(unsigned long long) * c->p.Ly)) != cudaSuccess) return bail(e, "cudaMalloc sums");
-  if ((e = dev_alloc(&c->d_mass, sizeof(unsigned long long))) != cudaSuccess) return bail(e, "cudaMalloc mass");
+  if ((e = dev_alloc(&c->d_mass, sizeof(unsigned long long) * (1 + size_t(c->p.Lx) + c->p.Ly))) != cudaSuccess)
+    return bail(e, "cudaMalloc sums");
+  c->d_col = c->d_mass + 1;
+  c->d_row = c->d_col + c->p.Lx;
+  if ((e = dev_alloc(&c->d_proj, sizeof(unsigned long long) * kProjScratchWords)) != cudaSuccess)
+    return bail(e, "cudaMalloc projections");
   if ((e = cudaMallocHost(&c->h_word, sizeof(unsigned long long) * kFailWords)) != cudaSuccess) return bail(e, "cudaMallocHost");
 
   std::vector<uint32_t> tables(block_words, 0u);
@@ -229,6 +231,7 @@ ilg_status ilg_create(const ilg_params* params, void* stream, ilg_ctx** out) {
   if (e != cudaSuccess) return bail(e, "copy tables");
   e = cudaMemsetAsync(c->d_fail, 0xFF, sizeof(unsigned long long), c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_fail + 1, 0, 2 * sizeof(unsigned long long), c->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->d_proj, 0, sizeof(unsigned long long) * kProjScratchWords, c->stream);
   if (e != cudaSuccess) return bail(e, "reset flag");
   e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return bail(e, "cudaStreamSynchronize");
@@ -301,15 +304,24 @@ ilg_status ilg_init(ilg_ctx* c) {
   return ILG_OK;
 }
 
+// Sums of the current state into d_mass / d_col (and d_row).
+static ilg_status queue_sums(ilg_ctx* c, bool want_rows) {
+  const uint32_t Lx = c->p.Lx, Ly = c->p.Ly;
+  ILG_CUDA(c, cudaMemsetAsync(c->d_mass, 0, sizeof(unsigned long long) * (1 + size_t(Lx) + (want_rows ? Ly : 0)), c->stream),
+           "clear sums");
+  ILG_CUDA(c, launch_sums(c->Q, c->buf[c->cur], Lx, Ly, c->d_col, c->d_row, c->d_mass, want_rows ? 1 : 0, uint32_t(c->sms),
+                          c->stream),
+           "sums kernel");
+  return ILG_OK;
+}
+
 // mean occupation of the current state decides between the collision paths
 static ilg_status update_path_choice(ilg_ctx* c) {
-  const uint32_t Lx = c->p.Lx, Ly = c->p.Ly;
-  ILG_CUDA(c, cudaMemsetAsync(c->d_col, 0, sizeof(unsigned long long) * Lx, c->stream), "clear sums");
-  ILG_CUDA(c, launch_sums(c->Q, c->buf[c->cur], Lx, Ly, c->d_col, c->d_row, 0, c->stream), "sums kernel");
-  ILG_CUDA(c, launch_project(c->d_col, c->d_row, Lx, Ly, nullptr, 0, nullptr, c->d_mass, c->stream), "mass kernel");
+  const ilg_status st = queue_sums(c, false);
+  if (st != ILG_OK) return st;
   ILG_CUDA(c, cudaMemcpyAsync(c->h_word, c->d_mass, sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream),
            "read mass");
-  ILG_CUDA(c, cudaStreamSynchronize(c->stream), "read mass");
+  ILG_CUDA(c, cudaStreamSynchronize(c->stream), "copy state in");
   c->general = general_path(c->p.lattice, c->p.theta, c->omega_star, double(*c->h_word) / (double(c->nodes) * c->Q));
   return ILG_OK;
 }
@@ -319,10 +331,9 @@ static ilg_status set_state_impl(ilg_ctx* c, const uint16_t* src, size_t n, uint
   if (n != c->nodes * c->Q) return fail(c, ILG_E_INVALID, "state size must be Q * Lx * Ly");
   if (t >= (uint64_t(1) << 32)) return fail(c, ILG_E_INVALID, "t must be below 2^32");
   ILG_CUDA(c, cudaMemcpyAsync(c->buf[c->cur], src, sizeof(uint16_t) * n, kind, c->stream), "copy state in");
-  ILG_CUDA(c, cudaStreamSynchronize(c->stream), "copy state in");
   c->t = t;
   c->has_state = true;
-  return update_path_choice(c);
+  return update_path_choice(c);  // (waits for the copy too)
 }
 
 static ilg_status get_state_impl(ilg_ctx* c, uint16_t* dst, size_t n, uint64_t* t, cudaMemcpyKind kind) {
@@ -662,35 +673,29 @@ ilg_status ilg_observables(ilg_ctx* c, const int32_t* modes, uint32_t nmodes, ui
     if (my != 0) want_rows = true;
   }
   if (nmodes > c->mode_cap) {
-    cudaFree(c->d_modes);
-    cudaFree(c->d_res);
-    c->d_modes = nullptr;
-    c->d_res = nullptr;
+    if (c->h_obs) cudaFreeHost(c->h_obs);
+    c->h_obs = nullptr;
     c->mode_cap = 0;
-    ILG_CUDA(c, dev_alloc(&c->d_modes, sizeof(int32_t) * 2 * nmodes), "cudaMalloc modes");
-    ILG_CUDA(c, dev_alloc(&c->d_res, sizeof(double) * 4 * nmodes), "cudaMalloc modes");
+    ILG_CUDA(c, cudaMallocHost(&c->h_obs, sizeof(unsigned long long) * (1 + 4 * size_t(nmodes))), "cudaMallocHost modes");
     c->mode_cap = nmodes;
   }
   const uint32_t Lx = c->p.Lx, Ly = c->p.Ly;
-  ILG_CUDA(c, cudaMemsetAsync(c->d_col, 0, sizeof(unsigned long long) * Lx, c->stream), "clear sums");
-  if (want_rows) ILG_CUDA(c, cudaMemsetAsync(c->d_row, 0, sizeof(unsigned long long) * Ly, c->stream), "clear sums");
+  const ilg_status st = queue_sums(c, want_rows);
+  if (st != ILG_OK) return st;
+  const double* const res = reinterpret_cast<const double*>(c->h_obs + 1);
   if (nmodes)
-    ILG_CUDA(c, cudaMemcpyAsync(c->d_modes, modes, sizeof(int32_t) * 2 * nmodes, cudaMemcpyHostToDevice, c->stream),
-             "copy modes");
-  ILG_CUDA(c, launch_sums(c->Q, c->buf[c->cur], Lx, Ly, c->d_col, c->d_row, want_rows ? 1 : 0, c->stream), "sums kernel");
-  ILG_CUDA(c, launch_project(c->d_col, c->d_row, Lx, Ly, c->d_modes, nmodes, c->d_res, c->d_mass, c->stream),
-           "projection kernel");
-  std::vector<double> res(size_t(4) * nmodes);
-  unsigned long long M = 0;
-  if (nmodes)
-    ILG_CUDA(c, cudaMemcpyAsync(res.data(), c->d_res, sizeof(double) * res.size(), cudaMemcpyDeviceToHost, c->stream),
-             "copy results");
-  ILG_CUDA(c, cudaMemcpyAsync(&M, c->d_mass, sizeof(M), cudaMemcpyDeviceToHost, c->stream), "copy mass");
+    ILG_CUDA(c, launch_project(ProjWork{c->d_col, c->d_row, c->d_mass, c->d_proj}, Lx, Ly, modes, nmodes,
+                               const_cast<double*>(res), c->h_obs, c->stream),
+             "projection kernel");
+  else
+    ILG_CUDA(c, cudaMemcpyAsync(c->h_word, c->d_mass, sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream),
+             "copy mass");
   if (col_sums)
     ILG_CUDA(c, cudaMemcpyAsync(col_sums, c->d_col, sizeof(int64_t) * Lx, cudaMemcpyDeviceToHost, c->stream), "copy sums");
   if (row_sums)
     ILG_CUDA(c, cudaMemcpyAsync(row_sums, c->d_row, sizeof(int64_t) * Ly, cudaMemcpyDeviceToHost, c->stream), "copy sums");
   ILG_CUDA(c, cudaStreamSynchronize(c->stream), "observables");
+  const unsigned long long M = nmodes ? c->h_obs[0] : *c->h_word;
   if (t) *t = c->t;
   if (mass) *mass = M;
   for (uint32_t i = 0; i < nmodes; ++i) {

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstring>
 
 #include "ilg_collide.cuh"
 #include "ilg_device.cuh"
@@ -230,52 +231,125 @@ cudaError_t launch_init(int Q, const InitArgs& a, uint16_t* out, int grid, cudaS
 }
 
 // --------------------------------------------------------------------------
-// integer sums: N(x,y) = sum_i n_i; column sums C(x) over a block of rows, one
-// 64-bit atomic per column and block; row sums R(y) by warp shuffles, one
-// atomic per warp and row.
+// integer sums: N(x,y) = sum_i n_i; column sums C(x), row sums R(y) and the mass.  A block
+// takes 32 vectors of VEC nodes (16-byte loads where rows are a multiple of 8 and the
+// state is aligned) by 8 R rows, adds its eight row groups in shared memory and issues one
+// 64-bit atomic per column; row sums by warp shuffles, one atomic per warp and row.
+// Bound: HBM for states beyond L2 (16384^2 D2Q5: 0.39 ms, 0.98 of the measured copy rate),
+// the latency of a thread's R dependent rows for small ones: R is as small as still gives
+// every SM four blocks (1024^2: 4 us where 64 rows in one thread took 45).
 // --------------------------------------------------------------------------
-constexpr int kSumRows = 64;
+constexpr uint32_t kSumGroups = 8;    // row groups (warps) of a block
+constexpr uint32_t kSumMaxRows = 64;  // rows per thread at most
+
+template <int Q, int VEC>
+__global__ void __launch_bounds__(32 * kSumGroups) sums_kernel(const uint16_t* __restrict__ in, uint32_t Lx, uint32_t Ly,
+                                                               uint32_t R, unsigned long long* __restrict__ col,
+                                                               unsigned long long* __restrict__ row,
+                                                               unsigned long long* __restrict__ mass, int want_rows) {
+  __shared__ uint32_t red[kSumGroups][32 * VEC];
+  __shared__ unsigned long long total[kSumGroups];
+  const uint32_t tx = threadIdx.x & 31u, ty = threadIdx.x >> 5;
+  const uint64_t x = (uint64_t(blockIdx.x) * 32 + tx) * VEC;
+  const size_t plane = size_t(Lx) * Ly;
+  const uint32_t chunks = (Ly + kSumGroups * R - 1) / (kSumGroups * R);
+  unsigned long long sum = 0;
+  for (uint32_t chunk = blockIdx.y; chunk < chunks; chunk += gridDim.y) {
+    const uint32_t y0 = chunk * kSumGroups * R;
+    uint32_t acc[VEC];  // at most 64 rows of 9 x 65535
+#pragma unroll
+    for (int j = 0; j < VEC; ++j) acc[j] = 0;
+#pragma unroll 2
+    for (uint32_t k = 0; k < R; ++k) {
+      const uint32_t y = y0 + ty + kSumGroups * k;
+      if (y >= Ly || y < y0) break;
+      uint32_t n[VEC];
+#pragma unroll
+      for (int j = 0; j < VEC; ++j) n[j] = 0;
+      if (x < Lx) {
+        const uint16_t* p = in + (size_t(y) * Lx + x);
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+          if constexpr (VEC == 8) {
+            const uint4 w = __ldg(reinterpret_cast<const uint4*>(p + i * plane));
+            n[0] += w.x & 0xFFFFu;
+            n[1] += w.x >> 16;
+            n[2] += w.y & 0xFFFFu;
+            n[3] += w.y >> 16;
+            n[4] += w.z & 0xFFFFu;
+            n[5] += w.z >> 16;
+            n[6] += w.w & 0xFFFFu;
+            n[7] += w.w >> 16;
+          } else {
+            n[0] += p[i * plane];
+          }
+        }
+      }
+      uint32_t N = 0;
+#pragma unroll
+      for (int j = 0; j < VEC; ++j) {
+        acc[j] += n[j];
+        N += n[j];
+      }
+      if (want_rows) {
+        N = __reduce_add_sync(0xFFFFFFFFu, N);  // at most 256 nodes of 9 x 65535
+        if (tx == 0 && N) atomicAdd(row + y, static_cast<unsigned long long>(N));
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < VEC; ++j) red[ty][tx * VEC + j] = acc[j];
+    __syncthreads();
+    const uint64_t c = uint64_t(blockIdx.x) * 32 * VEC + threadIdx.x;
+    if (threadIdx.x < 32 * VEC && c < Lx) {
+      unsigned long long C = 0;
+#pragma unroll
+      for (uint32_t g = 0; g < kSumGroups; ++g) C += red[g][threadIdx.x];
+      if (C) atomicAdd(col + c, C);
+      sum += C;
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xFFFFFFFFu, sum, o);
+  if (tx == 0) total[ty] = sum;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned long long M = 0;
+    for (uint32_t g = 0; g < kSumGroups; ++g) M += total[g];
+    if (M) atomicAdd(mass, M);
+  }
+}
 
 template <int Q>
-__global__ void __launch_bounds__(256) sums_kernel(const uint16_t* __restrict__ in, uint32_t Lx, uint32_t Ly,
-                                                   unsigned long long* __restrict__ col,
-                                                   unsigned long long* __restrict__ row, int want_rows) {
-  const uint32_t x = blockIdx.x * blockDim.x + threadIdx.x;
-  const uint32_t y0 = blockIdx.y * kSumRows;
-  const uint32_t y1 = min(Ly, y0 + kSumRows);
-  const size_t plane = size_t(Lx) * Ly;
-  uint64_t acc = 0;
-  for (uint32_t y = y0; y < y1; ++y) {
-    uint32_t N = 0;
-    if (x < Lx) {
-      const size_t at = size_t(y) * Lx + x;
-#pragma unroll
-      for (int i = 0; i < Q; ++i) N += in[i * plane + at];
-    }
-    acc += N;
-    if (want_rows) {
-      uint64_t v = N;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xFFFFFFFFu, v, o);
-      if ((threadIdx.x & 31) == 0 && v) atomicAdd(row + y, static_cast<unsigned long long>(v));
-    }
-  }
-  if (x < Lx && acc) atomicAdd(col + x, static_cast<unsigned long long>(acc));
+static void sums_launch(const uint16_t* in, uint32_t Lx, uint32_t Ly, unsigned long long* col, unsigned long long* row,
+                        unsigned long long* mass, int want_rows, uint32_t sms, cudaStream_t s) {
+  const bool wide = Lx % 8 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0;
+  const uint32_t width = wide ? 256 : 32;
+  const uint32_t gx = uint32_t((uint64_t(Lx) + width - 1) / width);
+  const uint64_t groups = (uint64_t(Ly) + kSumGroups - 1) / kSumGroups;  // rows per thread if one block took all
+  const uint32_t want = std::max<uint32_t>(1, 4 * sms / gx);            // blocks along y
+  const uint32_t R = uint32_t(std::min<uint64_t>(kSumMaxRows, std::max<uint64_t>(1, groups / want)));
+  const dim3 grid(gx, uint32_t(std::min<uint64_t>(65535, (groups + R - 1) / R)));
+  if (wide) sums_kernel<Q, 8><<<grid, 32 * kSumGroups, 0, s>>>(in, Lx, Ly, R, col, row, mass, want_rows);
+  else sums_kernel<Q, 1><<<grid, 32 * kSumGroups, 0, s>>>(in, Lx, Ly, R, col, row, mass, want_rows);
 }
 
 cudaError_t launch_sums(int Q, const uint16_t* in, uint32_t Lx, uint32_t Ly, unsigned long long* col,
-                        unsigned long long* row, int want_rows, cudaStream_t s) {
-  dim3 grid((Lx + 255) / 256, (Ly + kSumRows - 1) / kSumRows);
-  if (Q == 9) sums_kernel<9><<<grid, 256, 0, s>>>(in, Lx, Ly, col, row, want_rows);
-  else if (Q == 3) sums_kernel<3><<<grid, 256, 0, s>>>(in, Lx, Ly, col, row, want_rows);
-  else sums_kernel<5><<<grid, 256, 0, s>>>(in, Lx, Ly, col, row, want_rows);
+                        unsigned long long* row, unsigned long long* mass, int want_rows, uint32_t sms, cudaStream_t s) {
+  if (Q == 9) sums_launch<9>(in, Lx, Ly, col, row, mass, want_rows, sms, s);
+  else if (Q == 3) sums_launch<3>(in, Lx, Ly, col, row, mass, want_rows, sms, s);
+  else sums_launch<5>(in, Lx, Ly, col, row, mass, want_rows, sms, s);
   return cudaGetLastError();
 }
 
 // --------------------------------------------------------------------------
-// projections: one block per mode.  D(x) = L*S(x) - M in exact int64, then
-// compensated dot products (Ogita, Rump & Oishi 2005: error-free TwoProduct by
-// FMA, TwoSum) with cos and sin of 2 pi r / L, r = (m*x) mod L.
+// projections: the entries of a mode cut into chunks, one block each.  D(x) = L*S(x) - M
+// in exact int64, then compensated dot products (Ogita, Rump & Oishi 2005: error-free
+// TwoProduct by FMA, TwoSum) with cos and sin of 2 pi r / L, r = (m*x) mod L; the block
+// that finishes last adds the chunks' pairs in their order (the same result every time).
+// Bound: the fp64 pipe (about 65 double instructions per entry, 2 lanes per SM and cycle),
+// so a mode is spread over as many SMs as its length feeds (one block per mode before:
+// 64 modes of 16384 entries 0.33 -> 0.15 ms, one mode of 2^22 71 -> 1 ms).
 // --------------------------------------------------------------------------
 __device__ __forceinline__ void two_sum(double a, double b, double& s, double& e) {
   s = a + b;
@@ -299,40 +373,24 @@ struct Dot2 {
   }
 };
 
-__global__ void __launch_bounds__(256) project_kernel(const unsigned long long* __restrict__ colsum,
-                                                      const unsigned long long* __restrict__ rowsum,
-                                                      uint32_t Lx, uint32_t Ly, const int32_t* __restrict__ modes,
-                                                      double* __restrict__ res, unsigned long long* __restrict__ mass) {
-  __shared__ long long sM[8];
-  __shared__ double sv[4][8];
-  const int mi = blockIdx.x;
-  const int32_t mx = modes[2 * mi], my = modes[2 * mi + 1];
-  const bool along_x = (my == 0);
-  const unsigned long long* S = along_x ? colsum : rowsum;
-  const uint32_t L = along_x ? Lx : Ly;
-  const int64_t mraw = along_x ? mx : my;
-  const uint64_t m = uint64_t(((mraw % int64_t(L)) + int64_t(L)) % int64_t(L));
+constexpr int kProjThreads = 64;
+
+struct ProjArgs {
+  const unsigned long long* colsum;
+  const unsigned long long* rowsum;
+  const unsigned long long* mass_in;
+  uint32_t Lx, Ly;
+  uint32_t nmodes;
+  double* part;            // (re.s, re.c, im.s, im.c) per chunk and mode
+  unsigned int* ticket;    // per mode, 0 between launches
+  double* res;             // 4 per mode (device or mapped host memory)
+  unsigned long long* mass_out;
+  int32_t modes[2 * kProjModes];
+};
+
+// fixed tree over the block's threads: warp shuffles, then the warps' pairs
+__device__ __forceinline__ void block_dot2(Dot2& re, Dot2& im, double (*sv)[kProjThreads / 32]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-
-  long long part = 0;
-  for (uint32_t x = threadIdx.x; x < L; x += blockDim.x) part += static_cast<long long>(S[x]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(0xFFFFFFFFu, part, o);
-  if (lane == 0) sM[warp] = part;
-  __syncthreads();
-  long long M = 0;
-  for (int w = 0; w < int(blockDim.x >> 5); ++w) M += sM[w];
-
-  Dot2 re{0.0, 0.0}, im{0.0, 0.0};
-  for (uint32_t x = threadIdx.x; x < L; x += blockDim.x) {
-    const long long D = static_cast<long long>(L) * static_cast<long long>(S[x]) - M;
-    const uint32_t r = uint32_t((m * x) % L);
-    double sn, cs;
-    sincospi(2.0 * double(r) / double(L), &sn, &cs);
-    re.add_product(cs, double(D));
-    im.add_product(sn, double(D));
-  }
-  // tree over the block: warp shuffles, then the warps' partial pairs
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     Dot2 ore{__shfl_down_sync(0xFFFFFFFFu, re.s, o), __shfl_down_sync(0xFFFFFFFFu, re.c, o)};
@@ -340,49 +398,100 @@ __global__ void __launch_bounds__(256) project_kernel(const unsigned long long* 
     re.merge(ore);
     im.merge(oim);
   }
+  __syncthreads();
   if (lane == 0) {
-    sv[0][warp] = re.s; sv[1][warp] = re.c; sv[2][warp] = im.s; sv[3][warp] = im.c;
+    sv[0][warp] = re.s;
+    sv[1][warp] = re.c;
+    sv[2][warp] = im.s;
+    sv[3][warp] = im.c;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    Dot2 R{sv[0][0], sv[1][0]}, I{sv[2][0], sv[3][0]};
-    for (int w = 1; w < int(blockDim.x >> 5); ++w) {
-      R.merge(Dot2{sv[0][w], sv[1][w]});
-      I.merge(Dot2{sv[2][w], sv[3][w]});
+    for (int w = 1; w < kProjThreads / 32; ++w) {
+      re.merge(Dot2{sv[0][w], sv[1][w]});
+      im.merge(Dot2{sv[2][w], sv[3][w]});
     }
-    const double vre = (R.s + R.c) / double(L);
-    const double vim = (I.s + I.c) / double(L);
-    const double K = double(Lx) * double(Ly);
-    res[4 * mi + 0] = vre;
-    res[4 * mi + 1] = vim;
-    res[4 * mi + 2] = vim / (K / 2.0);
-    res[4 * mi + 3] = (vre * vre + vim * vim) / K;
-    if (mi == 0) *mass = static_cast<unsigned long long>(M);
   }
 }
 
-// mass alone (no modes requested)
-__global__ void mass_kernel(const unsigned long long* __restrict__ colsum, uint32_t Lx,
-                            unsigned long long* __restrict__ mass) {
-  __shared__ unsigned long long sM[8];
-  unsigned long long part = 0;
-  for (uint32_t x = threadIdx.x; x < Lx; x += blockDim.x) part += colsum[x];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(0xFFFFFFFFu, part, o);
-  if ((threadIdx.x & 31) == 0) sM[threadIdx.x >> 5] = part;
-  __syncthreads();
+__global__ void __launch_bounds__(kProjThreads) project_kernel(const __grid_constant__ ProjArgs a) {
+  __shared__ double sv[4][kProjThreads / 32];
+  __shared__ bool last;
+  const uint32_t mi = blockIdx.y, P = gridDim.x;
+  const int32_t mx = a.modes[2 * mi], my = a.modes[2 * mi + 1];
+  const bool along_x = (my == 0);
+  const unsigned long long* S = along_x ? a.colsum : a.rowsum;
+  const uint32_t L = along_x ? a.Lx : a.Ly;
+  const int64_t mraw = along_x ? mx : my;
+  const uint64_t m = uint64_t(((mraw % int64_t(L)) + int64_t(L)) % int64_t(L));
+  const long long M = static_cast<long long>(*a.mass_in);
+  const uint32_t x0 = uint32_t(uint64_t(L) * blockIdx.x / P), x1 = uint32_t(uint64_t(L) * (blockIdx.x + 1) / P);
+  Dot2 re{0.0, 0.0}, im{0.0, 0.0};
+  for (uint64_t x = uint64_t(x0) + threadIdx.x; x < x1; x += kProjThreads) {
+    const long long D = static_cast<long long>(L) * static_cast<long long>(S[x]) - M;
+    const uint32_t r = uint32_t((m * x) % L);
+    double sn, cs;
+    sincospi(2.0 * double(r) / double(L), &sn, &cs);
+    re.add_product(cs, double(D));
+    im.add_product(sn, double(D));
+  }
+  block_dot2(re, im, sv);
+  if (P > 1) {
+    volatile double* const part = a.part + size_t(mi) * P * 4;
+    if (threadIdx.x == 0) {
+      volatile double* const q = part + 4 * blockIdx.x;
+      q[0] = re.s;
+      q[1] = re.c;
+      q[2] = im.s;
+      q[3] = im.c;
+      __threadfence();
+      last = atomicAdd(a.ticket + mi, 1u) == P - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    re = im = Dot2{0.0, 0.0};
+    for (uint32_t k = threadIdx.x; k < P; k += kProjThreads) {
+      const volatile double* const q = part + 4 * k;
+      re.merge(Dot2{q[0], q[1]});
+      im.merge(Dot2{q[2], q[3]});
+    }
+    block_dot2(re, im, sv);
+  }
   if (threadIdx.x == 0) {
-    unsigned long long M = 0;
-    for (int w = 0; w < int(blockDim.x >> 5); ++w) M += sM[w];
-    *mass = M;
+    if (P > 1) a.ticket[mi] = 0;
+    const double vre = (re.s + re.c) / double(L);
+    const double vim = (im.s + im.c) / double(L);
+    const double K = double(a.Lx) * double(a.Ly);
+    a.res[4 * mi + 0] = vre;
+    a.res[4 * mi + 1] = vim;
+    a.res[4 * mi + 2] = vim / (K / 2.0);
+    a.res[4 * mi + 3] = (vre * vre + vim * vim) / K;
+    if (mi == 0) *a.mass_out = static_cast<unsigned long long>(M);
   }
 }
 
-cudaError_t launch_project(const unsigned long long* col, const unsigned long long* row, uint32_t Lx,
-                           uint32_t Ly, const int32_t* modes, uint32_t nmodes, double* res,
-                           unsigned long long* mass, cudaStream_t s) {
-  if (nmodes == 0) mass_kernel<<<1, 256, 0, s>>>(col, Lx, mass);
-  else project_kernel<<<nmodes, 256, 0, s>>>(col, row, Lx, Ly, modes, res, mass);
+cudaError_t launch_project(const ProjWork& w, uint32_t Lx, uint32_t Ly, const int32_t* modes, uint32_t nmodes,
+                           double* res, unsigned long long* mass, cudaStream_t s) {
+  ProjArgs a{};
+  a.colsum = w.col;
+  a.rowsum = w.row;
+  a.mass_in = w.mass;
+  a.Lx = Lx;
+  a.Ly = Ly;
+  a.part = reinterpret_cast<double*>(w.scratch);
+  a.ticket = reinterpret_cast<unsigned int*>(w.scratch + 4 * (kProjBlocks + kProjModes));
+  a.mass_out = mass;
+  for (uint32_t k = 0; k < nmodes; k += kProjModes) {
+    a.nmodes = std::min(nmodes - k, kProjModes);
+    a.res = res + size_t(4) * k;
+    std::memcpy(a.modes, modes + size_t(2) * k, sizeof(int32_t) * 2 * a.nmodes);
+    uint32_t L = 0;
+    for (uint32_t j = 0; j < a.nmodes; ++j) L = std::max(L, a.modes[2 * j + 1] == 0 ? Lx : Ly);
+    const uint32_t P = uint32_t(std::min<uint64_t>(std::max<uint32_t>(1, kProjBlocks / a.nmodes),
+                                                   (uint64_t(L) + kProjThreads - 1) / kProjThreads));
+    project_kernel<<<dim3(P, a.nmodes), kProjThreads, 0, s>>>(a);
+  }
   return cudaGetLastError();
 }
 

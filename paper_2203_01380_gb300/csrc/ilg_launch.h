@@ -60,11 +60,23 @@ uint32_t step9_threads();
 uint32_t step9_blocks_per_sm();
 cudaError_t launch_step9(const StepArgs& a, const uint16_t* in, uint16_t* out, uint32_t t, unsigned long long* fail,
                          int grid, cudaStream_t s);
+// adds to col (Lx words), row (Ly words; want_rows) and mass: zero them first
 cudaError_t launch_sums(int Q, const uint16_t* in, uint32_t Lx, uint32_t Ly, unsigned long long* col,
-                        unsigned long long* row, int want_rows, cudaStream_t s);
-cudaError_t launch_project(const unsigned long long* col, const unsigned long long* row, uint32_t Lx,
-                           uint32_t Ly, const int32_t* modes, uint32_t nmodes, double* res,
-                           unsigned long long* mass, cudaStream_t s);
+                        unsigned long long* row, unsigned long long* mass, int want_rows, uint32_t sms, cudaStream_t s);
+constexpr uint32_t kProjModes = 256;    // modes of one launch
+constexpr uint32_t kProjBlocks = 2048;  // blocks of one launch: chunks of a mode x modes
+constexpr size_t kProjScratchWords = 4 * (kProjBlocks + kProjModes) + kProjModes / 2;
+// the sums of a state, and kProjScratchWords 8-byte words whose last kProjModes / 2 (the
+// tickets) are 0 between launches
+struct ProjWork {
+  const unsigned long long* col;
+  const unsigned long long* row;
+  const unsigned long long* mass;
+  unsigned long long* scratch;
+};
+// modes: host, nmodes > 0 pairs; res (4 doubles per mode) and mass: device or mapped host memory
+cudaError_t launch_project(const ProjWork& w, uint32_t Lx, uint32_t Ly, const int32_t* modes, uint32_t nmodes,
+                           double* res, unsigned long long* mass, cudaStream_t s);
 cudaError_t launch_philox(const uint32_t* ctr, uint32_t k0, uint32_t k1, uint32_t* out, size_t n,
                           cudaStream_t s);
 

@@ -12,6 +12,7 @@
 // return the results.
 #include <cuda_runtime.h>
 
+#include <cstring>
 #include <mutex>
 #include <string>
 
@@ -24,13 +25,14 @@ constexpr uint32_t kMaxSide = 32768;   // largest Lx and Ly
 constexpr uint32_t kMaxModes = 256;    // largest number of modes per call
 constexpr int kMaxDevices = 64;
 
-// scratch layout, in 8-byte words: col[kMaxSide] | row[kMaxSide] | mass | res[4 kMaxModes] | modes
-constexpr size_t kColOff = 0;
+// scratch layout, in 8-byte words: mass | col[kMaxSide] | row[kMaxSide] | result mass and
+// res[4 kMaxModes] | the projections' scratch (zero between calls where they need it)
+constexpr size_t kMassOff = 0;
+constexpr size_t kColOff = kMassOff + 1;
 constexpr size_t kRowOff = kColOff + kMaxSide;
-constexpr size_t kMassOff = kRowOff + kMaxSide;
-constexpr size_t kResOff = kMassOff + 1;
-constexpr size_t kModesOff = kResOff + 4 * kMaxModes;
-constexpr size_t kScratchWords = kModesOff + kMaxModes;  // modes: kMaxModes int32 pairs
+constexpr size_t kResOff = kRowOff + kMaxSide;
+constexpr size_t kProjOff = kResOff + 1 + 4 * kMaxModes;
+constexpr size_t kScratchWords = kProjOff + ilg::kProjScratchWords;
 
 static __device__ __align__(256) unsigned long long noalloc_scratch[kScratchWords];
 
@@ -84,31 +86,30 @@ extern "C" ilg_status ilg_observables_noalloc(int32_t lattice, uint32_t Lx, uint
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int Q = lattice == ILG_D1Q3 ? 3 : (lattice == ILG_D2Q5 ? 5 : 9);
+  int sms = 0;
+  e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  unsigned long long* mass_sum = base + kMassOff;
   unsigned long long* col = base + kColOff;
   unsigned long long* row = base + kRowOff;
-  unsigned long long* d_mass = base + kMassOff;
-  double* res = reinterpret_cast<double*>(base + kResOff);
-  int32_t* d_modes = reinterpret_cast<int32_t*>(base + kModesOff);
+  unsigned long long* res = base + kResOff;
   // the array keeps the previous call's contents: clear the sums that accumulate
-  e = cudaMemsetAsync(col, 0, sizeof(unsigned long long) * Lx, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(mass_sum, 0, sizeof(unsigned long long) * (1 + size_t(Lx)), s);
   if (e == cudaSuccess && rows) e = cudaMemsetAsync(row, 0, sizeof(unsigned long long) * Ly, s);
+  if (e == cudaSuccess) e = ilg::launch_sums(Q, state, Lx, Ly, col, row, mass_sum, rows ? 1 : 0, uint32_t(sms), s);
   if (e == cudaSuccess && nmodes)
-    e = cudaMemcpyAsync(d_modes, modes, sizeof(int32_t) * 2 * nmodes, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = ilg::launch_sums(Q, state, Lx, Ly, col, row, rows ? 1 : 0, s);
-  if (e == cudaSuccess) e = ilg::launch_project(col, row, Lx, Ly, d_modes, nmodes, res, d_mass, s);
-  double h_res[4 * kMaxModes];
-  unsigned long long h_mass = 0;
-  if (e == cudaSuccess && nmodes)
-    e = cudaMemcpyAsync(h_res, res, sizeof(double) * 4 * nmodes, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&h_mass, d_mass, sizeof(h_mass), cudaMemcpyDeviceToHost, s);
+    e = ilg::launch_project(ilg::ProjWork{col, row, mass_sum, base + kProjOff}, Lx, Ly, modes, nmodes,
+                            reinterpret_cast<double*>(res + 1), res, s);
+  double h_res[1 + 4 * kMaxModes];
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(h_res, nmodes ? res : mass_sum, sizeof(double) * (1 + 4 * nmodes), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return context_free_fail(ILG_E_CUDA, std::string("ilg_observables_noalloc: ") + cudaGetErrorString(e));
-  if (mass) *mass = h_mass;
+  if (mass) std::memcpy(mass, h_res, sizeof(uint64_t));
   for (uint32_t i = 0; i < nmodes; ++i) {
-    if (re) re[i] = h_res[4 * i + 0];
-    if (im) im[i] = h_res[4 * i + 1];
-    if (amp) amp[i] = h_res[4 * i + 2];
-    if (Sk) Sk[i] = h_res[4 * i + 3];
+    if (re) re[i] = h_res[1 + 4 * i + 0];
+    if (im) im[i] = h_res[1 + 4 * i + 1];
+    if (amp) amp[i] = h_res[1 + 4 * i + 2];
+    if (Sk) Sk[i] = h_res[1 + 4 * i + 3];
   }
   return ILG_OK;
 }

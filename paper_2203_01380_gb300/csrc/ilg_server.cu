@@ -121,9 +121,8 @@ struct ilg_server {
   uint32_t* d_first = nullptr;         // sms + 1
   // of a round: barrier word, block cycles, failing steps, a word for a wait that gave up
   unsigned long long* d_round = nullptr;
-  unsigned long long* d_col = nullptr;
-  unsigned long long* d_row = nullptr;
-  int32_t* d_modes = nullptr;
+  unsigned long long* d_sums = nullptr;   // mass | column sums, kServerMaxSide
+  unsigned long long* d_proj = nullptr;   // scratch of the projections
   // observables of the requests a round finished, kOutWords words each: res[4], mass
   unsigned long long* d_out = nullptr;
   unsigned long long* h_out = nullptr;    // pinned
@@ -172,9 +171,8 @@ void free_server(ilg_server* s) {
   cudaFree(s->d_shares);
   cudaFree(s->d_first);
   cudaFree(s->d_round);
-  cudaFree(s->d_col);
-  cudaFree(s->d_row);
-  cudaFree(s->d_modes);
+  cudaFree(s->d_sums);
+  cudaFree(s->d_proj);
   cudaFree(s->d_out);
   if (s->h_out) cudaFreeHost(s->h_out);
   if (s->out_ev) cudaEventDestroy(s->out_ev);
@@ -340,10 +338,14 @@ cudaError_t queue_results(ilg_server* s, const std::vector<Resident>& out) {
     if (!has_result(r)) continue;
     const uint32_t Lx = r.rq.p.Lx, Ly = r.rq.p.Ly;
     unsigned long long* const to = s->d_out + kOutWords * i;
-    e = cudaMemsetAsync(s->d_col, 0, sizeof(unsigned long long) * Lx, s->stream);
-    if (e == cudaSuccess) e = launch_sums(5, state_of(s, r), Lx, Ly, s->d_col, s->d_row, 0, s->stream);
+    static const int32_t kMode[2] = {1, 0};
+    unsigned long long* const col = s->d_sums + 1;
+    e = cudaMemsetAsync(s->d_sums, 0, sizeof(unsigned long long) * (1 + size_t(Lx)), s->stream);
     if (e == cudaSuccess)
-      e = launch_project(s->d_col, s->d_row, Lx, Ly, s->d_modes, 1, reinterpret_cast<double*>(to), to + 4, s->stream);
+      e = launch_sums(5, state_of(s, r), Lx, Ly, col, nullptr, s->d_sums, 0, uint32_t(s->sms), s->stream);
+    if (e == cudaSuccess)
+      e = launch_project(ProjWork{col, nullptr, s->d_sums, s->d_proj}, Lx, Ly, kMode, 1, reinterpret_cast<double*>(to),
+                         to + 4, s->stream);
   }
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(s->h_out, s->d_out, sizeof(unsigned long long) * kOutWords * out.size(), cudaMemcpyDeviceToHost,
@@ -659,12 +661,10 @@ ilg_status ilg_server_create(uint64_t seed, uint64_t hbm_bytes, uint32_t max_slo
   if ((e = dev_alloc(&s->d_shares, sizeof(WorkShare) * (size_t(s->sms) + max_slots))) != cudaSuccess) return bail(e, "cudaMalloc");
   if ((e = dev_alloc(&s->d_first, sizeof(uint32_t) * (size_t(s->sms) + 1))) != cudaSuccess) return bail(e, "cudaMalloc");
   if ((e = dev_alloc(&s->d_round, round_bytes(s->sms, max_slots))) != cudaSuccess) return bail(e, "cudaMalloc");
-  if ((e = dev_alloc(&s->d_col, sizeof(unsigned long long) * kServerMaxSide)) != cudaSuccess) return bail(e, "cudaMalloc");
-  if ((e = dev_alloc(&s->d_row, sizeof(unsigned long long) * kServerMaxSide)) != cudaSuccess) return bail(e, "cudaMalloc");
+  if ((e = dev_alloc(&s->d_sums, sizeof(unsigned long long) * (1 + kServerMaxSide))) != cudaSuccess) return bail(e, "cudaMalloc");
+  if ((e = dev_alloc(&s->d_proj, sizeof(unsigned long long) * kProjScratchWords)) != cudaSuccess) return bail(e, "cudaMalloc");
+  if ((e = cudaMemset(s->d_proj, 0, sizeof(unsigned long long) * kProjScratchWords)) != cudaSuccess) return bail(e, "clear");
   if ((e = dev_alloc(&s->d_out, sizeof(unsigned long long) * kOutWords * max_slots)) != cudaSuccess) return bail(e, "cudaMalloc");
-  if ((e = dev_alloc(&s->d_modes, sizeof(int32_t) * 2)) != cudaSuccess) return bail(e, "cudaMalloc");
-  const int32_t mode1[2] = {1, 0};
-  if ((e = cudaMemcpy(s->d_modes, mode1, sizeof(mode1), cudaMemcpyHostToDevice)) != cudaSuccess) return bail(e, "upload");
   if ((e = cudaStreamCreateWithFlags(&s->init_stream, cudaStreamNonBlocking)) != cudaSuccess)
     return bail(e, "cudaStreamCreate");
   if ((e = cudaStreamCreateWithFlags(&s->out_stream, cudaStreamNonBlocking)) != cudaSuccess)
