@@ -113,13 +113,6 @@ void round_keys(uint64_t seed, uint32_t* rk) {
 namespace {
 using ilg::validate_params;
 
-// node-parallel kernels: `per_sm` resident blocks of `threads` threads on every SM
-int step_grid(const ilg_ctx* c, size_t per_sm, size_t threads = 256) {
-  const size_t blocks = (c->nodes + threads - 1) / threads;
-  const size_t cap = size_t(c->sms) * per_sm;
-  return int(blocks < cap ? blocks : cap);
-}
-
 // row-tiled step: one block per row at a time, per_sm blocks per SM
 int vec_grid(const ilg_ctx* c, size_t per_sm) {
   const size_t rows = c->p.Ly;
@@ -291,7 +284,7 @@ ilg_status ilg_init(ilg_ctx* c) {
   a.offset = d_off;
   a.count = d_cnt;
   a.table = d_tab;
-  if ((e = launch_init(c->Q, a, c->buf[c->cur], step_grid(c, 4), c->stream)) != cudaSuccess) {
+  if ((e = launch_init(c->Q, a, uint32_t(it.table.size()), c->buf[c->cur], uint32_t(c->sms), c->stream)) != cudaSuccess) {
     cleanup();
     return cuda_fail(c, e, "init kernel");
   }

@@ -225,8 +225,7 @@ ilg_status ilg_batch_init(ilg_batch* b) {
     a.offset = d_all + base[i];
     a.count = d_all + base[i] + cells;
     a.table = d_all + base[i] + 2 * cells;
-    const int grid = int(std::min<size_t>((q.Lx + 255) / 256, size_t(b->sms) * 4));
-    e = launch_init(3, a, b->d_state + b->desc[i].state_off, grid, b->stream);
+    e = launch_init(3, a, uint32_t(its[i].table.size()), b->d_state + b->desc[i].state_off, uint32_t(b->sms), b->stream);
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   cudaFree(d_all);

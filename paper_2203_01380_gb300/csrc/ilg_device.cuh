@@ -99,24 +99,29 @@ struct StepKeys {
   uint32_t A, G, H[NB], I[NB], J[NB];
 };
 
+// (of the stream with purpose tag `tag`, in its place in the fourth counter word)
 template <int NB>
-__device__ __forceinline__ StepKeys<NB> step_keys(const StepArgs& a, uint32_t t) {
+__device__ __forceinline__ StepKeys<NB> stream_keys(const uint32_t (&rk)[20], uint32_t t, uint32_t replica, uint32_t tag) {
   constexpr uint32_t M0 = 0xD2511F53u, M1 = 0xCD9E8D57u;
   StepKeys<NB> k;
-  const uint64_t P = uint64_t(M0) * t, R = uint64_t(M1) * a.replica;
-  k.A = uint32_t(R >> 32) ^ a.rk[0];
-  k.G = uint32_t(P) ^ a.rk[3];
+  const uint64_t P = uint64_t(M0) * t, R = uint64_t(M1) * replica;
+  k.A = uint32_t(R >> 32) ^ rk[0];
+  k.G = uint32_t(P) ^ rk[3];
 #pragma unroll
   for (int b = 0; b < NB; ++b) {
-    const uint32_t C = uint32_t(P >> 32) ^ (kDevTagStep | uint32_t(b)) ^ a.rk[1];  // round 2's x2
+    const uint32_t C = uint32_t(P >> 32) ^ (tag | uint32_t(b)) ^ rk[1];  // round 2's x2
     const uint64_t R1 = uint64_t(M1) * C;
-    const uint32_t E = uint32_t(R1 >> 32) ^ uint32_t(R) ^ a.rk[2];                  // round 3's x0
+    const uint32_t E = uint32_t(R1 >> 32) ^ uint32_t(R) ^ rk[2];          // round 3's x0
     const uint64_t P2 = uint64_t(M0) * E;
-    k.H[b] = uint32_t(R1) ^ a.rk[4];
-    k.I[b] = uint32_t(P2 >> 32) ^ a.rk[5];
+    k.H[b] = uint32_t(R1) ^ rk[4];
+    k.I[b] = uint32_t(P2 >> 32) ^ rk[5];
     k.J[b] = uint32_t(P2);
   }
   return k;
+}
+template <int NB>
+__device__ __forceinline__ StepKeys<NB> step_keys(const StepArgs& a, uint32_t t) {
+  return stream_keys<NB>(a.rk, t, a.replica, kDevTagStep);
 }
 
 // Words 0..4 NB - 1 of a node's tag-1 stream at the step its keys were made for.

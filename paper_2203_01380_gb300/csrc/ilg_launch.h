@@ -54,7 +54,8 @@ size_t step_tb_smem_bytes(uint32_t B, uint32_t Tb);
 cudaError_t prepare_step_tb_kernel(uint32_t B, uint32_t Tb);
 cudaError_t launch_step_tb(const StepArgs& a, const uint16_t* in, uint16_t* out, uint32_t t0, uint32_t Tb,
                            uint32_t B, unsigned long long* fail, int grid, cudaStream_t s);
-cudaError_t launch_init(int Q, const InitArgs& a, uint16_t* out, int grid, cudaStream_t s);
+// words: entries of a.table
+cudaError_t launch_init(int Q, const InitArgs& a, uint32_t words, uint16_t* out, uint32_t sms, cudaStream_t s);
 cudaError_t prepare_step9_kernel();  // D2Q9 (ilg_d2q9.cu)
 uint32_t step9_threads();
 uint32_t step9_blocks_per_sm();

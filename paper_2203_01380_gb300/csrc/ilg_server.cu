@@ -296,9 +296,8 @@ bool admit(ilg_server* s, const Request& rq, Resident* out, cudaError_t* cerr, s
     a.offset = d_init;
     a.count = d_init + it.offset.size();
     a.table = d_init + it.offset.size() + it.count.size();
-    const size_t nodes = size_t(rq.p.Lx) * rq.p.Ly;
-    const int grid = int(std::min<size_t>((nodes + 255) / 256, size_t(s->sms) * 4));
-    e = launch_init(5, a, reinterpret_cast<uint16_t*>(s->d_arena + r.off_state), grid, s->init_stream);
+    e = launch_init(5, a, uint32_t(it.table.size()), reinterpret_cast<uint16_t*>(s->d_arena + r.off_state),
+                    uint32_t(s->sms), s->init_stream);
   }
   cudaEvent_t ev = nullptr;
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
