@@ -8,16 +8,19 @@
 // So, per opposite pair (i, -i) with weight w_m and per rest velocity,
 //   post_i  = omega w_m rho + a1 f_i + a2 f_-i,  a1,2 = ((1 - omega) +- (1 - omega^j)) / 2
 //   post_0  = omega w_0 rho + (1 - omega) f_0
-// (15 double operations per D2Q5 node, 9 per D1Q3 node), then push-streaming to
-// x + v_i.  No moment matrix appears; the oracle uses the matrix.
+// (9 fused multiply-adds per D2Q5 node, 5 per D1Q3 node, and the density with its products,
+// formed in integers), then push-streaming to x + v_i.  No moment matrix appears; the
+// oracle uses the matrix.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <string>
 #include <vector>
 
 #include "ilg_internal.h"
+#include "ilg_sync.cuh"
 
 namespace {
 
@@ -33,54 +36,146 @@ struct LbCoef {
   double l2;   // 1 - omega
   double a1;   // ((1 - omega) + (1 - omega^j)) / 2
   double a2;   // ((1 - omega) - (1 - omega^j)) / 2
+  // cr, cm, cd as integers: m 2^e with the top bit of m set; whole: all of them are (positive
+  // and of ordinary size), so that their products with rho may be formed in integers
+  unsigned long long mr, mm, md;
+  int er, em, ed;
+  int whole;
 };
 
-// One step, one node per thread: blocks stride over rows (blockIdx.y) and over
-// x within a row (blockIdx.x); load the Q planes, relax, push.
+// ---- double-precision sums and products on the integer pipes ----
+// An SM has two fp64 lanes and 128 integer lanes, so the density sum and its products with
+// the equilibrium weights (six of a D2Q5 node's fifteen fp64 operations) are formed in
+// integers; the other nine, all fused multiply-adds, stay on the fp64 pipe, which bounds the
+// step.  D2Q5 16384^2 7.72 -> 4.93 ms (0.78 of the fp64 rate of the nine, 0.64 of HBM),
+// 1024^2 34.9 -> 22.0 us per step; D2Q9 1024^2 63.6 -> 40.3.
+
+// S (not 0, its top bit at least 2^53) rounded to 53 bits, ties to even: returns them (2^52 to
+// 2^53) and how many bits were dropped.
+__device__ __forceinline__ unsigned long long round53(unsigned long long S, int& dropped) {
+  const int p = 11 - __clzll(static_cast<long long>(S));
+  dropped = p;
+  S += (1ull << (p - 1)) - 1ull + ((S >> p) & 1ull);
+  return S >> p;
+}
+
+// The sum of Q doubles as M 2^E, rounded once (round to nearest even): exact shifts to the
+// largest exponent and one 64-bit integer sum.  False (and nothing else) unless all are
+// positive, of ordinary size, and within 2^kRoom of one another.
 template <int Q>
-__global__ void __launch_bounds__(kLbThreads) lb_step_kernel(LbCoef k, const double* __restrict__ in,
-                                                            double* __restrict__ out, uint32_t Lx, uint32_t Ly) {
-  const size_t plane = size_t(Lx) * Ly;
-  for (uint32_t y = blockIdx.y; y < Ly; y += gridDim.y) {
-    const size_t row = size_t(y) * Lx;
-    const uint32_t yp = y + 1 == Ly ? 0 : y + 1;
-    const uint32_t ym = y == 0 ? Ly - 1 : y - 1;
-    for (uint32_t x = blockIdx.x * blockDim.x + threadIdx.x; x < Lx; x += gridDim.x * blockDim.x) {
-      const size_t node = row + x;
-      double f[Q];
+__device__ __forceinline__ bool whole_sum(const double (&f)[Q], unsigned long long& M, int& E) {
+  constexpr int kRoom = Q == 3 ? 9 : (Q == 5 ? 8 : 7);  // Q 2^(53 + kRoom) < 2^64
+  int e[Q], top = 0, low = 1 << 20;
 #pragma unroll
-      for (int i = 0; i < Q; ++i) f[i] = in[i * plane + node];
-      double rho = f[0] + f[1] + f[2];
-      if constexpr (Q >= 5) rho = rho + f[3] + f[4];
-      if constexpr (Q == 9) rho = rho + f[5] + f[6] + f[7] + f[8];
-      const double c = k.cm * rho;
-      const double p0 = fma(k.l2, f[0], k.cr * rho);
-      const double p1 = fma(k.a1, f[1], fma(k.a2, f[2], c));
-      const double p2 = fma(k.a1, f[2], fma(k.a2, f[1], c));
-      const uint32_t xp = x + 1 == Lx ? 0 : x + 1;
-      const uint32_t xm = x == 0 ? Lx - 1 : x - 1;
-      out[node] = p0;
-      out[plane + row + xp] = p1;
-      out[2 * plane + row + xm] = p2;
-      if constexpr (Q >= 5) {
-        const double p3 = fma(k.a1, f[3], fma(k.a2, f[4], c));
-        const double p4 = fma(k.a1, f[4], fma(k.a2, f[3], c));
-        out[3 * plane + size_t(yp) * Lx + x] = p3;
-        out[4 * plane + size_t(ym) * Lx + x] = p4;
+  for (int i = 0; i < Q; ++i) {
+    e[i] = int(uint32_t(__double2hiint(f[i])) >> 20);  // with the sign bit: a negative value is above any limit
+    top = max(top, e[i]);
+    low = min(low, e[i]);
+  }
+  if (low < 64 || top > 1980 || top - low > kRoom) return false;
+  unsigned long long S = 0;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    const uint32_t hi = (uint32_t(__double2hiint(f[i])) & 0xFFFFFu) | 0x100000u;
+    S += ((static_cast<unsigned long long>(hi) << 32) | uint32_t(__double2loint(f[i]))) << (kRoom - top + e[i]);
+  }
+  int p;
+  M = round53(S, p);
+  E = top - 1075 - kRoom + p;
+  return true;
+}
+
+// (M 2^E)(m 2^e) as a double, rounded once: the 128-bit product, its low half folded into a
+// sticky bit.  M at most 2^53, m with its top bit set.
+__device__ __forceinline__ double whole_product(unsigned long long M, int E, unsigned long long m, int e) {
+  const unsigned long long a = M << 10;
+  const uint32_t a0 = uint32_t(a), a1 = uint32_t(a >> 32), b0 = uint32_t(m), b1 = uint32_t(m >> 32);
+  const unsigned long long p00 = static_cast<unsigned long long>(a0) * b0;
+  const unsigned long long p01 = static_cast<unsigned long long>(a0) * b1 + (p00 >> 32);
+  const unsigned long long p10 = static_cast<unsigned long long>(a1) * b0 + uint32_t(p01);
+  unsigned long long S = static_cast<unsigned long long>(a1) * b1 + (p01 >> 32) + (p10 >> 32);
+  if ((uint32_t(p00) | uint32_t(p10)) != 0u) S |= 1ull;
+  int p;
+  const unsigned long long r = round53(S, p);
+  const unsigned long long bits = (static_cast<unsigned long long>(E + e + 54 + p + 1074) << 52) + r;
+  return __longlong_as_double(static_cast<long long>(bits));
+}
+
+// T steps, one node per thread: load the Q planes, relax, push.  f0 holds the state, the
+// steps alternate the buffers; a barrier of all blocks (a cooperative launch) separates them.
+// sync[0]: barrier word, sync[1]: 1 once a wait gave up.
+template <int Q>
+__global__ void __launch_bounds__(kLbThreads, 4)
+    lb_run_kernel(const __grid_constant__ LbCoef k, double* f0, double* f1, uint32_t Lx, uint32_t Ly, uint32_t T,
+                  unsigned long long* sync) {
+  __shared__ int stop;
+  if (threadIdx.x == 0) stop = 0;
+  const uint32_t nodes = Lx * Ly;
+  const size_t plane = nodes;
+  const uint32_t stride = gridDim.x * kLbThreads, stride_y = stride / Lx, stride_x = stride - stride_y * Lx;
+  const uint32_t first = blockIdx.x * kLbThreads + threadIdx.x;
+  const uint32_t y0 = first / Lx, x0 = first - y0 * Lx;
+  for (uint32_t step = 0;; ++step) {
+    const double* const in = (step & 1) ? f1 : f0;
+    double* const out = (step & 1) ? f0 : f1;
+    uint32_t x = x0, y = y0, node = first;
+    while (node < nodes) {
+      double f[Q];
+      // (through L2 only: another SM wrote these lines in the step before)
+#pragma unroll
+      for (int i = 0; i < Q; ++i) f[i] = __ldcg(in + (i * plane + node));
+      double c, cr, cd = 0.0;
+      unsigned long long M;
+      int E;
+      if (k.whole && whole_sum<Q>(f, M, E)) {
+        c = whole_product(M, E, k.mm, k.em);
+        cr = whole_product(M, E, k.mr, k.er);
+        if constexpr (Q == 9) cd = whole_product(M, E, k.md, k.ed);
+      } else {
+        double rho = f[0] + f[1] + f[2];
+        if constexpr (Q >= 5) rho = rho + f[3] + f[4];
+        if constexpr (Q == 9) rho = rho + f[5] + f[6] + f[7] + f[8];
+        c = k.cm * rho;
+        cr = k.cr * rho;
+        if constexpr (Q == 9) cd = k.cd * rho;
       }
-      if constexpr (Q == 9) {
-        // diagonal pairs (+1,+1)/(-1,-1) and (+1,-1)/(-1,+1)
-        const double cdr = k.cd * rho;
-        const double p5 = fma(k.a1, f[5], fma(k.a2, f[6], cdr));
-        const double p6 = fma(k.a1, f[6], fma(k.a2, f[5], cdr));
-        const double p7 = fma(k.a1, f[7], fma(k.a2, f[8], cdr));
-        const double p8 = fma(k.a1, f[8], fma(k.a2, f[7], cdr));
-        out[5 * plane + size_t(yp) * Lx + xp] = p5;
-        out[6 * plane + size_t(ym) * Lx + xm] = p6;
-        out[7 * plane + size_t(ym) * Lx + xp] = p7;
-        out[8 * plane + size_t(yp) * Lx + xm] = p8;
+      const uint32_t yp = y + 1 == Ly ? 0 : y + 1;
+      const uint32_t ym = y == 0 ? Ly - 1 : y - 1;
+      double* const o = out + node;  // row y starts at node - x
+      const int64_t right = x + 1 == Lx ? -int64_t(x) : 1, left = x == 0 ? int64_t(Lx) - 1 : -1;
+      o[0] = fma(k.l2, f[0], cr);
+      o[int64_t(plane) + right] = fma(k.a1, f[1], fma(k.a2, f[2], c));
+      o[int64_t(2 * plane) + left] = fma(k.a1, f[2], fma(k.a2, f[1], c));
+      if constexpr (Q >= 5) {
+        double* const up = out + (size_t(yp) * Lx + x);
+        double* const down = out + (size_t(ym) * Lx + x);
+        up[3 * plane] = fma(k.a1, f[3], fma(k.a2, f[4], c));
+        down[4 * plane] = fma(k.a1, f[4], fma(k.a2, f[3], c));
+        if constexpr (Q == 9) {
+          // diagonal pairs (+1,+1)/(-1,-1) and (+1,-1)/(-1,+1)
+          up[int64_t(5 * plane) + right] = fma(k.a1, f[5], fma(k.a2, f[6], cd));
+          down[int64_t(6 * plane) + left] = fma(k.a1, f[6], fma(k.a2, f[5], cd));
+          down[int64_t(7 * plane) + right] = fma(k.a1, f[7], fma(k.a2, f[8], cd));
+          up[int64_t(8 * plane) + left] = fma(k.a1, f[8], fma(k.a2, f[7], cd));
+        }
+      }
+      if (nodes - node <= stride) break;  // (node + stride may pass 2^32)
+      node += stride;
+      x += stride_x;
+      y += stride_y;
+      if (x >= Lx) {
+        x -= Lx;
+        y += 1;
       }
     }
+    if (step + 1 == T) break;
+    __syncthreads();
+    if (threadIdx.x == 0 && ilg::run_barrier(sync, (step + 1) * gridDim.x) == ~0ull) {
+      atomicExch(sync + 1, 1ull);
+      stop = 1;
+    }
+    __syncthreads();
+    if (stop) break;
   }
 }
 
@@ -283,6 +378,9 @@ struct ilg_lb {
   double* d_out = nullptr;    // 1 + 2 kLbMaxModes
   double2* d_red = nullptr;   // projection partials, 2 kLbMaxModes x chunks
   int32_t* d_modes = nullptr; // 2 kLbMaxModes
+  unsigned long long* d_sync = nullptr;  // [0] barrier word of a several-step launch, [1] a wait gave up
+  unsigned long long* h_sync = nullptr;  // pinned: sync[1]
+  int run_blocks = 0;                    // resident blocks of the step kernel
   std::string err;
 };
 
@@ -327,15 +425,30 @@ int lb_grid(const ilg_lb* b) {
   return int(blocks < cap ? blocks : cap);
 }
 
-// step grid: x blocks cover a row (up to the resident total), y blocks share rows
-dim3 lb_step_grid(const ilg_lb* b) {
-  const uint32_t cap = uint32_t(b->sms) * (2048 / kLbThreads);
-  uint32_t gx = (b->p.Lx + kLbThreads - 1) / kLbThreads;
-  if (gx > cap) gx = cap;
-  uint32_t gy = cap / gx;
-  if (gy < 1) gy = 1;
-  if (gy > b->Ly) gy = b->Ly;
-  return dim3(gx, gy);
+const void* lb_run_fn(int Q) {
+  return Q == 3   ? reinterpret_cast<const void*>(lb_run_kernel<3>)
+         : Q == 5 ? reinterpret_cast<const void*>(lb_run_kernel<5>)
+                  : reinterpret_cast<const void*>(lb_run_kernel<9>);
+}
+
+// v = m 2^e with the top bit of m set; false unless v is positive and of ordinary size
+bool as_integer(double v, unsigned long long* m, int* e) {
+  if (!(v >= 1e-15 && v <= 1e3)) return false;
+  int x = 0;
+  const double f = std::frexp(v, &x);  // [1/2, 1)
+  *m = static_cast<unsigned long long>(std::ldexp(f, 53)) << 11;
+  *e = x - 64;
+  return true;
+}
+
+// A bounded wait between the blocks of a several-step launch gave up (read back with the
+// results): the buffers hold parts of different steps.
+ilg_status lb_gave_up(ilg_lb* b) {
+  b->has_state = false;
+  *b->h_sync = 0;
+  cudaMemsetAsync(b->d_sync, 0, 2 * sizeof(unsigned long long), b->stream);
+  cudaStreamSynchronize(b->stream);
+  return lb_fail(b, ILG_E_TIMEOUT, "a wait between the blocks of a several-step launch gave up: the state is lost");
 }
 
 }  // namespace
@@ -361,8 +474,15 @@ ilg_status ilg_lb_create(const ilg_lb_params* params, void* stream, ilg_lb** out
   double w[9];
   ilg::weights(p.lattice, p.theta, w);
   const double l2 = 1.0 - p.omega, lj = 1.0 - p.omega_j;
-  b->coef = LbCoef{p.omega * w[0], p.omega * w[1], b->Q == 9 ? p.omega * w[5] : 0.0, l2, 0.5 * (l2 + lj),
-                   0.5 * (l2 - lj)};
+  b->coef = LbCoef{};
+  b->coef.cr = p.omega * w[0];
+  b->coef.cm = p.omega * w[1];
+  b->coef.cd = b->Q == 9 ? p.omega * w[5] : 0.0;
+  b->coef.l2 = l2;
+  b->coef.a1 = 0.5 * (l2 + lj);
+  b->coef.a2 = 0.5 * (l2 - lj);
+  b->coef.whole = as_integer(b->coef.cr, &b->coef.mr, &b->coef.er) && as_integer(b->coef.cm, &b->coef.mm, &b->coef.em) &&
+                  (b->Q != 9 || as_integer(b->coef.cd, &b->coef.md, &b->coef.ed));
   b->chunks = (b->Ly + kLbRowChunk - 1) / kLbRowChunk;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -377,10 +497,17 @@ ilg_status ilg_lb_create(const ilg_lb_params* params, void* stream, ilg_lb** out
   if (e == cudaSuccess) e = ilg::dev_alloc(&b->d_modes, sizeof(int32_t) * 2 * kLbMaxModes);
   const size_t maxL = p.Lx > b->Ly ? p.Lx : b->Ly;
   if (e == cudaSuccess) e = ilg::dev_alloc(&b->d_red, sizeof(double2) * 2 * kLbMaxModes * ((maxL + kLbChunk - 1) / kLbChunk));
+  if (e == cudaSuccess) e = ilg::dev_alloc(&b->d_sync, 2 * sizeof(unsigned long long));
+  if (e == cudaSuccess) e = cudaMallocHost(&b->h_sync, sizeof(unsigned long long));
+  if (e == cudaSuccess) e = cudaMemsetAsync(b->d_sync, 0, 2 * sizeof(unsigned long long), b->stream);
+  int per_sm = 0;
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lb_run_fn(b->Q), kLbThreads, 0);
   if (e != cudaSuccess) {
     ilg_lb_destroy(b);
     return lb_cuda_fail(nullptr, e, "ilg_lb_create");
   }
+  *b->h_sync = 0;
+  b->run_blocks = int(std::min<size_t>(size_t(per_sm) * b->sms, (b->nodes + kLbThreads - 1) / kLbThreads));
   *out = b;
   return ILG_OK;
 }
@@ -396,6 +523,8 @@ ilg_status ilg_lb_destroy(ilg_lb* b) {
   cudaFree(b->d_out);
   cudaFree(b->d_modes);
   cudaFree(b->d_red);
+  cudaFree(b->d_sync);
+  if (b->h_sync) cudaFreeHost(b->h_sync);
   delete b;
   return ILG_OK;
 }
@@ -475,7 +604,10 @@ ilg_status ilg_lb_get_state(ilg_lb* b, double* host, size_t n, uint64_t* t) {
   if (!b->has_state) return lb_fail(b, ILG_E_STATE, "no state: call ilg_lb_init or ilg_lb_set_state first");
   if (!host || n != size_t(b->Q) * b->nodes) return lb_fail(b, ILG_E_INVALID, "state must hold Q*Lx*Ly doubles");
   LB_CUDA(b, cudaMemcpyAsync(host, b->f[b->cur], sizeof(double) * n, cudaMemcpyDeviceToHost, b->stream), "copy out");
+  LB_CUDA(b, cudaMemcpyAsync(b->h_sync, b->d_sync + 1, sizeof(unsigned long long), cudaMemcpyDeviceToHost, b->stream),
+          "copy out");
   LB_CUDA(b, cudaStreamSynchronize(b->stream), "copy out");
+  if (*b->h_sync != 0) return lb_gave_up(b);
   if (t) *t = b->t;
   return ILG_OK;
 }
@@ -483,17 +615,29 @@ ilg_status ilg_lb_get_state(ilg_lb* b, double* host, size_t n, uint64_t* t) {
 ilg_status ilg_lb_step(ilg_lb* b, uint32_t T) {
   if (!b) return ILG_E_INVALID;
   if (!b->has_state) return lb_fail(b, ILG_E_STATE, "no state: call ilg_lb_init or ilg_lb_set_state first");
-  const dim3 grid = lb_step_grid(b);
-  for (uint32_t k = 0; k < T; ++k) {
-    if (b->Q == 3)
-      lb_step_kernel<3><<<grid, kLbThreads, 0, b->stream>>>(b->coef, b->f[b->cur], b->f[b->cur ^ 1], b->p.Lx, b->Ly);
-    else if (b->Q == 5)
-      lb_step_kernel<5><<<grid, kLbThreads, 0, b->stream>>>(b->coef, b->f[b->cur], b->f[b->cur ^ 1], b->p.Lx, b->Ly);
-    else
-      lb_step_kernel<9><<<grid, kLbThreads, 0, b->stream>>>(b->coef, b->f[b->cur], b->f[b->cur ^ 1], b->p.Lx, b->Ly);
-    LB_CUDA(b, cudaGetLastError(), "lattice Boltzmann step");
-    b->cur ^= 1;
-    b->t += 1;
+  constexpr uint32_t kRunSteps = 4096;  // per launch
+  const void* fn = lb_run_fn(b->Q);
+  bool run = true;
+  for (uint32_t k = 0; k < T;) {
+    uint32_t n = run ? std::min(T - k, kRunSteps) : 1;
+    double *f0 = b->f[b->cur], *f1 = b->f[b->cur ^ 1];
+    void* args[] = {&b->coef, &f0, &f1, &b->p.Lx, &b->Ly, &n, &b->d_sync};
+    if (n > 1) {
+      LB_CUDA(b, cudaMemsetAsync(b->d_sync, 0, sizeof(unsigned long long), b->stream), "lattice Boltzmann step");
+      const cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(b->run_blocks), dim3(kLbThreads), args, 0, b->stream);
+      if (e == cudaErrorCooperativeLaunchTooLarge) {
+        // the device cannot hold all blocks at once (SMs reserved elsewhere): step by step
+        cudaGetLastError();
+        run = false;
+        continue;
+      }
+      LB_CUDA(b, e, "lattice Boltzmann step");
+    } else {
+      LB_CUDA(b, cudaLaunchKernel(fn, dim3(b->run_blocks), dim3(kLbThreads), args, 0, b->stream), "lattice Boltzmann step");
+    }
+    b->cur ^= int(n & 1u);
+    b->t += n;
+    k += n;
   }
   return ILG_OK;
 }
@@ -547,7 +691,10 @@ ilg_status ilg_lb_observables(ilg_lb* b, const int32_t* modes, uint32_t nmodes, 
   std::vector<double> h(1 + 2 * size_t(nmodes));
   LB_CUDA(b, cudaMemcpyAsync(h.data(), b->d_out, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, b->stream),
           "copy observables");
+  LB_CUDA(b, cudaMemcpyAsync(b->h_sync, b->d_sync + 1, sizeof(unsigned long long), cudaMemcpyDeviceToHost, b->stream),
+          "copy observables");
   LB_CUDA(b, cudaStreamSynchronize(b->stream), "observables");
+  if (*b->h_sync != 0) return lb_gave_up(b);
   if (t) *t = b->t;
   if (mass) *mass = h[0];
   const double half = double(Lx) * double(Ly) / 2.0;
