@@ -143,8 +143,9 @@ ilg_status ilg_set_temporal_blocking(ilg_ctx* ctx, uint32_t depth);
  * for later ilg_step calls:
  *   candidate 0  row-tiled step, 8 nodes per thread (16-byte vectors), 3 blocks per SM
  *   candidate 1  row-tiled step, 4 nodes per thread (8-byte vectors), 3 blocks per SM
- *   candidate 2  node-parallel step, one node per thread; D1Q3 and D2Q5: up to 4096
- *                steps per launch (the default on lattices of at most 8192 nodes per SM)
+ *   candidate 2  node-parallel step, one node per thread, up to 4096 steps per launch (the
+ *                default on small lattices, and wherever many nodes need the general
+ *                collision)
  *   candidate 3, 4  temporal blocking of depth 2, 4 (D2Q5; the remainder of a call
  *                takes the fastest single-step candidate)
  *   candidate 5  8-node vectors in warp segments: each warp walks 8192 nodes of a row,
@@ -156,11 +157,12 @@ ilg_status ilg_set_temporal_blocking(ilg_ctx* ctx, uint32_t depth);
  *                compile-time plane order, the fast collision branch-free, the
  *                values crossing a segment's ends written by the warp that computes
  *                them (no node computed twice); one block of 384 threads per SM
- *                (the default where it applies, on larger lattices)
+ *                (the default where it applies, on larger lattices); up to 4096 steps
+ *                per launch below 2^26 nodes
  *   candidate 7  as 6 with 4-node vectors (rows a multiple of 4), 640 threads per SM
- *                (the default where 6 does not apply and 7 does)
- *   D2Q9 lattices: candidate 2 (node-parallel, two nodes of a row per thread where
- *                rows are even) and the staged warp step with 4-node vectors (rows a
+ *                (the default on lattices between the small and the larger ones, and
+ *                where 6 does not apply)
+ *   D2Q9 lattices: candidate 2 and the staged warp step with 4-node vectors (rows a
  *                multiple of 4; all three probabilities strictly between 0 and 1),
  *                collided two nodes at a time in shared memory, in 512 threads per SM
  *                (candidate 6, the default where it applies) or 640 (candidate 7)

@@ -35,7 +35,9 @@ struct ilg_ctx {
   unsigned long long* d_col = nullptr;
   unsigned long long* d_row = nullptr;
   unsigned long long* d_proj = nullptr;    // scratch of the projections
-  unsigned long long* h_obs = nullptr;     // pinned, written by the projections: mass, 4 per mode
+  // pinned, written by the projections: mass, 4 per mode; after the words of h_word for up
+  // to kFirstModes modes, an allocation of its own for more
+  unsigned long long* h_obs = nullptr;
   uint32_t mode_cap = 0;
   uint32_t tb_depth = 0;                   // temporal blocking: steps per launch (0: off)
   uint32_t general = 0;                    // too many nodes would fail the fast collision: general at once
@@ -48,6 +50,7 @@ struct ilg_ctx {
 namespace {
 
 constexpr size_t kFailWords = 3;
+constexpr uint32_t kFirstModes = 64;
 
 thread_local std::string g_create_error;
 
@@ -145,7 +148,7 @@ void free_ctx(ilg_ctx* c) {
   cudaFree(c->d_fail);
   cudaFree(c->d_mass);
   cudaFree(c->d_proj);
-  if (c->h_obs) cudaFreeHost(c->h_obs);
+  if (c->mode_cap > kFirstModes) cudaFreeHost(c->h_obs);
   if (c->h_word) cudaFreeHost(c->h_word);
 }
 
@@ -212,11 +215,13 @@ ilg_status ilg_create(const ilg_params* params, void* stream, ilg_ctx** out) {
   c->d_row = c->d_col + c->p.Lx;
   if ((e = dev_alloc(&c->d_proj, sizeof(unsigned long long) * kProjScratchWords)) != cudaSuccess)
     return bail(e, "cudaMalloc projections");
-  if ((e = cudaMallocHost(&c->h_word, sizeof(unsigned long long) * kFailWords)) != cudaSuccess) return bail(e, "cudaMallocHost");
+  if ((e = cudaMallocHost(&c->h_word, sizeof(unsigned long long) * (kFailWords + 1 + 4 * kFirstModes))) != cudaSuccess)
+    return bail(e, "cudaMallocHost");
+  c->h_obs = c->h_word + kFailWords;
+  c->mode_cap = kFirstModes;
 
   std::vector<uint32_t> tables(block_words, 0u);
   build_table_block(c->Q, c->p.sampler, c->P_omega, c->P_rest, c->P_axis, tables.data());
-  if ((e = prepare_step9_kernel()) != cudaSuccess) return bail(e, "cudaFuncSetAttribute");
   if ((e = prepare_step_kernels()) != cudaSuccess) return bail(e, "cudaFuncSetAttribute");
   if ((e = prepare_step_vec_kernels()) != cudaSuccess) return bail(e, "cudaFuncSetAttribute");
   if ((e = prepare_step_warp_kernels()) != cudaSuccess) return bail(e, "cudaFuncSetAttribute");
@@ -386,75 +391,66 @@ bool kernel_applies(const ilg_ctx* c, const StepArgs& a, int kind) {
 // resident warps of the row-tiled kernels (3 blocks of 8 warps per SM)
 uint64_t vec_warps(const ilg_ctx* c) { return uint64_t(c->sms) * 3 * 8; }
 
-// D1Q3 and D2Q5 lattices of at most this many nodes per SM run node-parallel, several
-// steps per launch: there a launch, its table staging and its idle warps per step cost
-// the staged warp kernel more than its cheaper collision saves (D2Q5, 10 per velocity,
-// us per step node-parallel / staged warp: 64^2 2.3 / 24.7, 512^2 5.8 / 22.7, 1024^2
-// 15.3 / 22.7, 1448^2 27.5 / 24.9, 2048^2 50 / 37)
-constexpr uint64_t kRunNodesPerSm = 8192;
+// Lattices of at most this many nodes per SM run node-parallel: a tile of the staged warp
+// kernel (256 nodes of D2Q5, 128 of D2Q9, one after the other in a lane) lasts longer than
+// their whole step.  Beyond, D1Q3 and D2Q5 take the smaller tiles while a warp has few of
+// them.  Us per step, 10 per velocity, node-parallel / 4-node / 8-node vectors: D2Q5 512^2
+// 5.4 / 5.3 / 5.7, 768^2 8.8 / 8.1 / 8.6, 1024^2 13.4 / 10.5 / 11.8, 1448^2 24.4 / 19.4 /
+// 18.1, 2048^2 45 / 33 / 30; D2Q9 (4-node) 1024^2 21 / 31, 1448^2 39 / 50, 2048^2 84 / 75.
+constexpr uint64_t kRunNodesPerSm = 2048, kRunNodesPerSm9 = 16384, kWarp4NodesPerSm = 10240;
 
 // the kernel a step runs: the tuned one while it applies to the current state, else
 // the default: node-parallel on small lattices; the shared-memory-staged warp kernel
-// with 8-node, else 4-node vectors where the rows and probabilities allow; else 8-node
-// row tiles where the rows allow; node-parallel otherwise
+// with 4- or 8-node vectors where the rows and probabilities allow; else 8-node row tiles
+// where the rows allow; node-parallel otherwise
 int pick_kernel(const ilg_ctx* c, const StepArgs& a) {
   if (c->kernel_choice >= 0 && kernel_applies(c, a, c->kernel_choice)) return c->kernel_choice;
-  if (c->Q != 9 && c->nodes <= kRunNodesPerSm * uint64_t(c->sms)) return kKernelNode;
+  const uint64_t sms = uint64_t(c->sms);
+  if (c->nodes <= (c->Q == 9 ? kRunNodesPerSm9 : kRunNodesPerSm) * sms) return kKernelNode;
+  const bool w4 = kernel_applies(c, a, kKernelWarp4);
+  if (c->Q != 9 && w4 && c->nodes <= kWarp4NodesPerSm * sms) return kKernelWarp4;
   if (kernel_applies(c, a, kKernelWarp8)) return kKernelWarp8;
-  if (kernel_applies(c, a, kKernelWarp4)) return kKernelWarp4;
+  if (w4) return kKernelWarp4;
   if (!kernel_applies(c, a, kKernelVec8)) return kKernelNode;
   return step_seg_units(c->p.Lx, c->p.Ly) >= 2 * vec_warps(c) ? kKernelSeg : kKernelVec8;
 }
 
-cudaError_t launch_single(const ilg_ctx* c, int kind, const StepArgs& a, const uint16_t* in, uint16_t* out,
-                          uint64_t t, unsigned long long* fail_word) {
-  if (c->Q == 9 && kind != kKernelWarp8 && kind != kKernelWarp4) {
-    // rows of even length run two neighbouring nodes per thread (launch_step9)
-    const size_t work = c->p.Lx % 2 == 0 ? c->nodes / 2 : c->nodes;
-    const size_t blocks = (work + step9_threads() - 1) / step9_threads();
-    const size_t cap = size_t(c->sms) * step9_blocks_per_sm();
-    return launch_step9(a, in, out, uint32_t(t), fail_word, int(blocks < cap ? blocks : cap), c->stream);
+// kernels that take several steps per launch
+bool takes_runs(int kind) { return kind == kKernelNode || kind == kKernelWarp8 || kind == kKernelWarp4; }
+
+// T steps from step t (one, unless takes_runs), the state in b0
+cudaError_t launch_steps(const ilg_ctx* c, int kind, const StepArgs& a, uint16_t* b0, uint16_t* b1, uint64_t t, uint32_t T,
+                         unsigned long long* fail_word) {
+  const uint32_t sms = uint32_t(c->sms);
+  if (kind == kKernelVec8 || kind == kKernelVec4) {
+    const int npt = kind == kKernelVec8 ? 8 : 4;
+    return launch_step_vec(c->Q, a, b0, b1, uint32_t(t), fail_word, vec_grid(c, step_vec_blocks_per_sm(npt)), c->stream, npt);
   }
-  if (kind == kKernelVec8)
-    return launch_step_vec(c->Q, a, in, out, uint32_t(t), fail_word, vec_grid(c, step_vec_blocks_per_sm(8)), c->stream,
-                           8);
-  if (kind == kKernelVec4)
-    return launch_step_vec(c->Q, a, in, out, uint32_t(t), fail_word, vec_grid(c, step_vec_blocks_per_sm(4)), c->stream,
-                           4);
   if (kind == kKernelSeg) {
     const uint64_t blocks = (step_seg_units(c->p.Lx, c->p.Ly) + 7) / 8, cap = vec_warps(c) / 8;
-    return launch_step_seg(c->Q, a, in, out, uint32_t(t), fail_word, int(blocks < cap ? blocks : cap), c->stream);
+    return launch_step_seg(c->Q, a, b0, b1, uint32_t(t), fail_word, int(blocks < cap ? blocks : cap), c->stream);
   }
-  if (kind == kKernelWarp8 || kind == kKernelWarp4) {
-    const int shape = kind == kKernelWarp4 ? 1 : 0;
-    const uint32_t Ly = c->Q == 3 ? 1u : c->p.Ly;
-    return launch_step_warp(c->Q, shape, a, in, out, uint32_t(t), fail_word,
-                            int(step_warp_grid(c->Q, c->p.Lx, Ly, uint32_t(c->sms), shape)), c->stream);
-  }
-  return launch_step_run(c->Q, a, const_cast<uint16_t*>(in), out, uint32_t(t), 1, fail_word, fail_word + 1,
-                         uint32_t(c->sms), c->stream);
+  if (kind == kKernelWarp8 || kind == kKernelWarp4)
+    return launch_step_warp(c->Q, kind == kKernelWarp4 ? 1 : 0, a, b0, b1, uint32_t(t), T, fail_word, fail_word + 1, sms,
+                            c->stream);
+  return launch_step_run(c->Q, a, b0, b1, uint32_t(t), T, fail_word, fail_word + 1, sms, c->stream);
 }
 
-// T single steps from step t (the state in bufs[cur], the steps alternate the buffers);
-// the node-parallel kernel takes them in few launches of several steps each
+// T single steps from step t (the state in bufs[cur], the steps alternate the buffers), in
+// few launches of several steps each where the kernel takes them
 cudaError_t launch_singles(const ilg_ctx* c, int kind, const StepArgs& a, uint16_t* const* bufs, int cur, uint64_t t,
                            uint32_t T, unsigned long long* fail_word) {
-  constexpr uint32_t kRunSteps = 4096;  // per launch
-  bool run = kind == kKernelNode && c->Q != 9;
+  constexpr uint32_t kRunSteps = 4096;         // per launch
+  constexpr uint64_t kRunNodes = 1ull << 26;  // beyond: a step takes half a millisecond and more, a launch nothing of it
+  bool run = takes_runs(kind) && (kind == kKernelNode || c->nodes < kRunNodes);
   for (uint32_t k = 0; k < T;) {
     const uint32_t n = run ? std::min(T - k, kRunSteps) : 1;
-    cudaError_t e;
-    if (n > 1) {
-      e = launch_step_run(c->Q, a, bufs[cur], bufs[cur ^ 1], uint32_t(t + k), n, fail_word, fail_word + 1,
-                          uint32_t(c->sms), c->stream);
-      if (e == cudaErrorCooperativeLaunchTooLarge) {
-        // the device cannot hold all blocks at once (SMs reserved elsewhere): step by step
-        cudaGetLastError();
-        run = false;
-        continue;
-      }
-    } else {
-      e = launch_single(c, kind, a, bufs[cur], bufs[cur ^ 1], t + k, fail_word);
+    const cudaError_t e = launch_steps(c, kind, a, bufs[cur], bufs[cur ^ 1], t + k, n, fail_word);
+    if (e == cudaErrorCooperativeLaunchTooLarge && n > 1) {
+      // the device cannot hold all blocks at once (SMs reserved elsewhere): step by step
+      cudaGetLastError();
+      run = false;
+      continue;
     }
     if (e != cudaSuccess) return e;
     k += n;
@@ -666,10 +662,10 @@ ilg_status ilg_observables(ilg_ctx* c, const int32_t* modes, uint32_t nmodes, ui
     if (my != 0) want_rows = true;
   }
   if (nmodes > c->mode_cap) {
-    if (c->h_obs) cudaFreeHost(c->h_obs);
-    c->h_obs = nullptr;
-    c->mode_cap = 0;
-    ILG_CUDA(c, cudaMallocHost(&c->h_obs, sizeof(unsigned long long) * (1 + 4 * size_t(nmodes))), "cudaMallocHost modes");
+    unsigned long long* more = nullptr;
+    ILG_CUDA(c, cudaMallocHost(&more, sizeof(unsigned long long) * (1 + 4 * size_t(nmodes))), "cudaMallocHost modes");
+    if (c->mode_cap > kFirstModes) cudaFreeHost(c->h_obs);
+    c->h_obs = more;
     c->mode_cap = nmodes;
   }
   const uint32_t Lx = c->p.Lx, Ly = c->p.Ly;

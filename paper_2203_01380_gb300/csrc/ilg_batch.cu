@@ -249,7 +249,7 @@ __device__ __forceinline__ uint32_t run_ring(const BatchArgs& b, const StepArgs&
       }
       if ((REC || STATES) && s == T) continue;
       if (!TABLES && a.particle) collide_particle<3>(a, tables, x, d.t + s, m, post);
-      else collide_warp<3, S, BatchShape<THREADS>::kRing, TABLES>(a, k, to, tr, words, 4 * tid, x, m, post);
+      else collide_warp<3, S, BatchShape<THREADS>::kRing, TABLES>(a, k, to, tr, tr, words, 4 * tid, x, m, post);
       if (active) {
         bad |= (post[0] | post[1] | post[2]) > 65535u;
         dst[x] = uint16_t(post[0]);

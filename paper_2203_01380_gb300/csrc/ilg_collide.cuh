@@ -1,6 +1,6 @@
-// The collision of one node per lane by a whole warp (D1Q3, D2Q5; any occupations):
+// The collision of one node per lane by a whole warp (any occupations):
 // the node-parallel kernels' collision, where many nodes need more random words than
-// the eight slot words.
+// the slot words.
 //
 // What bounds it: the ALU pipe (two cycles per warp instruction and sub-partition),
 // then the wide products of Philox on the FMA-heavy pipe.  Per-lane loops over chunks
@@ -23,16 +23,20 @@ constexpr unsigned kFullWarp = 0xFFFFFFFFu;
 // What is the same for every node of a launch (or of a lattice and step) in the first
 // three Philox rounds (see StepKeys), and the two words an extension block's own part
 // of them starts from.
-struct WordKeys {
-  StepKeys<2> slot;
+template <int NB>
+struct NodeKeys {
+  StepKeys<NB> slot;
   uint32_t ext_c;  // round 2's x2 of extension block 0, without the block index
   uint32_t ext_e;  // round 3's x0 without the block's product
 };
 
-__device__ __forceinline__ WordKeys word_keys(const StepArgs& a, uint32_t t) {
+using WordKeys = NodeKeys<2>;  // D1Q3, D2Q5 (two slot blocks; D2Q9: four)
+
+template <int NB = 2>
+__device__ __forceinline__ NodeKeys<NB> word_keys(const StepArgs& a, uint32_t t) {
   constexpr uint32_t M0 = 0xD2511F53u, M1 = 0xCD9E8D57u;
-  WordKeys k;
-  k.slot = step_keys<2>(a, t);
+  NodeKeys<NB> k;
+  k.slot = step_keys<NB>(a, t);
   k.ext_c = uint32_t((uint64_t(M0) * t) >> 32) ^ kDevTagExt ^ a.rk[1];
   k.ext_e = uint32_t(uint64_t(M1) * a.replica) ^ a.rk[2];
   return k;
@@ -61,7 +65,8 @@ struct NodeWords {
   uint32_t r2h, r2l, p1l;  // the node's part of rounds 1-3
   uint32_t blk;            // next extension block
 
-  __device__ __forceinline__ void begin(const WordKeys& k, unsigned char* ring_, uint32_t lane_off, uint32_t node) {
+  template <class Keys>
+  __device__ __forceinline__ void begin(const Keys& k, unsigned char* ring_, uint32_t lane_off, uint32_t node) {
     const uint64_t P1 = uint64_t(0xD2511F53u) * (node ^ k.slot.A);
     const uint64_t R2 = uint64_t(0xCD9E8D57u) * (uint32_t(P1 >> 32) ^ k.slot.G);
     r2h = uint32_t(R2 >> 32);
@@ -71,11 +76,13 @@ struct NodeWords {
     rd = wr = lane_off;
     blk = 0;
   }
-  __device__ __forceinline__ uint4 slot(const WordKeys& k, const uint32_t (&rk)[20], int b) const {
+  template <class Keys>
+  __device__ __forceinline__ uint4 slot(const Keys& k, const uint32_t (&rk)[20], int b) const {
     return philox_tail(make_uint4(r2h ^ k.slot.H[b], r2l, p1l ^ k.slot.I[b], k.slot.J[b]), rk);
   }
   // the next extension block into the ring
-  __device__ __forceinline__ void fill(const WordKeys& k, const uint32_t (&rk)[20]) {
+  template <class Keys>
+  __device__ __forceinline__ void fill(const Keys& k, const uint32_t (&rk)[20]) {
     const uint64_t R1 = uint64_t(0xCD9E8D57u) * (k.ext_c ^ blk);
     const uint64_t P2 = uint64_t(0xD2511F53u) * (uint32_t(R1 >> 32) ^ k.ext_e);
     const uint4 b = philox_tail(make_uint4(r2h ^ uint32_t(R1) ^ rk[4], r2l, p1l ^ uint32_t(P2 >> 32) ^ rk[5], uint32_t(P2)), rk);
@@ -89,7 +96,8 @@ struct NodeWords {
   }
   // every lane has at least `bytes` of words afterwards (bytes <= (K - 4) S, a multiple of
   // S); lanes with room fill together
-  __device__ __forceinline__ void ensure(const WordKeys& k, const uint32_t (&rk)[20], uint32_t bytes) {
+  template <class Keys>
+  __device__ __forceinline__ void ensure(const Keys& k, const uint32_t (&rk)[20], uint32_t bytes) {
     while (__any_sync(kFullWarp, wr - rd < bytes)) {
       if (wr - rd <= (K - 4) * S) fill(k, rk);
     }
@@ -103,8 +111,8 @@ struct NodeWords {
 // Binomial(x, P) beyond its first chunk: chunks of 63 trials, each with the lane's next
 // extension word, two per pass; left = x - 63 (negative or zero: none).  A lane that is
 // done draws from row 0: nothing.
-template <uint32_t S, uint32_t K, class Tab>
-__device__ __forceinline__ uint32_t more_chunks(NodeWords<S, K>& e, const WordKeys& k, const uint32_t (&rk)[20],
+template <uint32_t S, uint32_t K, class Keys, class Tab>
+__device__ __forceinline__ uint32_t more_chunks(NodeWords<S, K>& e, const Keys& k, const uint32_t (&rk)[20],
                                                 const Tab& A, int32_t left) {
   uint32_t r = 0;
   while (__any_sync(kFullWarp, left > 0)) {
@@ -119,24 +127,57 @@ __device__ __forceinline__ uint32_t more_chunks(NodeWords<S, K>& e, const WordKe
   return r;
 }
 
+// Bits of c particles' two direction words, 32 particles at a time: the first words A, B,
+// every further group the lane's next two extension words (a mask of no bits once a lane is
+// done).  Returns the numbers of particles with A set, with both set, and with B alone.
+struct BitCounts {
+  uint32_t a, both, b;
+};
+template <uint32_t S, uint32_t K, class Keys>
+__device__ __forceinline__ BitCounts count_bits(NodeWords<S, K>& e, const Keys& k, const uint32_t (&rk)[20], uint32_t c,
+                                                uint32_t A, uint32_t B) {
+  constexpr uint32_t kPass = (K - 4 < 8 ? K - 4 : 8) / 2;  // groups whose words are asked for at once
+  int32_t left = int32_t(c);
+  uint32_t mask = __funnelshift_lc(kFullWarp, 0u, uint32_t(left));
+  left = max(left - 32, 0);
+  A &= mask;
+  B &= mask;
+  BitCounts n{uint32_t(__popc(A)), uint32_t(__popc(A & B)), uint32_t(__popc(B & ~A))};
+  while (__any_sync(kFullWarp, left > 0)) {
+    e.ensure(k, rk, min(uint32_t(left + 31) >> 5, kPass) * (2 * S));
+    for (uint32_t u = 0; u < kPass && __any_sync(kFullWarp, left > 0); ++u) {
+      mask = __funnelshift_lc(kFullWarp, 0u, uint32_t(left));
+      A = e.peek() & mask;
+      B = e.peek(1) & mask;
+      n.a += __popc(A);
+      n.both += __popc(A & B);
+      n.b += __popc(B & ~A);
+      if (left > 0) e.rd += 2 * S;
+      left = max(left - 32, 0);
+    }
+  }
+  return n;
+}
+
 // The collision of one node per lane (m: its occupations after the flip, all zero for a
 // lane without a node); all 32 lanes call it together.  The same words and results as
-// collide().  ring: the block's ring of K words per thread in shared memory, lane_off:
-// 4 x the thread's index.  TABLES: both probabilities lie strictly between 0 and 1 and are
-// drawn through their tables (known outside the loop over nodes: the tests for the other
-// cases would be made for every node).
-template <int Q, uint32_t S, uint32_t K, bool TABLES, class Tab>
-__device__ __forceinline__ void collide_warp(const StepArgs& a, const WordKeys& k, const Tab& to, const Tab& tr,
+// collide() (D2Q9: collide9_general()).  ring: the block's ring of K words per thread in
+// shared memory, lane_off: 4 x the thread's index; ta: D2Q9's axis-share table (others: any).
+// TABLES: every probability lies strictly between 0 and 1 and is drawn through its table
+// (known outside the loop over nodes: the tests for the other cases would be made for every
+// node).
+template <int Q, uint32_t S, uint32_t K, bool TABLES, class Keys, class Tab>
+__device__ __forceinline__ void collide_warp(const StepArgs& a, const Keys& k, const Tab& to, const Tab& tr, const Tab& ta,
                                              unsigned char* ring, uint32_t lane_off, uint32_t node,
                                              const uint32_t (&m)[Q], uint32_t (&out)[Q]) {
-  static_assert(Q == 3 || Q == 5, "D1Q3 and D2Q5");
   static_assert(K >= 4 + uint32_t(Q), "a word for each velocity beside the block being written");
+  constexpr int NB = Q == 9 ? 4 : 2;
   constexpr int32_t kN = int32_t(kDevNmax);
   NodeWords<S, K> e;
   e.begin(k, ring, lane_off, node);
-  uint32_t W[8];
+  uint32_t W[4 * NB];
 #pragma unroll
-  for (int b = 0; b < 2; ++b) {
+  for (int b = 0; b < NB; ++b) {
     const uint4 v = e.slot(k, a.rk, b);
     W[4 * b] = v.x;
     W[4 * b + 1] = v.y;
@@ -179,30 +220,30 @@ __device__ __forceinline__ void collide_warp(const StepArgs& a, const WordKeys& 
     removed += r[i];
   }
 
+  // a share of x through a table: the first chunk with its slot word, then extension words
+  auto share = [&](uint32_t mode, const Tab& A, uint32_t x, uint32_t slot) -> uint32_t {
+    if (TABLES || mode == kTable) {
+      const uint32_t s = A(min(x, kDevNmax), slot);
+      return s + more_chunks(e, k, a.rk, A, int32_t(x) - kN);
+    }
+    return mode == kAlways ? x : 0u;
+  };
   // share sent to rest
-  uint32_t to_rest;
-  if (TABLES || a.rest_mode == kTable) {
-    to_rest = tr(min(removed, kDevNmax), W[Q]);
-    to_rest += more_chunks(e, k, a.rk, tr, int32_t(removed) - kN);
-  } else {
-    to_rest = a.rest_mode == kAlways ? removed : 0u;
-  }
+  const uint32_t to_rest = share(a.rest_mode, tr, removed, W[Q]);
   out[0] += to_rest;
 
-  // directions of the moving particles, 32 at a time (a mask of no bits once a lane is done)
+  // directions of the moving particles, 32 at a time
   const uint32_t moving = removed - to_rest;
-  int32_t left = int32_t(moving);
-  uint32_t mask = __funnelshift_lc(kFullWarp, 0u, uint32_t(left));
-  left = max(left - 32, 0);
-  constexpr uint32_t kWords = Q == 3 ? 1 : 2;               // per group
-  // groups whose words are asked for at once
-  constexpr int32_t kPass = int32_t((K - 4 < 8 ? K - 4 : 8) / kWords);
-  auto ask = [&](int32_t l) { return min(uint32_t(l + 31) >> 5, uint32_t(kPass)) * (kWords * S); };
   if constexpr (Q == 3) {
+    // one sign word per group
+    constexpr uint32_t kPass = K - 4 < 8 ? K - 4 : 8;
+    int32_t left = int32_t(moving);
+    uint32_t mask = __funnelshift_lc(kFullWarp, 0u, uint32_t(left));
     uint32_t minus = __popc(W[Q + 1] & mask);
+    left = max(left - 32, 0);
     while (__any_sync(kFullWarp, left > 0)) {
-      e.ensure(k, a.rk, ask(left));
-      for (int u = 0; u < kPass && __any_sync(kFullWarp, left > 0); ++u) {
+      e.ensure(k, a.rk, min(uint32_t(left + 31) >> 5, kPass) * S);
+      for (uint32_t u = 0; u < kPass && __any_sync(kFullWarp, left > 0); ++u) {
         mask = __funnelshift_lc(kFullWarp, 0u, uint32_t(left));
         minus += __popc(e.peek() & mask);
         if (left > 0) e.rd += S;
@@ -212,25 +253,22 @@ __device__ __forceinline__ void collide_warp(const StepArgs& a, const WordKeys& 
     out[1] += moving - minus;
     out[2] += minus;
   } else {
-    uint32_t A = W[Q + 1] & mask, B = W[Q + 2] & mask;
-    uint32_t ny = __popc(A), nmy = __popc(A & B), nmx = __popc(B & ~A);
-    while (__any_sync(kFullWarp, left > 0)) {
-      e.ensure(k, a.rk, ask(left));
-      for (int u = 0; u < kPass && __any_sync(kFullWarp, left > 0); ++u) {
-        mask = __funnelshift_lc(kFullWarp, 0u, uint32_t(left));
-        A = e.peek() & mask;
-        B = e.peek(1) & mask;
-        ny += __popc(A);
-        nmy += __popc(A & B);
-        nmx += __popc(B & ~A);
-        if (left > 0) e.rd += 2 * S;
-        left = max(left - 32, 0);
-      }
+    // axis bit (0: x, 1: y), sign bit (0: +, 1: -); on D2Q9 of the axis particles
+    const uint32_t axis = Q == 9 ? share(a.axis_mode, ta, moving, W[10]) : moving;
+    const BitCounts n = count_bits(e, k, a.rk, axis, W[Q == 9 ? 11 : Q + 1], W[Q == 9 ? 12 : Q + 2]);
+    out[1] += axis - n.a - n.b;
+    out[2] += n.b;
+    out[3] += n.a - n.both;
+    out[4] += n.both;
+    if constexpr (Q == 9) {
+      // diagonal particles: x-sign bit, y-sign bit
+      const uint32_t diag = moving - axis;
+      const BitCounts d = count_bits(e, k, a.rk, diag, W[13], W[14]);
+      out[5] += diag - d.a - d.b;
+      out[6] += d.both;
+      out[7] += d.b;
+      out[8] += d.a - d.both;
     }
-    out[1] += moving - ny - nmx;
-    out[2] += nmx;
-    out[3] += ny - nmy;
-    out[4] += nmy;
   }
 }
 

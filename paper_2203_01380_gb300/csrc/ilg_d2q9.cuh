@@ -1,10 +1,9 @@
-// D2Q9 collision of one node (shared by the node-parallel D2Q9 kernels and the
-// staged warp kernel): the collision thins every velocity, sends a binomial share of
-// the removed particles to rest, splits the moving ones binomially into axis and
-// diagonal particles, and gives each axis particle an axis bit and a sign bit and
-// each diagonal particle an x-sign and a y-sign bit (slot words 11/12 and 13/14 for
-// the first group of 32).  The table block holds the thinning, rest and axis-share
-// alias tables, one after the other.
+// D2Q9 general collision of one node (out of line in the staged warp kernel): it thins every
+// velocity, sends a binomial share of the removed particles to rest, splits the moving ones
+// binomially into axis and diagonal particles, and gives each axis particle an axis bit and
+// a sign bit and each diagonal particle an x-sign and a y-sign bit (slot words 11/12 and
+// 13/14 for the first group of 32).  The table block holds the thinning, rest and
+// axis-share alias tables, one after the other.
 #pragma once
 
 #include <cstdint>
@@ -12,10 +11,6 @@
 #include "ilg_device.cuh"
 
 namespace ilg {
-
-// velocity order: rest, +x, -x, +y, -y, (+1,+1), (-1,-1), (+1,-1), (-1,+1)
-__device__ __forceinline__ int d9_vx(int i) { return (i == 1 || i == 5 || i == 7) ? 1 : ((i == 2 || i == 6 || i == 8) ? -1 : 0); }
-__device__ __forceinline__ int d9_vy(int i) { return (i == 3 || i == 5 || i == 8) ? 1 : ((i == 4 || i == 6 || i == 7) ? -1 : 0); }
 
 __device__ __forceinline__ const uint2* axis_table(const uint32_t* s) {
   return reinterpret_cast<const uint2*>(s) + 2 * kDevAliasEntries;
@@ -45,44 +40,6 @@ __device__ __forceinline__ void add_diag(uint32_t c, uint32_t X, uint32_t Y, uin
   out[6] += nmm;
   out[7] += npm;
   out[8] += nmp;
-}
-
-// Fast path: every occupation <= 63, at most 63 removed, at most 32 axis and 32
-// diagonal movers, all three probabilities drawn through tables.  False outside.
-__device__ __forceinline__ bool collide9_try_fast(const StepArgs& a, const uint32_t* s, uint32_t node, uint32_t t,
-                                                  const uint32_t (&m)[9], uint32_t (&out)[9]) {
-  if (a.omega_mode != kTable || a.rest_mode != kTable || a.axis_mode != kTable) return false;
-  uint32_t any = 0;
-#pragma unroll
-  for (int i = 0; i < 9; ++i) any |= m[i];
-  if (any >> 6) return false;
-  uint32_t W[16];
-#pragma unroll
-  for (int b = 0; b < 4; ++b) {
-    const uint4 w = philox_rk(counter(node, t, a.replica, kDevTagStep | uint32_t(b)), a.rk);
-    W[4 * b] = w.x;
-    W[4 * b + 1] = w.y;
-    W[4 * b + 2] = w.z;
-    W[4 * b + 3] = w.w;
-  }
-  const uint2* to = thinning_table(s);
-  uint32_t removed = 0;
-#pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    const uint32_t r = binomial_alias(to, m[i], W[i]);
-    out[i] = m[i] - r;
-    removed += r;
-  }
-  if (removed >> 6) return false;
-  const uint32_t to_rest = binomial_alias(rest_table(s), removed, W[9]);
-  const uint32_t moving = removed - to_rest;
-  const uint32_t axis = binomial_alias(axis_table(s), moving, W[10]);
-  const uint32_t diag = moving - axis;
-  if (axis > 32 || diag > 32) return false;
-  out[0] += to_rest;
-  add_axis(axis, W[11], W[12], out);
-  add_diag(diag, W[13], W[14], out);
-  return true;
 }
 
 // General path: any occupations, extension words read lazily in the order

@@ -30,6 +30,8 @@ namespace ilg {
 // --------------------------------------------------------------------------
 constexpr uint32_t kStepRing = 16;  // extension words per lane
 
+__host__ __device__ constexpr uint32_t run_table_words(int Q) { return Q == 9 ? kDevBlockWords9 : kDevStagedWords; }
+
 // sync[0]: the barrier word, sync[1]: set to 1 when a wait gave up.  TABLES: the binomial
 // sampler with both probabilities strictly between 0 and 1; false: anything else.
 template <int Q, int THREADS, bool TABLES>
@@ -40,16 +42,17 @@ __global__ void __launch_bounds__(THREADS, 1)
   __shared__ int stop;
   uint32_t* s = reinterpret_cast<uint32_t*>(smem4);
   if (threadIdx.x == 0) stop = (*reinterpret_cast<volatile unsigned long long*>(fail) != ~0ull);
+  constexpr uint32_t kTables = run_table_words(Q);
   {
-    // the block's first words: the two alias tables, or the particle sampler's boundaries
+    // the block's first words: the alias tables, or the particle sampler's boundaries
     const uint4* g4 = reinterpret_cast<const uint4*>(a.tables);
 #pragma unroll 8
-    for (uint32_t i = threadIdx.x; i < kDevStagedWords / 4; i += THREADS) smem4[i] = g4[i];
+    for (uint32_t i = threadIdx.x; i < kTables / 4; i += THREADS) smem4[i] = g4[i];
   }
   __syncthreads();
   if (stop) return;
-  unsigned char* const ring = reinterpret_cast<unsigned char*>(smem4) + 4 * kDevStagedWords;
-  const Alias8 to = Alias8::of(s, 0), tr = Alias8::of(s, 1);
+  unsigned char* const ring = reinterpret_cast<unsigned char*>(smem4) + 4 * kTables;
+  const Alias8 to = Alias8::of(s, 0), tr = Alias8::of(s, 1), ta = Alias8::of(s, Q == 9 ? 2 : 1);
 
   const uint32_t nodes = a.Lx * a.Ly;
   const size_t plane = nodes;
@@ -70,7 +73,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     const uint16_t* from[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) from[i] = in + (i == 0 || !a.flip ? i : (i & 1 ? i + 1 : i - 1)) * plane;
-    const WordKeys keys = word_keys(a, t);  // the launch-wide Philox rounds
+    const auto keys = word_keys<Q == 9 ? 4 : 2>(a, t);  // the launch-wide Philox rounds
     while (base < nodes) {
       const uint32_t node = base + lane;
       const bool active = node < nodes && node >= base;
@@ -79,7 +82,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 #pragma unroll
       for (int i = 0; i < Q; ++i) m[i] = active ? __ldcg(from[i] + node) : 0u;
       if (!TABLES && a.particle) collide_particle<Q>(a, s, node, t, m, post);
-      else collide_warp<Q, 4 * THREADS, kStepRing, TABLES>(a, keys, to, tr, ring, 4 * threadIdx.x, node, m, post);
+      else collide_warp<Q, 4 * THREADS, kStepRing, TABLES>(a, keys, to, tr, ta, ring, 4 * threadIdx.x, node, m, post);
       if (active) {
         uint32_t high = 0;
 #pragma unroll
@@ -87,13 +90,20 @@ __global__ void __launch_bounds__(THREADS, 1)
         bad |= high > 65535u;
         uint16_t* const o = out + node;  // row y starts at node - x
         o[0] = uint16_t(post[0]);
-        (o + plane)[x + 1 == a.Lx ? -int64_t(x) : 1] = uint16_t(post[1]);
-        (o + 2 * plane)[x == 0 ? int64_t(a.Lx) - 1 : -1] = uint16_t(post[2]);
-        if constexpr (Q == 5) {
-          const uint32_t yp = y + 1 == a.Ly ? 0 : y + 1;
-          const uint32_t ym = y == 0 ? a.Ly - 1 : y - 1;
-          out[3 * plane + size_t(yp) * a.Lx + x] = uint16_t(post[3]);
-          out[4 * plane + size_t(ym) * a.Lx + x] = uint16_t(post[4]);
+        const int64_t right = x + 1 == a.Lx ? -int64_t(x) : 1, left = x == 0 ? int64_t(a.Lx) - 1 : -1;
+        (o + plane)[right] = uint16_t(post[1]);
+        (o + 2 * plane)[left] = uint16_t(post[2]);
+        if constexpr (Q >= 5) {
+          uint16_t* const up = out + (size_t(y + 1 == a.Ly ? 0 : y + 1) * a.Lx + x);
+          uint16_t* const down = out + (size_t(y == 0 ? a.Ly - 1 : y - 1) * a.Lx + x);
+          up[3 * plane] = uint16_t(post[3]);
+          down[4 * plane] = uint16_t(post[4]);
+          if constexpr (Q == 9) {
+            (up + 5 * plane)[right] = uint16_t(post[5]);
+            (down + 6 * plane)[left] = uint16_t(post[6]);
+            (down + 7 * plane)[right] = uint16_t(post[7]);
+            (up + 8 * plane)[left] = uint16_t(post[8]);
+          }
         }
       }
       x += stride_x;
@@ -127,10 +137,12 @@ __global__ void __launch_bounds__(THREADS, 1)
   }
 }
 
-constexpr size_t run_smem(int threads) { return sizeof(uint32_t) * (kDevStagedWords + size_t(kStepRing) * threads); }
+constexpr size_t run_smem(int Q, int threads) {
+  return sizeof(uint32_t) * (run_table_words(Q) + size_t(kStepRing) * threads);
+}
 
 // Shapes: one block per SM of as few threads (128, 512, 1024) as give every node a lane of
-// its own; 1024 beyond that.
+// its own; beyond that 1024 (D2Q9: 512, a node's nine planes need the registers).
 struct RunShape {
   const void* fn;
   int threads;
@@ -141,27 +153,33 @@ static const void* run_fn(int Q, bool tables) {
   if (Q == 3)
     return tables ? reinterpret_cast<const void*>(step_run_kernel<3, THREADS, true>)
                   : reinterpret_cast<const void*>(step_run_kernel<3, THREADS, false>);
-  return tables ? reinterpret_cast<const void*>(step_run_kernel<5, THREADS, true>)
-                : reinterpret_cast<const void*>(step_run_kernel<5, THREADS, false>);
+  if (Q == 5)
+    return tables ? reinterpret_cast<const void*>(step_run_kernel<5, THREADS, true>)
+                  : reinterpret_cast<const void*>(step_run_kernel<5, THREADS, false>);
+  if constexpr (THREADS <= 512)
+    return tables ? reinterpret_cast<const void*>(step_run_kernel<9, THREADS, true>)
+                  : reinterpret_cast<const void*>(step_run_kernel<9, THREADS, false>);
+  return nullptr;
 }
 
 static RunShape run_shape(int Q, const StepArgs& a, uint64_t nodes, uint32_t sms) {
-  const bool tables = !a.particle && a.omega_mode == kTable && a.rest_mode == kTable;
+  const bool tables = !a.particle && a.omega_mode == kTable && a.rest_mode == kTable && (Q != 9 || a.axis_mode == kTable);
   if (nodes <= uint64_t(sms) * 128) return {run_fn<128>(Q, tables), 128};
-  if (nodes <= uint64_t(sms) * 512) return {run_fn<512>(Q, tables), 512};
+  if (Q == 9 || nodes <= uint64_t(sms) * 512) return {run_fn<512>(Q, tables), 512};
   return {run_fn<1024>(Q, tables), 1024};
 }
 
 cudaError_t prepare_step_kernels() {
   cudaError_t e = cudaSuccess;
-  auto set = [&](const void* f, int threads) {
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(run_smem(threads)));
+  auto set = [&](const void* f, int Q, int threads) {
+    if (f && e == cudaSuccess)
+      e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(run_smem(Q, threads)));
   };
-  for (int Q : {3, 5})
+  for (int Q : {3, 5, 9})
     for (bool tables : {false, true}) {
-      set(run_fn<128>(Q, tables), 128);
-      set(run_fn<512>(Q, tables), 512);
-      set(run_fn<1024>(Q, tables), 1024);
+      set(run_fn<128>(Q, tables), Q, 128);
+      set(run_fn<512>(Q, tables), Q, 512);
+      set(run_fn<1024>(Q, tables), Q, 1024);
     }
   return e;
 }
@@ -173,10 +191,10 @@ cudaError_t launch_step_run(int Q, const StepArgs& a, uint16_t* buf0, uint16_t* 
   const dim3 grid(uint32_t(std::min<uint64_t>((nodes + r.threads - 1) / r.threads, sms)));
   StepArgs args = a;
   void* p[] = {&args, &buf0, &buf1, &t, &T, &fail, &sync};
-  if (T == 1) return cudaLaunchKernel(r.fn, grid, dim3(r.threads), p, run_smem(r.threads), s);
+  if (T == 1) return cudaLaunchKernel(r.fn, grid, dim3(r.threads), p, run_smem(Q, r.threads), s);
   const cudaError_t e = cudaMemsetAsync(sync, 0, sizeof(unsigned long long), s);
   if (e != cudaSuccess) return e;
-  return cudaLaunchCooperativeKernel(r.fn, grid, dim3(r.threads), p, run_smem(r.threads), s);
+  return cudaLaunchCooperativeKernel(r.fn, grid, dim3(r.threads), p, run_smem(Q, r.threads), s);
 }
 
 // --------------------------------------------------------------------------

@@ -43,24 +43,18 @@ cudaError_t launch_step_seg(int Q, const StepArgs& a, const uint16_t* in, uint16
 // every probability drawn through its table; D1Q3 and D2Q5: shape 0 = 8 nodes per
 // lane, one block of 384 threads per SM, shape 1 = 4 nodes per lane, 640 threads;
 // D2Q9: 4 nodes per lane collided in shared memory, 512 (shape 0) or 640 (shape 1)
-// threads; step_warp_grid =
-// blocks of a launch
+// threads
 cudaError_t prepare_step_warp_kernels();
 uint32_t step_warp_width(int Q, int shape);  // nodes per lane (rows must be a multiple)
-uint32_t step_warp_grid(int Q, uint32_t Lx, uint32_t Ly, uint32_t sms, int shape);
-cudaError_t launch_step_warp(int Q, int shape, const StepArgs& a, const uint16_t* in, uint16_t* out, uint32_t t,
-                             unsigned long long* fail, int grid, cudaStream_t s);
+// T steps from step t in one launch, as launch_step_run
+cudaError_t launch_step_warp(int Q, int shape, const StepArgs& a, uint16_t* buf0, uint16_t* buf1, uint32_t t, uint32_t T,
+                             unsigned long long* fail, unsigned long long* sync, uint32_t sms, cudaStream_t s);
 size_t step_tb_smem_bytes(uint32_t B, uint32_t Tb);
 cudaError_t prepare_step_tb_kernel(uint32_t B, uint32_t Tb);
 cudaError_t launch_step_tb(const StepArgs& a, const uint16_t* in, uint16_t* out, uint32_t t0, uint32_t Tb,
                            uint32_t B, unsigned long long* fail, int grid, cudaStream_t s);
 // words: entries of a.table
 cudaError_t launch_init(int Q, const InitArgs& a, uint32_t words, uint16_t* out, uint32_t sms, cudaStream_t s);
-cudaError_t prepare_step9_kernel();  // D2Q9 (ilg_d2q9.cu)
-uint32_t step9_threads();
-uint32_t step9_blocks_per_sm();
-cudaError_t launch_step9(const StepArgs& a, const uint16_t* in, uint16_t* out, uint32_t t, unsigned long long* fail,
-                         int grid, cudaStream_t s);
 // adds to col (Lx words), row (Ly words; want_rows) and mass: zero them first
 cudaError_t launch_sums(int Q, const uint16_t* in, uint32_t Lx, uint32_t Ly, unsigned long long* col,
                         unsigned long long* row, unsigned long long* mass, int want_rows, uint32_t sms, cudaStream_t s);

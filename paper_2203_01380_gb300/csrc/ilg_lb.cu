@@ -379,7 +379,7 @@ struct ilg_lb {
   double2* d_red = nullptr;   // projection partials, 2 kLbMaxModes x chunks
   int32_t* d_modes = nullptr; // 2 kLbMaxModes
   unsigned long long* d_sync = nullptr;  // [0] barrier word of a several-step launch, [1] a wait gave up
-  unsigned long long* h_sync = nullptr;  // pinned: sync[1]
+  unsigned long long h_sync = 0;         // sync[1] as read back with the last results
   int run_blocks = 0;                    // resident blocks of the step kernel
   std::string err;
 };
@@ -445,7 +445,7 @@ bool as_integer(double v, unsigned long long* m, int* e) {
 // results): the buffers hold parts of different steps.
 ilg_status lb_gave_up(ilg_lb* b) {
   b->has_state = false;
-  *b->h_sync = 0;
+  b->h_sync = 0;
   cudaMemsetAsync(b->d_sync, 0, 2 * sizeof(unsigned long long), b->stream);
   cudaStreamSynchronize(b->stream);
   return lb_fail(b, ILG_E_TIMEOUT, "a wait between the blocks of a several-step launch gave up: the state is lost");
@@ -498,7 +498,6 @@ ilg_status ilg_lb_create(const ilg_lb_params* params, void* stream, ilg_lb** out
   const size_t maxL = p.Lx > b->Ly ? p.Lx : b->Ly;
   if (e == cudaSuccess) e = ilg::dev_alloc(&b->d_red, sizeof(double2) * 2 * kLbMaxModes * ((maxL + kLbChunk - 1) / kLbChunk));
   if (e == cudaSuccess) e = ilg::dev_alloc(&b->d_sync, 2 * sizeof(unsigned long long));
-  if (e == cudaSuccess) e = cudaMallocHost(&b->h_sync, sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaMemsetAsync(b->d_sync, 0, 2 * sizeof(unsigned long long), b->stream);
   int per_sm = 0;
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lb_run_fn(b->Q), kLbThreads, 0);
@@ -506,7 +505,6 @@ ilg_status ilg_lb_create(const ilg_lb_params* params, void* stream, ilg_lb** out
     ilg_lb_destroy(b);
     return lb_cuda_fail(nullptr, e, "ilg_lb_create");
   }
-  *b->h_sync = 0;
   b->run_blocks = int(std::min<size_t>(size_t(per_sm) * b->sms, (b->nodes + kLbThreads - 1) / kLbThreads));
   *out = b;
   return ILG_OK;
@@ -524,7 +522,6 @@ ilg_status ilg_lb_destroy(ilg_lb* b) {
   cudaFree(b->d_modes);
   cudaFree(b->d_red);
   cudaFree(b->d_sync);
-  if (b->h_sync) cudaFreeHost(b->h_sync);
   delete b;
   return ILG_OK;
 }
@@ -604,10 +601,10 @@ ilg_status ilg_lb_get_state(ilg_lb* b, double* host, size_t n, uint64_t* t) {
   if (!b->has_state) return lb_fail(b, ILG_E_STATE, "no state: call ilg_lb_init or ilg_lb_set_state first");
   if (!host || n != size_t(b->Q) * b->nodes) return lb_fail(b, ILG_E_INVALID, "state must hold Q*Lx*Ly doubles");
   LB_CUDA(b, cudaMemcpyAsync(host, b->f[b->cur], sizeof(double) * n, cudaMemcpyDeviceToHost, b->stream), "copy out");
-  LB_CUDA(b, cudaMemcpyAsync(b->h_sync, b->d_sync + 1, sizeof(unsigned long long), cudaMemcpyDeviceToHost, b->stream),
+  LB_CUDA(b, cudaMemcpyAsync(&b->h_sync, b->d_sync + 1, sizeof(unsigned long long), cudaMemcpyDeviceToHost, b->stream),
           "copy out");
   LB_CUDA(b, cudaStreamSynchronize(b->stream), "copy out");
-  if (*b->h_sync != 0) return lb_gave_up(b);
+  if (b->h_sync != 0) return lb_gave_up(b);
   if (t) *t = b->t;
   return ILG_OK;
 }
@@ -691,10 +688,10 @@ ilg_status ilg_lb_observables(ilg_lb* b, const int32_t* modes, uint32_t nmodes, 
   std::vector<double> h(1 + 2 * size_t(nmodes));
   LB_CUDA(b, cudaMemcpyAsync(h.data(), b->d_out, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, b->stream),
           "copy observables");
-  LB_CUDA(b, cudaMemcpyAsync(b->h_sync, b->d_sync + 1, sizeof(unsigned long long), cudaMemcpyDeviceToHost, b->stream),
+  LB_CUDA(b, cudaMemcpyAsync(&b->h_sync, b->d_sync + 1, sizeof(unsigned long long), cudaMemcpyDeviceToHost, b->stream),
           "copy observables");
   LB_CUDA(b, cudaStreamSynchronize(b->stream), "observables");
-  if (*b->h_sync != 0) return lb_gave_up(b);
+  if (b->h_sync != 0) return lb_gave_up(b);
   if (t) *t = b->t;
   if (mass) *mass = h[0];
   const double half = double(Lx) * double(Ly) / 2.0;

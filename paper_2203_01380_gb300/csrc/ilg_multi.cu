@@ -54,7 +54,7 @@ __device__ __forceinline__ bool step_share(const StepArgs& a, const LatDesc& d, 
 #pragma unroll
     for (int i = 0; i < Q; ++i) m[i] = active ? __ldcg(from[i] + node) : 0u;
     if (!TABLES && a.particle) collide_particle<Q>(a, s, node, t, m, post);
-    else collide_warp<Q, 4 * kMultiThreads, kMultiRing, TABLES>(a, keys, to, tr, ring, 4 * threadIdx.x, node, m, post);
+    else collide_warp<Q, 4 * kMultiThreads, kMultiRing, TABLES>(a, keys, to, tr, tr, ring, 4 * threadIdx.x, node, m, post);
     if (active) {
       uint32_t high = 0;
 #pragma unroll

@@ -12,11 +12,9 @@
 //  - the fast collision runs branch-free on every node of a vector whose
 //    occupations are all below ROWS (64: the rows of the alias tables, staged in
 //    shared memory once per SM); the rare node outside that domain is redone by the
-//    general collision, out of line (its registers do not weigh on the fast path),
-//    which reads the tables from global memory;
-//  - warp w takes the w-th of equal shares of the row-major sequence of all
-//    vectors (so every warp has the same work to within one vector) and walks it
-//    tile by tile, as segments that end at row ends; neighbouring lanes trade
+//    general collision, out of line (its registers do not weigh on the fast path);
+//  - warp w takes the w-th of equal shares of the row-major sequence of all tiles (32
+//    vectors of a row) and walks it tile by tile, as segments that end at row ends; neighbouring lanes trade
 //    edge values by shuffles, and the two values that cross a segment's ends are
 //    written as single 16-bit stores by the warp that computes them, so no node is
 //    computed twice and no warp waits for another;
@@ -33,6 +31,7 @@
 #include "ilg_d2q9.cuh"
 #include "ilg_device.cuh"
 #include "ilg_launch.h"
+#include "ilg_sync.cuh"
 
 namespace ilg {
 namespace {
@@ -173,10 +172,11 @@ __device__ __forceinline__ uint32_t fast_draws9(const uint2* to, const uint2* tr
 // slot of the warp's scratch in shared memory, or the slot itself when the vector is
 // collided in place.  Both live in shared memory so that no register array of the
 // caller has its address taken (which would keep it in local memory on every tile).
-// gt: the full Alias8 tables in global memory.  Returns true when a result exceeds
-// 65535.
+// st: the staged tables (all rows of each, laid out as the table block; from global memory a
+// node's dozen dependent draws would keep its warp ten times longer).  Returns true when a
+// result exceeds 65535.
 template <int Q, int NPT>
-__device__ __noinline__ bool slow_nodes(const StepArgs& a, const uint32_t* gt, uint32_t node0, uint32_t t,
+__device__ __noinline__ bool slow_nodes(const StepArgs& a, const uint32_t* st, uint32_t node0, uint32_t t,
                                         const VN<NPT>* N, VN<NPT>* R, uint32_t slow) {
   bool bad = false;
   while (slow) {
@@ -185,8 +185,8 @@ __device__ __noinline__ bool slow_nodes(const StepArgs& a, const uint32_t* gt, u
     uint32_t m[Q], o[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) m[i] = node_of(N[32 * i], k);
-    if constexpr (Q == 9) collide9_general(a, gt, node0 + k, t, m, o);
-    else collide<Q>(a, gt, node0 + k, t, m, o);
+    if constexpr (Q == 9) collide9_general(a, st, node0 + k, t, m, o);
+    else collide<Q>(a, st, node0 + k, t, m, o);
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
       bad |= o[i] > 65535u;
@@ -205,7 +205,7 @@ __device__ __noinline__ bool slow_nodes(const StepArgs& a, const uint32_t* gt, u
 template <int Q, int ROWS, int NPT>
 __device__ __forceinline__ void collide_vec(const StepArgs& a, const StepKeys<Q == 9 ? 4 : 2>& keys, const uint2* to,
                                             const uint2* tr, const uint2* ta, uint32_t node0, uint32_t t,
-                                            const VN<NPT> (&N)[Q], VN<NPT> (&P)[Q], const VN<NPT>* slot,
+                                            VN<NPT> (&N)[Q], VN<NPT> (&P)[Q], const VN<NPT>* slot,
                                             VN<NPT>* scratch, bool& bad) {
   constexpr uint32_t kHigh = ROWS == 32 ? 0xFFE0FFE0u : 0xFFC0FFC0u;  // bits of values >= ROWS
   uint32_t any = 0;
@@ -213,14 +213,28 @@ __device__ __forceinline__ void collide_vec(const StepArgs& a, const StepKeys<Q 
   for (int i = 0; i < Q; ++i)
 #pragma unroll
     for (int j = 0; j < NPT / 2; ++j) any |= N[i].w[j];
-  // the fast collision needs every probability drawn through its table
-  if (a.omega_mode != kTable || a.rest_mode != kTable || (Q == 9 && a.axis_mode != kTable)) any = 0xFFFFFFFFu;
-  uint32_t slow = (any & kHigh) ? (1u << NPT) - 1u : 0u;
+  uint32_t slow = 0;
+  if (any & kHigh) {
+    // nodes beyond the fast collision's rows: marked for the general one, and their values
+    // cut to six bits so that they pass through the fast one without harm
+    constexpr uint32_t kLow = ~kHigh;
+#pragma unroll
+    for (int j = 0; j < NPT / 2; ++j) {
+      uint32_t w = 0;
+#pragma unroll
+      for (int i = 0; i < Q; ++i) {
+        w |= N[i].w[j];
+        N[i].w[j] &= kLow;
+      }
+      w &= kHigh;
+      slow |= ((w & 0xFFFFu) ? 1u : 0u) << (2 * j) | ((w >> 16) ? 2u : 0u) << (2 * j);
+    }
+  }
 #pragma unroll
   for (int i = 0; i < Q; ++i)
 #pragma unroll
     for (int j = 0; j < NPT / 2; ++j) P[i].w[j] = 0u;
-  if (!slow) {
+  {
 #pragma unroll
     for (int k = 0; k < NPT; ++k) {
       uint32_t m[Q], o[Q];
@@ -265,7 +279,7 @@ __device__ __forceinline__ void collide_vec(const StepArgs& a, const StepKeys<Q 
     }
   }
   if (slow) {
-    bad |= slow_nodes<Q, NPT>(a, a.tables, node0, t, slot, scratch, slow);
+    bad |= slow_nodes<Q, NPT>(a, reinterpret_cast<const uint32_t*>(to), node0, t, slot, scratch, slow);
     // take the general collision's half-words for the nodes it redid
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
@@ -342,7 +356,7 @@ __device__ __forceinline__ void collide_vec_res(const StepArgs& a, const StepKey
 #pragma unroll
     for (int i = 0; i < Q; ++i) sts32(sn + i * kPlane + 4 * j, __byte_perm(o[0][i], o[1][i], 0x5410));
   }
-  if (slow) bad |= slow_nodes<Q, NPT>(a, a.tables, node0, t, slot, slot, slow);
+  if (slow) bad |= slow_nodes<Q, NPT>(a, reinterpret_cast<const uint32_t*>(to), node0, t, slot, slot, slow);
 }
 
 // The segment that starts at vector g of the row-major sequence of all vectors
@@ -386,24 +400,28 @@ __device__ __forceinline__ constexpr int vel_dy(int i) {
                 : (Q == 5 ? (i == 3 ? 1 : (i == 4 ? -1 : 0)) : 0);
 }
 
-template <int Q, bool FLIP, int ROWS, int NPT, int THREADS, int MINB, bool RES>
+// T steps from t0, the state in buf0, a barrier of all blocks between them (a cooperative
+// launch) that alternate the buffers; !RUN: one step (the loop costs 0.5 % of a step's time,
+// more than a launch does on lattices of 2^26 nodes and beyond).  sync: as launch_step_run.
+template <int Q, bool FLIP, int ROWS, int NPT, int THREADS, int MINB, bool RES, bool RUN>
 __global__ void __launch_bounds__(THREADS, MINB)
-    step_warp_kernel(const __grid_constant__ StepArgs a, const uint16_t* __restrict__ in,
-                     uint16_t* __restrict__ out, uint32_t t, unsigned long long* __restrict__ fail) {
+    step_warp_kernel(const __grid_constant__ StepArgs a, uint16_t* buf0, uint16_t* buf1, uint32_t t0, uint32_t T,
+                     unsigned long long* fail, unsigned long long* sync) {
   extern __shared__ uint4 smem4[];
-  __shared__ int skip;
-  if (threadIdx.x == 0) skip = (*reinterpret_cast<const volatile unsigned long long*>(fail) != ~0ull);
+  __shared__ int stop;
+  if (threadIdx.x == 0) stop = (*reinterpret_cast<const volatile unsigned long long*>(fail) != ~0ull);
   constexpr uint32_t kTables = Q == 9 ? 3 : 2;           // thinning, rest (D2Q9: and the axis share)
   constexpr uint32_t kRow4 = ROWS * kDevAliasCols / 2;  // uint4 per staged table
   {
     // rows 0..ROWS-1 of each alias table (uint2 entries, two per uint4)
     const uint4* g4 = reinterpret_cast<const uint4*>(a.tables);
     constexpr uint32_t kTab4 = kDevAliasEntries / 2;  // uint4 per full table
+#pragma unroll 8
     for (uint32_t i = threadIdx.x; i < kTables * kRow4; i += THREADS)
       smem4[i] = g4[(i / kRow4) * kTab4 + (i % kRow4)];
   }
   __syncthreads();
-  if (skip) return;
+  if (stop) return;
   const uint2* to = reinterpret_cast<const uint2*>(smem4);
   const uint2* tr = to + ROWS * kDevAliasCols;
   const uint2* ta = tr + ROWS * kDevAliasCols;  // D2Q9 only
@@ -420,13 +438,25 @@ __global__ void __launch_bounds__(THREADS, MINB)
   // all tile buffers)
   VN<NPT>* const scratch = reinterpret_cast<VN<NPT>*>(smem4 + kTables * kRow4) + (THREADS / 32) * (2 * Q * 32) +
                            (threadIdx.x >> 5) * (Q * 32) + lane;
-  // this warp's share of the row-major sequence of all vectors: [g, end)
-  const uint64_t total = uint64_t(vpr) * Ly, nwarps = (uint64_t(gridDim.x) * THREADS) >> 5;
-  const uint64_t w = (uint64_t(blockIdx.x) * THREADS + threadIdx.x) >> 5;
-  const uint32_t end = uint32_t((w + 1) * total / nwarps);
-  uint32_t g = uint32_t(w * total / nwarps);
-  if (g >= end) return;
+  for (uint32_t step = 0;; ++step) {
+  const uint32_t t = t0 + step;
+  const uint16_t* const __restrict__ in = RUN && (step & 1) ? buf1 : buf0;
+  uint16_t* const __restrict__ out = RUN && (step & 1) ? buf0 : buf1;
   bool bad = false;
+  // this warp's share of the row-major sequence of all vectors, [g, end): an equal share of
+  // the tiles (a row's vectors, 32 at a time; one that is not full costs as much as one that
+  // is), worked out anew each step to keep its registers free meanwhile
+  uint32_t w = (blockIdx.x * THREADS + threadIdx.x) >> 5;
+  asm volatile("" : "+r"(w));
+  const uint32_t tpr = (vpr + 31) >> 5, nwarps = gridDim.x * (THREADS / 32);
+  const uint64_t tiles = uint64_t(tpr) * Ly;
+  auto vector_of = [&](uint64_t tile) {
+    const uint32_t ty = uint32_t(tile / tpr);
+    return ty * vpr + (uint32_t(tile) - ty * tpr) * 32;
+  };
+  uint32_t g = vector_of(w * tiles / nwarps);
+  const uint32_t end = vector_of((w + 1) * tiles / nwarps);
+  if (g < end) {
   const StepKeys<Q == 9 ? 4 : 2> keys = step_keys<Q == 9 ? 4 : 2>(a, t);  // the launch-uniform Philox rounds
 
   uint32_t y, v0, v1;
@@ -580,7 +610,27 @@ __global__ void __launch_bounds__(THREADS, MINB)
     buf ^= 1;
   }
   cp_async_wait_all();  // the last (empty) group: nothing lands after the warp exits
-  if (bad) atomicMin(fail, static_cast<unsigned long long>(t));
+  }
+  if (bad) {
+    atomicMin(fail, static_cast<unsigned long long>(t));
+    __threadfence();
+    atomicOr(sync, kRunMark);
+  }
+  if (!RUN || step + 1 == T) break;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const unsigned long long v = run_barrier(sync, (step + 1) * gridDim.x);
+    if (v == ~0ull) {
+      atomicExch(sync + 1, 1ull);
+      stop = 1;
+    } else if (v >= kRunMark) {
+      // a step overflowed: this one, or already the next one (a faster block's)
+      stop = *reinterpret_cast<const volatile unsigned long long*>(fail) <= t;
+    }
+  }
+  __syncthreads();
+  if (stop) break;
+  }
 }
 
 // Shapes (the autotuner's two candidates): one block per SM, so the 64 staged table
@@ -639,28 +689,40 @@ constexpr size_t warp_smem() {
          size_t(S::kThreads / 32) * (S::kRes ? 2 : 3) * Q * 32 * (2 * S::kNpt);
 }
 
-template <int Q, bool FLIP, int SHAPE>
-constexpr auto warp_kernel() {
+template <int Q, bool FLIP, int SHAPE, bool RUN>
+const void* warp_kernel() {
   using S = WarpShapeQ<Q, SHAPE>;
-  return step_warp_kernel<Q, FLIP, kRows, S::kNpt, S::kThreads, S::kBlocks, S::kRes>;
+  return reinterpret_cast<const void*>(step_warp_kernel<Q, FLIP, kRows, S::kNpt, S::kThreads, S::kBlocks, S::kRes, RUN>);
+}
+
+template <int Q, int SHAPE>
+const void* warp_fn(bool flip, bool run) {
+  if (run) return flip ? warp_kernel<Q, true, SHAPE, true>() : warp_kernel<Q, false, SHAPE, true>();
+  return flip ? warp_kernel<Q, true, SHAPE, false>() : warp_kernel<Q, false, SHAPE, false>();
 }
 
 template <int Q, int SHAPE>
 cudaError_t warp_attr() {
-  cudaError_t e = cudaFuncSetAttribute(warp_kernel<Q, false, SHAPE>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       int(warp_smem<Q, SHAPE>()));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(warp_kernel<Q, true, SHAPE>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(warp_smem<Q, SHAPE>()));
+  cudaError_t e = cudaSuccess;
+  for (bool flip : {false, true})
+    for (bool run : {false, true})
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(warp_fn<Q, SHAPE>(flip, run), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 int(warp_smem<Q, SHAPE>()));
   return e;
 }
 
 template <int Q, int SHAPE>
-void warp_launch(const StepArgs& a, const uint16_t* in, uint16_t* out, uint32_t t, unsigned long long* fail, int grid,
-                 cudaStream_t s) {
-  constexpr int kThreads = WarpShapeQ<Q, SHAPE>::kThreads;
-  if (a.flip) warp_kernel<Q, true, SHAPE>()<<<grid, kThreads, warp_smem<Q, SHAPE>(), s>>>(a, in, out, t, fail);
-  else warp_kernel<Q, false, SHAPE>()<<<grid, kThreads, warp_smem<Q, SHAPE>(), s>>>(a, in, out, t, fail);
+cudaError_t warp_launch(const StepArgs& a, uint16_t* buf0, uint16_t* buf1, uint32_t t, uint32_t T,
+                        unsigned long long* fail, unsigned long long* sync, int grid, cudaStream_t s) {
+  const void* fn = warp_fn<Q, SHAPE>(a.flip != 0, T > 1);
+  StepArgs args = a;
+  void* p[] = {&args, &buf0, &buf1, &t, &T, &fail, &sync};
+  const dim3 threads(WarpShapeQ<Q, SHAPE>::kThreads);
+  if (T == 1) return cudaLaunchKernel(fn, dim3(grid), threads, p, warp_smem<Q, SHAPE>(), s);
+  const cudaError_t e = cudaMemsetAsync(sync, 0, sizeof(unsigned long long), s);
+  if (e != cudaSuccess) return e;
+  return cudaLaunchCooperativeKernel(fn, dim3(grid), threads, p, warp_smem<Q, SHAPE>(), s);
 }
 
 template <int Q>
@@ -699,29 +761,26 @@ uint32_t step_warp_width(int Q, int shape) {
   return npt;
 }
 
-// Blocks of a launch: one per SM, or fewer on lattices too small to give each warp
-// at least four tiles.
-uint32_t step_warp_grid(int Q, uint32_t Lx, uint32_t Ly, uint32_t sms, int shape) {
+// Blocks of a launch: one per SM, or fewer on lattices too small to give each warp a tile.
+static uint32_t step_warp_grid(int Q, uint32_t Lx, uint32_t Ly, uint32_t sms, int shape) {
   uint32_t npt, threads, per_sm;
   shape_of(Q, shape, &npt, &threads, &per_sm);
   const uint64_t cap = uint64_t(sms) * per_sm;
-  const uint64_t warps = std::max<uint64_t>(1, uint64_t(Lx / npt) * Ly / 128);
+  const uint64_t warps = std::max<uint64_t>(1, uint64_t(Lx / npt) * Ly / 32);
   return uint32_t(std::min<uint64_t>(cap, (warps + threads / 32 - 1) / (threads / 32)));
 }
 
-cudaError_t launch_step_warp(int Q, int shape, const StepArgs& a, const uint16_t* in, uint16_t* out, uint32_t t,
-                             unsigned long long* fail, int grid, cudaStream_t s) {
-  if (Q == 3) {
-    if (shape == 1) warp_launch<3, 1>(a, in, out, t, fail, grid, s);
-    else warp_launch<3, 0>(a, in, out, t, fail, grid, s);
-  } else if (Q == 5) {
-    if (shape == 1) warp_launch<5, 1>(a, in, out, t, fail, grid, s);
-    else warp_launch<5, 0>(a, in, out, t, fail, grid, s);
-  } else {
-    if (shape == 1) warp_launch<9, 1>(a, in, out, t, fail, grid, s);
-    else warp_launch<9, 0>(a, in, out, t, fail, grid, s);
-  }
-  return cudaGetLastError();
+cudaError_t launch_step_warp(int Q, int shape, const StepArgs& a, uint16_t* buf0, uint16_t* buf1, uint32_t t, uint32_t T,
+                             unsigned long long* fail, unsigned long long* sync, uint32_t sms, cudaStream_t s) {
+  const int grid = int(step_warp_grid(Q, a.Lx, a.Ly, sms, shape));
+  if (Q == 3)
+    return shape == 1 ? warp_launch<3, 1>(a, buf0, buf1, t, T, fail, sync, grid, s)
+                      : warp_launch<3, 0>(a, buf0, buf1, t, T, fail, sync, grid, s);
+  if (Q == 5)
+    return shape == 1 ? warp_launch<5, 1>(a, buf0, buf1, t, T, fail, sync, grid, s)
+                      : warp_launch<5, 0>(a, buf0, buf1, t, T, fail, sync, grid, s);
+  return shape == 1 ? warp_launch<9, 1>(a, buf0, buf1, t, T, fail, sync, grid, s)
+                    : warp_launch<9, 0>(a, buf0, buf1, t, T, fail, sync, grid, s);
 }
 
 }  // namespace ilg

@@ -186,25 +186,29 @@ double poisson_tail(double lambda, int k) {
 }  // namespace
 
 // The fast collision needs every occupation below 64, at most 63 removed and at most 32
-// moving particles (D2Q9: 32 axis and 32 diagonal).  With Poisson occupations of the
-// given mean, removals and movers are thinned Poisson counts; the lattice goes straight
-// to the general collision when the expected share of nodes that fail the fast one is
-// above kGeneralShare: trying the fast collision first then costs more than it saves,
-// since the warp that holds a failing node runs both collisions.
+// moving particles (D2Q9: 32 axis and 32 diagonal).  With Poisson occupations of the given
+// mean, shared out by the weights as in equilibrium, removals and movers are thinned Poisson
+// counts; the lattice goes straight to the general collision (the node-parallel kernel, which
+// takes such nodes as it takes any) when the expected share of nodes that fail the fast one
+// is above a limit: the staged warp kernel redoes each of them alone.  Measured on 2048^2
+// (D1Q3 2^22), node-parallel / staged warp us per step: D2Q5 46 / 35 at a share of 0.0003,
+// 48 / 47 at 0.005, 53 / 54 at 0.011; D1Q3 44 / 42 at 0.016, 52 / 70 at 0.16; D2Q9 84 / 75
+// at 0.0003, 85 / 147 at 0.009.
 uint32_t general_path(int lattice, double theta, double omega_star, double mean_occupation) {
-  constexpr double kGeneralShare = 0.02;
+  const double limit = lattice == ILG_D2Q9 ? 0.001 : 0.006;
   double w[9];
   weights(lattice, theta, w);
   const int Q = lattice == ILG_D1Q3 ? 3 : (lattice == ILG_D2Q9 ? 9 : 5);
   const double removed = omega_star * Q * mean_occupation, moving = removed * (1.0 - w[0]);
-  double fail = Q * poisson_tail(mean_occupation, 64) + poisson_tail(removed, 64);
+  double fail = poisson_tail(removed, 64);
+  for (int i = 0; i < Q; ++i) fail += poisson_tail(Q * mean_occupation * w[i], 64);
   if (lattice == ILG_D2Q9) {
     const double a = axis_share(theta);
     fail += poisson_tail(moving * a, 33) + poisson_tail(moving * (1.0 - a), 33);
   } else {
     fail += poisson_tail(moving, 33);
   }
-  return fail > kGeneralShare ? 1u : 0u;
+  return fail > limit ? 1u : 0u;
 }
 
 uint64_t quantise_probability(double p) {
