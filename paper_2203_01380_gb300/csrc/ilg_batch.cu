@@ -123,22 +123,26 @@ struct ModeSums {
   }
 };
 
-// One thread: out[0..3] = the 128-bit sums (L 2^62 re, L 2^62 im) of a state as (lo, hi)
-// pairs, from the warps' partials red[4 warp + k] and the ring's c[k] = sum_x of the
-// parts of its trigonometric values.
-__device__ void write_sums(const long long* red, uint32_t warps, const long long* c, uint32_t L, uint64_t mass,
-                           long long* out) {
-  long long v[4] = {0, 0, 0, 0};
-  for (uint32_t w = 0; w < warps; ++w)
+// One warp: the 128-bit sums (L 2^62 re, L 2^62 im) of `count` <= 8 states, each as two (lo,
+// hi) pairs in out[4 i .. 4 i + 3], from the partial sums red(i)[4 j + k] of R warps and the
+// ring's c[k] = sum_x of the parts of its trigonometric values.  Lane 4 i + k adds up part k
+// of state i.
+template <uint32_t R, class Red>
+__device__ __forceinline__ void write_sums(const Red& red, uint32_t count, const long long* c, uint32_t L, uint64_t mass,
+                                           long long* out) {
+  const uint32_t lane = threadIdx.x & 31u, i = lane >> 2, k = lane & 3u;
+  long long v = 0;
+  if (i < count) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] += red[4 * w + k];
-#pragma unroll
-  for (int k = 0; k < 4; k += 2) {
-    const __int128 S = (__int128(v[k + 1]) << 32) + v[k];
+    for (uint32_t j = 0; j < R; ++j) v += red(i)[4 * j + k];
+  }
+  const long long high = __shfl_down_sync(kFullWarp, v, 1);  // even lanes: the high part beside the low one
+  if (i < count && (k & 1u) == 0) {
+    const __int128 S = (__int128(high) << 32) + v;
     const __int128 C = (__int128(c[k + 1]) << 32) + c[k];
     const __int128 r = S * __int128(L) - C * __int128((long long)mass);
-    out[k] = (long long)(unsigned long long)r;
-    out[k + 1] = (long long)(r >> 64);
+    out[lane] = (long long)(unsigned long long)r;
+    out[lane + 1] = (long long)(r >> 64);
   }
 }
 
@@ -164,55 +168,111 @@ __device__ __forceinline__ void make_step_keys(const StepArgs& a, uint32_t t0, u
 // draw takes two instructions fewer), packed where several share an SM.  Measured
 // against per-lane loops and one 128-bit projection per node and step: 2048 rings of 64 to
 // 8192 nodes x 2000 steps 205 ms / 249 ms; 512 rings of 320 nodes x 2000 steps with
-// statistics 7.9 / 10.6 ms; one ring of 256 nodes with its records 1.45 / 2.0 us per step.
+// statistics 7.0 / 10.6 ms; one ring of 256 nodes with its records 1.07 / 2.06 us per step.
 template <int THREADS>
 struct BatchShape {
   static constexpr int kPerSm = 1024 / THREADS;
   static constexpr bool kPairs = THREADS == 1024;
   static constexpr uint32_t kTableWords = kPairs ? kDevStagedWords : kDevTableWords4;
   static constexpr uint32_t kRing = kBatchExtWords;
-  // states whose partial sums are written out together: by one warp each, every kGroup
-  // steps, so that no step waits for one thread to add them up
-  static constexpr uint32_t kGroup = THREADS == 1024 ? 2 : (THREADS == 512 ? 4 : 8);
+  // Warps that only record (the mode's sums, the states), beside those that collide: a
+  // state's sums are taken while the next one is made, off the step's chain of waits, and
+  // added up across these few warps instead of all.  Bound by the loads of the
+  // trigonometric values (16 bytes per node; 131 KB for 8192 nodes come from L2), hence
+  // their number: with one to three, rings of 8192 nodes at 10 per velocity took 19.7 us
+  // per step.  Against colliding warps that record as well, per step: one ring of 256 nodes
+  // 1.01 / 1.28 us, with its states 1.07 / 1.41; 512 rings of 320 nodes 3.51 / 3.91; 152
+  // rings of 8192 nodes at 10 per velocity 10.5 / 11.6, at 100 25.6 / 25.4.
+  static constexpr uint32_t kRecorders = THREADS == 1024 ? 8 : (THREADS == 512 ? 4 : 2);
+  // most threads of a block: the recording warps come on top where a 256-thread block has
+  // an SM to itself
+  static constexpr int kMost = THREADS + (THREADS == 256 ? 64 : 0);
 };
 
 // The shared memory of a batch block beside its dynamic part.
 template <int THREADS>
 struct BatchShared {
-  static constexpr uint32_t kSlots = 2 * BatchShape<THREADS>::kGroup;
+  // states whose partial sums are written out together, and room for as many again
+  static constexpr uint32_t kGroup = 8, kSlots = 2 * kGroup;
   uint32_t task;
   uint32_t fail;  // first step that would overflow
   unsigned long long mass;
-  long long c[4];                                // sums of the mode's trigonometric values
-  long long red[kSlots][4 * (THREADS / 32)];     // partial sums of the last states
-  BatchStepKeys keys[2][32];                     // of 64 steps
+  long long c[4];  // sums of the mode's trigonometric values
+  long long red[kSlots][4 * BatchShape<THREADS>::kRecorders];  // partial sums of the last states
+  BatchStepKeys keys[2][32];                                   // of 64 steps
 };
 
-// All steps of one ring that lies in src (3 planes of L; dst: the other buffer), by the
-// first `warps` warps of the block.  REC: the mode's sums at every state; STATES: every
-// state to b.states; TABLES: see collide_warp (and the binomial sampler).  Returns the
-// steps done; src is the buffer that holds the state.
+// All steps of one ring that lies in src (3 planes of L; dst: the other buffer): the first
+// `colliders` warps of the block collide, the recording warps (REC: the mode's sums at every
+// state; STATES: every state to b.states) follow them and see a state's planes in the step
+// that reads them.  TABLES: see collide_warp (and the binomial sampler).  Returns the steps
+// done; src is the buffer that holds the state.
 template <int THREADS, bool REC, bool STATES, bool TABLES, class Tab>
 __device__ __forceinline__ uint32_t run_ring(const BatchArgs& b, const StepArgs& a, const ReplicaDesc& d, uint32_t r,
                                              const uint32_t* tables, const Tab& to, const Tab& tr, unsigned char* words,
-                                             BatchShared<THREADS>& sh, uint16_t*& src, uint16_t* dst, uint32_t warps) {
+                                             BatchShared<THREADS>& sh, uint16_t*& src, uint16_t* dst, uint32_t colliders) {
   constexpr uint32_t S = 4 * THREADS;
-  constexpr uint32_t kGroup = BatchShape<THREADS>::kGroup, kSlots = BatchShared<THREADS>::kSlots;
-  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, threads = blockDim.x;
+  constexpr uint32_t R = REC || STATES ? BatchShape<THREADS>::kRecorders : 0;
+  constexpr uint32_t kGroup = BatchShared<THREADS>::kGroup, kSlots = BatchShared<THREADS>::kSlots;
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   const uint32_t L = d.L, T = b.T;
   const uint64_t mass = sh.mass;
   // no occupation can pass 65535 while the whole ring holds no more than that
   const bool safe = mass <= 65535ull;
-  const longlong2* trig = REC ? b.trig + d.state_off / 3 : nullptr;  // this ring's values
-  const auto bar = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(warps * 32) : "memory"); };
+  const auto bar = [&]() { asm volatile("bar.sync 1, %0;" ::"r"((colliders + R) * 32) : "memory"); };
+  // (a faster warp may already have marked the next step)
+  const auto stopped = [&](uint32_t s) { return !safe && *reinterpret_cast<volatile uint32_t*>(&sh.fail) <= s; };
   // the flip F_i(n) = n_{-i}: velocity i of the collision reads plane -i
   const uint32_t p1 = d.flip ? 2 * L : L, p2 = d.flip ? L : 2 * L;
+  uint32_t s = 0;
+  if (R != 0 && warp >= colliders) {
+    const uint32_t j = warp - colliders;
+    const longlong2* trig = REC ? b.trig + d.state_off / 3 : nullptr;  // this ring's values
+    const auto red = [&](uint32_t st) { return sh.red[st % kSlots]; };
+    const auto write_group = [&](uint32_t s0, uint32_t count) {
+      write_sums<R>([&](uint32_t i) { return red(s0 + i); }, count, sh.c, L, mass,
+                    b.record + (size_t(r) * (T + 1) + s0) * 4);
+    };
+    for (;; ++s) {
+      ModeSums ms;
+      if constexpr (REC) ms.clear();
+      // the state after step s - 1, planes rest, +1, -1
+      uint16_t* const rs = STATES && s > 0 ? b.states + d.state_off * T + size_t(s - 1) * 3 * L : nullptr;
+#pragma unroll 4
+      for (uint32_t x = 32 * j + lane; x < L; x += 32 * R) {
+        const uint32_t m0 = src[x], m1 = src[L + x], m2 = src[2 * L + x];
+        if constexpr (REC) ms.add(trig[x], m0 + m1 + m2);
+        if constexpr (STATES) {
+          if (s > 0) {
+            rs[x] = uint16_t(m0);
+            rs[L + x] = uint16_t(m1);
+            rs[2 * L + x] = uint16_t(m2);
+          }
+        }
+      }
+      if constexpr (REC) {
+        const long long v = ms.warp_sum(lane);
+        if ((lane & 7) == 0) red(s)[4 * j + (lane >> 3)] = v;
+      }
+      if (s == T) break;
+      bar();
+      if (stopped(s)) break;  // src still holds the state
+      uint16_t* tmp = src;
+      src = dst;
+      dst = tmp;
+      if (REC && (s % kGroup) == kGroup - 1 && j == 0) write_group(s - (kGroup - 1), kGroup);
+    }
+    bar();
+    if constexpr (REC) {
+      // the states since the last group (s: the last state whose sums exist)
+      if (j == 0) write_group(s / kGroup * kGroup, s % kGroup + 1);
+    }
+    return s;
+  }
   WordKeys k;
   k.slot.A = uint32_t((uint64_t(0xCD9E8D57u) * a.replica) >> 32) ^ a.rk[0];
   k.ext_e = uint32_t(uint64_t(0xCD9E8D57u) * a.replica) ^ a.rk[2];
-  uint32_t s = 0;
-  for (;; ++s) {
-    if (!REC && !STATES && s == T) break;
+  for (; s < T; ++s) {
     {
       const uint4* q = reinterpret_cast<const uint4*>(&sh.keys[(s >> 5) & 1][s & 31]);
       const uint4 k0 = q[0], k1 = q[1];
@@ -226,28 +286,13 @@ __device__ __forceinline__ uint32_t run_ring(const BatchArgs& b, const StepArgs&
       k.ext_c = k1.w;
     }
     bool bad = false;
-    ModeSums ms;
-    if constexpr (REC) ms.clear();
-    for (uint32_t x0 = warp * 32; x0 < L; x0 += threads) {
+    for (uint32_t x0 = warp * 32; x0 < L; x0 += colliders * 32) {
       const uint32_t x = x0 + lane;
       const bool active = x < L;
       uint32_t m[3], post[3];
       m[0] = active ? src[x] : 0u;
       m[1] = active ? src[p1 + x] : 0u;
       m[2] = active ? src[p2 + x] : 0u;
-      if constexpr (REC) {
-        if (active) ms.add(trig[x], m[0] + m[1] + m[2]);
-      }
-      if constexpr (STATES) {
-        if (s > 0 && active) {
-          // the state after step s - 1, planes rest, +1, -1
-          uint16_t* rs = b.states + d.state_off * T + size_t(s - 1) * 3 * L + x;
-          rs[0] = uint16_t(m[0]);
-          rs[p1] = uint16_t(m[1]);
-          rs[p2] = uint16_t(m[2]);
-        }
-      }
-      if ((REC || STATES) && s == T) continue;
       if (!TABLES && a.particle) collide_particle<3>(a, tables, x, d.t + s, m, post);
       else collide_warp<3, S, BatchShape<THREADS>::kRing, TABLES>(a, k, to, tr, tr, words, 4 * tid, x, m, post);
       if (active) {
@@ -257,42 +302,22 @@ __device__ __forceinline__ uint32_t run_ring(const BatchArgs& b, const StepArgs&
         dst[2 * L + (x == 0 ? L - 1 : x - 1)] = uint16_t(post[2]);
       }
     }
-    if constexpr (REC) {
-      // the partial sums of state s; kGroup states at a time are written out, one per
-      // warp, after the barrier that follows the last of them
-      const long long v = ms.warp_sum(lane);
-      if ((lane & 7) == 0) sh.red[s % kSlots][4 * warp + (lane >> 3)] = v;
-    }
-    if ((REC || STATES) && s == T) break;
     if (bad) atomicMin(&sh.fail, s);
     bar();
-    // (a faster warp may already have marked the next step)
-    if (!safe && *reinterpret_cast<volatile uint32_t*>(&sh.fail) <= s) break;  // src still holds the state
+    if (stopped(s)) break;  // src still holds the state
     // the steps' launch-wide Philox words, over those of the 32 steps just done
     if (warp == 0 && (s & 31) == 31) make_step_keys(a, d.t, s + 33, sh.keys);
     uint16_t* tmp = src;
     src = dst;
     dst = tmp;
-    if (REC && (s % kGroup) == kGroup - 1) {
-      for (uint32_t g = warp; g < kGroup; g += warps)
-        if (lane == 0) {
-          const uint32_t st = s - (kGroup - 1) + g;
-          write_sums(sh.red[st % kSlots], warps, sh.c, L, mass, b.record + (size_t(r) * (T + 1) + st) * 4);
-        }
-    }
   }
   bar();
-  if constexpr (REC) {
-    // the states since the last group (s: the last state whose sums exist)
-    for (uint32_t st = s / kGroup * kGroup + warp; st <= s; st += warps)
-      if (lane == 0)
-        write_sums(sh.red[st % kSlots], warps, sh.c, L, mass, b.record + (size_t(r) * (T + 1) + st) * 4);
-  }
   return s;
 }
 
 template <int THREADS, bool REC, bool STATES>
-__global__ void __launch_bounds__(THREADS, BatchShape<THREADS>::kPerSm)
+__global__ void __launch_bounds__(REC || STATES ? BatchShape<THREADS>::kMost : THREADS,
+                                  REC || STATES ? 65536 / (64 * BatchShape<THREADS>::kMost) : BatchShape<THREADS>::kPerSm)
     batch_d1q3_kernel(const __grid_constant__ BatchArgs b, const __grid_constant__ StepArgs common) {
   using Shape = BatchShape<THREADS>;
   using Tab = std::conditional_t<Shape::kPairs, Alias8, Alias4>;
@@ -356,15 +381,17 @@ __global__ void __launch_bounds__(THREADS, BatchShape<THREADS>::kPerSm)
       make_step_keys(a, d.t, 32, sh.keys);
     }
     __syncthreads();
-    const uint32_t warps = (min(L, threads) + 31) >> 5;  // the others have no node of this ring
-    if (warp < warps) {
+    // the ring's colliding warps, and those that record it; the others have nothing to do
+    constexpr uint32_t R = REC || STATES ? Shape::kRecorders : 0;
+    const uint32_t colliders = min((L + 31) >> 5, threads / 32 - R);
+    if (warp < colliders + R) {
       uint16_t* src = ring;
       const bool plain = !a.particle && a.omega_mode == kTable && a.rest_mode == kTable;
       const uint32_t done =
-          plain ? run_ring<THREADS, REC, STATES, true>(b, a, d, r, tables, to, tr, words, sh, src, ring + 3 * L, warps)
-                : run_ring<THREADS, REC, STATES, false>(b, a, d, r, tables, to, tr, words, sh, src, ring + 3 * L, warps);
+          plain ? run_ring<THREADS, REC, STATES, true>(b, a, d, r, tables, to, tr, words, sh, src, ring + 3 * L, colliders)
+                : run_ring<THREADS, REC, STATES, false>(b, a, d, r, tables, to, tr, words, sh, src, ring + 3 * L, colliders);
       // ring back to global memory; the replica's step counter moves on
-      for (uint32_t i = tid; i < 3 * L; i += warps * 32) gs[i] = src[i];
+      for (uint32_t i = tid; i < 3 * L; i += (colliders + R) * 32) gs[i] = src[i];
       if (tid == 0) {
         b.desc[r].t = d.t + done;
         if (sh.fail != ~0u) b.failed[r] = 1u;
@@ -425,11 +452,19 @@ cudaError_t prepare_batch_kernel(uint32_t Lmax, int threads) {
 
 // Persistent grid: as many blocks as fit on every SM (shared memory and registers
 // decide), at most one per ring.  A block has as many of its shape's threads as the longest
-// ring keeps equally busy (320 nodes on the 256-thread shape: 160 threads, two nodes each).
+// ring keeps equally busy (320 nodes on the 256-thread shape: 160 threads, two nodes each),
+// and the recording warps.
 cudaError_t launch_batch(const BatchArgs& b, const StepArgs& common, int sms, cudaStream_t s, int shape) {
   const size_t smem = batch_smem_bytes(b.Lmax, shape);
-  const uint32_t rounds = (b.Lmax + uint32_t(shape) - 1) / uint32_t(shape);
-  const int threads = int(((b.Lmax + rounds - 1) / rounds + 31) / 32 * 32);
+  const bool rec = b.record != nullptr || b.states != nullptr;
+  const uint32_t most = uint32_t(shape) / 32, tiles = (b.Lmax + 31) / 32;
+  const uint32_t recorders = !rec ? 0u : shape == 1024 ? BatchShape<1024>::kRecorders
+                                      : shape == 512   ? BatchShape<512>::kRecorders
+                                                       : BatchShape<256>::kRecorders;
+  // all of the shape's warps collide where a block has an SM to itself
+  const uint32_t room = shape == 256 && b.n <= uint32_t(sms) ? most : most - recorders;
+  const uint32_t rounds = (tiles + room - 1) / room;
+  const int threads = int(((tiles + rounds - 1) / rounds + recorders) * 32);
   const void* fn = batch_fn(shape, b.record != nullptr, b.states != nullptr);
   int per_sm = 1;
   const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem);
