@@ -10,6 +10,15 @@
 // result without a branch.  The words beyond the slot words wait in a ring of K words
 // per lane in shared memory (lane-interleaved, so no access conflicts), filled one
 // Philox block at a time by all lanes together when one of them runs short.
+//
+// A vote costs some 40 cycles of latency and three issue slots, so few stand in a node's
+// chain: one asks whether any occupation exceeds a chunk; behind it three are asked at once,
+// the first block is made without asking, and the rest velocity (which holds the most in
+// equilibrium) takes its further chunks by itself.  Against a vote for every block and a
+// second chunk drawn for all velocities, us per step: D2Q5 1024^2 at 50 per velocity 25.5 /
+// 27.5 (omega* = 0.5), 16.2 / 18.4 (0.1), 1501 x 777 at 100 44.8 / 52.2; D2Q9 1024^2 at 50
+// 49.6 / 56.0; where nothing exceeds a chunk it is the same (D2Q5 768^2 at 10: 8.25) up to
+// 5 % slower (rings of 8192 nodes at 10: 8.56 / 8.13).
 #pragma once
 
 #include <cstdint>
@@ -94,12 +103,21 @@ struct NodeWords {
     wr += 4 * S;
     blk += 1;
   }
-  // every lane has at least `bytes` of words afterwards (bytes <= (K - 4) S, a multiple of
-  // S); lanes with room fill together
-  template <class Keys>
+  // every lane has at least `bytes` of words afterwards (at most MAX words, MAX <= K - 4);
+  // lanes with room fill together.  A lane without room has more than K - 8 words, so one
+  // block is enough for four words in a ring of more than 8; in a ring of 8 the single test
+  // gained nothing (rings of 256 nodes 0.85 instead of 0.83 us per step).
+  template <uint32_t MAX, class Keys>
   __device__ __forceinline__ void ensure(const Keys& k, const uint32_t (&rk)[20], uint32_t bytes) {
-    while (__any_sync(kFullWarp, wr - rd < bytes)) {
-      if (wr - rd <= (K - 4) * S) fill(k, rk);
+    static_assert(MAX <= K - 4, "whole blocks must fit beside what is asked for");
+    if constexpr (MAX <= 4 && K > 8) {
+      if (__any_sync(kFullWarp, wr - rd < bytes)) {
+        if (wr - rd <= (K - 4) * S) fill(k, rk);
+      }
+    } else {
+      while (__any_sync(kFullWarp, wr - rd < bytes)) {
+        if (wr - rd <= (K - 4) * S) fill(k, rk);
+      }
     }
   }
   // the word `ahead` places after the next one
@@ -116,7 +134,7 @@ __device__ __forceinline__ uint32_t more_chunks(NodeWords<S, K>& e, const Keys& 
                                                 const Tab& A, int32_t left) {
   uint32_t r = 0;
   while (__any_sync(kFullWarp, left > 0)) {
-    e.ensure(k, rk, left > int32_t(kDevNmax) ? 2 * S : (left > 0 ? S : 0u));
+    e.template ensure<2>(k, rk, left > int32_t(kDevNmax) ? 2 * S : (left > 0 ? S : 0u));
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
       r += A(uint32_t(__vimin_s32_relu(left, int32_t(kDevNmax))), e.peek());
@@ -136,25 +154,27 @@ struct BitCounts {
 template <uint32_t S, uint32_t K, class Keys>
 __device__ __forceinline__ BitCounts count_bits(NodeWords<S, K>& e, const Keys& k, const uint32_t (&rk)[20], uint32_t c,
                                                 uint32_t A, uint32_t B) {
-  constexpr uint32_t kPass = (K - 4 < 8 ? K - 4 : 8) / 2;  // groups whose words are asked for at once
+  constexpr uint32_t kPass = 2;  // groups whose words (one block) are asked for at once
   int32_t left = int32_t(c);
   uint32_t mask = __funnelshift_lc(kFullWarp, 0u, uint32_t(left));
   left = max(left - 32, 0);
   A &= mask;
   B &= mask;
   BitCounts n{uint32_t(__popc(A)), uint32_t(__popc(A & B)), uint32_t(__popc(B & ~A))};
+  const auto group = [&]() {
+    mask = __funnelshift_lc(kFullWarp, 0u, uint32_t(left));
+    A = e.peek() & mask;
+    B = e.peek(1) & mask;
+    n.a += __popc(A);
+    n.both += __popc(A & B);
+    n.b += __popc(B & ~A);
+    if (left > 0) e.rd += 2 * S;
+    left = max(left - 32, 0);
+  };
   while (__any_sync(kFullWarp, left > 0)) {
-    e.ensure(k, rk, min(uint32_t(left + 31) >> 5, kPass) * (2 * S));
-    for (uint32_t u = 0; u < kPass && __any_sync(kFullWarp, left > 0); ++u) {
-      mask = __funnelshift_lc(kFullWarp, 0u, uint32_t(left));
-      A = e.peek() & mask;
-      B = e.peek(1) & mask;
-      n.a += __popc(A);
-      n.both += __popc(A & B);
-      n.b += __popc(B & ~A);
-      if (left > 0) e.rd += 2 * S;
-      left = max(left - 32, 0);
-    }
+    e.template ensure<2 * kPass>(k, rk, min(uint32_t(left + 31) >> 5, kPass) * (2 * S));
+    group();
+    for (uint32_t u = 1; u < kPass && __any_sync(kFullWarp, left > 0); ++u) group();
   }
   return n;
 }
@@ -188,26 +208,39 @@ __device__ __forceinline__ void collide_warp(const StepArgs& a, const Keys& k, c
   // thinning
   uint32_t r[Q], removed = 0;
   if (TABLES || a.omega_mode == kTable) {
-    uint32_t most = m[0];
+    uint32_t most = m[1];
 #pragma unroll
-    for (int i = 1; i < Q; ++i) most = max(most, m[i]);
+    for (int i = 2; i < Q; ++i) most = max(most, m[i]);
 #pragma unroll
     for (int i = 0; i < Q; ++i) r[i] = to(min(m[i], kDevNmax), W[i]);
-    if (__any_sync(kFullWarp, most > uint32_t(kN))) {
-      if (!__any_sync(kFullWarp, most > uint32_t(2 * kN))) {
-        // one more chunk at most: no loop
-        uint32_t need = 0;
+    if (__any_sync(kFullWarp, max(most, m[0]) > uint32_t(kN))) {
+      const bool rest1 = __any_sync(kFullWarp, m[0] > uint32_t(kN)), move1 = __any_sync(kFullWarp, most > uint32_t(kN)),
+                 move2 = __any_sync(kFullWarp, most > uint32_t(2 * kN));
+      e.fill(k, a.rk);  // no lane has a word yet
+      if (rest1) {
+        // the rest velocity by itself: it holds the most in equilibrium, often alone
+        const int32_t left = int32_t(m[0]) - kN;
+        const bool two = __any_sync(kFullWarp, left > kN);
+        r[0] += to(uint32_t(__vimin_s32_relu(left, kN)), e.peek());
+        if (left > 0) e.rd += S;
+        if (two) r[0] += more_chunks(e, k, a.rk, to, left - kN);
+      }
+      if (move1) {
+        if (!move2) {
+          // one more chunk at most: no loop
+          uint32_t need = 0;
 #pragma unroll
-        for (int i = 0; i < Q; ++i) need += m[i] > uint32_t(kN) ? S : 0u;
-        e.ensure(k, a.rk, need);
+          for (int i = 1; i < Q; ++i) need += m[i] > uint32_t(kN) ? S : 0u;
+          e.template ensure<Q - 1>(k, a.rk, need);
 #pragma unroll
-        for (int i = 0; i < Q; ++i) {
-          r[i] += to(uint32_t(max(int32_t(m[i]) - kN, 0)), e.peek());
-          if (m[i] > uint32_t(kN)) e.rd += S;
+          for (int i = 1; i < Q; ++i) {
+            r[i] += to(uint32_t(max(int32_t(m[i]) - kN, 0)), e.peek());
+            if (m[i] > uint32_t(kN)) e.rd += S;
+          }
+        } else {
+#pragma unroll
+          for (int i = 1; i < Q; ++i) r[i] += more_chunks(e, k, a.rk, to, int32_t(m[i]) - kN);
         }
-      } else {
-#pragma unroll
-        for (int i = 0; i < Q; ++i) r[i] += more_chunks(e, k, a.rk, to, int32_t(m[i]) - kN);
       }
     }
   } else {
@@ -236,13 +269,13 @@ __device__ __forceinline__ void collide_warp(const StepArgs& a, const Keys& k, c
   const uint32_t moving = removed - to_rest;
   if constexpr (Q == 3) {
     // one sign word per group
-    constexpr uint32_t kPass = K - 4 < 8 ? K - 4 : 8;
+    constexpr uint32_t kPass = 4;
     int32_t left = int32_t(moving);
     uint32_t mask = __funnelshift_lc(kFullWarp, 0u, uint32_t(left));
     uint32_t minus = __popc(W[Q + 1] & mask);
     left = max(left - 32, 0);
     while (__any_sync(kFullWarp, left > 0)) {
-      e.ensure(k, a.rk, min(uint32_t(left + 31) >> 5, kPass) * S);
+      e.template ensure<kPass>(k, a.rk, min(uint32_t(left + 31) >> 5, kPass) * S);
       for (uint32_t u = 0; u < kPass && __any_sync(kFullWarp, left > 0); ++u) {
         mask = __funnelshift_lc(kFullWarp, 0u, uint32_t(left));
         minus += __popc(e.peek() & mask);

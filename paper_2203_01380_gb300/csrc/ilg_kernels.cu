@@ -25,8 +25,8 @@ namespace ilg {
 // once, in the 64-bit form whose draw takes two instructions fewer than the packed one
 // (29.1 against 31.0 us per step for two blocks of 512, 33 with packed tables).  Us per
 // step against one launch per step with a collision that loops per lane: 1024^2 at 50 per
-// velocity 28.6 / 37.3 (omega* 0.5), 19.8 / 26.8 (0.1); 1501 x 777 at 100 per velocity
-// 55 / 66; 1024^2 at 200 per velocity, omega* = 1, 93 / 241; 96 x 40 2.2 / 18.7.
+// velocity 25.5 / 37.3 (omega* 0.5), 16.2 / 26.8 (0.1); 1501 x 777 at 100 per velocity
+// 44.8 / 66; 1024^2 at 200 per velocity, omega* = 1, 85 / 241; 96 x 40 2.2 / 18.7.
 // --------------------------------------------------------------------------
 constexpr uint32_t kStepRing = 16;  // extension words per lane
 
