@@ -26,6 +26,10 @@ namespace {
 
 constexpr int kLbThreads = 256;
 constexpr uint32_t kLbMaxModes = 256;
+constexpr int kLbModeThreads = 64;     // of a projection's blocks
+constexpr uint32_t kLbCols = 32;       // columns of a block of their sums (or kLbThreads)
+constexpr uint32_t kLbFewRows = 8;
+constexpr uint32_t kLbFirstModes = 64; // passed as a kernel argument
 constexpr uint32_t kLbRowChunk = 64;   // rows per partial column sum
 constexpr uint32_t kLbChunk = 4096;    // entries per partial of a projection
 
@@ -200,35 +204,6 @@ __global__ void __launch_bounds__(kLbThreads) lb_init_kernel(const double* __res
   }
 }
 
-// Partial column sums of rho over a chunk of kLbRowChunk rows (fixed order).
-template <int Q>
-__global__ void __launch_bounds__(kLbThreads) lb_colpart_kernel(const double* __restrict__ f, uint32_t Lx,
-                                                               uint32_t Ly, double* __restrict__ part) {
-  const uint32_t x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= Lx) return;
-  const size_t plane = size_t(Lx) * Ly;
-  const uint32_t y0 = blockIdx.y * kLbRowChunk;
-  const uint32_t y1 = y0 + kLbRowChunk < Ly ? y0 + kLbRowChunk : Ly;
-  double s = 0.0;
-  for (uint32_t y = y0; y < y1; ++y) {
-    const size_t at = size_t(y) * Lx + x;
-    double n = f[at];
-#pragma unroll
-    for (int i = 1; i < Q; ++i) n += f[i * plane + at];
-    s += n;
-  }
-  part[size_t(blockIdx.y) * Lx + x] = s;
-}
-
-__global__ void lb_colsum_kernel(const double* __restrict__ part, uint32_t Lx, uint32_t chunks,
-                                 double* __restrict__ col) {
-  const uint32_t x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= Lx) return;
-  double s = 0.0;
-  for (uint32_t g = 0; g < chunks; ++g) s += part[size_t(g) * Lx + x];
-  col[x] = s;
-}
-
 // Row sums of rho: one block per row, strided accumulation, fixed tree.
 template <int Q>
 __global__ void __launch_bounds__(kLbThreads) lb_rowsum_kernel(const double* __restrict__ f, uint32_t Lx,
@@ -278,23 +253,94 @@ struct Acc {
 };
 
 // Fixed-order block reduction of the threads' accumulators (the same tree for
-// every launch shape with kLbThreads threads).
+// every launch shape with N threads).
+template <int N>
 __device__ Acc block_acc(Acc a, double* ss, double* se) {
   ss[threadIdx.x] = a.s;
   se[threadIdx.x] = a.e;
   __syncthreads();
-  for (int h = kLbThreads / 2; h > 0; h >>= 1) {
+  for (int h = N / 2; h > 0; h >>= 1) {
     if (int(threadIdx.x) < h) {
-      Acc l{ss[threadIdx.x], se[threadIdx.x]};
-      l.merge(Acc{ss[threadIdx.x + h], se[threadIdx.x + h]});
-      ss[threadIdx.x] = l.s;
-      se[threadIdx.x] = l.e;
+      a.merge(Acc{ss[threadIdx.x + h], se[threadIdx.x + h]});
+      ss[threadIdx.x] = a.s;
+      se[threadIdx.x] = a.e;
     }
     __syncthreads();
   }
   const Acc r{ss[0], se[0]};
   __syncthreads();
   return r;
+}
+
+// True in every thread of the last of `blocks` blocks to come here (which sees what the
+// others wrote, through L2); it leaves the counter at zero for the next launch.
+__device__ bool last_block(uint32_t* counter, uint32_t blocks) {
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    last = atomicAdd(counter, 1u) == blocks - 1;
+    if (last) *counter = 0;
+  }
+  __syncthreads();
+  __threadfence();
+  return last;
+}
+
+// Column sums of rho: a block adds kLbRowChunk rows of COLS columns, every kLbThreads / COLS-th
+// part of the rows in other warps (one thread for all 64 rows waited 43 us for its loads on
+// a 64 x 64 lattice, with its mass and one mode 95 us, here 58), the last block of the
+// columns adds those partial sums, in a fixed order each, and, with mass != NULL (at most
+// kLbChunk columns), the last block of all the columns: one launch instead of four.  Bound
+// on small lattices: the launch and the loads' latency; on large ones the state's bytes.
+template <int Q, uint32_t COLS>
+__global__ void __launch_bounds__(kLbThreads) lb_col_kernel(const double* __restrict__ f, uint32_t Lx, uint32_t Ly,
+                                                           double* __restrict__ part, double* __restrict__ col,
+                                                           uint32_t* __restrict__ count, double* __restrict__ mass) {
+  constexpr uint32_t kGroups = kLbThreads / COLS, kRows = kLbRowChunk / kGroups;
+  __shared__ double ss[kLbThreads], se[kLbThreads];
+  const uint32_t c = threadIdx.x % COLS, g = threadIdx.x / COLS;
+  const uint32_t x = blockIdx.x * COLS + c;
+  const size_t plane = size_t(Lx) * Ly;
+  const auto groups_sum = [&](double v) {  // (valid in the first group)
+    if constexpr (kGroups > 1) {
+      ss[threadIdx.x] = v;
+      __syncthreads();
+#pragma unroll
+      for (uint32_t i = 1; i < kGroups; ++i) v += ss[(threadIdx.x + i * COLS) % kLbThreads];
+      __syncthreads();
+    }
+    return v;
+  };
+  double s = 0.0;
+  const uint32_t y0 = blockIdx.y * kLbRowChunk + g * kRows;
+  if (x < Lx) {
+#pragma unroll 8
+    for (uint32_t y = y0; y < min(y0 + kRows, Ly); ++y) {
+      const double* const p = f + (size_t(y) * Lx + x);
+      double n = p[0];
+#pragma unroll
+      for (int i = 1; i < Q; ++i) n += p[i * plane];
+      s += n;
+    }
+  }
+  s = groups_sum(s);
+  if (gridDim.y > 1) {
+    if (g == 0 && x < Lx) part[size_t(blockIdx.y) * Lx + x] = s;
+    if (!last_block(count + blockIdx.x, gridDim.y)) return;
+    s = 0.0;
+    if (x < Lx) {
+#pragma unroll 4
+      for (uint32_t i = g; i < gridDim.y; i += kGroups) s += __ldcg(part + size_t(i) * Lx + x);
+    }
+    s = groups_sum(s);
+  }
+  if (g == 0 && x < Lx) col[x] = s;
+  if (!mass || !last_block(count + gridDim.x, gridDim.x)) return;
+  Acc a;
+  for (uint32_t i = threadIdx.x; i < Lx; i += kLbThreads) a.add(__ldcg(col + i));
+  const Acc r = block_acc<kLbThreads>(a, ss, se);
+  if (threadIdx.x == 0) *mass = r.s + r.e;
 }
 
 // Partial sums over chunks of kLbChunk consecutive entries; part[c] = (s, e).
@@ -305,30 +351,53 @@ __global__ void __launch_bounds__(kLbThreads) lb_mass_partial_kernel(const doubl
   const uint32_t x1 = x0 + kLbChunk < Lx ? x0 + kLbChunk : Lx;
   Acc a;
   for (uint32_t x = x0 + threadIdx.x; x < x1; x += kLbThreads) a.add(col[x]);
-  const Acc r = block_acc(a, ss, se);
+  const Acc r = block_acc<kLbThreads>(a, ss, se);
   if (threadIdx.x == 0) part[blockIdx.x] = make_double2(r.s, r.e);
 }
 
-// Block (c, j): chunk c of mode j; part[(2j) P + c] = re, part[(2j+1) P + c] = im.
-// The mean M / L comes from out[0] (the mass, already combined).
-__global__ void __launch_bounds__(kLbThreads) lb_mode_partial_kernel(const double* __restrict__ col,
-                                                                    const double* __restrict__ row, uint32_t Lx,
-                                                                    uint32_t Ly, const int32_t* __restrict__ modes,
-                                                                    const double* __restrict__ out,
-                                                                    double2* __restrict__ part) {
-  __shared__ double ss[kLbThreads], se[kLbThreads];
-  const uint32_t j = blockIdx.y, P = gridDim.x;
-  const int32_t mx = modes[2 * j], my = modes[2 * j + 1];
+// The first modes of a call travel with the launch, without a copy of their own.
+struct LbModes {
+  int32_t m[2 * kLbFirstModes];
+};
+
+// Entries per block of a projection: one per thread while that makes at most 256 blocks (the
+// sines and cosines in double precision bound it: 1024 entries in one block of 256 threads
+// took 20 us), at most kLbChunk.
+__host__ __device__ inline uint32_t lb_mode_chunk(uint32_t L) {
+  if (L > 256u * kLbChunk) return kLbChunk;
+  return ((L + 255) / 256 + kLbModeThreads - 1) / kLbModeThreads * kLbModeThreads;
+}
+
+// Blocks of a projection along any side of at most maxL entries (a side just past a multiple
+// of 256 kLbModeThreads has fewer than a somewhat shorter one).
+inline uint32_t lb_mode_blocks(uint32_t maxL) {
+  return maxL > 256u * kLbChunk ? (maxL + kLbChunk - 1) / kLbChunk
+                                : std::min((maxL + kLbModeThreads - 1) / kLbModeThreads, 256u);
+}
+
+// Block (c, j): chunk c of mode j; part[(2j) P + c] = re, part[(2j+1) P + c] = im, and
+// the last block of a mode adds its P <= gridDim.x partials in a fixed order into
+// out[1 + 2 j], out[2 + 2 j].  The mean M / L comes from out[0] (the mass).  modes: NULL for
+// those in `first`.
+__global__ void __launch_bounds__(kLbModeThreads) lb_mode_kernel(const double* __restrict__ col, const double* __restrict__ row,
+                                                            uint32_t Lx, uint32_t Ly, const __grid_constant__ LbModes first,
+                                                            const int32_t* __restrict__ modes, double* __restrict__ out,
+                                                            double2* __restrict__ part, uint32_t* __restrict__ count) {
+  __shared__ double ss[kLbModeThreads], se[kLbModeThreads];
+  const uint32_t j = blockIdx.y;
+  const int32_t mx = modes ? modes[2 * j] : first.m[2 * j], my = modes ? modes[2 * j + 1] : first.m[2 * j + 1];
   const bool along_x = mx != 0;
   const uint32_t L = along_x ? Lx : Ly;
+  const uint32_t chunk = lb_mode_chunk(L), P = (L + chunk - 1) / chunk;
+  if (blockIdx.x >= P) return;
   const double* C = along_x ? col : row;
   const int64_t mr = along_x ? mx : my;
   const uint64_t mode = uint64_t(((mr % int64_t(L)) + int64_t(L)) % int64_t(L));
   const double mean = out[0] / double(L);
-  const uint32_t x0 = blockIdx.x * kLbChunk;
-  const uint32_t x1 = x0 + kLbChunk < L ? x0 + kLbChunk : L;
+  const uint32_t x0 = blockIdx.x * chunk;
+  const uint32_t x1 = x0 + chunk < L ? x0 + chunk : L;
   Acc re, im;
-  for (uint32_t x = x0 + threadIdx.x; x < x1; x += kLbThreads) {
+  for (uint32_t x = x0 + threadIdx.x; x < x1; x += kLbModeThreads) {
     const uint64_t r = (mode * x) % L;
     double sn, cs;
     sincospi(2.0 * double(r) / double(L), &sn, &cs);
@@ -336,25 +405,42 @@ __global__ void __launch_bounds__(kLbThreads) lb_mode_partial_kernel(const doubl
     re.add_product(cs, d);
     im.add_product(sn, d);
   }
-  const Acc a = block_acc(re, ss, se);
-  const Acc b = block_acc(im, ss, se);
+  Acc a = block_acc<kLbModeThreads>(re, ss, se);
+  Acc b = block_acc<kLbModeThreads>(im, ss, se);
+  if (P > 1) {
+    double2* const pr = part + size_t(2 * j) * gridDim.x;
+    double2* const pi = pr + gridDim.x;
+    if (threadIdx.x == 0) {
+      pr[blockIdx.x] = make_double2(a.s, a.e);
+      pi[blockIdx.x] = make_double2(b.s, b.e);
+    }
+    if (!last_block(count + j, P)) return;
+    re = im = Acc{};
+    for (uint32_t c = threadIdx.x; c < P; c += kLbModeThreads) {
+      const double2 u = __ldcg(pr + c), v = __ldcg(pi + c);
+      re.merge(Acc{u.x, u.y});
+      im.merge(Acc{v.x, v.y});
+    }
+    a = block_acc<kLbModeThreads>(re, ss, se);
+    b = block_acc<kLbModeThreads>(im, ss, se);
+  }
   if (threadIdx.x == 0) {
-    part[size_t(2 * j) * P + blockIdx.x] = make_double2(a.s, a.e);
-    part[size_t(2 * j + 1) * P + blockIdx.x] = make_double2(b.s, b.e);
+    out[1 + 2 * j] = a.s + a.e;
+    out[2 + 2 * j] = b.s + b.e;
   }
 }
 
-// Block q combines part[q P .. q P + P) in a fixed order into out[first + q].
+// Combines part[0 .. P) in a fixed order into *out (one block).
 __global__ void __launch_bounds__(kLbThreads) lb_combine_kernel(const double2* __restrict__ part, uint32_t P,
-                                                               double* __restrict__ out, uint32_t first) {
+                                                               double* __restrict__ out) {
   __shared__ double ss[kLbThreads], se[kLbThreads];
   Acc a;
   for (uint32_t c = threadIdx.x; c < P; c += kLbThreads) {
-    const double2 v = part[size_t(blockIdx.x) * P + c];
+    const double2 v = part[c];
     a.merge(Acc{v.x, v.y});
   }
-  const Acc r = block_acc(a, ss, se);
-  if (threadIdx.x == 0) out[first + blockIdx.x] = r.s + r.e;
+  const Acc r = block_acc<kLbThreads>(a, ss, se);
+  if (threadIdx.x == 0) *out = r.s + r.e;
 }
 
 }  // namespace
@@ -375,11 +461,14 @@ struct ilg_lb {
   double* d_part = nullptr;   // chunks x Lx partial column sums
   double* d_col = nullptr;    // Lx
   double* d_row = nullptr;    // Ly
-  double* d_out = nullptr;    // 1 + 2 kLbMaxModes
   double2* d_red = nullptr;   // projection partials, 2 kLbMaxModes x chunks
   int32_t* d_modes = nullptr; // 2 kLbMaxModes
-  unsigned long long* d_sync = nullptr;  // [0] barrier word of a several-step launch, [1] a wait gave up
+  // one allocation: [0] barrier word of a several-step launch, [1] a wait gave up, d_out, d_count
+  unsigned long long* d_sync = nullptr;
+  double* d_out = nullptr;               // mass, then re and im of each mode
+  uint32_t* d_count = nullptr;           // arrivals: kLbMaxModes, then the column blocks and one; zero between launches
   unsigned long long h_sync = 0;         // sync[1] as read back with the last results
+  bool waits = false;                    // several-step launches since sync[1] was read
   int run_blocks = 0;                    // resident blocks of the step kernel
   std::string err;
 };
@@ -431,6 +520,16 @@ const void* lb_run_fn(int Q) {
                   : reinterpret_cast<const void*>(lb_run_kernel<9>);
 }
 
+const void* lb_col_fn(int Q, bool wide) {
+  if (wide)
+    return Q == 3   ? reinterpret_cast<const void*>(lb_col_kernel<3, kLbThreads>)
+           : Q == 5 ? reinterpret_cast<const void*>(lb_col_kernel<5, kLbThreads>)
+                    : reinterpret_cast<const void*>(lb_col_kernel<9, kLbThreads>);
+  return Q == 3   ? reinterpret_cast<const void*>(lb_col_kernel<3, kLbCols>)
+         : Q == 5 ? reinterpret_cast<const void*>(lb_col_kernel<5, kLbCols>)
+                  : reinterpret_cast<const void*>(lb_col_kernel<9, kLbCols>);
+}
+
 // v = m 2^e with the top bit of m set; false unless v is positive and of ordinary size
 bool as_integer(double v, unsigned long long* m, int* e) {
   if (!(v >= 1e-15 && v <= 1e3)) return false;
@@ -446,6 +545,7 @@ bool as_integer(double v, unsigned long long* m, int* e) {
 ilg_status lb_gave_up(ilg_lb* b) {
   b->has_state = false;
   b->h_sync = 0;
+  b->waits = false;
   cudaMemsetAsync(b->d_sync, 0, 2 * sizeof(unsigned long long), b->stream);
   cudaStreamSynchronize(b->stream);
   return lb_fail(b, ILG_E_TIMEOUT, "a wait between the blocks of a several-step launch gave up: the state is lost");
@@ -493,12 +593,17 @@ ilg_status ilg_lb_create(const ilg_lb_params* params, void* stream, ilg_lb** out
   if (e == cudaSuccess) e = ilg::dev_alloc(&b->d_part, sizeof(double) * b->chunks * p.Lx);
   if (e == cudaSuccess) e = ilg::dev_alloc(&b->d_col, sizeof(double) * p.Lx);
   if (e == cudaSuccess) e = ilg::dev_alloc(&b->d_row, sizeof(double) * b->Ly);
-  if (e == cudaSuccess) e = ilg::dev_alloc(&b->d_out, sizeof(double) * (1 + 2 * kLbMaxModes));
   if (e == cudaSuccess) e = ilg::dev_alloc(&b->d_modes, sizeof(int32_t) * 2 * kLbMaxModes);
-  const size_t maxL = p.Lx > b->Ly ? p.Lx : b->Ly;
-  if (e == cudaSuccess) e = ilg::dev_alloc(&b->d_red, sizeof(double2) * 2 * kLbMaxModes * ((maxL + kLbChunk - 1) / kLbChunk));
-  if (e == cudaSuccess) e = ilg::dev_alloc(&b->d_sync, 2 * sizeof(unsigned long long));
-  if (e == cudaSuccess) e = cudaMemsetAsync(b->d_sync, 0, 2 * sizeof(unsigned long long), b->stream);
+  const uint32_t maxL = p.Lx > b->Ly ? p.Lx : b->Ly;
+  if (e == cudaSuccess) e = ilg::dev_alloc(&b->d_red, sizeof(double2) * 2 * kLbMaxModes * lb_mode_blocks(maxL));
+  const size_t words = 2 + 1 + 2 * kLbMaxModes, counters = kLbMaxModes + (p.Lx + kLbCols - 1) / kLbCols + 1;
+  const size_t small = sizeof(double) * words + sizeof(uint32_t) * counters;
+  if (e == cudaSuccess) e = ilg::dev_alloc(&b->d_sync, small);
+  if (e == cudaSuccess) {
+    b->d_out = reinterpret_cast<double*>(b->d_sync + 2);
+    b->d_count = reinterpret_cast<uint32_t*>(b->d_sync + words);
+    e = cudaMemsetAsync(b->d_sync, 0, small, b->stream);
+  }
   int per_sm = 0;
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lb_run_fn(b->Q), kLbThreads, 0);
   if (e != cudaSuccess) {
@@ -518,7 +623,6 @@ ilg_status ilg_lb_destroy(ilg_lb* b) {
   cudaFree(b->d_part);
   cudaFree(b->d_col);
   cudaFree(b->d_row);
-  cudaFree(b->d_out);
   cudaFree(b->d_modes);
   cudaFree(b->d_red);
   cudaFree(b->d_sync);
@@ -601,9 +705,11 @@ ilg_status ilg_lb_get_state(ilg_lb* b, double* host, size_t n, uint64_t* t) {
   if (!b->has_state) return lb_fail(b, ILG_E_STATE, "no state: call ilg_lb_init or ilg_lb_set_state first");
   if (!host || n != size_t(b->Q) * b->nodes) return lb_fail(b, ILG_E_INVALID, "state must hold Q*Lx*Ly doubles");
   LB_CUDA(b, cudaMemcpyAsync(host, b->f[b->cur], sizeof(double) * n, cudaMemcpyDeviceToHost, b->stream), "copy out");
-  LB_CUDA(b, cudaMemcpyAsync(&b->h_sync, b->d_sync + 1, sizeof(unsigned long long), cudaMemcpyDeviceToHost, b->stream),
-          "copy out");
+  if (b->waits)
+    LB_CUDA(b, cudaMemcpyAsync(&b->h_sync, b->d_sync + 1, sizeof(unsigned long long), cudaMemcpyDeviceToHost, b->stream),
+            "copy out");
   LB_CUDA(b, cudaStreamSynchronize(b->stream), "copy out");
+  b->waits = false;
   if (b->h_sync != 0) return lb_gave_up(b);
   if (t) *t = b->t;
   return ILG_OK;
@@ -629,6 +735,7 @@ ilg_status ilg_lb_step(ilg_lb* b, uint32_t T) {
         continue;
       }
       LB_CUDA(b, e, "lattice Boltzmann step");
+      b->waits = true;
     } else {
       LB_CUDA(b, cudaLaunchKernel(fn, dim3(b->run_blocks), dim3(kLbThreads), args, 0, b->stream), "lattice Boltzmann step");
     }
@@ -654,13 +761,21 @@ ilg_status ilg_lb_observables(ilg_lb* b, const int32_t* modes, uint32_t nmodes, 
   }
   const uint32_t Lx = b->p.Lx, Ly = b->Ly;
   const double* f = b->f[b->cur];
-  const dim3 pg((Lx + kLbThreads - 1) / kLbThreads, b->chunks);
-  if (b->Q == 3) lb_colpart_kernel<3><<<pg, kLbThreads, 0, b->stream>>>(f, Lx, Ly, b->d_part);
-  else if (b->Q == 5) lb_colpart_kernel<5><<<pg, kLbThreads, 0, b->stream>>>(f, Lx, Ly, b->d_part);
-  else lb_colpart_kernel<9><<<pg, kLbThreads, 0, b->stream>>>(f, Lx, Ly, b->d_part);
-  LB_CUDA(b, cudaGetLastError(), "column sums");
-  lb_colsum_kernel<<<pg.x, kLbThreads, 0, b->stream>>>(b->d_part, Lx, b->chunks, b->d_col);
-  LB_CUDA(b, cudaGetLastError(), "column sums");
+  const uint32_t Pm = (Lx + kLbChunk - 1) / kLbChunk;
+  {
+    double* f_ = b->f[b->cur];
+    uint32_t* count = b->d_count + kLbMaxModes;
+    double* whole = Pm == 1 ? b->d_out : nullptr;
+    void* args[] = {&f_, &b->p.Lx, &b->Ly, &b->d_part, &b->d_col, &count, &whole};
+    // a thread for all rows of a chunk where there are few, or where such blocks fill the
+    // SMs' warps twice over (8192^2: 804 us, 833 with eight threads)
+    const bool wide = Ly <= kLbFewRows ||
+                      uint64_t((Lx + kLbThreads - 1) / kLbThreads) * b->chunks >= uint64_t(b->sms) * 2 * (2048 / kLbThreads);
+    const uint32_t cols = wide ? uint32_t(kLbThreads) : kLbCols;
+    LB_CUDA(b, cudaLaunchKernel(lb_col_fn(b->Q, wide), dim3((Lx + cols - 1) / cols, b->chunks), dim3(kLbThreads), args, 0,
+                                b->stream),
+            "column sums");
+  }
   if (any_y) {
     const int rg = int(Ly < uint32_t(b->sms) * 8 ? Ly : uint32_t(b->sms) * 8);
     if (b->Q == 3) lb_rowsum_kernel<3><<<rg, kLbThreads, 0, b->stream>>>(f, Lx, Ly, b->d_row);
@@ -668,30 +783,32 @@ ilg_status ilg_lb_observables(ilg_lb* b, const int32_t* modes, uint32_t nmodes, 
     else lb_rowsum_kernel<9><<<rg, kLbThreads, 0, b->stream>>>(f, Lx, Ly, b->d_row);
     LB_CUDA(b, cudaGetLastError(), "row sums");
   }
-  if (nmodes)
-    LB_CUDA(b, cudaMemcpyAsync(b->d_modes, modes, sizeof(int32_t) * 2 * nmodes, cudaMemcpyHostToDevice, b->stream),
-            "copy modes");
-  const uint32_t Pm = (Lx + kLbChunk - 1) / kLbChunk;
-  lb_mass_partial_kernel<<<Pm, kLbThreads, 0, b->stream>>>(b->d_col, Lx, b->d_red);
-  LB_CUDA(b, cudaGetLastError(), "mass");
-  lb_combine_kernel<<<1, kLbThreads, 0, b->stream>>>(b->d_red, Pm, b->d_out, 0);
-  LB_CUDA(b, cudaGetLastError(), "mass");
+  if (Pm > 1) {
+    lb_mass_partial_kernel<<<Pm, kLbThreads, 0, b->stream>>>(b->d_col, Lx, b->d_red);
+    LB_CUDA(b, cudaGetLastError(), "mass");
+    lb_combine_kernel<<<1, kLbThreads, 0, b->stream>>>(b->d_red, Pm, b->d_out);
+    LB_CUDA(b, cudaGetLastError(), "mass");
+  }
   if (nmodes) {
-    const uint32_t maxL = Lx > Ly ? Lx : Ly;
-    const uint32_t P = (maxL + kLbChunk - 1) / kLbChunk;
-    lb_mode_partial_kernel<<<dim3(P, nmodes), kLbThreads, 0, b->stream>>>(b->d_col, b->d_row, Lx, Ly, b->d_modes,
-                                                                          b->d_out, b->d_red);
-    LB_CUDA(b, cudaGetLastError(), "projection");
-    lb_combine_kernel<<<2 * nmodes, kLbThreads, 0, b->stream>>>(b->d_red, P, b->d_out, 1);
+    LbModes first{};
+    const bool few = nmodes <= kLbFirstModes;
+    if (few) std::copy(modes, modes + 2 * nmodes, first.m);
+    else
+      LB_CUDA(b, cudaMemcpyAsync(b->d_modes, modes, sizeof(int32_t) * 2 * nmodes, cudaMemcpyHostToDevice, b->stream),
+              "copy modes");
+    lb_mode_kernel<<<dim3(lb_mode_blocks(Lx > Ly ? Lx : Ly), nmodes), kLbModeThreads, 0, b->stream>>>(
+        b->d_col, b->d_row, Lx, Ly, first, few ? nullptr : b->d_modes, b->d_out, b->d_red, b->d_count);
     LB_CUDA(b, cudaGetLastError(), "projection");
   }
-  std::vector<double> h(1 + 2 * size_t(nmodes));
-  LB_CUDA(b, cudaMemcpyAsync(h.data(), b->d_out, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, b->stream),
-          "copy observables");
-  LB_CUDA(b, cudaMemcpyAsync(&b->h_sync, b->d_sync + 1, sizeof(unsigned long long), cudaMemcpyDeviceToHost, b->stream),
+  // sync[1] lies before the results
+  std::vector<double> got(2 + 2 * size_t(nmodes));
+  LB_CUDA(b, cudaMemcpyAsync(got.data(), b->d_sync + 1, sizeof(double) * got.size(), cudaMemcpyDeviceToHost, b->stream),
           "copy observables");
   LB_CUDA(b, cudaStreamSynchronize(b->stream), "observables");
+  std::memcpy(&b->h_sync, got.data(), sizeof b->h_sync);
+  b->waits = false;
   if (b->h_sync != 0) return lb_gave_up(b);
+  const double* const h = got.data() + 1;
   if (t) *t = b->t;
   if (mass) *mass = h[0];
   const double half = double(Lx) * double(Ly) / 2.0;
