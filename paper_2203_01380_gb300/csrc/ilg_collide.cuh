@@ -63,6 +63,29 @@ __device__ __forceinline__ uint4 philox_tail(uint4 c, const uint32_t (&rk)[20]) 
   return c;
 }
 
+// A node's slot words at a step, and its part of rounds 1-3.  They depend on the node and
+// the step alone: a kernel that waits for the step before makes its first node's meanwhile.
+template <int NB>
+struct SlotWords {
+  uint32_t W[4 * NB], r2h, r2l, p1l;
+  template <class Keys>
+  __device__ __forceinline__ void make(const Keys& k, const uint32_t (&rk)[20], uint32_t node) {
+    const uint64_t P1 = uint64_t(0xD2511F53u) * (node ^ k.slot.A);
+    const uint64_t R2 = uint64_t(0xCD9E8D57u) * (uint32_t(P1 >> 32) ^ k.slot.G);
+    r2h = uint32_t(R2 >> 32);
+    r2l = uint32_t(R2);
+    p1l = uint32_t(P1);
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      const uint4 v = philox_tail(make_uint4(r2h ^ k.slot.H[b], r2l, p1l ^ k.slot.I[b], k.slot.J[b]), rk);
+      W[4 * b] = v.x;
+      W[4 * b + 1] = v.y;
+      W[4 * b + 2] = v.z;
+      W[4 * b + 3] = v.w;
+    }
+  }
+};
+
 // The words of one node and step.  S: bytes between a lane's consecutive words in the
 // ring (4 x the threads that share it), K: words per lane (a power of two).
 template <uint32_t S, uint32_t K>
@@ -88,6 +111,15 @@ struct NodeWords {
   template <class Keys>
   __device__ __forceinline__ uint4 slot(const Keys& k, const uint32_t (&rk)[20], int b) const {
     return philox_tail(make_uint4(r2h ^ k.slot.H[b], r2l, p1l ^ k.slot.I[b], k.slot.J[b]), rk);
+  }
+  template <int NB>
+  __device__ __forceinline__ void begin(const SlotWords<NB>& w, unsigned char* ring_, uint32_t lane_off) {
+    r2h = w.r2h;
+    r2l = w.r2l;
+    p1l = w.p1l;
+    ring = ring_;
+    rd = wr = lane_off;
+    blk = 0;
   }
   // the next extension block into the ring
   template <class Keys>
@@ -182,27 +214,35 @@ __device__ __forceinline__ BitCounts count_bits(NodeWords<S, K>& e, const Keys& 
 // The collision of one node per lane (m: its occupations after the flip, all zero for a
 // lane without a node); all 32 lanes call it together.  The same words and results as
 // collide() (D2Q9: collide9_general()).  ring: the block's ring of K words per thread in
-// shared memory, lane_off: 4 x the thread's index; ta: D2Q9's axis-share table (others: any).
+// shared memory, lane_off: 4 x the thread's index; ta: D2Q9's axis-share table (others: any);
+// made: the node's slot words, if they are there already.
 // TABLES: every probability lies strictly between 0 and 1 and is drawn through its table
 // (known outside the loop over nodes: the tests for the other cases would be made for every
 // node).
 template <int Q, uint32_t S, uint32_t K, bool TABLES, class Keys, class Tab>
 __device__ __forceinline__ void collide_warp(const StepArgs& a, const Keys& k, const Tab& to, const Tab& tr, const Tab& ta,
                                              unsigned char* ring, uint32_t lane_off, uint32_t node,
-                                             const uint32_t (&m)[Q], uint32_t (&out)[Q]) {
+                                             const uint32_t (&m)[Q], uint32_t (&out)[Q],
+                                             const SlotWords<Q == 9 ? 4 : 2>* made = nullptr) {
   static_assert(K >= 4 + uint32_t(Q), "a word for each velocity beside the block being written");
   constexpr int NB = Q == 9 ? 4 : 2;
   constexpr int32_t kN = int32_t(kDevNmax);
   NodeWords<S, K> e;
-  e.begin(k, ring, lane_off, node);
   uint32_t W[4 * NB];
+  if (made) {
+    e.begin(*made, ring, lane_off);
 #pragma unroll
-  for (int b = 0; b < NB; ++b) {
-    const uint4 v = e.slot(k, a.rk, b);
-    W[4 * b] = v.x;
-    W[4 * b + 1] = v.y;
-    W[4 * b + 2] = v.z;
-    W[4 * b + 3] = v.w;
+    for (int i = 0; i < 4 * NB; ++i) W[i] = made->W[i];
+  } else {
+    e.begin(k, ring, lane_off, node);
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      const uint4 v = e.slot(k, a.rk, b);
+      W[4 * b] = v.x;
+      W[4 * b + 1] = v.y;
+      W[4 * b + 2] = v.z;
+      W[4 * b + 3] = v.w;
+    }
   }
 
   // thinning

@@ -19,14 +19,14 @@ namespace ilg {
 // x + v_i (periodic).  One launch takes T steps: the alias tables are staged in shared
 // memory once, and a barrier of all blocks (a cooperative launch) separates the steps,
 // instead of a launch, a staging pass and an idle tail per step.
-// Bound: integer issue (72 % of it, ~720 warp instructions per 32 nodes at 50 per
-// velocity and omega* = 0.5) on large lattices; the barrier and the latency of one node
-// (about 2 us a step) on small ones.  One block of 1024 threads per SM holds the tables
+// Bound: integer issue (65 % of it over all, about 75 % between the barriers; some 650 warp
+// instructions per 32 nodes at 50 per velocity and omega* = 0.5) on large lattices; the
+// barrier and the latency of one node (about 2 us a step) on small ones.  One block of 1024 threads per SM holds the tables
 // once, in the 64-bit form whose draw takes two instructions fewer than the packed one
 // (29.1 against 31.0 us per step for two blocks of 512, 33 with packed tables).  Us per
 // step against one launch per step with a collision that loops per lane: 1024^2 at 50 per
-// velocity 25.5 / 37.3 (omega* 0.5), 16.2 / 26.8 (0.1); 1501 x 777 at 100 per velocity
-// 44.8 / 66; 1024^2 at 200 per velocity, omega* = 1, 85 / 241; 96 x 40 2.2 / 18.7.
+// velocity 25.0 / 37.3 (omega* 0.5), 15.7 / 26.8 (0.1); 1501 x 777 at 100 per velocity
+// 44.5 / 66; 1024^2 at 200 per velocity, omega* = 1, 83 / 241; 96 x 40 2.2 / 18.7.
 // --------------------------------------------------------------------------
 constexpr uint32_t kStepRing = 16;  // extension words per lane
 
@@ -61,6 +61,15 @@ __global__ void __launch_bounds__(THREADS, 1)
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t base0 = blockIdx.x * THREADS + (threadIdx.x - lane);  // the warp's first node
   const uint32_t y0 = (base0 + lane) / a.Lx, x0 = base0 + lane - y0 * a.Lx;
+  // the launch-wide Philox rounds of a step, and the first node's words: made for the next
+  // step between a block's arrival at the barrier and its wait there (1024^2 at 50 per
+  // velocity 25.0 instead of 25.5 us per step, 15.7 instead of 16.2 at omega* = 0.1).  D2Q9
+  // has no registers for sixteen more words (768^2 at 10 per velocity 15.5 instead of 13.0)
+  constexpr int NB = Q == 9 ? 4 : 2;
+  constexpr bool kAhead = Q != 9;
+  NodeKeys<NB> keys = word_keys<NB>(a, t0);
+  SlotWords<NB> first;
+  if (kAhead && (TABLES || !a.particle)) first.make(keys, a.rk, base0 + lane);
   for (uint32_t step = 0;; ++step) {
     const uint32_t t = t0 + step;
     const uint16_t* const in = (step & 1) ? buf1 : buf0;
@@ -73,7 +82,6 @@ __global__ void __launch_bounds__(THREADS, 1)
     const uint16_t* from[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) from[i] = in + (i == 0 || !a.flip ? i : (i & 1 ? i + 1 : i - 1)) * plane;
-    const auto keys = word_keys<Q == 9 ? 4 : 2>(a, t);  // the launch-wide Philox rounds
     while (base < nodes) {
       const uint32_t node = base + lane;
       const bool active = node < nodes && node >= base;
@@ -82,7 +90,13 @@ __global__ void __launch_bounds__(THREADS, 1)
 #pragma unroll
       for (int i = 0; i < Q; ++i) m[i] = active ? __ldcg(from[i] + node) : 0u;
       if (!TABLES && a.particle) collide_particle<Q>(a, s, node, t, m, post);
-      else collide_warp<Q, 4 * THREADS, kStepRing, TABLES>(a, keys, to, tr, ta, ring, 4 * threadIdx.x, node, m, post);
+      else if constexpr (kAhead) {
+        SlotWords<NB> w = first;
+        if (base != base0) w.make(keys, a.rk, node);
+        collide_warp<Q, 4 * THREADS, kStepRing, TABLES>(a, keys, to, tr, ta, ring, 4 * threadIdx.x, node, m, post, &w);
+      } else {
+        collide_warp<Q, 4 * THREADS, kStepRing, TABLES>(a, keys, to, tr, ta, ring, 4 * threadIdx.x, node, m, post);
+      }
       if (active) {
         uint32_t high = 0;
 #pragma unroll
@@ -122,8 +136,12 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
     if (step + 1 == T) break;
     __syncthreads();
+    if (threadIdx.x == 0) run_arrive(sync);
+    // while the other blocks finish: the next step's words that need nothing of theirs
+    keys = word_keys<NB>(a, t + 1);
+    if (kAhead && (TABLES || !a.particle)) first.make(keys, a.rk, base0 + lane);
     if (threadIdx.x == 0) {
-      const unsigned long long v = run_barrier(sync, (step + 1) * gridDim.x);
+      const unsigned long long v = run_wait(sync, (step + 1) * gridDim.x);
       if (v == ~0ull) {
         atomicExch(sync + 1, 1ull);
         stop = 1;

@@ -10,18 +10,26 @@ namespace ilg {
 constexpr unsigned long long kRunMark = 1ull << 32;
 constexpr uint32_t kRunPolls = 1u << 23;  // seconds; the blocks of a step differ by far less
 
-// One thread per block, after the block's own barrier: arrive, and wait until `target`
-// arrivals.  Returns the word, or ~0 when the wait gave up (bounded: the kernel then
-// returns and the host reports it).
-__device__ __forceinline__ unsigned long long run_barrier(unsigned long long* word, uint32_t target) {
+// One thread per block, after the block's own barrier: arrive.
+__device__ __forceinline__ void run_arrive(unsigned long long* word) {
   __threadfence();
   atomicAdd(word, 1ull);
+}
+
+// The same thread: wait until `target` arrivals.  Returns the word, or ~0 when the wait gave
+// up (bounded: the kernel then returns and the host reports it).
+__device__ __forceinline__ unsigned long long run_wait(unsigned long long* word, uint32_t target) {
   unsigned long long v = 0;
   for (uint32_t k = 0; k < kRunPolls; ++k) {
     asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(word) : "memory");
     if (uint32_t(v) >= target) return v;
   }
   return ~0ull;
+}
+
+__device__ __forceinline__ unsigned long long run_barrier(unsigned long long* word, uint32_t target) {
+  run_arrive(word);
+  return run_wait(word, target);
 }
 
 }  // namespace ilg
