@@ -12,6 +12,7 @@
 #include "ilg_batch.h"
 #include "ilg_collide.cuh"
 #include "ilg_device.cuh"
+#include "ilg_fixed.cuh"
 
 namespace ilg {
 
@@ -54,40 +55,11 @@ __device__ double block_dot2(double s, double c, double* red) {
   return r;  // valid in thread 0
 }
 
-// A 128-bit integer as the record holds it.
-struct I128 {
-  unsigned long long lo = 0;
-  long long hi = 0;
-};
-
-// v * 2^-62 rounded once to double (round to nearest even).
-__device__ double i128_to_double_2m62(I128 v) {
-  const bool neg = v.hi < 0;
-  unsigned long long lo = v.lo, hi = (unsigned long long)v.hi;
-  if (neg) {  // two's complement negation
-    lo = ~lo + 1ull;
-    hi = ~hi + (lo == 0 ? 1ull : 0ull);
-  }
-  double mag;
-  if (hi == 0) {
-    mag = __ull2double_rn(lo);
-  } else {
-    // keep the top 64 bits, fold the rest into a sticky bit: one correct rounding
-    const int k = 64 - __clzll((long long)hi);  // significant bits of hi, 1..64
-    unsigned long long m = k == 64 ? hi : ((hi << (64 - k)) | (lo >> k));
-    const unsigned long long dropped = k == 64 ? lo : (lo << (64 - k));
-    if (dropped) m |= 1ull;
-    mag = ldexp(__ull2double_rn(m), k);
-  }
-  const double r = ldexp(mag, -62);
-  return neg ? -r : r;
-}
-
 // Fixed-point (2^-62) cosine and sine of 2 pi r / L.
 __device__ __forceinline__ longlong2 trig_fixed(uint32_t r, uint32_t L) {
   double sn, cs;
   sincospi(2.0 * double(r) / double(L), &sn, &cs);
-  return make_longlong2(__double2ll_rn(ldexp(cs, 62)), __double2ll_rn(ldexp(sn, 62)));
+  return make_longlong2(fixed62(cs), fixed62(sn));
 }
 
 // Complex amplitude of axis mode m of a ring: with D(x) = L N(x) - M and r = (m x) mod L,

@@ -8,6 +8,7 @@
 
 #include "ilg_collide.cuh"
 #include "ilg_device.cuh"
+#include "ilg_fixed.cuh"
 #include "ilg_launch.h"
 #include "ilg_sync.cuh"
 
@@ -490,12 +491,15 @@ cudaError_t launch_sums(int Q, const uint16_t* in, uint32_t Lx, uint32_t Ly, uns
 
 // --------------------------------------------------------------------------
 // projections: the entries of a mode cut into chunks, one block each.  D(x) = L*S(x) - M
-// in exact int64, then compensated dot products (Ogita, Rump & Oishi 2005: error-free
-// TwoProduct by FMA, TwoSum) with cos and sin of 2 pi r / L, r = (m*x) mod L; the block
-// that finishes last adds the chunks' pairs in their order (the same result every time).
-// Bound: the fp64 pipe (about 65 double instructions per entry, 2 lanes per SM and cycle),
-// so a mode is spread over as many SMs as its length feeds (one block per mode before:
-// 64 modes of 16384 entries 0.33 -> 0.15 ms, one mode of 2^22 71 -> 1 ms).
+// in exact int64, times cos and sin of 2 pi r / L, r = (m*x) mod L; the block that finishes
+// last adds the chunks' sums (the same result every time).
+// Bound: the fp64 pipe: a warp's double instruction takes 64 cycles of its sub-partition,
+// whatever lanes are active, so a mode is spread over as many SMs as its length feeds and
+// the products are summed in 128-bit integers (FixedSums): the sine and cosine, some 70
+// double instructions, are all that is left.  Against compensated double sums (DoubleSums,
+// still taken where 128 bits might not do), whose trees took most of a short mode's time:
+// mass and one mode of a ring of 256 nodes 27 / 35 us, of 1024^2 31 / 39, 64 modes of 16384^2
+// 482 / 556, two modes of 2^22 nodes 707 / 1011; the results are the same to the last bit.
 // --------------------------------------------------------------------------
 __device__ __forceinline__ void two_sum(double a, double b, double& s, double& e) {
   s = a + b;
@@ -512,14 +516,16 @@ struct Dot2 {
     two_sum(s, p, s, q);
     c += q + pe;
   }
-  __device__ void merge(const Dot2& o) {
+  __device__ void merge(double os, double oc) {
     double q;
-    two_sum(s, o.s, s, q);
-    c += o.c + q;
+    two_sum(s, os, s, q);
+    c += oc + q;
   }
 };
 
 constexpr int kProjThreads = 64;
+constexpr int kProjWarps = kProjThreads / 32;
+constexpr int kProjWords = 4;  // 8-byte words of a chunk's sums
 
 struct ProjArgs {
   const unsigned long long* colsum;
@@ -527,94 +533,157 @@ struct ProjArgs {
   const unsigned long long* mass_in;
   uint32_t Lx, Ly;
   uint32_t nmodes;
-  double* part;            // (re.s, re.c, im.s, im.c) per chunk and mode
-  unsigned int* ticket;    // per mode, 0 between launches
-  double* res;             // 4 per mode (device or mapped host memory)
+  unsigned long long* part;  // kProjWords per chunk and mode
+  unsigned int* ticket;      // per mode, 0 between launches
+  double* res;               // 4 per mode (device or mapped host memory)
   unsigned long long* mass_out;
-  int32_t modes[2 * kProjModes];
+  uint32_t modes[kProjModes];  // modulo the side's length
+  uint32_t along_y[kProjModes / 32];
 };
 
-// fixed tree over the block's threads: warp shuffles, then the warps' pairs
-__device__ __forceinline__ void block_dot2(Dot2& re, Dot2& im, double (*sv)[kProjThreads / 32]) {
+// The two sums as 128-bit integers, the trigonometric values rounded to 2^-62 (those of
+// 2^-9 and more are that already): exact while 2 L M 2^62 < 2^127.
+struct FixedSums {
+  __int128 re = 0, im = 0;
+  __device__ void add(double cs, double sn, long long D) {
+    re += __int128(fixed62(cs)) * D;
+    im += __int128(fixed62(sn)) * D;
+  }
+  __device__ void pack(unsigned long long (&w)[kProjWords]) const {
+    w[0] = (unsigned long long)re;
+    w[1] = (unsigned long long)(re >> 64);
+    w[2] = (unsigned long long)im;
+    w[3] = (unsigned long long)(im >> 64);
+  }
+  __device__ void merge(const unsigned long long (&w)[kProjWords]) {
+    re += (__int128(static_cast<long long>(w[1])) << 64) + w[0];
+    im += (__int128(static_cast<long long>(w[3])) << 64) + w[2];
+  }
+  // of a part as packed
+  __device__ static double value(unsigned long long lo, unsigned long long hi) {
+    return i128_to_double_2m62(I128{lo, (long long)hi});
+  }
+};
+
+// The two sums compensated in double precision (Ogita, Rump & Oishi 2005: error-free
+// TwoProduct by FMA, TwoSum), for any L and M.
+struct DoubleSums {
+  Dot2 re{0.0, 0.0}, im{0.0, 0.0};
+  __device__ void add(double cs, double sn, long long D) {
+    re.add_product(cs, double(D));
+    im.add_product(sn, double(D));
+  }
+  __device__ void pack(unsigned long long (&w)[kProjWords]) const {
+    w[0] = (unsigned long long)__double_as_longlong(re.s);
+    w[1] = (unsigned long long)__double_as_longlong(re.c);
+    w[2] = (unsigned long long)__double_as_longlong(im.s);
+    w[3] = (unsigned long long)__double_as_longlong(im.c);
+  }
+  __device__ void merge(const unsigned long long (&w)[kProjWords]) {
+    re.merge(__longlong_as_double((long long)w[0]), __longlong_as_double((long long)w[1]));
+    im.merge(__longlong_as_double((long long)w[2]), __longlong_as_double((long long)w[3]));
+  }
+  __device__ static double value(unsigned long long s, unsigned long long c) {
+    return __longlong_as_double((long long)s) + __longlong_as_double((long long)c);
+  }
+};
+
+// fixed tree over the block's threads: warp shuffles, then the warps' sums (in thread 0)
+template <class Sums>
+__device__ __forceinline__ void block_sums(Sums& v, unsigned long long (*sw)[kProjWords]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned long long w[kProjWords];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    Dot2 ore{__shfl_down_sync(0xFFFFFFFFu, re.s, o), __shfl_down_sync(0xFFFFFFFFu, re.c, o)};
-    Dot2 oim{__shfl_down_sync(0xFFFFFFFFu, im.s, o), __shfl_down_sync(0xFFFFFFFFu, im.c, o)};
-    re.merge(ore);
-    im.merge(oim);
+    v.pack(w);
+#pragma unroll
+    for (int i = 0; i < kProjWords; ++i) w[i] = __shfl_down_sync(0xFFFFFFFFu, w[i], o);
+    v.merge(w);
   }
+  v.pack(w);
   __syncthreads();
   if (lane == 0) {
-    sv[0][warp] = re.s;
-    sv[1][warp] = re.c;
-    sv[2][warp] = im.s;
-    sv[3][warp] = im.c;
+#pragma unroll
+    for (int i = 0; i < kProjWords; ++i) sw[warp][i] = w[i];
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    for (int w = 1; w < kProjThreads / 32; ++w) {
-      re.merge(Dot2{sv[0][w], sv[1][w]});
-      im.merge(Dot2{sv[2][w], sv[3][w]});
+    for (int k = 1; k < kProjWarps; ++k) {
+#pragma unroll
+      for (int i = 0; i < kProjWords; ++i) w[i] = sw[k][i];
+      v.merge(w);
+    }
+  }
+}
+
+template <class Sums>
+__device__ __forceinline__ void project_chunk(const ProjArgs& a, const unsigned long long* S, uint32_t L, uint32_t m,
+                                              long long M, unsigned long long (*sw)[kProjWords], bool* last) {
+  const uint32_t mi = blockIdx.y, P = gridDim.x;
+  const uint32_t x0 = uint32_t(uint64_t(L) * blockIdx.x / P), x1 = uint32_t(uint64_t(L) * (blockIdx.x + 1) / P);
+  Sums v;
+  for (uint64_t x = uint64_t(x0) + threadIdx.x; x < x1; x += kProjThreads) {
+    const long long D = static_cast<long long>(L) * static_cast<long long>(S[x]) - M;
+    // (m, x < L)
+    const uint32_t r = L <= 65536u ? (m * uint32_t(x)) % L : uint32_t((uint64_t(m) * x) % L);
+    double sn, cs;
+    sincospi(2.0 * double(r) / double(L), &sn, &cs);
+    v.add(cs, sn, D);
+  }
+  block_sums(v, sw);
+  if (P > 1) {
+    volatile unsigned long long* const part = a.part + size_t(mi) * P * kProjWords;
+    unsigned long long w[kProjWords];
+    if (threadIdx.x == 0) {
+      v.pack(w);
+#pragma unroll
+      for (int i = 0; i < kProjWords; ++i) part[size_t(kProjWords) * blockIdx.x + i] = w[i];
+      __threadfence();
+      *last = atomicAdd(a.ticket + mi, 1u) == P - 1;
+    }
+    __syncthreads();
+    if (!*last) return;
+    __threadfence();
+    v = Sums{};
+    for (uint32_t k = threadIdx.x; k < P; k += kProjThreads) {
+#pragma unroll
+      for (int i = 0; i < kProjWords; ++i) w[i] = part[size_t(kProjWords) * k + i];
+      v.merge(w);
+    }
+    block_sums(v, sw);
+  }
+  // lane 0 the real part, lane 1 the imaginary one: two divisions one after the other, not four
+  if (threadIdx.x < 32) {
+    unsigned long long w[kProjWords];
+    v.pack(w);
+#pragma unroll
+    for (int i = 0; i < kProjWords; ++i) w[i] = __shfl_sync(0xFFFFFFFFu, w[i], 0);
+    const bool first = threadIdx.x == 0;
+    const double q = Sums::value(first ? w[0] : w[2], first ? w[1] : w[3]) / double(L);
+    const double re = __shfl_sync(0xFFFFFFFFu, q, 0), im = __shfl_sync(0xFFFFFFFFu, q, 1);
+    const double K = double(a.Lx) * double(a.Ly);
+    const double p = (first ? re * re + im * im : im) / (first ? K : K / 2.0);
+    if (threadIdx.x < 2) {
+      a.res[4 * mi + threadIdx.x] = q;
+      a.res[4 * mi + 3 - threadIdx.x] = p;  // S(k), amplitude
+    }
+    if (first) {
+      if (P > 1) a.ticket[mi] = 0;
+      if (mi == 0) *a.mass_out = static_cast<unsigned long long>(M);
     }
   }
 }
 
 __global__ void __launch_bounds__(kProjThreads) project_kernel(const __grid_constant__ ProjArgs a) {
-  __shared__ double sv[4][kProjThreads / 32];
+  __shared__ unsigned long long sw[kProjWarps][kProjWords];
   __shared__ bool last;
-  const uint32_t mi = blockIdx.y, P = gridDim.x;
-  const int32_t mx = a.modes[2 * mi], my = a.modes[2 * mi + 1];
-  const bool along_x = (my == 0);
+  const bool along_x = !((a.along_y[blockIdx.y / 32] >> (blockIdx.y % 32)) & 1u);
   const unsigned long long* S = along_x ? a.colsum : a.rowsum;
-  const uint32_t L = along_x ? a.Lx : a.Ly;
-  const int64_t mraw = along_x ? mx : my;
-  const uint64_t m = uint64_t(((mraw % int64_t(L)) + int64_t(L)) % int64_t(L));
+  const uint32_t L = along_x ? a.Lx : a.Ly, m = a.modes[blockIdx.y];
   const long long M = static_cast<long long>(*a.mass_in);
-  const uint32_t x0 = uint32_t(uint64_t(L) * blockIdx.x / P), x1 = uint32_t(uint64_t(L) * (blockIdx.x + 1) / P);
-  Dot2 re{0.0, 0.0}, im{0.0, 0.0};
-  for (uint64_t x = uint64_t(x0) + threadIdx.x; x < x1; x += kProjThreads) {
-    const long long D = static_cast<long long>(L) * static_cast<long long>(S[x]) - M;
-    const uint32_t r = uint32_t((m * x) % L);
-    double sn, cs;
-    sincospi(2.0 * double(r) / double(L), &sn, &cs);
-    re.add_product(cs, double(D));
-    im.add_product(sn, double(D));
-  }
-  block_dot2(re, im, sv);
-  if (P > 1) {
-    volatile double* const part = a.part + size_t(mi) * P * 4;
-    if (threadIdx.x == 0) {
-      volatile double* const q = part + 4 * blockIdx.x;
-      q[0] = re.s;
-      q[1] = re.c;
-      q[2] = im.s;
-      q[3] = im.c;
-      __threadfence();
-      last = atomicAdd(a.ticket + mi, 1u) == P - 1;
-    }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    re = im = Dot2{0.0, 0.0};
-    for (uint32_t k = threadIdx.x; k < P; k += kProjThreads) {
-      const volatile double* const q = part + 4 * k;
-      re.merge(Dot2{q[0], q[1]});
-      im.merge(Dot2{q[2], q[3]});
-    }
-    block_dot2(re, im, sv);
-  }
-  if (threadIdx.x == 0) {
-    if (P > 1) a.ticket[mi] = 0;
-    const double vre = (re.s + re.c) / double(L);
-    const double vim = (im.s + im.c) / double(L);
-    const double K = double(a.Lx) * double(a.Ly);
-    a.res[4 * mi + 0] = vre;
-    a.res[4 * mi + 1] = vim;
-    a.res[4 * mi + 2] = vim / (K / 2.0);
-    a.res[4 * mi + 3] = (vre * vre + vim * vim) / K;
-    if (mi == 0) *a.mass_out = static_cast<unsigned long long>(M);
-  }
+  // sum |D| <= 2 L M
+  if (__umul64hi(L, (unsigned long long)M) == 0) project_chunk<FixedSums>(a, S, L, m, M, sw, &last);
+  else project_chunk<DoubleSums>(a, S, L, m, M, sw, &last);
 }
 
 cudaError_t launch_project(const ProjWork& w, uint32_t Lx, uint32_t Ly, const int32_t* modes, uint32_t nmodes,
@@ -625,15 +694,21 @@ cudaError_t launch_project(const ProjWork& w, uint32_t Lx, uint32_t Ly, const in
   a.mass_in = w.mass;
   a.Lx = Lx;
   a.Ly = Ly;
-  a.part = reinterpret_cast<double*>(w.scratch);
+  a.part = w.scratch;
   a.ticket = reinterpret_cast<unsigned int*>(w.scratch + 4 * (kProjBlocks + kProjModes));
   a.mass_out = mass;
   for (uint32_t k = 0; k < nmodes; k += kProjModes) {
     a.nmodes = std::min(nmodes - k, kProjModes);
     a.res = res + size_t(4) * k;
-    std::memcpy(a.modes, modes + size_t(2) * k, sizeof(int32_t) * 2 * a.nmodes);
+    std::memset(a.along_y, 0, sizeof a.along_y);
     uint32_t L = 0;
-    for (uint32_t j = 0; j < a.nmodes; ++j) L = std::max(L, a.modes[2 * j + 1] == 0 ? Lx : Ly);
+    for (uint32_t j = 0; j < a.nmodes; ++j) {
+      const int32_t mx = modes[2 * (k + j)], my = modes[2 * (k + j) + 1];
+      const int64_t side = my == 0 ? Lx : Ly, m = my == 0 ? mx : my;
+      a.modes[j] = uint32_t((m % side + side) % side);
+      if (my != 0) a.along_y[j / 32] |= 1u << (j % 32);
+      L = std::max(L, uint32_t(side));
+    }
     const uint32_t P = uint32_t(std::min<uint64_t>(std::max<uint32_t>(1, kProjBlocks / a.nmodes),
                                                    (uint64_t(L) + kProjThreads - 1) / kProjThreads));
     project_kernel<<<dim3(P, a.nmodes), kProjThreads, 0, s>>>(a);

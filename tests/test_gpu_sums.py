@@ -68,3 +68,24 @@ def test_unaligned_state(B):
         torch.cuda.synchronize()
         modes = [(1, 0), (0, 2)]
         check(s0, B.observables_noalloc(2, Lx, Ly, buf.data_ptr() + 2 * off, modes), modes, Lx, Ly)
+
+
+@pytest.mark.parametrize("low,high", [(20000, 21000), (65000, 65535)])
+def test_products_near_and_beyond_128_bits(B, low, high):
+    # L * M just below 2^64 (integer sums) and beyond (double sums), eight phases
+    L = 1 << 24
+    s0 = np.full((3, 1, L), low, np.uint16)
+    s0[:, 0, 1::8] = high
+    s0[1, 0, 2::8] = high
+    with B.Lattice(1, L, 1, omega_eff=1.5, seed=1) as lat:
+        lat.set_state(s0)
+        got = lat.observables([(L // 8, 0)])
+    S = [3 * low, 3 * high, 2 * low + high] + [3 * low] * 5  # column sums of the phase classes
+    M = sum(S) * (L // 8)
+    assert got["mass"] == M and (L * M < 2**64) == (low == 20000)
+    D = [np.longdouble(L // 8) * (np.longdouble(8 * s - sum(S)) / 8) for s in S]
+    ph = [4 * np.arctan(np.longdouble(1)) * c / 4 for c in range(8)]
+    re, im = (sum(f(p) * d for p, d in zip(ph, D)) for f in (np.cos, np.sin))
+    # the sines and cosines are off by two ulps at most, the sums are rounded once
+    tol = 8 * 2.0**-53 * float(sum(abs(d) for d in D))
+    assert abs(got["re"][0] - re) <= tol and abs(got["im"][0] - im) <= tol
