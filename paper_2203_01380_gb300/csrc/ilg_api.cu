@@ -222,9 +222,9 @@ ilg_status ilg_create(const ilg_params* params, void* stream, ilg_ctx** out) {
 
   std::vector<uint32_t> tables(block_words, 0u);
   build_table_block(c->Q, c->p.sampler, c->P_omega, c->P_rest, c->P_axis, tables.data());
-  if ((e = prepare_step_kernels()) != cudaSuccess) return bail(e, "cudaFuncSetAttribute");
-  if ((e = prepare_step_vec_kernels()) != cudaSuccess) return bail(e, "cudaFuncSetAttribute");
-  if ((e = prepare_step_warp_kernels()) != cudaSuccess) return bail(e, "cudaFuncSetAttribute");
+  if ((e = prepare_step_kernels(c->Q)) != cudaSuccess) return bail(e, "cudaFuncSetAttribute");
+  if (c->Q != 9 && (e = prepare_step_vec_kernels()) != cudaSuccess) return bail(e, "cudaFuncSetAttribute");
+  if ((e = prepare_step_warp_kernels(c->Q)) != cudaSuccess) return bail(e, "cudaFuncSetAttribute");
   e = cudaMemcpyAsync(c->d_tables, tables.data(), sizeof(uint32_t) * tables.size(), cudaMemcpyHostToDevice, c->stream);
   if (e != cudaSuccess) return bail(e, "copy tables");
   e = cudaMemsetAsync(c->d_fail, 0xFF, sizeof(unsigned long long), c->stream);
@@ -305,8 +305,6 @@ ilg_status ilg_init(ilg_ctx* c) {
 // Sums of the current state into d_mass / d_col (and d_row).
 static ilg_status queue_sums(ilg_ctx* c, bool want_rows) {
   const uint32_t Lx = c->p.Lx, Ly = c->p.Ly;
-  ILG_CUDA(c, cudaMemsetAsync(c->d_mass, 0, sizeof(unsigned long long) * (1 + size_t(Lx) + (want_rows ? Ly : 0)), c->stream),
-           "clear sums");
   ILG_CUDA(c, launch_sums(c->Q, c->buf[c->cur], Lx, Ly, c->d_col, c->d_row, c->d_mass, want_rows ? 1 : 0, uint32_t(c->sms),
                           c->stream),
            "sums kernel");

@@ -44,14 +44,12 @@ __global__ void __launch_bounds__(THREADS, 1)
   uint32_t* s = reinterpret_cast<uint32_t*>(smem4);
   if (threadIdx.x == 0) stop = (*reinterpret_cast<volatile unsigned long long*>(fail) != ~0ull);
   constexpr uint32_t kTables = run_table_words(Q);
-  {
-    // the block's first words: the alias tables, or the particle sampler's boundaries
-    const uint4* g4 = reinterpret_cast<const uint4*>(a.tables);
-#pragma unroll 8
-    for (uint32_t i = threadIdx.x; i < kTables / 4; i += THREADS) smem4[i] = g4[i];
-  }
-  __syncthreads();
-  if (stop) return;
+  // the block's first words: the alias tables, or the particle sampler's boundaries (all
+  // copies in flight at once, the first node's words made meanwhile)
+  for (uint32_t i = threadIdx.x; i < kTables / 4; i += THREADS)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(uint32_t(__cvta_generic_to_shared(smem4 + i))),
+                 "l"(reinterpret_cast<const uint4*>(a.tables) + i)
+                 : "memory");
   unsigned char* const ring = reinterpret_cast<unsigned char*>(smem4) + 4 * kTables;
   const Alias8 to = Alias8::of(s, 0), tr = Alias8::of(s, 1), ta = Alias8::of(s, Q == 9 ? 2 : 1);
 
@@ -71,6 +69,9 @@ __global__ void __launch_bounds__(THREADS, 1)
   NodeKeys<NB> keys = word_keys<NB>(a, t0);
   SlotWords<NB> first;
   if (kAhead && (TABLES || !a.particle)) first.make(keys, a.rk, base0 + lane);
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
+  __syncthreads();
+  if (stop) return;
   for (uint32_t step = 0;; ++step) {
     const uint32_t t = t0 + step;
     const uint16_t* const in = (step & 1) ? buf1 : buf0;
@@ -188,18 +189,17 @@ static RunShape run_shape(int Q, const StepArgs& a, uint64_t nodes, uint32_t sms
   return {run_fn<1024>(Q, tables), 1024};
 }
 
-cudaError_t prepare_step_kernels() {
+cudaError_t prepare_step_kernels(int Q) {
   cudaError_t e = cudaSuccess;
-  auto set = [&](const void* f, int Q, int threads) {
+  auto set = [&](const void* f, int threads) {
     if (f && e == cudaSuccess)
       e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(run_smem(Q, threads)));
   };
-  for (int Q : {3, 5, 9})
-    for (bool tables : {false, true}) {
-      set(run_fn<128>(Q, tables), Q, 128);
-      set(run_fn<512>(Q, tables), Q, 512);
-      set(run_fn<1024>(Q, tables), Q, 1024);
-    }
+  for (bool tables : {false, true}) {
+    set(run_fn<128>(Q, tables), 128);
+    set(run_fn<512>(Q, tables), 512);
+    set(run_fn<1024>(Q, tables), 1024);
+  }
   return e;
 }
 
@@ -400,6 +400,8 @@ __global__ void __launch_bounds__(32 * kSumGroups) sums_kernel(const uint16_t* _
   const uint64_t x = (uint64_t(blockIdx.x) * 32 + tx) * VEC;
   const size_t plane = size_t(Lx) * Ly;
   const uint32_t chunks = (Ly + kSumGroups * R - 1) / (kSumGroups * R);
+  // a block that has the lattice to itself writes its sums over what was there
+  const bool alone = gridDim.x == 1 && gridDim.y == 1;
   unsigned long long sum = 0;
   for (uint32_t chunk = blockIdx.y; chunk < chunks; chunk += gridDim.y) {
     const uint32_t y0 = chunk * kSumGroups * R;
@@ -440,7 +442,10 @@ __global__ void __launch_bounds__(32 * kSumGroups) sums_kernel(const uint16_t* _
       }
       if (want_rows) {
         N = __reduce_add_sync(0xFFFFFFFFu, N);  // at most 256 nodes of 9 x 65535
-        if (tx == 0 && N) atomicAdd(row + y, static_cast<unsigned long long>(N));
+        if (tx == 0) {
+          if (alone) row[y] = N;
+          else if (N) atomicAdd(row + y, static_cast<unsigned long long>(N));
+        }
       }
     }
 #pragma unroll
@@ -451,7 +456,8 @@ __global__ void __launch_bounds__(32 * kSumGroups) sums_kernel(const uint16_t* _
       unsigned long long C = 0;
 #pragma unroll
       for (uint32_t g = 0; g < kSumGroups; ++g) C += red[g][threadIdx.x];
-      if (C) atomicAdd(col + c, C);
+      if (alone) col[c] = C;
+      else if (C) atomicAdd(col + c, C);
       sum += C;
     }
     __syncthreads();
@@ -463,13 +469,15 @@ __global__ void __launch_bounds__(32 * kSumGroups) sums_kernel(const uint16_t* _
   if (threadIdx.x == 0) {
     unsigned long long M = 0;
     for (uint32_t g = 0; g < kSumGroups; ++g) M += total[g];
-    if (M) atomicAdd(mass, M);
+    if (alone) *mass = M;
+    else if (M) atomicAdd(mass, M);
   }
 }
 
 template <int Q>
-static void sums_launch(const uint16_t* in, uint32_t Lx, uint32_t Ly, unsigned long long* col, unsigned long long* row,
-                        unsigned long long* mass, int want_rows, uint32_t sms, cudaStream_t s) {
+static cudaError_t sums_launch(const uint16_t* in, uint32_t Lx, uint32_t Ly, unsigned long long* col,
+                               unsigned long long* row, unsigned long long* mass, int want_rows, uint32_t sms,
+                               cudaStream_t s) {
   const bool wide = Lx % 8 == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0;
   const uint32_t width = wide ? 256 : 32;
   const uint32_t gx = uint32_t((uint64_t(Lx) + width - 1) / width);
@@ -477,16 +485,22 @@ static void sums_launch(const uint16_t* in, uint32_t Lx, uint32_t Ly, unsigned l
   const uint32_t want = std::max<uint32_t>(1, 4 * sms / gx);            // blocks along y
   const uint32_t R = uint32_t(std::min<uint64_t>(kSumMaxRows, std::max<uint64_t>(1, groups / want)));
   const dim3 grid(gx, uint32_t(std::min<uint64_t>(65535, (groups + R - 1) / R)));
+  if (grid.x > 1 || grid.y > 1) {  // (one block: nothing to clear; giving it 40 rows instead of 8 took longer than that)
+    const bool together = want_rows && row == col + Lx;
+    cudaError_t e = cudaMemsetAsync(mass, 0, sizeof(unsigned long long) * (1 + size_t(Lx) + (together ? Ly : 0)), s);
+    if (e == cudaSuccess && want_rows && !together) e = cudaMemsetAsync(row, 0, sizeof(unsigned long long) * Ly, s);
+    if (e != cudaSuccess) return e;
+  }
   if (wide) sums_kernel<Q, 8><<<grid, 32 * kSumGroups, 0, s>>>(in, Lx, Ly, R, col, row, mass, want_rows);
   else sums_kernel<Q, 1><<<grid, 32 * kSumGroups, 0, s>>>(in, Lx, Ly, R, col, row, mass, want_rows);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_sums(int Q, const uint16_t* in, uint32_t Lx, uint32_t Ly, unsigned long long* col,
                         unsigned long long* row, unsigned long long* mass, int want_rows, uint32_t sms, cudaStream_t s) {
-  if (Q == 9) sums_launch<9>(in, Lx, Ly, col, row, mass, want_rows, sms, s);
-  else if (Q == 3) sums_launch<3>(in, Lx, Ly, col, row, mass, want_rows, sms, s);
-  else sums_launch<5>(in, Lx, Ly, col, row, mass, want_rows, sms, s);
-  return cudaGetLastError();
+  if (Q == 9) return sums_launch<9>(in, Lx, Ly, col, row, mass, want_rows, sms, s);
+  if (Q == 3) return sums_launch<3>(in, Lx, Ly, col, row, mass, want_rows, sms, s);
+  return sums_launch<5>(in, Lx, Ly, col, row, mass, want_rows, sms, s);
 }
 
 // --------------------------------------------------------------------------

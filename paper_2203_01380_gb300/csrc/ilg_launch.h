@@ -22,7 +22,7 @@ struct InitArgs {
   const uint32_t* table;
 };
 
-cudaError_t prepare_step_kernels();  // opt in to the table block's shared memory
+cudaError_t prepare_step_kernels(int Q);  // opt in to the table block's shared memory
 // T node-parallel steps from step t in one launch (buf0 holds the state; the steps
 // alternate the buffers).  sync: two words, zeroed sync[1] on entry; sync[1] becomes 1 if
 // a wait between blocks gave up
@@ -44,7 +44,7 @@ cudaError_t launch_step_seg(int Q, const StepArgs& a, const uint16_t* in, uint16
 // lane, one block of 384 threads per SM, shape 1 = 4 nodes per lane, 640 threads;
 // D2Q9: 4 nodes per lane collided in shared memory, 512 (shape 0) or 640 (shape 1)
 // threads
-cudaError_t prepare_step_warp_kernels();
+cudaError_t prepare_step_warp_kernels(int Q);
 uint32_t step_warp_width(int Q, int shape);  // nodes per lane (rows must be a multiple)
 // T steps from step t in one launch, as launch_step_run
 cudaError_t launch_step_warp(int Q, int shape, const StepArgs& a, uint16_t* buf0, uint16_t* buf1, uint32_t t, uint32_t T,
@@ -55,7 +55,7 @@ cudaError_t launch_step_tb(const StepArgs& a, const uint16_t* in, uint16_t* out,
                            uint32_t B, unsigned long long* fail, int grid, cudaStream_t s);
 // words: entries of a.table
 cudaError_t launch_init(int Q, const InitArgs& a, uint32_t words, uint16_t* out, uint32_t sms, cudaStream_t s);
-// adds to col (Lx words), row (Ly words; want_rows) and mass: zero them first
+// col (Lx words, the ones after mass), row (Ly words; want_rows) and mass
 cudaError_t launch_sums(int Q, const uint16_t* in, uint32_t Lx, uint32_t Ly, unsigned long long* col,
                         unsigned long long* row, unsigned long long* mass, int want_rows, uint32_t sms, cudaStream_t s);
 constexpr uint32_t kProjModes = 256;    // modes of one launch

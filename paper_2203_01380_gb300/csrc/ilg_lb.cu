@@ -458,15 +458,15 @@ struct ilg_lb {
   bool has_state = false;
   LbCoef coef{};
   uint32_t chunks = 1;
-  double* d_part = nullptr;   // chunks x Lx partial column sums
-  double* d_col = nullptr;    // Lx
-  double* d_row = nullptr;    // Ly
-  double2* d_red = nullptr;   // projection partials, 2 kLbMaxModes x chunks
-  int32_t* d_modes = nullptr; // 2 kLbMaxModes
-  // one allocation: [0] barrier word of a several-step launch, [1] a wait gave up, d_out, d_count
+  double2* d_red = nullptr;              // projection partials, 2 kLbMaxModes x chunks
+  // one allocation: [0] barrier word of a several-step launch, [1] a wait gave up, then these
   unsigned long long* d_sync = nullptr;
   double* d_out = nullptr;               // mass, then re and im of each mode
   uint32_t* d_count = nullptr;           // arrivals: kLbMaxModes, then the column blocks and one; zero between launches
+  int32_t* d_modes = nullptr;            // 2 kLbMaxModes
+  double* d_col = nullptr;               // Lx
+  double* d_row = nullptr;               // Ly
+  double* d_part = nullptr;              // chunks x Lx partial column sums
   unsigned long long h_sync = 0;         // sync[1] as read back with the last results
   bool waits = false;                    // several-step launches since sync[1] was read
   int run_blocks = 0;                    // resident blocks of the step kernel
@@ -590,19 +590,21 @@ ilg_status ilg_lb_create(const ilg_lb_params* params, void* stream, ilg_lb** out
   const size_t bytes = sizeof(double) * b->Q * b->nodes;
   if (e == cudaSuccess) e = ilg::dev_alloc(&b->f[0], bytes);
   if (e == cudaSuccess) e = ilg::dev_alloc(&b->f[1], bytes);
-  if (e == cudaSuccess) e = ilg::dev_alloc(&b->d_part, sizeof(double) * b->chunks * p.Lx);
-  if (e == cudaSuccess) e = ilg::dev_alloc(&b->d_col, sizeof(double) * p.Lx);
-  if (e == cudaSuccess) e = ilg::dev_alloc(&b->d_row, sizeof(double) * b->Ly);
-  if (e == cudaSuccess) e = ilg::dev_alloc(&b->d_modes, sizeof(int32_t) * 2 * kLbMaxModes);
   const uint32_t maxL = p.Lx > b->Ly ? p.Lx : b->Ly;
   if (e == cudaSuccess) e = ilg::dev_alloc(&b->d_red, sizeof(double2) * 2 * kLbMaxModes * lb_mode_blocks(maxL));
+  // one allocation: what has to be zero, then the modes and the sums
   const size_t words = 2 + 1 + 2 * kLbMaxModes, counters = kLbMaxModes + (p.Lx + kLbCols - 1) / kLbCols + 1;
-  const size_t small = sizeof(double) * words + sizeof(uint32_t) * counters;
-  if (e == cudaSuccess) e = ilg::dev_alloc(&b->d_sync, small);
+  const size_t clear = words + (counters + 1) / 2;
+  const size_t all = clear + kLbMaxModes + p.Lx + size_t(b->Ly) + size_t(b->chunks) * p.Lx;
+  if (e == cudaSuccess) e = ilg::dev_alloc(&b->d_sync, sizeof(unsigned long long) * all);
   if (e == cudaSuccess) {
     b->d_out = reinterpret_cast<double*>(b->d_sync + 2);
     b->d_count = reinterpret_cast<uint32_t*>(b->d_sync + words);
-    e = cudaMemsetAsync(b->d_sync, 0, small, b->stream);
+    b->d_modes = reinterpret_cast<int32_t*>(b->d_sync + clear);
+    b->d_col = reinterpret_cast<double*>(b->d_sync + clear + kLbMaxModes);
+    b->d_row = b->d_col + p.Lx;
+    b->d_part = b->d_row + b->Ly;
+    e = cudaMemsetAsync(b->d_sync, 0, sizeof(unsigned long long) * clear, b->stream);
   }
   int per_sm = 0;
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lb_run_fn(b->Q), kLbThreads, 0);
@@ -620,10 +622,6 @@ ilg_status ilg_lb_destroy(ilg_lb* b) {
   if (b->f[0] || b->f[1]) cudaStreamSynchronize(b->stream);
   cudaFree(b->f[0]);
   cudaFree(b->f[1]);
-  cudaFree(b->d_part);
-  cudaFree(b->d_col);
-  cudaFree(b->d_row);
-  cudaFree(b->d_modes);
   cudaFree(b->d_red);
   cudaFree(b->d_sync);
   delete b;

@@ -92,9 +92,6 @@ extern "C" ilg_status ilg_observables_noalloc(int32_t lattice, uint32_t Lx, uint
   unsigned long long* col = base + kColOff;
   unsigned long long* row = base + kRowOff;
   unsigned long long* res = base + kResOff;
-  // the array keeps the previous call's contents: clear the sums that accumulate
-  if (e == cudaSuccess) e = cudaMemsetAsync(mass_sum, 0, sizeof(unsigned long long) * (1 + size_t(Lx)), s);
-  if (e == cudaSuccess && rows) e = cudaMemsetAsync(row, 0, sizeof(unsigned long long) * Ly, s);
   if (e == cudaSuccess) e = ilg::launch_sums(Q, state, Lx, Ly, col, row, mass_sum, rows ? 1 : 0, uint32_t(sms), s);
   if (e == cudaSuccess && nmodes)
     e = ilg::launch_project(ilg::ProjWork{col, row, mass_sum, base + kProjOff}, Lx, Ly, modes, nmodes,

@@ -339,9 +339,7 @@ cudaError_t queue_results(ilg_server* s, const std::vector<Resident>& out) {
     unsigned long long* const to = s->d_out + kOutWords * i;
     static const int32_t kMode[2] = {1, 0};
     unsigned long long* const col = s->d_sums + 1;
-    e = cudaMemsetAsync(s->d_sums, 0, sizeof(unsigned long long) * (1 + size_t(Lx)), s->stream);
-    if (e == cudaSuccess)
-      e = launch_sums(5, state_of(s, r), Lx, Ly, col, nullptr, s->d_sums, 0, uint32_t(s->sms), s->stream);
+    e = launch_sums(5, state_of(s, r), Lx, Ly, col, nullptr, s->d_sums, 0, uint32_t(s->sms), s->stream);
     if (e == cudaSuccess)
       e = launch_project(ProjWork{col, nullptr, s->d_sums, s->d_proj}, Lx, Ly, kMode, 1, reinterpret_cast<double*>(to),
                          to + 4, s->stream);

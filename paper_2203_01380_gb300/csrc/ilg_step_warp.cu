@@ -745,14 +745,14 @@ void shape_of(int Q, int shape, uint32_t* npt, uint32_t* threads, uint32_t* per_
 
 }  // namespace
 
-cudaError_t prepare_step_warp_kernels() {
-  cudaError_t e = warp_attr<3, 0>();
-  if (e == cudaSuccess) e = warp_attr<3, 1>();
-  if (e == cudaSuccess) e = warp_attr<5, 0>();
-  if (e == cudaSuccess) e = warp_attr<5, 1>();
-  if (e == cudaSuccess) e = warp_attr<9, 0>();
-  if (e == cudaSuccess) e = warp_attr<9, 1>();
-  return e;
+template <int Q>
+static cudaError_t warp_attrs() {
+  const cudaError_t e = warp_attr<Q, 0>();
+  return e == cudaSuccess ? warp_attr<Q, 1>() : e;
+}
+
+cudaError_t prepare_step_warp_kernels(int Q) {
+  return Q == 3 ? warp_attrs<3>() : Q == 5 ? warp_attrs<5>() : warp_attrs<9>();
 }
 
 uint32_t step_warp_width(int Q, int shape) {
