@@ -197,49 +197,51 @@ __device__ __forceinline__ uint32_t run_ring(const BatchArgs& b, const StepArgs&
   // the flip F_i(n) = n_{-i}: velocity i of the collision reads plane -i
   const uint32_t p1 = d.flip ? 2 * L : L, p2 = d.flip ? L : 2 * L;
   uint32_t s = 0;
-  if (R != 0 && warp >= colliders) {
-    const uint32_t j = warp - colliders;
-    const longlong2* trig = REC ? b.trig + d.state_off / 3 : nullptr;  // this ring's values
-    const auto red = [&](uint32_t st) { return sh.red[st % kSlots]; };
-    const auto write_group = [&](uint32_t s0, uint32_t count) {
-      write_sums<R>([&](uint32_t i) { return red(s0 + i); }, count, sh.c, L, mass,
-                    b.record + (size_t(r) * (T + 1) + s0) * 4);
-    };
-    for (;; ++s) {
-      ModeSums ms;
-      if constexpr (REC) ms.clear();
-      // the state after step s - 1, planes rest, +1, -1
-      uint16_t* const rs = STATES && s > 0 ? b.states + d.state_off * T + size_t(s - 1) * 3 * L : nullptr;
+  if constexpr (R != 0) {
+    if (warp >= colliders) {
+      const uint32_t j = warp - colliders;
+      const longlong2* trig = REC ? b.trig + d.state_off / 3 : nullptr;  // this ring's values
+      const auto red = [&](uint32_t st) { return sh.red[st % kSlots]; };
+      const auto write_group = [&](uint32_t s0, uint32_t count) {
+        write_sums<R>([&](uint32_t i) { return red(s0 + i); }, count, sh.c, L, mass,
+                      b.record + (size_t(r) * (T + 1) + s0) * 4);
+      };
+      for (;; ++s) {
+        ModeSums ms;
+        if constexpr (REC) ms.clear();
+        // the state after step s - 1, planes rest, +1, -1
+        uint16_t* const rs = STATES && s > 0 ? b.states + d.state_off * T + size_t(s - 1) * 3 * L : nullptr;
 #pragma unroll 4
-      for (uint32_t x = 32 * j + lane; x < L; x += 32 * R) {
-        const uint32_t m0 = src[x], m1 = src[L + x], m2 = src[2 * L + x];
-        if constexpr (REC) ms.add(trig[x], m0 + m1 + m2);
-        if constexpr (STATES) {
-          if (s > 0) {
-            rs[x] = uint16_t(m0);
-            rs[L + x] = uint16_t(m1);
-            rs[2 * L + x] = uint16_t(m2);
+        for (uint32_t x = 32 * j + lane; x < L; x += 32 * R) {
+          const uint32_t m0 = src[x], m1 = src[L + x], m2 = src[2 * L + x];
+          if constexpr (REC) ms.add(trig[x], m0 + m1 + m2);
+          if constexpr (STATES) {
+            if (s > 0) {
+              rs[x] = uint16_t(m0);
+              rs[L + x] = uint16_t(m1);
+              rs[2 * L + x] = uint16_t(m2);
+            }
           }
         }
+        if constexpr (REC) {
+          const long long v = ms.warp_sum(lane);
+          if ((lane & 7) == 0) red(s)[4 * j + (lane >> 3)] = v;
+        }
+        if (s == T) break;
+        bar();
+        if (stopped(s)) break;  // src still holds the state
+        uint16_t* tmp = src;
+        src = dst;
+        dst = tmp;
+        if (REC && (s % kGroup) == kGroup - 1 && j == 0) write_group(s - (kGroup - 1), kGroup);
       }
-      if constexpr (REC) {
-        const long long v = ms.warp_sum(lane);
-        if ((lane & 7) == 0) red(s)[4 * j + (lane >> 3)] = v;
-      }
-      if (s == T) break;
       bar();
-      if (stopped(s)) break;  // src still holds the state
-      uint16_t* tmp = src;
-      src = dst;
-      dst = tmp;
-      if (REC && (s % kGroup) == kGroup - 1 && j == 0) write_group(s - (kGroup - 1), kGroup);
+      if constexpr (REC) {
+        // the states since the last group (s: the last state whose sums exist)
+        if (j == 0) write_group(s / kGroup * kGroup, s % kGroup + 1);
+      }
+      return s;
     }
-    bar();
-    if constexpr (REC) {
-      // the states since the last group (s: the last state whose sums exist)
-      if (j == 0) write_group(s / kGroup * kGroup, s % kGroup + 1);
-    }
-    return s;
   }
   WordKeys k;
   k.slot.A = uint32_t((uint64_t(0xCD9E8D57u) * a.replica) >> 32) ^ a.rk[0];

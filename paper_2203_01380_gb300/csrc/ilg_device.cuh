@@ -24,7 +24,6 @@ constexpr uint32_t kDevTagStep = 1u << 24;
 constexpr uint32_t kDevTagExt = 2u << 24;
 constexpr uint32_t kDevTagInit = 3u << 24;
 constexpr uint32_t kDevTagParticle = 4u << 24;
-constexpr int kExtWords = 20;        // extension words per thread held in shared memory
 
 // How a probability P/2^32 is drawn: never (P = 0), by table (0 < P < 2^32),
 // always (P = 2^32).
@@ -148,24 +147,18 @@ __device__ __forceinline__ void step_blocks(const StepKeys<NB>& k, const uint32_
   }
 }
 
-// A node's eight slot words (two blocks): from its launch's StepKeys where the caller
-// made them, else from the full rounds.
-__device__ __forceinline__ void slot_words8(const StepArgs& a, const StepKeys<2>* keys, uint32_t node, uint32_t t,
-                                            uint32_t (&W)[8]) {
-  if (keys) {
-    step_blocks<2>(*keys, a.rk, node, W);
-  } else {
-    const uint4 b0 = philox_rk(counter(node, t, a.replica, kDevTagStep | 0u), a.rk);
-    const uint4 b1 = philox_rk(counter(node, t, a.replica, kDevTagStep | 1u), a.rk);
-    W[0] = b0.x;
-    W[1] = b0.y;
-    W[2] = b0.z;
-    W[3] = b0.w;
-    W[4] = b1.x;
-    W[5] = b1.y;
-    W[6] = b1.z;
-    W[7] = b1.w;
-  }
+// A node's eight slot words (two blocks).
+__device__ __forceinline__ void slot_words8(const StepArgs& a, uint32_t node, uint32_t t, uint32_t (&W)[8]) {
+  const uint4 b0 = philox_rk(counter(node, t, a.replica, kDevTagStep | 0u), a.rk);
+  const uint4 b1 = philox_rk(counter(node, t, a.replica, kDevTagStep | 1u), a.rk);
+  W[0] = b0.x;
+  W[1] = b0.y;
+  W[2] = b0.z;
+  W[3] = b0.w;
+  W[4] = b1.x;
+  W[5] = b1.y;
+  W[6] = b1.z;
+  W[7] = b1.w;
 }
 
 __device__ __forceinline__ uint32_t lane_of(const uint4& b, uint32_t i) {
@@ -187,14 +180,6 @@ __device__ __forceinline__ uint32_t ext_word(const StepArgs& a, ExtStream& e) {
   const uint32_t w = lane_of(e.blk, e.next & 3u);
   e.next += 1;
   return w;
-}
-
-// Word e of a node's extension stream, computed alone and out of line: the rare
-// word beyond a thread's shared-memory buffer, kept out of the loops that read the
-// buffer (inlined there, its Philox rounds weigh on every iteration).
-static __device__ __noinline__ uint32_t ext_word_at(const StepArgs& a, uint32_t node, uint32_t t, uint32_t e) {
-  const uint4 b = philox_rk(counter(node, t, a.replica, kDevTagExt | (e >> 2)), a.rk);
-  return lane_of(b, e & 3u);
 }
 
 // The two alias tables of the block (shared memory).
@@ -316,22 +301,18 @@ __device__ __forceinline__ void collide(const StepArgs& a, const uint32_t* s, ui
 // groups), a whole Philox block at a time, into this thread's shared-memory
 // buffer (word e at xb[e * S]; threads interleaved with stride S, so a warp's
 // accesses hit distinct banks), so a warp runs its blocks together; words beyond K
-// are read lazily, inline, or with OOL one at a time out of line (which keeps the
-// loops that read the buffer small, where a kernel has registers for the call).  A
-// probability of 0 or 2^32 draws nothing.
-template <int Q, int K, int S, class Tab = Alias8, bool OOL = false>
+// are read lazily.  A probability of 0 or 2^32 draws nothing.
+template <int Q, int K, int S>
 __device__ __forceinline__ void collide_buffered(const StepArgs& a, const uint32_t* s, uint32_t node, uint32_t t,
-                                                 const uint32_t (&m)[Q], uint32_t (&out)[Q], uint32_t* xb,
-                                                 const StepKeys<2>* keys = nullptr) {
+                                                 const uint32_t (&m)[Q], uint32_t (&out)[Q], uint32_t* xb) {
   static_assert(K % 4 == 0, "whole Philox blocks");
-  const Tab to = Tab::of(s, 0);
-  const Tab tr = Tab::of(s, 1);
+  const Alias8 to = Alias8::of(s, 0), tr = Alias8::of(s, 1);
   auto extra = [](uint32_t mode, uint32_t x) -> uint32_t { return mode == kTable && x > kDevNmax ? (x - 1) / kDevNmax : 0u; };
   uint32_t need = 0;
 #pragma unroll
   for (int i = 0; i < Q; ++i) need += extra(a.omega_mode, m[i]);
   uint32_t W[8];
-  slot_words8(a, keys, node, t, W);
+  slot_words8(a, node, t, W);
   uint32_t filled = 0;
   auto gen = [&](uint32_t upto) {
     upto = upto < uint32_t(K) ? upto : uint32_t(K);
@@ -347,14 +328,13 @@ __device__ __forceinline__ void collide_buffered(const StepArgs& a, const uint32
   ExtStream lazy{node, t, 0u, 0xFFFFFFFFu, make_uint4(0, 0, 0, 0)};
   auto word = [&](uint32_t e) -> uint32_t {
     if (e < uint32_t(K)) return xb[e * S];
-    if constexpr (OOL) return ext_word_at(a, node, t, e);
     lazy.next = e;
     return ext_word(a, lazy);
   };
   uint32_t e = 0;
   // Binomial(x, P) in chunks of 63 trials: the first with the slot word, the others
   // with the next extension words
-  auto draw = [&](uint32_t mode, const Tab& A, uint32_t x, uint32_t slot) -> uint32_t {
+  auto draw = [&](uint32_t mode, const Alias8& A, uint32_t x, uint32_t slot) -> uint32_t {
     if (mode == kNever) return 0u;
     if (mode == kAlways) return x;
     uint32_t r = A(x < kDevNmax ? x : kDevNmax, slot);
@@ -461,12 +441,11 @@ __device__ void collide_particle(const StepArgs& a, const uint32_t* s, uint32_t 
 }
 
 // The general collision in whichever sampler the lattice uses.
-template <int Q, int K, int S, class Tab = Alias8, bool OOL = false>
+template <int Q, int K, int S>
 __device__ __forceinline__ void collide_general(const StepArgs& a, const uint32_t* s, uint32_t node, uint32_t t,
-                                                const uint32_t (&m)[Q], uint32_t (&out)[Q], uint32_t* xb,
-                                                const StepKeys<2>* keys = nullptr) {
+                                                const uint32_t (&m)[Q], uint32_t (&out)[Q], uint32_t* xb) {
   if (a.particle) collide_particle<Q>(a, s, node, t, m, out);
-  else collide_buffered<Q, K, S, Tab, OOL>(a, s, node, t, m, out, xb, keys);
+  else collide_buffered<Q, K, S>(a, s, node, t, m, out, xb);
 }
 
 // The collision of one node, fast path: every occupation <= 63, at most 63
@@ -475,12 +454,10 @@ __device__ __forceinline__ void collide_general(const StepArgs& a, const uint32_
 // (out undefined) when the node falls outside that domain; the caller then runs
 // collide().  Same result as collide() wherever it returns true.  No result can
 // exceed 65535 here (mass is conserved and at most 5 * 63).
-template <int Q, class Tab = Alias8>
+template <int Q>
 __device__ __forceinline__ bool collide_try_fast(const StepArgs& a, const uint32_t* s, uint32_t node,
-                                                 uint32_t t, const uint32_t (&m)[Q], uint32_t (&out)[Q],
-                                                 const StepKeys<2>* keys = nullptr) {
-  const Tab to = Tab::of(s, 0);
-  const Tab tr = Tab::of(s, 1);
+                                                 uint32_t t, const uint32_t (&m)[Q], uint32_t (&out)[Q]) {
+  const Alias8 to = Alias8::of(s, 0), tr = Alias8::of(s, 1);
   if (a.omega_mode != kTable || a.rest_mode != kTable) return false;
   uint32_t any = m[0];
 #pragma unroll
@@ -488,7 +465,7 @@ __device__ __forceinline__ bool collide_try_fast(const StepArgs& a, const uint32
   if (any >> 6) return false;
   // slot words: thinning 0..Q-1, rest Q, moving Q+1 (and Q+2)
   uint32_t W[8];
-  slot_words8(a, keys, node, t, W);
+  slot_words8(a, node, t, W);
   uint32_t r[Q];
 #pragma unroll
   for (int i = 0; i < Q; ++i) r[i] = to(m[i], W[i]);
