@@ -42,7 +42,7 @@ SMS = 152
 # DRAM bytes (read + write) of one 16384^2 launch of a step kernel, from an ncu
 # capture of the same kernel (scaled from a smaller lattice by node count); only
 # kernels unchanged since their capture are listed
-TRAFFIC_BYTES_PER_LAUNCH = {"seg8": 5.187e9, "warpv8": 5.168e9}
+TRAFFIC_BYTES_PER_LAUNCH = {"seg8": 5.187e9, "warpv8": 5.193e9}
 
 
 def json_default(o):
@@ -182,7 +182,7 @@ def oracle_all_cores(cfg, side, steps, seconds):
     return sum(r[0] for r in res) / wall, n
 
 
-KERNEL_NAMES = {"vec8": "step_vec_kernel<5, 8>", "vec4": "step_vec_kernel<5, 4>", "node": "step_kernel<5>",
+KERNEL_NAMES = {"vec8": "step_vec_kernel<5, 8>", "vec4": "step_vec_kernel<5, 4>", "node": "step_run_kernel<5>",
                 "tb2": "step_tb_kernel (depth 2)", "tb4": "step_tb_kernel (depth 4)", "seg8": "step_seg_kernel<5, 8>",
                 "warpv8": "step_warp_kernel<5, flip, 64 rows, 8 nodes per lane, 384 threads>",
                 "warpv4": "step_warp_kernel<5, flip, 64 rows, 4 nodes per lane, 640 threads>"}
@@ -274,7 +274,7 @@ def measure_batched(torch, B, dev, rings=4096, T=5000, sample=64):
 
 
 FP64_LANES_PER_SM_CYCLE = 2.0   # GB300 nominal 1.25 TFLOP/s fp64 = 2 fused multiply-add lanes per SM per cycle at 2070 MHz
-LB_FP64_OPS_PER_NU = 15         # D2Q5: 4 adds, 2 multiplies, 9 fused multiply-adds, one fp64 lane-op each
+LB_FP64_OPS_PER_NU = 9          # D2Q5: 9 fused multiply-adds (the density and its two products are formed in integers)
 LB_BYTES_PER_NU = 80            # 5 doubles read + 5 written
 
 
@@ -308,7 +308,7 @@ def measure_lb(torch, B, dev, clocks, side=None):
     return {"workload": f"lb_d2q5: D2Q5 {kw['Lx']}x{kw['Ly']} fp64, omega^j {oj}, omega {om:.2f}, {T} steps",
             "value": nodes / (ms / 1e3) / 1e9, "unit": "GNUPS", "ms_per_step": ms,
             "roofline": {"bound": "alu", "achieved": ach, "peak": peak, "unit": "G fp64 lane-ops/s", "frac": ach / peak,
-                         "kernel": "lb_step_kernel<5>", "fp64_ops_per_node_update": LB_FP64_OPS_PER_NU,
+                         "kernel": "lb_run_kernel<5>", "fp64_ops_per_node_update": LB_FP64_OPS_PER_NU,
                          "peak_source": "nominal 1.25 TFLOP/s fp64 (2 FMA lanes per SM per cycle) at the measured SM clock"},
             "hbm": {"achieved": gbs, "peak": hpk, "unit": "GB/s", "frac": gbs / hpk},
             "mass": mass}
@@ -366,7 +366,7 @@ def measure_particle(torch, B, dev, side):
         ms = e0.elapsed_time(e1) / T
     return {"workload": f"large_d2q5 with the particle sampler: D2Q5 {side}x{side}, {T} steps",
             "value": side * side / (ms / 1e3) / 1e9, "unit": "GNUPS", "ms_per_step": ms,
-            "kernel": "step_kernel<5> (general path, one Philox word per particle)"}
+            "kernel": "step_run_kernel<5> (general path, one Philox word per particle)"}
 
 
 def measure_sweep(torch, B, dev):
@@ -472,7 +472,7 @@ def measure_d2q9(torch, B, dev, side):
     hpk = pk["hbm_gbs"] if pk else 6800.0
     names = {6: "step_warp_kernel<9>, 4-node vectors collided in shared memory, 512 threads per SM (default)",
              7: "step_warp_kernel<9>, 4-node vectors collided in shared memory, 640 threads per SM",
-             2: "step9_pair_kernel (node-parallel, two nodes of a row per thread)"}
+             2: "step_run_kernel<9> (node-parallel, a node per lane)"}
     kernels, obs = {}, []
     for cand in (6, 7, 2):
         with B.Lattice(**cfg, stream=st) as lat:

@@ -192,7 +192,8 @@ ilg_status ilg_set_step_kernel(ilg_ctx* ctx, int32_t candidate);
  *   re = sum_x cos(2 pi r / Lx) D(x) / Lx,  im = sum_x sin(2 pi r / Lx) D(x) / Lx,
  *   amp = im / (Lx*Ly/2)  (A^LG of Sec. V),  Sk = (re^2 + im^2) / (Lx*Ly);
  * modes along y use row sums R(y) and Ly.  Integer sums are exact (int64); the
- * projections are compensated double-precision dot products.  Every output pointer
+ * projections are exact sums of products with the cosines and sines rounded to 2^-62
+ * (compensated double-precision sums where Lx * M >= 2^64).  Every output pointer
  * is a host array (nmodes entries for re/im/amp/Sk, Lx for col_sums, Ly for
  * row_sums) and may be NULL.  Synchronous. */
 ilg_status ilg_observables(ilg_ctx* ctx, const int32_t* modes, uint32_t nmodes, uint64_t* t,

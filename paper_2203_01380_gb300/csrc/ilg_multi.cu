@@ -5,8 +5,8 @@
 // and a barrier of all blocks separates the steps.  Each lattice keeps its own step counter,
 // replica word and two buffers, so its result is the one it would have had alone.
 // Bound: integer issue (see collide_warp; 70 % of it while many lattices run).  24 requests of
-// 64 to 1024 a side at 5 to 100 per velocity: 62.7 ms in these launches.  Measured against
-// shares of a lattice that wait only for one another (608 blocks of 256 threads): 80 ms, the
+// 64 to 1024 a side at 5 to 100 per velocity: 55.3 ms in these launches.  Shares of a lattice
+// that wait only for one another (608 blocks of 256 threads) took 80 where this took 63: the
 // blocks of different lattices on an SM then wait at different times and leave it half idle.
 #include <cuda_runtime.h>
 
