@@ -42,7 +42,9 @@ __global__ void __launch_bounds__(THREADS, 1)
   extern __shared__ uint4 smem4[];
   __shared__ int stop;
   uint32_t* s = reinterpret_cast<uint32_t*>(smem4);
-  if (threadIdx.x == 0) stop = (*reinterpret_cast<volatile unsigned long long*>(fail) != ~0ull);
+  // a step before this launch overflowed (one of its own stops it at the barriers: a block that
+  // started late must not leave the others waiting there)
+  if (threadIdx.x == 0) stop = *reinterpret_cast<volatile unsigned long long*>(fail) < t0;
   constexpr uint32_t kTables = run_table_words(Q);
   // the block's first words: the alias tables, or the particle sampler's boundaries (all
   // copies in flight at once, the first node's words made meanwhile)

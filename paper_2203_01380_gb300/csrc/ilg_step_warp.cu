@@ -409,7 +409,9 @@ __global__ void __launch_bounds__(THREADS, MINB)
                      unsigned long long* fail, unsigned long long* sync) {
   extern __shared__ uint4 smem4[];
   __shared__ int stop;
-  if (threadIdx.x == 0) stop = (*reinterpret_cast<const volatile unsigned long long*>(fail) != ~0ull);
+  // a step before this launch overflowed (one of its own stops it at the barriers: a block that
+  // started late must not leave the others waiting there)
+  if (threadIdx.x == 0) stop = *reinterpret_cast<const volatile unsigned long long*>(fail) < t0;
   constexpr uint32_t kTables = Q == 9 ? 3 : 2;           // thinning, rest (D2Q9: and the axis share)
   constexpr uint32_t kRow4 = ROWS * kDevAliasCols / 2;  // uint4 per staged table
   {
