@@ -22,12 +22,12 @@ namespace ilg {
 // instead of a launch, a staging pass and an idle tail per step.
 // Bound: integer issue (65 % of it over all, about 75 % between the barriers; some 650 warp
 // instructions per 32 nodes at 50 per velocity and omega* = 0.5) on large lattices; the
-// barrier and the latency of one node (about 2 us a step) on small ones.  One block of 1024 threads per SM holds the tables
+// barrier and the latency of one node (1 to 2 us a step) on small ones.  One block of 1024 threads per SM holds the tables
 // once, in the 64-bit form whose draw takes two instructions fewer than the packed one
 // (29.1 against 31.0 us per step for two blocks of 512, 33 with packed tables).  Us per
 // step against one launch per step with a collision that loops per lane: 1024^2 at 50 per
 // velocity 25.0 / 37.3 (omega* 0.5), 15.7 / 26.8 (0.1); 1501 x 777 at 100 per velocity
-// 44.5 / 66; 1024^2 at 200 per velocity, omega* = 1, 83 / 241; 96 x 40 2.2 / 18.7.
+// 44.5 / 66; 1024^2 at 200 per velocity, omega* = 1, 83 / 241; 96 x 40 1.6 / 18.7.
 // --------------------------------------------------------------------------
 constexpr uint32_t kStepRing = 16;  // extension words per lane
 
@@ -35,7 +35,8 @@ __host__ __device__ constexpr uint32_t run_table_words(int Q) { return Q == 9 ? 
 
 // sync[0]: the barrier word, sync[1]: set to 1 when a wait gave up.  TABLES: the binomial
 // sampler with both probabilities strictly between 0 and 1; false: anything else.
-template <int Q, int THREADS, bool TABLES>
+// CLUSTER: the launch is one cluster of blocks and its barrier the cluster's.
+template <int Q, int THREADS, bool TABLES, bool CLUSTER>
 __global__ void __launch_bounds__(THREADS, 1)
     step_run_kernel(const __grid_constant__ StepArgs a, uint16_t* buf0, uint16_t* buf1, uint32_t t0, uint32_t T,
                     unsigned long long* fail, unsigned long long* sync) {
@@ -44,7 +45,11 @@ __global__ void __launch_bounds__(THREADS, 1)
   uint32_t* s = reinterpret_cast<uint32_t*>(smem4);
   // a step before this launch overflowed (one of its own stops it at the barriers: a block that
   // started late must not leave the others waiting there)
-  if (threadIdx.x == 0) stop = *reinterpret_cast<volatile unsigned long long*>(fail) < t0;
+  __shared__ uint32_t mark;  // CLUSTER: the first step of this launch that overflowed
+  if (threadIdx.x == 0) {
+    stop = *reinterpret_cast<volatile unsigned long long*>(fail) < t0;
+    mark = ~0u;
+  }
   constexpr uint32_t kTables = run_table_words(Q);
   // the block's first words: the alias tables, or the particle sampler's boundaries (all
   // copies in flight at once, the first node's words made meanwhile)
@@ -74,6 +79,11 @@ __global__ void __launch_bounds__(THREADS, 1)
   asm volatile("cp.async.wait_all;\n" ::: "memory");
   __syncthreads();
   if (stop) return;
+  if constexpr (CLUSTER) {
+    // the marks are written by other blocks from here on
+    cluster_arrive();
+    cluster_wait();
+  }
   for (uint32_t step = 0;; ++step) {
     const uint32_t t = t0 + step;
     const uint16_t* const in = (step & 1) ? buf1 : buf0;
@@ -135,15 +145,31 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
     if (bad) {
       atomicMin(fail, static_cast<unsigned long long>(t));
-      __threadfence();
-      atomicOr(sync, kRunMark);
+      if constexpr (CLUSTER) {
+        // (in the last step nobody waits for the mark, and a block may have ended)
+        if (step + 1 < T) cluster_mark(&mark, step, gridDim.x);
+      } else {
+        __threadfence();
+        atomicOr(sync, kRunMark);
+      }
     }
     if (step + 1 == T) break;
-    __syncthreads();
-    if (threadIdx.x == 0) run_arrive(sync);
+    if constexpr (CLUSTER) {
+      __syncwarp();
+      cluster_arrive();
+    } else {
+      __syncthreads();
+      if (threadIdx.x == 0) run_arrive(sync);
+    }
     // while the other blocks finish: the next step's words that need nothing of theirs
     keys = word_keys<NB>(a, t + 1);
     if (kAhead && (TABLES || !a.particle)) first.make(keys, a.rk, base0 + lane);
+    if constexpr (CLUSTER) {
+      cluster_wait();
+      // (a faster block may already have marked the next step)
+      if (*reinterpret_cast<volatile uint32_t*>(&mark) <= step) break;
+      continue;
+    }
     if (threadIdx.x == 0) {
       const unsigned long long v = run_wait(sync, (step + 1) * gridDim.x);
       if (v == ~0ull) {
@@ -173,19 +199,44 @@ struct RunShape {
 template <int THREADS>
 static const void* run_fn(int Q, bool tables) {
   if (Q == 3)
-    return tables ? reinterpret_cast<const void*>(step_run_kernel<3, THREADS, true>)
-                  : reinterpret_cast<const void*>(step_run_kernel<3, THREADS, false>);
+    return tables ? reinterpret_cast<const void*>(step_run_kernel<3, THREADS, true, false>)
+                  : reinterpret_cast<const void*>(step_run_kernel<3, THREADS, false, false>);
   if (Q == 5)
-    return tables ? reinterpret_cast<const void*>(step_run_kernel<5, THREADS, true>)
-                  : reinterpret_cast<const void*>(step_run_kernel<5, THREADS, false>);
+    return tables ? reinterpret_cast<const void*>(step_run_kernel<5, THREADS, true, false>)
+                  : reinterpret_cast<const void*>(step_run_kernel<5, THREADS, false, false>);
   if constexpr (THREADS <= 512)
-    return tables ? reinterpret_cast<const void*>(step_run_kernel<9, THREADS, true>)
-                  : reinterpret_cast<const void*>(step_run_kernel<9, THREADS, false>);
+    return tables ? reinterpret_cast<const void*>(step_run_kernel<9, THREADS, true, false>)
+                  : reinterpret_cast<const void*>(step_run_kernel<9, THREADS, false, false>);
   return nullptr;
 }
 
+template <int THREADS>
+static const void* cluster_fn(int Q) {
+  return Q == 3   ? reinterpret_cast<const void*>(step_run_kernel<3, THREADS, true, true>)
+         : Q == 5 ? reinterpret_cast<const void*>(step_run_kernel<5, THREADS, true, true>)
+                  : reinterpret_cast<const void*>(step_run_kernel<9, THREADS, true, true>);
+}
+
+// Several steps of a lattice that one cluster holds, a lane per node: the cluster's barrier
+// takes a few hundred cycles where arriving at and polling a word in L2 takes two thousand.
+// Sixteen blocks of 128 or 256 threads, as few as hold the lattice (rounded to a power of two);
+// in fewer and larger blocks the steps of more warps per SM cost what the barrier gains (64^2
+// at 50 per velocity 2.84 us per step in 8 blocks of 512, 2.33 in 16 of 256, 2.58 by the grid
+// barrier).  Us per step, grid barrier / cluster: 256 nodes of D1Q3 1.75 / 1.10, D2Q5 32^2
+// 1.75 / 1.15, 96 x 40 1.88 / 1.63, D2Q9 32^2 1.97 / 1.34, 64^2 2.08 / 1.93.
+constexpr uint32_t kClusterBlocks = 16;  // (beyond 8 a kernel opts in)
+static bool cluster_shape(int Q, bool tables, uint64_t nodes, RunShape* r) {
+  if (!tables || nodes > kClusterBlocks * 256) return false;
+  *r = nodes <= kClusterBlocks * 128 ? RunShape{cluster_fn<128>(Q), 128} : RunShape{cluster_fn<256>(Q), 256};
+  return true;
+}
+
+static bool run_tables(int Q, const StepArgs& a) {
+  return !a.particle && a.omega_mode == kTable && a.rest_mode == kTable && (Q != 9 || a.axis_mode == kTable);
+}
+
 static RunShape run_shape(int Q, const StepArgs& a, uint64_t nodes, uint32_t sms) {
-  const bool tables = !a.particle && a.omega_mode == kTable && a.rest_mode == kTable && (Q != 9 || a.axis_mode == kTable);
+  const bool tables = run_tables(Q, a);
   if (nodes <= uint64_t(sms) * 128) return {run_fn<128>(Q, tables), 128};
   if (Q == 9 || nodes <= uint64_t(sms) * 512) return {run_fn<512>(Q, tables), 512};
   return {run_fn<1024>(Q, tables), 1024};
@@ -202,12 +253,36 @@ cudaError_t prepare_step_kernels(int Q) {
     set(run_fn<512>(Q, tables), 512);
     set(run_fn<1024>(Q, tables), 1024);
   }
+  set(cluster_fn<128>(Q), 128);
+  set(cluster_fn<256>(Q), 256);
+  for (const void* f : {cluster_fn<128>(Q), cluster_fn<256>(Q)})
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   return e;
 }
 
 cudaError_t launch_step_run(int Q, const StepArgs& a, uint16_t* buf0, uint16_t* buf1, uint32_t t, uint32_t T,
                             unsigned long long* fail, unsigned long long* sync, uint32_t sms, cudaStream_t s) {
   const uint64_t nodes = uint64_t(a.Lx) * a.Ly;
+  RunShape cr;
+  if (T > 1 && cluster_shape(Q, run_tables(Q, a), nodes, &cr)) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr = {};
+    uint32_t blocks = 1;
+    while (uint64_t(blocks) * cr.threads < nodes) blocks *= 2;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = blocks;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(cr.threads);
+    cfg.dynamicSmemBytes = run_smem(Q, cr.threads);
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    StepArgs ca = a;
+    void* p[] = {&ca, &buf0, &buf1, &t, &T, &fail, &sync};
+    if (cudaLaunchKernelExC(&cfg, cr.fn, p) == cudaSuccess) return cudaSuccess;
+    cudaGetLastError();  // no room for a cluster (SMs reserved elsewhere): the grid barrier instead
+  }
   const RunShape r = run_shape(Q, a, nodes, sms);
   const dim3 grid(uint32_t(std::min<uint64_t>((nodes + r.threads - 1) / r.threads, sms)));
   StepArgs args = a;

@@ -32,4 +32,19 @@ __device__ __forceinline__ unsigned long long run_barrier(unsigned long long* wo
   return run_wait(word, target);
 }
 
+// The same between the blocks of one cluster (the whole launch): the hardware's cluster barrier,
+// and an overflow's step marked in every block's shared memory.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_mark(uint32_t* mark, uint32_t step, uint32_t blocks) {
+  const uint32_t own = static_cast<uint32_t>(__cvta_generic_to_shared(mark));
+  for (uint32_t r = 0; r < blocks; ++r)
+    asm volatile(
+        "{\n.reg .b32 at;\n"
+        "mapa.shared::cluster.u32 at, %0, %1;\n"
+        "red.relaxed.cluster.shared::cluster.min.u32 [at], %2;\n}"
+        ::"r"(own), "r"(r), "r"(step)
+        : "memory");
+}
+
 }  // namespace ilg
