@@ -27,6 +27,7 @@ namespace {
 constexpr int kLbThreads = 256;
 constexpr uint32_t kLbMaxModes = 256;
 constexpr int kLbModeThreads = 64;     // of a projection's blocks
+constexpr int kLbClusterBlocks = 16;   // (beyond 8 a kernel opts in)
 constexpr uint32_t kLbCols = 32;       // columns of a block of their sums (or kLbThreads)
 constexpr uint32_t kLbFewRows = 8;
 constexpr uint32_t kLbFirstModes = 64; // passed as a kernel argument
@@ -107,8 +108,11 @@ __device__ __forceinline__ double whole_product(unsigned long long M, int E, uns
 
 // T steps, one node per thread: load the Q planes, relax, push.  f0 holds the state, the
 // steps alternate the buffers; a barrier of all blocks (a cooperative launch) separates them.
-// sync[0]: barrier word, sync[1]: 1 once a wait gave up.
-template <int Q>
+// sync[0]: barrier word, sync[1]: 1 once a wait gave up.  CLUSTER: the launch is one cluster
+// (at most kLbClusterBlocks blocks, a node per thread) and its barrier the cluster's.  Us per
+// step, grid barrier / cluster: 500 nodes of D1Q3 2.0 / 1.3, D2Q5 64^2 2.5 / 2.1, D2Q9 56 x 66
+// 3.4 / 3.0 (one launch per step: 4.1).
+template <int Q, bool CLUSTER>
 __global__ void __launch_bounds__(kLbThreads, 4)
     lb_run_kernel(const __grid_constant__ LbCoef k, double* f0, double* f1, uint32_t Lx, uint32_t Ly, uint32_t T,
                   unsigned long long* sync) {
@@ -116,8 +120,9 @@ __global__ void __launch_bounds__(kLbThreads, 4)
   if (threadIdx.x == 0) stop = 0;
   const uint32_t nodes = Lx * Ly;
   const size_t plane = nodes;
-  const uint32_t stride = gridDim.x * kLbThreads, stride_y = stride / Lx, stride_x = stride - stride_y * Lx;
-  const uint32_t first = blockIdx.x * kLbThreads + threadIdx.x;
+  const uint32_t threads = CLUSTER ? blockDim.x : uint32_t(kLbThreads);
+  const uint32_t stride = gridDim.x * threads, stride_y = stride / Lx, stride_x = stride - stride_y * Lx;
+  const uint32_t first = blockIdx.x * threads + threadIdx.x;
   const uint32_t y0 = first / Lx, x0 = first - y0 * Lx;
   for (uint32_t step = 0;; ++step) {
     const double* const in = (step & 1) ? f1 : f0;
@@ -173,6 +178,12 @@ __global__ void __launch_bounds__(kLbThreads, 4)
       }
     }
     if (step + 1 == T) break;
+    if constexpr (CLUSTER) {
+      __syncwarp();
+      ilg::cluster_arrive();
+      ilg::cluster_wait();
+      continue;
+    }
     __syncthreads();
     if (threadIdx.x == 0 && ilg::run_barrier(sync, (step + 1) * gridDim.x) == ~0ull) {
       atomicExch(sync + 1, 1ull);
@@ -514,10 +525,37 @@ int lb_grid(const ilg_lb* b) {
   return int(blocks < cap ? blocks : cap);
 }
 
-const void* lb_run_fn(int Q) {
-  return Q == 3   ? reinterpret_cast<const void*>(lb_run_kernel<3>)
-         : Q == 5 ? reinterpret_cast<const void*>(lb_run_kernel<5>)
-                  : reinterpret_cast<const void*>(lb_run_kernel<9>);
+const void* lb_run_fn(int Q, bool cluster = false) {
+  if (cluster)
+    return Q == 3   ? reinterpret_cast<const void*>(lb_run_kernel<3, true>)
+           : Q == 5 ? reinterpret_cast<const void*>(lb_run_kernel<5, true>)
+                    : reinterpret_cast<const void*>(lb_run_kernel<9, true>);
+  return Q == 3   ? reinterpret_cast<const void*>(lb_run_kernel<3, false>)
+         : Q == 5 ? reinterpret_cast<const void*>(lb_run_kernel<5, false>)
+                  : reinterpret_cast<const void*>(lb_run_kernel<9, false>);
+}
+
+bool lb_fits_cluster(const ilg_lb* b) { return b->nodes <= size_t(kLbClusterBlocks) * kLbThreads; }
+
+// Several steps as one cluster; false where there is no room for it (SMs reserved elsewhere).
+bool lb_launch_cluster(const ilg_lb* b, void** args) {
+  // many small blocks: the fp64 pipe of as many SMs as there are
+  uint32_t threads = 64, blocks = 1;
+  while (size_t(kLbClusterBlocks) * threads < b->nodes) threads *= 2;
+  while (size_t(blocks) * threads < b->nodes) blocks *= 2;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = blocks;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(threads);
+  cfg.stream = b->stream;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  if (cudaLaunchKernelExC(&cfg, lb_run_fn(b->Q, true), args) == cudaSuccess) return true;
+  cudaGetLastError();
+  return false;
 }
 
 const void* lb_col_fn(int Q, bool wide) {
@@ -608,6 +646,8 @@ ilg_status ilg_lb_create(const ilg_lb_params* params, void* stream, ilg_lb** out
   }
   int per_sm = 0;
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lb_run_fn(b->Q), kLbThreads, 0);
+  if (e == cudaSuccess && lb_fits_cluster(b))
+    e = cudaFuncSetAttribute(lb_run_fn(b->Q, true), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) {
     ilg_lb_destroy(b);
     return lb_cuda_fail(nullptr, e, "ilg_lb_create");
@@ -723,7 +763,9 @@ ilg_status ilg_lb_step(ilg_lb* b, uint32_t T) {
     uint32_t n = run ? std::min(T - k, kRunSteps) : 1;
     double *f0 = b->f[b->cur], *f1 = b->f[b->cur ^ 1];
     void* args[] = {&b->coef, &f0, &f1, &b->p.Lx, &b->Ly, &n, &b->d_sync};
-    if (n > 1) {
+    if (n > 1 && lb_fits_cluster(b) && lb_launch_cluster(b, args)) {
+      // (no wait that could give up)
+    } else if (n > 1) {
       LB_CUDA(b, cudaMemsetAsync(b->d_sync, 0, sizeof(unsigned long long), b->stream), "lattice Boltzmann step");
       const cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(b->run_blocks), dim3(kLbThreads), args, 0, b->stream);
       if (e == cudaErrorCooperativeLaunchTooLarge) {

@@ -64,3 +64,17 @@ def test_overflow_marked_by_one_block(B, lattice, Lx, Ly, seed):
         assert e.value.status == B.ILG_E_OVERFLOW
         got, t = lat.get_state()
         assert t == fail_t and np.array_equal(got, cur)
+
+
+@pytest.mark.parametrize("lattice,Lx,Ly", [(1, 255, 1), (1, 257, 1), (2, 64, 64), (2, 241, 17), (3, 43, 41), (3, 64, 64)])
+def test_comparator_several_steps_at_once(B, lattice, Lx, Ly):
+    """One call of 11 steps and eleven calls of one step (plain launches): the same doubles."""
+    states = []
+    f0 = np.random.default_rng(Lx).uniform(1.0, 30.0, (Q[lattice], Ly, Lx))
+    for calls in ((11,), (1,) * 11):
+        with B.LB(lattice, Lx, Ly, omega_j=1.7, omega=0.3) as lb:
+            lb.set_state(f0)
+            for T in calls:
+                lb.step(T)
+            states.append(lb.get_state()[0])
+    assert np.array_equal(states[0], states[1])
