@@ -139,8 +139,8 @@ __device__ __forceinline__ void make_step_keys(const StepArgs& a, uint32_t t0, u
 // the alias tables in 64-bit form where one block per SM is resident (1024 threads; a
 // draw takes two instructions fewer), packed where several share an SM.  Measured
 // against per-lane loops and one 128-bit projection per node and step: 2048 rings of 64 to
-// 8192 nodes x 2000 steps 193 ms / 249 ms; 512 rings of 320 nodes x 2000 steps with
-// statistics 6.5 / 10.6 ms; one ring of 256 nodes with its records 1.0 / 2.06 us per step.
+// 8192 nodes x 2000 steps 190 ms / 249 ms; 512 rings of 320 nodes x 2000 steps with
+// statistics 6.2 / 10.6 ms; one ring of 256 nodes with its records 1.0 / 2.06 us per step.
 template <int THREADS>
 struct BatchShape {
   static constexpr int kPerSm = 1024 / THREADS;
