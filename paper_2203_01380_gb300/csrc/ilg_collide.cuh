@@ -168,20 +168,24 @@ struct NodeWords {
 template <uint32_t S, uint32_t K, class Keys, class Tab>
 __device__ __forceinline__ uint32_t more_chunks(NodeWords<S, K>& e, const Keys& k, const uint32_t (&rk)[20],
                                                 const Tab& A, int32_t left) {
-  constexpr int32_t kN = int32_t(kDevNmax);
   uint32_t r = 0;
-  const auto chunk = [&]() {
-    r += A(uint32_t(__vimin_s32_relu(left, kN)), e.peek());
-    if (left > 0) e.rd += S;
-    left -= kN;
-  };
   if constexpr (K > 8) {
     while (__any_sync(kFullWarp, left > 0)) {
-      e.template ensure<2>(k, rk, left > kN ? 2 * S : (left > 0 ? S : 0u));
-      chunk();
-      chunk();
+      e.template ensure<2>(k, rk, left > int32_t(kDevNmax) ? 2 * S : (left > 0 ? S : 0u));
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        r += A(uint32_t(__vimin_s32_relu(left, int32_t(kDevNmax))), e.peek());
+        if (left > 0) e.rd += S;
+        left -= int32_t(kDevNmax);
+      }
     }
   } else {
+    constexpr int32_t kN = int32_t(kDevNmax);
+    const auto chunk = [&]() {
+      r += A(uint32_t(__vimin_s32_relu(left, kN)), e.peek());
+      if (left > 0) e.rd += S;
+      left -= kN;
+    };
     bool some = __any_sync(kFullWarp, left > 0);
     if (!some) return 0;
     while (__any_sync(kFullWarp, left > 2 * kN)) {
