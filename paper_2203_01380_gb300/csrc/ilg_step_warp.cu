@@ -7,7 +7,7 @@
 //    warp covers 32 NPT nodes of a row per tile); the next tile's occupations are
 //    copied into the warp's shared-memory buffer by cp.async while the current tile
 //    collides, so the copy holds no registers;
-//  - the flip is a compile-time choice of which plane is loaded as which
+//  - the flip is a compile-time choice of which plane of the buffer is read as which
 //    velocity, so it costs nothing;
 //  - the fast collision runs branch-free on every node of a vector whose
 //    occupations are all below ROWS (64: the rows of the alias tables, staged in
@@ -18,10 +18,8 @@
 //    edge values by shuffles, and the two values that cross a segment's ends are
 //    written as single 16-bit stores by the warp that computes them, so no node is
 //    computed twice and no warp waits for another;
-//  - D1Q3 and D2Q5 hold a lane's vector and its results in registers; D2Q9 (nine
-//    planes, four Philox blocks and eleven draws per node) leaves the vector in the
-//    tile buffer and collides it two nodes at a time in place, which frees the
-//    registers for more warps.
+//  - a lane's vector and its results stay in registers, and it collides two nodes at a
+//    time (fast_pair), so that sums and results are formed for both at once.
 // Every random number is keyed by node and step, so the bits equal those of every
 // other step kernel.
 #include <cuda_runtime.h>
@@ -74,140 +72,167 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 __device__ __forceinline__ void cp_async_wait_prior() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
-// Binomial(n, P) for n < 64 with one draw u through the alias table A (rows of 64
-// columns, column u >> 26): the column's own outcome below its threshold, else its
-// alias.  HI: the column as the high word of u * 64 (a multiply, on the FMA pipe,
-// where the ALU pipe is the busier one: D2Q9) instead of a shift.
-template <bool HI = false>
-__device__ __forceinline__ uint32_t draw(const uint2* A, uint32_t n, uint32_t u) {
-  const uint2 e = A[__funnelshift_l(u, n, 6)];
-  return u < e.x ? (HI ? __umulhi(u, 64u) : (u >> 26)) : e.y;
+// the flip F_i(n) = n_{-i}: velocity i of the collision reads plane -i
+template <bool FLIP>
+__device__ __forceinline__ constexpr int source_plane(int i) {
+  return !FLIP || i == 0 ? i : (i & 1 ? i + 1 : i - 1);
 }
 
-// Fast collision of one node whose occupations are all below ROWS, branch-free, from
-// its slot words W.  Returns nonzero when the node needs the general collision (more than ROWS - 1
-// removed, or for ROWS = 64 more than 32 moving particles); out is then garbage,
-// but every table index stayed inside the staged rows.
-template <int Q, int ROWS>
-__device__ __forceinline__ uint32_t fast_draws(const uint2* to, const uint2* tr, const uint32_t (&W)[8],
-                                               const uint32_t (&m)[Q], uint32_t (&out)[Q]) {
-  uint32_t r[Q];
-  uint32_t removed = 0;
+// a b + c on the FMA pipe
+__device__ __forceinline__ uint32_t mad(uint32_t a, uint32_t b, uint32_t c) {
+  uint32_t d;
+  asm("mad.lo.u32 %0, %1, %2, %3;\n" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+  return d;
+}
+
+// Binomial(n, P) for n < 64 with one draw u through the alias table at shared address
+// `table` (rows of 64 columns, column u >> 26): the column's own outcome below its
+// threshold, else its alias.
+__device__ __forceinline__ uint32_t draw(uint32_t table, uint32_t n, uint32_t u) {
+  const uint32_t j = u >> 26;
+  uint32_t thr, r;
+  asm("ld.shared.v2.u32 {%0, %1}, [%2];\n" : "=r"(thr), "=r"(r) : "r"(mad(j, 8, mad(n, 512, table))));
+  return u < thr ? j : r;
+}
+
+// Shared addresses of the staged tables: thinning, rest, D2Q9's axis share.
+struct FastTables {
+  uint32_t to, tr, ta;
+};
+
+// Axis bit A (0: x, 1: y) and sign bit B (0: +, 1: -) of the first `c` <= 32 particles:
+// how many have A set, both, B alone.
+__device__ __forceinline__ void count3(uint32_t c, uint32_t A, uint32_t B, uint32_t& a, uint32_t& both, uint32_t& b) {
+  const uint32_t mask = __funnelshift_lc(0xFFFFFFFFu, 0u, c);  // (1 << c) - 1, c <= 32
+  a = __popc(A & mask);
+  both = __popc(A & B & mask);
+  b = __popc(~A & B & mask);
+}
+
+// What bounds it: the ALU and FMA-heavy pipes.  Each takes two cycles per warp instruction and
+// sub-partition; a 32 x 32 -> 64 product takes four of the FMA-heavy pipe and, measured beside
+// 3-input logic, two of the ALU pipe as well, so a node's 30 products fill 120 and 60 cycles
+// before anything else, and the two pipes are as full as they get (collisions alone, D2Q5: 220
+// cycles per 32 nodes, 208 of them the ALU pipe's, 165 the FMA-heavy pipe's).  Hence: what can be a
+// multiply-add is one (table addresses, halves packed and parted), and sums, differences, limits
+// and the checks on them are made once for the two nodes, in 16-bit halves.  GNUPS against one node
+// at a time, 16384^2 D2Q5 165 / 159; 8192^2 4-node vectors 149 / 138; 8192^2 D2Q9 77.4 / 72.7 (there
+// one pair at a time from the tile buffer).  Not faster: the table's outcome selected by a
+// predicated multiply-add instead of on the ALU pipe (D2Q5 166 for some of the draws, 159 for all).
+//
+// Fast collision of two neighbouring nodes whose occupations (w: the even node's in the low
+// halves) are all below 64, branch-free: node0 the even node, p their results packed alike.
+// Returns bits 12 and 28: the even / the odd node needs the general collision (more than 63
+// removed, or more than 32 moving particles of a kind); its half of p is then garbage in
+// [0, 126], but every table index stayed inside the staged rows.
+template <int Q>
+__device__ __forceinline__ uint32_t fast_pair(const FastTables& T, const StepKeys<Q == 9 ? 4 : 2>& keys,
+                                              const uint32_t (&rk)[20], uint32_t node0, const uint32_t (&w)[Q],
+                                              uint32_t (&p)[Q]) {
+  constexpr int NB = Q == 9 ? 4 : 2;
+  uint32_t W[2][4 * NB], r[Q], D[Q];
 #pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    r[i] = draw(to, m[i], W[i]);
-    removed += r[i];
+  for (int h = 0; h < 2; ++h) {
+    step_blocks<NB>(keys, rk, node0 + h, W[h]);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      const uint32_t high = w[i] >> 16;
+      const uint32_t m = h ? high : mad(high, 0xFFFF0000u, w[i]);
+      const uint32_t x = draw(T.to, m, W[h][i]);
+      if (h) D[i] = mad(x, 65536u, r[i]);
+      else r[i] = x;
+    }
   }
-  uint32_t fail = removed >= uint32_t(ROWS) ? 1u : 0u;
-  const uint32_t rr = min(removed, uint32_t(ROWS - 1));
-  const uint32_t to_rest = draw(tr, rr, W[Q]);
-  const uint32_t moving = rr - to_rest;
-  if constexpr (ROWS > 33) fail |= moving > 32u ? 1u : 0u;
-  const uint32_t mask = __funnelshift_lc(0xFFFFFFFFu, 0u, moving);  // (1 << moving) - 1, moving <= 32
-  out[0] = m[0] - r[0] + to_rest;
+  uint32_t removed = D[0];
+#pragma unroll
+  for (int i = 1; i < Q; ++i) removed += D[i];
+  const uint32_t rr = __vminu2(removed, 0x003F003Fu);
+  const uint32_t rr1 = rr >> 16, rr0 = mad(rr1, 0xFFFF0000u, rr);
+  const uint32_t rest0 = draw(T.tr, rr0, W[0][Q]), rest1 = draw(T.tr, rr1, W[1][Q]);
+  const uint32_t rest = mad(rest1, 65536u, rest0);
+  const uint32_t mv = rr - rest, mv1 = rr1 - rest1, mv0 = rr0 - rest0;
+  p[0] = w[0] - D[0] + rest;
+  // 4096 - 64 + removed and 4096 - 33 + moving reach bit 12 beyond the limits
+  uint32_t over = removed + 0x0FC00FC0u;
   if constexpr (Q == 3) {
-    const uint32_t minus = __popc(W[Q + 1] & mask);
-    out[1] = m[1] - r[1] + (moving - minus);
-    out[2] = m[2] - r[2] + minus;
+    over |= mv + 0x0FDF0FDFu;
+    const uint32_t k0 = __popc(W[0][Q + 1] & __funnelshift_lc(0xFFFFFFFFu, 0u, mv0));
+    const uint32_t k1 = __popc(W[1][Q + 1] & __funnelshift_lc(0xFFFFFFFFu, 0u, mv1));
+    const uint32_t minus = mad(k1, 65536u, k0);
+    p[1] = w[1] - D[1] + (mv - minus);
+    p[2] = w[2] - D[2] + minus;
   } else {
-    const uint32_t ax = W[Q + 1] & mask, sg = W[Q + 2];
-    const uint32_t ny = __popc(ax);                // to +y or -y
-    const uint32_t nmy = __popc(ax & sg);          // to -y
-    const uint32_t nmx = __popc(sg & mask & ~ax);  // to -x
-    out[1] = m[1] - r[1] + (moving - ny - nmx);
-    out[2] = m[2] - r[2] + nmx;
-    out[3] = m[3] - r[3] + (ny - nmy);
-    out[4] = m[4] - r[4] + nmy;
+    uint32_t ax = mv, ax0 = mv0, ax1 = mv1;
+    if constexpr (Q == 9) {
+      ax0 = draw(T.ta, mv0, W[0][10]);
+      ax1 = draw(T.ta, mv1, W[1][10]);
+      ax = mad(ax1, 65536u, ax0);
+    }
+    over |= ax + 0x0FDF0FDFu;
+    constexpr int A = Q == 9 ? 11 : Q + 1;
+    uint32_t a[2], both[2], b[2];
+    count3(ax0, W[0][A], W[0][A + 1], a[0], both[0], b[0]);
+    count3(ax1, W[1][A], W[1][A + 1], a[1], both[1], b[1]);
+    const uint32_t ny = mad(a[1], 65536u, a[0]), nmy = mad(both[1], 65536u, both[0]), nmx = mad(b[1], 65536u, b[0]);
+    p[1] = (w[1] - D[1] + ax) - ny - nmx;
+    p[2] = w[2] - D[2] + nmx;
+    p[3] = w[3] - D[3] + (ny - nmy);
+    p[4] = w[4] - D[4] + nmy;
+    if constexpr (Q == 9) {
+      // diagonal particles: x-sign bit X, y-sign bit Y (0: +, 1: -)
+      const uint32_t dg = mv - ax;
+      over |= dg + 0x0FDF0FDFu;
+      count3(mv0 - ax0, W[0][13], W[0][14], a[0], both[0], b[0]);
+      count3(mv1 - ax1, W[1][13], W[1][14], a[1], both[1], b[1]);
+      const uint32_t x = mad(a[1], 65536u, a[0]), xy = mad(both[1], 65536u, both[0]), yo = mad(b[1], 65536u, b[0]);
+      p[5] = (w[5] - D[5] + dg) - x - yo;
+      p[6] = w[6] - D[6] + xy;
+      p[7] = w[7] - D[7] + yo;
+      p[8] = w[8] - D[8] + (x - xy);
+    }
   }
-  return fail;
-}
-
-// D2Q9 fast collision of one node whose occupations are all below ROWS, branch-free
-// (the fast path of ilg_d2q9.cuh with the same words and results): thinning W0..W8,
-// rest W9, axis share W10, axis particles (A, B) = (W11, W12), diagonal particles
-// (X, Y) = (W13, W14).  Nonzero when the node needs the general collision (more than
-// ROWS - 1 removed, more than 32 axis or diagonal movers).
-template <int ROWS>
-__device__ __forceinline__ uint32_t fast_draws9(const uint2* to, const uint2* tr, const uint2* ta,
-                                                const uint32_t (&W)[16], const uint32_t (&m)[9], uint32_t (&out)[9]) {
-  uint32_t r[9];
-  uint32_t removed = 0;
-#pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    r[i] = draw<true>(to, m[i], W[i]);
-    removed += r[i];
-  }
-  uint32_t fail = removed >= uint32_t(ROWS) ? 1u : 0u;
-  const uint32_t rr = min(removed, uint32_t(ROWS - 1));
-  const uint32_t to_rest = draw<true>(tr, rr, W[9]);
-  const uint32_t moving = rr - to_rest;
-  const uint32_t axis = draw<true>(ta, moving, W[10]);
-  const uint32_t diag = moving - axis;
-  fail |= (axis > 32u || diag > 32u) ? 1u : 0u;
-  const uint32_t ma = __funnelshift_lc(0xFFFFFFFFu, 0u, axis);  // (1 << c) - 1, c <= 32
-  const uint32_t md = __funnelshift_lc(0xFFFFFFFFu, 0u, diag);
-#pragma unroll
-  for (int i = 0; i < 9; ++i) out[i] = m[i] - r[i];
-  out[0] += to_rest;
-  // axis particles: axis bit A (0: x, 1: y), sign bit B (0: +, 1: -)
-  const uint32_t A = W[11] & ma, B = W[12] & ma;
-  const uint32_t ny = __popc(A), nmy = __popc(A & B), nmx = __popc(B & ~A);
-  out[1] += axis - ny - nmx;
-  out[2] += nmx;
-  out[3] += ny - nmy;
-  out[4] += nmy;
-  // diagonal particles: x-sign bit X, y-sign bit Y (0: +, 1: -)
-  const uint32_t X = W[13] & md, Y = W[14] & md;
-  const uint32_t nmm = __popc(X & Y), npm = __popc(Y) - nmm, nmp = __popc(X) - nmm;
-  out[5] += diag - nmm - npm - nmp;
-  out[6] += nmm;
-  out[7] += npm;
-  out[8] += nmp;
-  return fail;
+  return over & 0x10001000u;
 }
 
 // The general collision of the nodes of a vector marked in `slow`, out of line.  N:
-// the lane's slot of the current tile buffer in shared memory (plane i at N[32 i],
-// flip applied); node k's results are written to half-word k of R[32 i]: the lane's
-// slot of the warp's scratch in shared memory, or the slot itself when the vector is
-// collided in place.  Both live in shared memory so that no register array of the
-// caller has its address taken (which would keep it in local memory on every tile).
+// the lane's slot of the current tile buffer in shared memory (plane i at N[32 i], before
+// the flip); velocity i's result of node k replaces half-word k of N[32 i].  In shared memory
+// so that no register array of the caller has its address taken (which would keep it in local
+// memory on every tile).
 // st: the staged tables (all rows of each, laid out as the table block; from global memory a
 // node's dozen dependent draws would keep its warp ten times longer).  Returns true when a
 // result exceeds 65535.
-template <int Q, int NPT>
+template <int Q, bool FLIP, int NPT>
 __device__ __noinline__ bool slow_nodes(const StepArgs& a, const uint32_t* st, uint32_t node0, uint32_t t,
-                                        const VN<NPT>* N, VN<NPT>* R, uint32_t slow) {
+                                        VN<NPT>* N, uint32_t slow) {
   bool bad = false;
   while (slow) {
     const int k = __ffs(slow) - 1;
     slow &= slow - 1;
     uint32_t m[Q], o[Q];
 #pragma unroll
-    for (int i = 0; i < Q; ++i) m[i] = node_of(N[32 * i], k);
+    for (int i = 0; i < Q; ++i) m[i] = node_of(N[32 * source_plane<FLIP>(i)], k);
     if constexpr (Q == 9) collide9_general(a, st, node0 + k, t, m, o);
     else collide<Q>(a, st, node0 + k, t, m, o);
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
       bad |= o[i] > 65535u;
-      reinterpret_cast<uint16_t*>(&R[32 * i])[k] = uint16_t(o[i]);
+      reinterpret_cast<uint16_t*>(&N[32 * i])[k] = uint16_t(o[i]);
     }
   }
   return bad;
 }
 
-// Flip and collide the NPT nodes of one vector (first node `node0`) into the packed
-// post-collision planes P.  N holds the vector's occupations with the flip already
-// applied (plane i loaded from the flipped source); slot is where they came from in
-// the tile buffer and scratch the lane's slot for the general collision's results
-// (both read only by the out-of-line general collision); keys: the launch-wide part
-// of every node's slot blocks.
-template <int Q, int ROWS, int NPT>
-__device__ __forceinline__ void collide_vec(const StepArgs& a, const StepKeys<Q == 9 ? 4 : 2>& keys, const uint2* to,
-                                            const uint2* tr, const uint2* ta, uint32_t node0, uint32_t t,
-                                            VN<NPT> (&N)[Q], VN<NPT> (&P)[Q], const VN<NPT>* slot,
-                                            VN<NPT>* scratch, bool& bad) {
-  constexpr uint32_t kHigh = ROWS == 32 ? 0xFFE0FFE0u : 0xFFC0FFC0u;  // bits of values >= ROWS
+// Collide the NPT nodes of one vector (first node `node0`) into the packed post-collision
+// planes P.  N holds the vector's occupations with the flip already applied; slot is where
+// they came from in the tile buffer (for the out-of-line general collision, which leaves its
+// results there); keys: the launch-wide part of every node's slot blocks.
+template <int Q, bool FLIP, int ROWS, int NPT>
+__device__ __forceinline__ void collide_vec(const StepArgs& a, const StepKeys<Q == 9 ? 4 : 2>& keys, const uint32_t* tables,
+                                            const FastTables& T, uint32_t node0, uint32_t t,
+                                            VN<NPT> (&N)[Q], VN<NPT> (&P)[Q], VN<NPT>* slot, bool& bad) {
+  static_assert(ROWS == 64 && NPT <= 8, "six-bit rows; the pairs' marks stay in their halves");
+  constexpr uint32_t kHigh = 0xFFC0FFC0u;  // bits of values >= ROWS
   uint32_t any = 0;
 #pragma unroll
   for (int i = 0; i < Q; ++i)
@@ -230,60 +255,30 @@ __device__ __forceinline__ void collide_vec(const StepArgs& a, const StepKeys<Q 
       slow |= ((w & 0xFFFFu) ? 1u : 0u) << (2 * j) | ((w >> 16) ? 2u : 0u) << (2 * j);
     }
   }
+  uint32_t over = 0;  // pair j's bits end at 12 + H - 1 - j and 28 + H - 1 - j
 #pragma unroll
-  for (int i = 0; i < Q; ++i)
+  for (int j = 0; j < NPT / 2; ++j) {
+    uint32_t w[Q], p[Q];
 #pragma unroll
-    for (int j = 0; j < NPT / 2; ++j) P[i].w[j] = 0u;
-  {
+    for (int i = 0; i < Q; ++i) w[i] = N[i].w[j];
+    const uint32_t e = fast_pair<Q>(T, keys, a.rk, node0 + 2 * j, w, p);
+    over = j == 0 ? e : mad(over, 2u, e);
 #pragma unroll
-    for (int k = 0; k < NPT; ++k) {
-      uint32_t m[Q], o[Q];
+    for (int i = 0; i < Q; ++i) P[i].w[j] = p[i];
+  }
+  if (over) {
 #pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        // the odd node is the high half; the even node the word minus it times 2^16,
-        // a multiply-add (FMA pipe) where a mask would take the busier ALU pipe
-        const uint32_t w = N[i].w[k >> 1], high = w >> 16;
-        if (k & 1) {
-          m[i] = high;
-        } else {
-          uint32_t low;
-          asm("mad.lo.u32 %0, %1, %2, %3;\n" : "=r"(low) : "r"(high), "r"(0xFFFF0000u), "r"(w));
-          m[i] = low;
-        }
-      }
-      if constexpr (Q == 9) {
-        uint32_t W[16];
-        step_blocks<4>(keys, a.rk, node0 + k, W);
-        slow |= fast_draws9<ROWS>(to, tr, ta, W, m, o) << k;
-      } else {
-        uint32_t W[8];
-        step_blocks<2>(keys, a.rk, node0 + k, W);
-        slow |= fast_draws<Q, ROWS>(to, tr, W, m, o) << k;
-      }
-      // pack the node's results into its half-words as soon as they exist: an odd
-      // node's by a multiply-add (the FMA pipe: the ALU pipe is the busier one), which
-      // is exact because every fast-path result, even a failing node's, lies in
-      // [0, 126] (no draw exceeds its trials, and at most min(moving, 32) of the
-      // moving particles are sorted), so the even node's high half is zero
-#pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        uint32_t& w = P[i].w[k >> 1];
-        if (k & 1) {
-          uint32_t packed;
-          asm("mad.lo.u32 %0, %1, 65536, %2;\n" : "=r"(packed) : "r"(o[i]), "r"(w));
-          w = packed;
-        } else {
-          w = o[i];
-        }
-      }
+    for (int j = 0; j < NPT / 2; ++j) {
+      const uint32_t e = over >> (NPT / 2 - 1 - j);
+      slow |= ((e >> 12) & 1u) << (2 * j) | ((e >> 28) & 1u) << (2 * j + 1);
     }
   }
   if (slow) {
-    bad |= slow_nodes<Q, NPT>(a, reinterpret_cast<const uint32_t*>(to), node0, t, slot, scratch, slow);
+    bad |= slow_nodes<Q, FLIP, NPT>(a, tables, node0, t, slot, slow);
     // take the general collision's half-words for the nodes it redid
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-      const VN<NPT> r = scratch[32 * i];
+      const VN<NPT> r = slot[32 * i];
 #pragma unroll
       for (int j = 0; j < NPT / 2; ++j) {
         const uint32_t mask = ((slow >> (2 * j)) & 1u ? 0x0000FFFFu : 0u) | ((slow >> (2 * j + 1)) & 1u ? 0xFFFF0000u : 0u);
@@ -291,72 +286,6 @@ __device__ __forceinline__ void collide_vec(const StepArgs& a, const StepKeys<Q 
       }
     }
   }
-}
-
-// 32-bit shared-memory load and store at a shared-window address, kept in program
-// order with the other shared accesses of the lane's slots
-__device__ __forceinline__ uint32_t lds32(uint32_t addr) {
-  uint32_t v;
-  asm volatile("ld.shared.u32 %0, [%1];\n" : "=r"(v) : "r"(addr) : "memory");
-  return v;
-}
-__device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) {
-  asm volatile("st.shared.u32 [%0], %1;\n" ::"r"(addr), "r"(v) : "memory");
-}
-
-// collide_vec with the vector left in shared memory: the nodes are taken two at a
-// time (one 32-bit word per plane) from the lane's slot of the tile buffer (plane i at
-// slot[32 i]), and their packed results replace the occupations they came from, so
-// only one pair's occupations and results are held in registers at a time.  A pair is
-// written only when both its nodes passed the fast collision; otherwise both are
-// redone by the general collision, which still finds their occupations in the slot.
-template <int Q, int ROWS, int NPT>
-__device__ __forceinline__ void collide_vec_res(const StepArgs& a, const StepKeys<Q == 9 ? 4 : 2>& keys,
-                                                const uint2* to, const uint2* tr, const uint2* ta, uint32_t node0,
-                                                uint32_t t, VN<NPT>* slot, bool& bad) {
-  constexpr uint32_t kHigh = ROWS == 32 ? 0xFFE0FFE0u : 0xFFC0FFC0u;  // bits of values >= ROWS
-  constexpr uint32_t kPlane = 32 * sizeof(VN<NPT>);                     // bytes between planes
-  const bool tables = a.omega_mode == kTable && a.rest_mode == kTable && (Q != 9 || a.axis_mode == kTable);
-  const uint32_t sn = static_cast<uint32_t>(__cvta_generic_to_shared(slot));
-  uint32_t slow = 0;
-#pragma unroll
-  for (int j = 0; j < NPT / 2; ++j) {
-    uint32_t w[Q];
-    uint32_t any = 0;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      w[i] = lds32(sn + i * kPlane + 4 * j);
-      any |= w[i];
-    }
-    if (!tables || (any & kHigh)) {
-      slow |= 3u << (2 * j);
-      continue;
-    }
-    uint32_t o[2][Q];
-    uint32_t f = 0;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      uint32_t m[Q];
-#pragma unroll
-      for (int i = 0; i < Q; ++i) m[i] = h ? (w[i] >> 16) : (w[i] & 0xFFFFu);
-      if constexpr (Q == 9) {
-        uint32_t W[16];
-        step_blocks<4>(keys, a.rk, node0 + 2 * j + h, W);
-        f |= fast_draws9<ROWS>(to, tr, ta, W, m, o[h]) << h;
-      } else {
-        uint32_t W[8];
-        step_blocks<2>(keys, a.rk, node0 + 2 * j + h, W);
-        f |= fast_draws<Q, ROWS>(to, tr, W, m, o[h]) << h;
-      }
-    }
-    if (f) {
-      slow |= 3u << (2 * j);
-      continue;
-    }
-#pragma unroll
-    for (int i = 0; i < Q; ++i) sts32(sn + i * kPlane + 4 * j, __byte_perm(o[0][i], o[1][i], 0x5410));
-  }
-  if (slow) bad |= slow_nodes<Q, NPT>(a, reinterpret_cast<const uint32_t*>(to), node0, t, slot, slot, slow);
 }
 
 // The segment that starts at vector g of the row-major sequence of all vectors
@@ -371,20 +300,13 @@ __device__ __forceinline__ void segment_at(uint32_t g, uint32_t end, uint32_t vp
 
 // Queue the copies of one lane's vector (tile row rowoff, vector v) into its slots of
 // the warp's tile buffer tb (Q planes of 32 vectors).
-template <int Q, bool FLIP, int NPT>
+template <int Q, int NPT>
 __device__ __forceinline__ void stage_tile(VN<NPT>* tb, const uint16_t* __restrict__ in, size_t plane, size_t rowoff,
                                            uint32_t v, bool active, uint32_t lane) {
-  constexpr int kBytes = 2 * NPT < 16 ? 2 * NPT : 16;  // per copy
+  static_assert(2 * NPT <= 16, "one copy per vector");
 #pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    // the flip F_i(n) = n_{-i}: velocity i of the collision reads plane -i
-    const int src = !FLIP || i == 0 ? i : (i & 1 ? i + 1 : i - 1);
-    const uint16_t* p = active ? in + src * plane + rowoff + size_t(v) * NPT : in;
-#pragma unroll
-    for (int c = 0; c < 2 * NPT / kBytes; ++c)
-      cp_async<kBytes>(reinterpret_cast<char*>(tb + i * 32 + lane) + c * kBytes, active ? p + c * (kBytes / 2) : p,
-                       active);
-  }
+  for (int i = 0; i < Q; ++i)
+    cp_async<2 * NPT>(tb + i * 32 + lane, active ? in + i * plane + rowoff + size_t(v) * NPT : in, active);
   cp_async_commit();
 }
 
@@ -403,8 +325,8 @@ __device__ __forceinline__ constexpr int vel_dy(int i) {
 // T steps from t0, the state in buf0, a barrier of all blocks between them (a cooperative
 // launch) that alternate the buffers; !RUN: one step (the loop costs 0.5 % of a step's time,
 // more than a launch does on lattices of 2^26 nodes and beyond).  sync: as launch_step_run.
-template <int Q, bool FLIP, int ROWS, int NPT, int THREADS, int MINB, bool RES, bool RUN>
-__global__ void __launch_bounds__(THREADS, MINB)
+template <int Q, bool FLIP, int ROWS, int NPT, int THREADS, bool RUN>
+__global__ void __launch_bounds__(THREADS, 1)
     step_warp_kernel(const __grid_constant__ StepArgs a, uint16_t* buf0, uint16_t* buf1, uint32_t t0, uint32_t T,
                      unsigned long long* fail, unsigned long long* sync) {
   extern __shared__ uint4 smem4[];
@@ -424,9 +346,9 @@ __global__ void __launch_bounds__(THREADS, MINB)
   }
   __syncthreads();
   if (stop) return;
-  const uint2* to = reinterpret_cast<const uint2*>(smem4);
-  const uint2* tr = to + ROWS * kDevAliasCols;
-  const uint2* ta = tr + ROWS * kDevAliasCols;  // D2Q9 only
+  const uint32_t* const tables = reinterpret_cast<const uint32_t*>(smem4);
+  const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(smem4));
+  const FastTables tab{base, base + ROWS * kDevAliasCols * 8, base + 2 * ROWS * kDevAliasCols * 8};
 
   constexpr unsigned kFull = 0xFFFFFFFFu;
   constexpr int H = NPT / 2;  // words per vector
@@ -436,10 +358,6 @@ __global__ void __launch_bounds__(THREADS, MINB)
   const uint32_t lane = threadIdx.x & 31u;
   // this warp's two tile buffers (Q planes of 32 vectors each) after the tables
   VN<NPT>* tbuf = reinterpret_cast<VN<NPT>*>(smem4 + kTables * kRow4) + (threadIdx.x >> 5) * (2 * Q * 32);
-  // this lane's slot of the warp's scratch for the general collision's results (after
-  // all tile buffers)
-  VN<NPT>* const scratch = reinterpret_cast<VN<NPT>*>(smem4 + kTables * kRow4) + (THREADS / 32) * (2 * Q * 32) +
-                           (threadIdx.x >> 5) * (Q * 32) + lane;
   for (uint32_t step = 0;; ++step) {
   const uint32_t t = t0 + step;
   const uint16_t* const __restrict__ in = RUN && (step & 1) ? buf1 : buf0;
@@ -465,7 +383,7 @@ __global__ void __launch_bounds__(THREADS, MINB)
   segment_at(g, end, vpr, y, v0, v1);
   uint32_t vb = v0;
   int buf = 0;
-  stage_tile<Q, FLIP, NPT>(tbuf, in, plane, size_t(y) * Lx, vb + lane, vb + lane < v1, lane);
+  stage_tile<Q, NPT>(tbuf, in, plane, size_t(y) * Lx, vb + lane, vb + lane < v1, lane);
   uint32_t carry[Q];   // +x planes: the value of the previous tile's lane 31
   VN<NPT> held[Q];     // -x planes, lane 31: the vector waiting for the next tile's first node
 #pragma unroll
@@ -492,25 +410,17 @@ __global__ void __launch_bounds__(THREADS, MINB)
       segment_at(g_next, end, vpr, ny, nv0, nv1);
       nvb = nv0;
     }
-    stage_tile<Q, FLIP, NPT>(tbuf + (buf ^ 1) * (Q * 32), in, plane, size_t(ny) * Lx, nvb + lane,
-                             more && nvb + lane < nv1, lane);
+    stage_tile<Q, NPT>(tbuf + (buf ^ 1) * (Q * 32), in, plane, size_t(ny) * Lx, nvb + lane, more && nvb + lane < nv1, lane);
     cp_async_wait_prior();
+    VN<NPT>* const slot = tbuf + buf * (Q * 32) + lane;
     const uint32_t v = vb + lane;
     const bool active = v < v1;
     const uint32_t x0 = v * NPT;
     VN<NPT> P[Q];
-    if constexpr (RES) {
-      VN<NPT>* const slot = tbuf + buf * (Q * 32) + lane;
-      collide_vec_res<Q, ROWS, NPT>(a, keys, to, tr, ta, uint32_t(size_t(y) * Lx) + x0, t, slot, bad);
+    VN<NPT> cur[Q];
 #pragma unroll
-      for (int i = 0; i < Q; ++i) P[i] = slot[32 * i];
-    } else {
-      VN<NPT> cur[Q];
-#pragma unroll
-      for (int i = 0; i < Q; ++i) cur[i] = tbuf[buf * (Q * 32) + i * 32 + lane];
-      collide_vec<Q, ROWS, NPT>(a, keys, to, tr, ta, uint32_t(size_t(y) * Lx) + x0, t, cur, P,
-                                tbuf + buf * (Q * 32) + lane, scratch, bad);
-    }
+    for (int i = 0; i < Q; ++i) cur[i] = slot[32 * source_plane<FLIP>(i)];
+    collide_vec<Q, FLIP, ROWS, NPT>(a, keys, tables, tab, uint32_t(size_t(y) * Lx) + x0, t, cur, P, slot, bad);
     const uint32_t yp = y + 1 == Ly ? 0 : y + 1;
     const uint32_t ym = y == 0 ? Ly - 1 : y - 1;
     // streaming: velocity i lands in row y + dy of its plane, shifted by dx within it
@@ -638,10 +548,9 @@ __global__ void __launch_bounds__(THREADS, MINB)
 // Shapes (the autotuner's two candidates): one block per SM, so the 64 staged table
 // rows exist once per SM; kNpt nodes per lane, kThreads threads, a multiple of 128 so
 // that the four sub-partitions of an SM hold equally many warps.  Few warps with room
-// for all their registers beat more warps that spill (measured on the 16384^2 D2Q5
-// lattice: 8 nodes per lane, 12 warps at up to 168 registers each, 158 G node
-// updates/s; 8 nodes per lane in 16 warps at 128 registers (spills), 153; 4 nodes per
-// lane, 20 warps at up to 96 registers, 142).
+// for all their registers (16384^2 D2Q5, 8 nodes per lane, G node updates/s: 12 warps at up
+// to 168 registers 162, 16 at 128 158.7, 20 at 96 157.2, all without spills; the pipes are as
+// full in each, and more warps stage and stream beside one another).
 constexpr int kRows = 64;
 template <int SHAPE>
 struct WarpShape;
@@ -649,52 +558,41 @@ template <>
 struct WarpShape<0> {
   static constexpr int kNpt = 8;
   static constexpr int kThreads = 384;
-  static constexpr int kBlocks = 1;
-  static constexpr bool kRes = false;
 };
 template <>
 struct WarpShape<1> {
   static constexpr int kNpt = 4;
   static constexpr int kThreads = 640;
-  static constexpr int kBlocks = 1;
-  static constexpr bool kRes = false;
 };
 
-// D2Q9 (nine planes, four Philox blocks and eleven draws per node): 4 nodes per lane
-// left in shared memory and collided two at a time (nine planes of vectors in
-// registers would cost 36 of them), 512 or 640 threads (measured on the 16384^2
-// lattice: 72.6 and 68.9 G node updates/s; with the vectors in registers, 512
-// threads: 62.9 before the launch-wide Philox rounds were split off)
+// D2Q9 (nine planes, four Philox blocks and eleven draws per node): 4 nodes per lane, 384 or
+// 512 threads (8192^2: 77.4 and 77.0 G node updates/s; 640, at 96 registers, spill: 59; 8 nodes
+// per lane in 384 threads 70)
 template <int Q, int SHAPE>
 struct WarpShapeQ : WarpShape<SHAPE> {};
 template <>
 struct WarpShapeQ<9, 0> {
   static constexpr int kNpt = 4;
-  static constexpr int kThreads = 512;
-  static constexpr int kBlocks = 1;
-  static constexpr bool kRes = true;
+  static constexpr int kThreads = 384;
 };
 template <>
 struct WarpShapeQ<9, 1> {
   static constexpr int kNpt = 4;
-  static constexpr int kThreads = 640;
-  static constexpr int kBlocks = 1;
-  static constexpr bool kRes = true;
+  static constexpr int kThreads = 512;
 };
 
-// tables, then two tile buffers of Q planes x 32 vectors per warp, then (vectors in
-// registers only) one scratch buffer of the same shape per warp
+// tables, then two tile buffers of Q planes x 32 vectors per warp
 template <int Q, int SHAPE>
 constexpr size_t warp_smem() {
   using S = WarpShapeQ<Q, SHAPE>;
   return sizeof(uint2) * (Q == 9 ? 3 : 2) * kRows * kDevAliasCols +
-         size_t(S::kThreads / 32) * (S::kRes ? 2 : 3) * Q * 32 * (2 * S::kNpt);
+         size_t(S::kThreads / 32) * 2 * Q * 32 * (2 * S::kNpt);
 }
 
 template <int Q, bool FLIP, int SHAPE, bool RUN>
 const void* warp_kernel() {
   using S = WarpShapeQ<Q, SHAPE>;
-  return reinterpret_cast<const void*>(step_warp_kernel<Q, FLIP, kRows, S::kNpt, S::kThreads, S::kBlocks, S::kRes, RUN>);
+  return reinterpret_cast<const void*>(step_warp_kernel<Q, FLIP, kRows, S::kNpt, S::kThreads, RUN>);
 }
 
 template <int Q, int SHAPE>
@@ -728,21 +626,19 @@ cudaError_t warp_launch(const StepArgs& a, uint16_t* buf0, uint16_t* buf1, uint3
 }
 
 template <int Q>
-void shape_of(int shape, uint32_t* npt, uint32_t* threads, uint32_t* per_sm) {
+void shape_of(int shape, uint32_t* npt, uint32_t* threads) {
   if (shape == 1) {
     *npt = WarpShapeQ<Q, 1>::kNpt;
     *threads = WarpShapeQ<Q, 1>::kThreads;
-    *per_sm = WarpShapeQ<Q, 1>::kBlocks;
   } else {
     *npt = WarpShapeQ<Q, 0>::kNpt;
     *threads = WarpShapeQ<Q, 0>::kThreads;
-    *per_sm = WarpShapeQ<Q, 0>::kBlocks;
   }
 }
 
-void shape_of(int Q, int shape, uint32_t* npt, uint32_t* threads, uint32_t* per_sm) {
-  if (Q == 9) shape_of<9>(shape, npt, threads, per_sm);
-  else shape_of<5>(shape, npt, threads, per_sm);
+void shape_of(int Q, int shape, uint32_t* npt, uint32_t* threads) {
+  if (Q == 9) shape_of<9>(shape, npt, threads);
+  else shape_of<5>(shape, npt, threads);
 }
 
 }  // namespace
@@ -758,16 +654,16 @@ cudaError_t prepare_step_warp_kernels(int Q) {
 }
 
 uint32_t step_warp_width(int Q, int shape) {
-  uint32_t npt, threads, per_sm;
-  shape_of(Q, shape, &npt, &threads, &per_sm);
+  uint32_t npt, threads;
+  shape_of(Q, shape, &npt, &threads);
   return npt;
 }
 
 // Blocks of a launch: one per SM, or fewer on lattices too small to give each warp a tile.
 static uint32_t step_warp_grid(int Q, uint32_t Lx, uint32_t Ly, uint32_t sms, int shape) {
-  uint32_t npt, threads, per_sm;
-  shape_of(Q, shape, &npt, &threads, &per_sm);
-  const uint64_t cap = uint64_t(sms) * per_sm;
+  uint32_t npt, threads;
+  shape_of(Q, shape, &npt, &threads);
+  const uint64_t cap = sms;
   const uint64_t warps = std::max<uint64_t>(1, uint64_t(Lx / npt) * Ly / 32);
   return uint32_t(std::min<uint64_t>(cap, (warps + threads / 32 - 1) / (threads / 32)));
 }
