@@ -8,9 +8,9 @@
 // So, per opposite pair (i, -i) with weight w_m and per rest velocity,
 //   post_i  = omega w_m rho + a1 f_i + a2 f_-i,  a1,2 = ((1 - omega) +- (1 - omega^j)) / 2
 //   post_0  = omega w_0 rho + (1 - omega) f_0
-// (9 fused multiply-adds per D2Q5 node, 5 per D1Q3 node, and the density with its products,
-// formed in integers), then push-streaming to x + v_i.  No moment matrix appears; the
-// oracle uses the matrix.
+// then push-streaming to x + v_i.  It is computed in 64-bit integers (relax_fixed), where a
+// node's values are of like size, and in double precision elsewhere.  No moment matrix appears;
+// the oracle uses the matrix.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -34,42 +34,51 @@ constexpr uint32_t kLbFirstModes = 64; // passed as a kernel argument
 constexpr uint32_t kLbRowChunk = 64;   // rows per partial column sum
 constexpr uint32_t kLbChunk = 4096;    // entries per partial of a projection
 
+// The kernels read the planes of a pair (i, -i) exchanged where swap is set (1 - omega^j < 0):
+// with the signs of a1's and a2's odd parts the odd part of f - f^0 then relaxes with
+// |1 - omega^j|.
 struct LbCoef {
   double cr;   // omega w_0
   double cm;   // omega w_m (moving, D2Q9: axis)
   double cd;   // D2Q9: omega w_diagonal
   double l2;   // 1 - omega
-  double a1;   // ((1 - omega) + (1 - omega^j)) / 2
-  double a2;   // ((1 - omega) - (1 - omega^j)) / 2
-  // cr, cm, cd as integers: m 2^e with the top bit of m set; whole: all of them are (positive
-  // and of ordinary size), so that their products with rho may be formed in integers
-  unsigned long long mr, mm, md;
-  int er, em, ed;
-  int whole;
+  double a1;   // ((1 - omega) + |1 - omega^j|) / 2
+  double a2;   // ((1 - omega) - |1 - omega^j|) / 2
+  // times 2^64: omega w_0 / 2, omega w_m, omega w_diagonal, |1 - omega| / 2, |1 - omega^j| / 2
+  unsigned long long hr, hm, hd, he, ho;
+  // what relax_fixed adds to the products with rho, and takes from those with a pair's difference
+  unsigned long long more, less;
+  int minus;   // 1 - omega < 0
+  int swap;    // 1 - omega^j < 0
 };
 
-// ---- double-precision sums and products on the integer pipes ----
-// An SM has two fp64 lanes and 128 integer lanes, so the density sum and its products with
-// the equilibrium weights (six of a D2Q5 node's fifteen fp64 operations) are formed in
-// integers; the other nine, all fused multiply-adds, stay on the fp64 pipe, which bounds the
-// step.  D2Q5 16384^2 7.72 -> 4.93 ms (0.78 of the fp64 rate of the nine, 0.64 of HBM),
-// 1024^2 34.9 -> 22.0 us per step; D2Q9 1024^2 63.6 -> 40.3.
+// ---- the relaxation on the integer pipes ----
+// An SM has two fp64 lanes: a warp's fp64 operation takes 64 cycles of its sub-partition, and
+// a D2Q5 node has 15 of them (9 with the density and its products in integers).  A 64-bit
+// integer sum takes two instructions and the upper half of a 64-bit product five, so the
+// whole node is relaxed in fixed point: the values shifted to the largest one's exponent
+// (exact), sums exact, products to two units of 2^-61 of the largest value, and each result
+// rounded once to 53 bits (the fp64 form rounds it three times).  A D2Q5 node takes 278 warp
+// instructions per 32 nodes.  Us per step against nine fp64 operations per node with the
+// density's sums and products in integers: D2Q5 1024^2 13.9 / 22.0 (the barrier, the loads'
+// latency and the ALU pipe), 4096^2 222 / 317 (0.89 of the measured copy bandwidth), 16384^2
+// 3.69 / 4.94 ms (0.85); D2Q9 1024^2 25.7 / 40.5.  Error after 200 steps of a sine against
+// extended precision: D2Q5 5e-16 / 1.2e-14 of a value at the rates (1.8, 0.2).
 
-// S (not 0, its top bit at least 2^53) rounded to 53 bits, ties to even: returns them (2^52 to
-// 2^53) and how many bits were dropped.
-__device__ __forceinline__ unsigned long long round53(unsigned long long S, int& dropped) {
-  const int p = 11 - __clzll(static_cast<long long>(S));
-  dropped = p;
-  S += (1ull << (p - 1)) - 1ull + ((S >> p) & 1ull);
-  return S >> p;
+// The upper half of a 128-bit product less 0 to 2 units, 1.25 on average.
+__device__ __forceinline__ unsigned long long upper_product(unsigned long long a, unsigned long long b) {
+  const uint32_t a0 = uint32_t(a), a1 = uint32_t(a >> 32), b0 = uint32_t(b), b1 = uint32_t(b >> 32);
+  return static_cast<unsigned long long>(a1) * b1 + __umulhi(a0, b1) + __umulhi(a1, b0);
 }
 
-// The sum of Q doubles as M 2^E, rounded once (round to nearest even): exact shifts to the
-// largest exponent and one 64-bit integer sum.  False (and nothing else) unless all are
-// positive, of ordinary size, and within 2^kRoom of one another.
-template <int Q>
-__device__ __forceinline__ bool whole_sum(const double (&f)[Q], unsigned long long& M, int& E) {
+// False (and nothing else) unless all values are positive, of ordinary size and within 2^kRoom
+// of one another, and the results between some 2^-5 of the largest value and four times it.
+// MINUS: 1 - omega < 0.
+template <int Q, bool MINUS>
+__device__ __forceinline__ bool relax_fixed(const LbCoef& k, const double (&f)[Q], double (&post)[Q]) {
+  using u64 = unsigned long long;
   constexpr int kRoom = Q == 3 ? 9 : (Q == 5 ? 8 : 7);  // Q 2^(53 + kRoom) < 2^64
+  constexpr uint32_t kLeast = Q == 9 ? 1u << 22 : 1u << 24;  // times 2^32: a result's least size
   int e[Q], top = 0, low = 1 << 20;
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
@@ -78,32 +87,60 @@ __device__ __forceinline__ bool whole_sum(const double (&f)[Q], unsigned long lo
     low = min(low, e[i]);
   }
   if (low < 64 || top > 1980 || top - low > kRoom) return false;
-  unsigned long long S = 0;
+  u64 F[Q], rho = 0, V[Q];
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
     const uint32_t hi = (uint32_t(__double2hiint(f[i])) & 0xFFFFFu) | 0x100000u;
-    S += ((static_cast<unsigned long long>(hi) << 32) | uint32_t(__double2loint(f[i]))) << (kRoom - top + e[i]);
+    F[i] = ((u64(hi) << 32) | uint32_t(__double2loint(f[i]))) << (kRoom - top + e[i]);
+    rho += F[i];
   }
-  int p;
-  M = round53(S, p);
-  E = top - 1075 - kRoom + p;
+  const auto even = [&](u64 c, u64 s) { return MINUS ? c - s : c + s; };
+  const u64 half = even(upper_product(rho, k.hr) + k.more, upper_product(F[0], k.he));
+  V[0] = 2 * half;
+  u64 c = upper_product(rho, k.hm) + k.more;
+#pragma unroll
+  for (int i = 1; i < Q; i += 2) {
+    if (Q == 9 && i == 5) c = upper_product(rho, k.hd) + k.more;
+    const u64 B = even(c, upper_product(F[i] + F[i + 1], k.he));
+    // (f_i - f_-i) |1 - omega^j| / 2 from the difference plus 2^62
+    const u64 t = upper_product(F[i] - F[i + 1] + (1ull << 62), k.ho) - k.less;
+    V[i] = B + t;
+    V[i + 1] = B - t;
+  }
+  // (no sum reaches 2^64 but twice `half`; a negative result passes any limit)
+  uint32_t least = uint32_t(V[0] >> 32), most = 0;
+#pragma unroll
+  for (int i = 1; i < Q; ++i) {
+    least = min(least, uint32_t(V[i] >> 32));
+    most = max(most, uint32_t(V[i] >> 32));
+  }
+  if (least < kLeast || most >= (1u << 31) || uint32_t(half >> 32) >= (1u << 30)) return false;
+  const uint32_t scale = uint32_t(top - kRoom - 1) << 20;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    // p >= 2 bits dropped, half a unit rounded up
+    const uint32_t p = 11 - __clz(int(V[i] >> 32));
+    const u64 r = V[i] + (1u << (p - 1));
+    const uint32_t lo = __funnelshift_r(uint32_t(r), uint32_t(r >> 32), p);
+    const uint32_t hi = (uint32_t(r >> 32) >> p) + scale + (p << 20);
+    post[i] = __hiloint2double(int(hi), int(lo));
+  }
   return true;
 }
 
-// (M 2^E)(m 2^e) as a double, rounded once: the 128-bit product, its low half folded into a
-// sticky bit.  M at most 2^53, m with its top bit set.
-__device__ __forceinline__ double whole_product(unsigned long long M, int E, unsigned long long m, int e) {
-  const unsigned long long a = M << 10;
-  const uint32_t a0 = uint32_t(a), a1 = uint32_t(a >> 32), b0 = uint32_t(m), b1 = uint32_t(m >> 32);
-  const unsigned long long p00 = static_cast<unsigned long long>(a0) * b0;
-  const unsigned long long p01 = static_cast<unsigned long long>(a0) * b1 + (p00 >> 32);
-  const unsigned long long p10 = static_cast<unsigned long long>(a1) * b0 + uint32_t(p01);
-  unsigned long long S = static_cast<unsigned long long>(a1) * b1 + (p01 >> 32) + (p10 >> 32);
-  if ((uint32_t(p00) | uint32_t(p10)) != 0u) S |= 1ull;
-  int p;
-  const unsigned long long r = round53(S, p);
-  const unsigned long long bits = (static_cast<unsigned long long>(E + e + 54 + p + 1074) << 52) + r;
-  return __longlong_as_double(static_cast<long long>(bits));
+template <int Q>
+__device__ __forceinline__ void relax(const LbCoef& k, const double (&f)[Q], double (&post)[Q]) {
+  if (k.minus ? relax_fixed<Q, true>(k, f, post) : relax_fixed<Q, false>(k, f, post)) return;
+  double rho = f[0] + f[1] + f[2];
+  if constexpr (Q >= 5) rho = rho + f[3] + f[4];
+  if constexpr (Q == 9) rho = rho + f[5] + f[6] + f[7] + f[8];
+  post[0] = fma(k.l2, f[0], k.cr * rho);
+#pragma unroll
+  for (int i = 1; i < Q; i += 2) {
+    const double c = (Q == 9 && i >= 5 ? k.cd : k.cm) * rho;
+    post[i] = fma(k.a1, f[i], fma(k.a2, f[i + 1], c));
+    post[i + 1] = fma(k.a1, f[i + 1], fma(k.a2, f[i], c));
+  }
 }
 
 // T steps, one node per thread: load the Q planes, relax, push.  f0 holds the state, the
@@ -128,44 +165,33 @@ __global__ void __launch_bounds__(kLbThreads, 4)
     const double* const in = (step & 1) ? f1 : f0;
     double* const out = (step & 1) ? f0 : f1;
     uint32_t x = x0, y = y0, node = first;
+    const double* from[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) from[i] = in + (i == 0 || !k.swap ? i : (i & 1 ? i + 1 : i - 1)) * plane;
     while (node < nodes) {
-      double f[Q];
+      double f[Q], post[Q];
       // (through L2 only: another SM wrote these lines in the step before)
 #pragma unroll
-      for (int i = 0; i < Q; ++i) f[i] = __ldcg(in + (i * plane + node));
-      double c, cr, cd = 0.0;
-      unsigned long long M;
-      int E;
-      if (k.whole && whole_sum<Q>(f, M, E)) {
-        c = whole_product(M, E, k.mm, k.em);
-        cr = whole_product(M, E, k.mr, k.er);
-        if constexpr (Q == 9) cd = whole_product(M, E, k.md, k.ed);
-      } else {
-        double rho = f[0] + f[1] + f[2];
-        if constexpr (Q >= 5) rho = rho + f[3] + f[4];
-        if constexpr (Q == 9) rho = rho + f[5] + f[6] + f[7] + f[8];
-        c = k.cm * rho;
-        cr = k.cr * rho;
-        if constexpr (Q == 9) cd = k.cd * rho;
-      }
+      for (int i = 0; i < Q; ++i) f[i] = __ldcg(from[i] + node);
+      relax<Q>(k, f, post);
       const uint32_t yp = y + 1 == Ly ? 0 : y + 1;
       const uint32_t ym = y == 0 ? Ly - 1 : y - 1;
       double* const o = out + node;  // row y starts at node - x
       const int64_t right = x + 1 == Lx ? -int64_t(x) : 1, left = x == 0 ? int64_t(Lx) - 1 : -1;
-      o[0] = fma(k.l2, f[0], cr);
-      o[int64_t(plane) + right] = fma(k.a1, f[1], fma(k.a2, f[2], c));
-      o[int64_t(2 * plane) + left] = fma(k.a1, f[2], fma(k.a2, f[1], c));
+      o[0] = post[0];
+      o[int64_t(plane) + right] = post[1];
+      o[int64_t(2 * plane) + left] = post[2];
       if constexpr (Q >= 5) {
         double* const up = out + (size_t(yp) * Lx + x);
         double* const down = out + (size_t(ym) * Lx + x);
-        up[3 * plane] = fma(k.a1, f[3], fma(k.a2, f[4], c));
-        down[4 * plane] = fma(k.a1, f[4], fma(k.a2, f[3], c));
+        up[3 * plane] = post[3];
+        down[4 * plane] = post[4];
         if constexpr (Q == 9) {
           // diagonal pairs (+1,+1)/(-1,-1) and (+1,-1)/(-1,+1)
-          up[int64_t(5 * plane) + right] = fma(k.a1, f[5], fma(k.a2, f[6], cd));
-          down[int64_t(6 * plane) + left] = fma(k.a1, f[6], fma(k.a2, f[5], cd));
-          down[int64_t(7 * plane) + right] = fma(k.a1, f[7], fma(k.a2, f[8], cd));
-          up[int64_t(8 * plane) + left] = fma(k.a1, f[8], fma(k.a2, f[7], cd));
+          up[int64_t(5 * plane) + right] = post[5];
+          down[int64_t(6 * plane) + left] = post[6];
+          down[int64_t(7 * plane) + right] = post[7];
+          up[int64_t(8 * plane) + left] = post[8];
         }
       }
       if (nodes - node <= stride) break;  // (node + stride may pass 2^32)
@@ -568,15 +594,8 @@ const void* lb_col_fn(int Q, bool wide) {
                   : reinterpret_cast<const void*>(lb_col_kernel<9, kLbCols>);
 }
 
-// v = m 2^e with the top bit of m set; false unless v is positive and of ordinary size
-bool as_integer(double v, unsigned long long* m, int* e) {
-  if (!(v >= 1e-15 && v <= 1e3)) return false;
-  int x = 0;
-  const double f = std::frexp(v, &x);  // [1/2, 1)
-  *m = static_cast<unsigned long long>(std::ldexp(f, 53)) << 11;
-  *e = x - 64;
-  return true;
-}
+// v 2^bits, v not negative and the result below 2^65: exact but for bits below 1
+unsigned __int128 scaled(double v, int bits) { return static_cast<unsigned __int128>(std::ldexp(v, bits)); }
 
 // A bounded wait between the blocks of a several-step launch gave up (read back with the
 // results): the buffers hold parts of different steps.
@@ -611,16 +630,30 @@ ilg_status ilg_lb_create(const ilg_lb_params* params, void* stream, ilg_lb** out
   b->stream = static_cast<cudaStream_t>(stream);
   double w[9];
   ilg::weights(p.lattice, p.theta, w);
-  const double l2 = 1.0 - p.omega, lj = 1.0 - p.omega_j;
-  b->coef = LbCoef{};
-  b->coef.cr = p.omega * w[0];
-  b->coef.cm = p.omega * w[1];
-  b->coef.cd = b->Q == 9 ? p.omega * w[5] : 0.0;
-  b->coef.l2 = l2;
-  b->coef.a1 = 0.5 * (l2 + lj);
-  b->coef.a2 = 0.5 * (l2 - lj);
-  b->coef.whole = as_integer(b->coef.cr, &b->coef.mr, &b->coef.er) && as_integer(b->coef.cm, &b->coef.mm, &b->coef.em) &&
-                  (b->Q != 9 || as_integer(b->coef.cd, &b->coef.md, &b->coef.ed));
+  LbCoef& k = b->coef;
+  k = LbCoef{};
+  k.minus = p.omega > 1.0;
+  k.swap = p.omega_j > 1.0;
+  const double lj = k.swap ? p.omega_j - 1.0 : 1.0 - p.omega_j;
+  k.cr = p.omega * w[0];
+  k.cm = p.omega * w[1];
+  k.cd = b->Q == 9 ? p.omega * w[5] : 0.0;
+  k.l2 = 1.0 - p.omega;
+  k.a1 = 0.5 * (k.l2 + lj);
+  k.a2 = 0.5 * (k.l2 - lj);
+  // the same weights and rates in fixed point, exact but for the last bit of the products
+  using u128 = unsigned __int128;
+  const u128 half = scaled(p.omega, 63), one = u128(1) << 63;
+  k.hr = static_cast<unsigned long long>((half * scaled(w[0], 64)) >> 64);
+  k.hm = static_cast<unsigned long long>((half * scaled(w[1], 64)) >> 63);
+  k.hd = b->Q == 9 ? static_cast<unsigned long long>((half * scaled(w[5], 64)) >> 63) : 0ull;
+  k.he = static_cast<unsigned long long>(k.minus ? half - one : one - half);
+  const u128 hj = scaled(p.omega_j, 63);
+  k.ho = static_cast<unsigned long long>(k.swap ? hj - one : one - hj) & ~3ull;  // its product with 2^62 is whole
+  // a product with a factor lacks about one unit
+  const unsigned long long lacks = k.he != 0, odd = k.ho != 0;
+  k.more = (k.hm != 0) + (k.minus ? 0 - lacks : lacks);
+  k.less = (k.ho >> 2) - odd;
   b->chunks = (b->Ly + kLbRowChunk - 1) / kLbRowChunk;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
