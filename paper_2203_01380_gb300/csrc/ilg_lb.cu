@@ -25,6 +25,9 @@
 namespace {
 
 constexpr int kLbThreads = 256;
+// threads of a step kernel's block: four blocks per SM, or (wide) one, whose loads run ahead and
+// need the registers (D2Q5 1024^2, us per step: 1024 threads 13.3, 768 12.4, 512 12.6)
+__host__ __device__ constexpr int lb_run_threads(int Q, bool wide) { return !wide ? 256 : (Q == 9 ? 512 : 768); }
 constexpr uint32_t kLbMaxModes = 256;
 constexpr int kLbModeThreads = 64;     // of a projection's blocks
 constexpr int kLbClusterBlocks = 16;   // (beyond 8 a kernel opts in)
@@ -60,9 +63,9 @@ struct LbCoef {
 // (exact), sums exact, products to two units of 2^-61 of the largest value, and each result
 // rounded once to 53 bits (the fp64 form rounds it three times).  A D2Q5 node takes 278 warp
 // instructions per 32 nodes.  Us per step against nine fp64 operations per node with the
-// density's sums and products in integers: D2Q5 1024^2 13.9 / 22.0 (the barrier, the loads'
-// latency and the ALU pipe), 4096^2 222 / 317 (0.89 of the measured copy bandwidth), 16384^2
-// 3.69 / 4.94 ms (0.85); D2Q9 1024^2 25.7 / 40.5.  Error after 200 steps of a sine against
+// density's sums and products in integers: D2Q5 1024^2 12.3 / 22.0 (the barrier, the loads'
+// latency and the ALU pipe), 4096^2 215 / 317 (0.92 of the measured copy bandwidth), 16384^2
+// 3.57 / 4.94 ms (0.88); D2Q9 1024^2 25.5 / 40.5.  Error after 200 steps of a sine against
 // extended precision: D2Q5 5e-16 / 1.2e-14 of a value at the rates (1.8, 0.2).
 
 // The upper half of a 128-bit product less 0 to 2 units, 1.25 on average.
@@ -149,15 +152,15 @@ __device__ __forceinline__ void relax(const LbCoef& k, const double (&f)[Q], dou
 // (at most kLbClusterBlocks blocks, a node per thread) and its barrier the cluster's.  Us per
 // step, grid barrier / cluster: 500 nodes of D1Q3 2.0 / 1.3, D2Q5 64^2 2.5 / 2.1, D2Q9 56 x 66
 // 3.4 / 3.0 (one launch per step: 4.1).
-template <int Q, bool CLUSTER>
-__global__ void __launch_bounds__(kLbThreads, 4)
+template <int Q, bool CLUSTER, bool WIDE>
+__global__ void __launch_bounds__(lb_run_threads(Q, WIDE), WIDE ? 1 : 4)
     lb_run_kernel(const __grid_constant__ LbCoef k, double* f0, double* f1, uint32_t Lx, uint32_t Ly, uint32_t T,
                   unsigned long long* sync) {
   __shared__ int stop;
   if (threadIdx.x == 0) stop = 0;
   const uint32_t nodes = Lx * Ly;
   const size_t plane = nodes;
-  const uint32_t threads = CLUSTER ? blockDim.x : uint32_t(kLbThreads);
+  const uint32_t threads = CLUSTER ? blockDim.x : uint32_t(lb_run_threads(Q, WIDE));
   const uint32_t stride = gridDim.x * threads, stride_y = stride / Lx, stride_x = stride - stride_y * Lx;
   const uint32_t first = blockIdx.x * threads + threadIdx.x;
   const uint32_t y0 = first / Lx, x0 = first - y0 * Lx;
@@ -168,11 +171,19 @@ __global__ void __launch_bounds__(kLbThreads, 4)
     const double* from[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) from[i] = in + (i == 0 || !k.swap ? i : (i & 1 ? i + 1 : i - 1)) * plane;
+    // (through L2 only: another SM wrote these lines in the step before)
+    double next[Q];
+    const auto load = [&](uint32_t at) {
+#pragma unroll
+      for (int i = 0; i < Q; ++i) next[i] = __ldcg(from[i] + at);
+    };
+    if (WIDE && node < nodes) load(node);
     while (node < nodes) {
       double f[Q], post[Q];
-      // (through L2 only: another SM wrote these lines in the step before)
+      if (!WIDE) load(node);
 #pragma unroll
-      for (int i = 0; i < Q; ++i) f[i] = __ldcg(from[i] + node);
+      for (int i = 0; i < Q; ++i) f[i] = next[i];
+      if (WIDE && nodes - node > stride) load(node + stride);
       relax<Q>(k, f, post);
       const uint32_t yp = y + 1 == Ly ? 0 : y + 1;
       const uint32_t ym = y == 0 ? Ly - 1 : y - 1;
@@ -551,15 +562,21 @@ int lb_grid(const ilg_lb* b) {
   return int(blocks < cap ? blocks : cap);
 }
 
-const void* lb_run_fn(int Q, bool cluster = false) {
-  if (cluster)
-    return Q == 3   ? reinterpret_cast<const void*>(lb_run_kernel<3, true>)
-           : Q == 5 ? reinterpret_cast<const void*>(lb_run_kernel<5, true>)
-                    : reinterpret_cast<const void*>(lb_run_kernel<9, true>);
-  return Q == 3   ? reinterpret_cast<const void*>(lb_run_kernel<3, false>)
-         : Q == 5 ? reinterpret_cast<const void*>(lb_run_kernel<5, false>)
-                  : reinterpret_cast<const void*>(lb_run_kernel<9, false>);
+template <bool CLUSTER, bool WIDE>
+const void* lb_run_of(int Q) {
+  return Q == 3   ? reinterpret_cast<const void*>(lb_run_kernel<3, CLUSTER, WIDE>)
+         : Q == 5 ? reinterpret_cast<const void*>(lb_run_kernel<5, CLUSTER, WIDE>)
+                  : reinterpret_cast<const void*>(lb_run_kernel<9, CLUSTER, WIDE>);
 }
+
+// Lattices of more nodes than this per SM: one wide block per SM, its threads' next values
+// loaded while the present ones relax.  Us per step, narrow / wide: D2Q5 350^2 3.85 / 4.09,
+// 400^2 5.08 / 4.25, 700^2 8.57 / 7.71, 1024^2 13.9 / 12.3; D1Q3 2^20 9.80 / 8.33; D2Q9 700^2
+// 13.6 / 11.5.
+constexpr size_t kLbWideNodesPerSm = 1024;
+bool lb_wide(const ilg_lb* b) { return b->nodes > kLbWideNodesPerSm * b->sms; }
+int lb_threads(const ilg_lb* b) { return lb_run_threads(b->Q, lb_wide(b)); }
+const void* lb_run_fn(const ilg_lb* b) { return lb_wide(b) ? lb_run_of<false, true>(b->Q) : lb_run_of<false, false>(b->Q); }
 
 bool lb_fits_cluster(const ilg_lb* b) { return b->nodes <= size_t(kLbClusterBlocks) * kLbThreads; }
 
@@ -579,7 +596,7 @@ bool lb_launch_cluster(const ilg_lb* b, void** args) {
   cfg.stream = b->stream;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  if (cudaLaunchKernelExC(&cfg, lb_run_fn(b->Q, true), args) == cudaSuccess) return true;
+  if (cudaLaunchKernelExC(&cfg, lb_run_of<true, false>(b->Q), args) == cudaSuccess) return true;
   cudaGetLastError();
   return false;
 }
@@ -678,14 +695,14 @@ ilg_status ilg_lb_create(const ilg_lb_params* params, void* stream, ilg_lb** out
     e = cudaMemsetAsync(b->d_sync, 0, sizeof(unsigned long long) * clear, b->stream);
   }
   int per_sm = 0;
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lb_run_fn(b->Q), kLbThreads, 0);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lb_run_fn(b), lb_threads(b), 0);
   if (e == cudaSuccess && lb_fits_cluster(b))
-    e = cudaFuncSetAttribute(lb_run_fn(b->Q, true), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    e = cudaFuncSetAttribute(lb_run_of<true, false>(b->Q), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) {
     ilg_lb_destroy(b);
     return lb_cuda_fail(nullptr, e, "ilg_lb_create");
   }
-  b->run_blocks = int(std::min<size_t>(size_t(per_sm) * b->sms, (b->nodes + kLbThreads - 1) / kLbThreads));
+  b->run_blocks = int(std::min<size_t>(size_t(per_sm) * b->sms, (b->nodes + lb_threads(b) - 1) / lb_threads(b)));
   *out = b;
   return ILG_OK;
 }
@@ -790,7 +807,7 @@ ilg_status ilg_lb_step(ilg_lb* b, uint32_t T) {
   if (!b) return ILG_E_INVALID;
   if (!b->has_state) return lb_fail(b, ILG_E_STATE, "no state: call ilg_lb_init or ilg_lb_set_state first");
   constexpr uint32_t kRunSteps = 4096;  // per launch
-  const void* fn = lb_run_fn(b->Q);
+  const void* fn = lb_run_fn(b);
   bool run = true;
   for (uint32_t k = 0; k < T;) {
     uint32_t n = run ? std::min(T - k, kRunSteps) : 1;
@@ -800,7 +817,7 @@ ilg_status ilg_lb_step(ilg_lb* b, uint32_t T) {
       // (no wait that could give up)
     } else if (n > 1) {
       LB_CUDA(b, cudaMemsetAsync(b->d_sync, 0, sizeof(unsigned long long), b->stream), "lattice Boltzmann step");
-      const cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(b->run_blocks), dim3(kLbThreads), args, 0, b->stream);
+      const cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(b->run_blocks), dim3(lb_threads(b)), args, 0, b->stream);
       if (e == cudaErrorCooperativeLaunchTooLarge) {
         // the device cannot hold all blocks at once (SMs reserved elsewhere): step by step
         cudaGetLastError();
@@ -810,7 +827,7 @@ ilg_status ilg_lb_step(ilg_lb* b, uint32_t T) {
       LB_CUDA(b, e, "lattice Boltzmann step");
       b->waits = true;
     } else {
-      LB_CUDA(b, cudaLaunchKernel(fn, dim3(b->run_blocks), dim3(kLbThreads), args, 0, b->stream), "lattice Boltzmann step");
+      LB_CUDA(b, cudaLaunchKernel(fn, dim3(b->run_blocks), dim3(lb_threads(b)), args, 0, b->stream), "lattice Boltzmann step");
     }
     b->cur ^= int(n & 1u);
     b->t += n;
