@@ -35,8 +35,7 @@ __host__ __device__ constexpr uint32_t run_table_words(int Q) { return Q == 9 ? 
 
 // sync[0]: the barrier word, sync[1]: set to 1 when a wait gave up.  TABLES: the binomial
 // sampler with both probabilities strictly between 0 and 1; false: anything else.
-// CLUSTER: the launch is one cluster of blocks and its barrier the cluster's.
-template <int Q, int THREADS, bool TABLES, bool CLUSTER>
+template <int Q, int THREADS, bool TABLES>
 __global__ void __launch_bounds__(THREADS, 1)
     step_run_kernel(const __grid_constant__ StepArgs a, uint16_t* buf0, uint16_t* buf1, uint32_t t0, uint32_t T,
                     unsigned long long* fail, unsigned long long* sync) {
@@ -45,11 +44,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   uint32_t* s = reinterpret_cast<uint32_t*>(smem4);
   // a step before this launch overflowed (one of its own stops it at the barriers: a block that
   // started late must not leave the others waiting there)
-  __shared__ uint32_t mark;  // CLUSTER: the first step of this launch that overflowed
-  if (threadIdx.x == 0) {
-    stop = *reinterpret_cast<volatile unsigned long long*>(fail) < t0;
-    mark = ~0u;
-  }
+  if (threadIdx.x == 0) stop = *reinterpret_cast<volatile unsigned long long*>(fail) < t0;
   constexpr uint32_t kTables = run_table_words(Q);
   // the block's first words: the alias tables, or the particle sampler's boundaries (all
   // copies in flight at once, the first node's words made meanwhile)
@@ -79,11 +74,6 @@ __global__ void __launch_bounds__(THREADS, 1)
   asm volatile("cp.async.wait_all;\n" ::: "memory");
   __syncthreads();
   if (stop) return;
-  if constexpr (CLUSTER) {
-    // the marks are written by other blocks from here on
-    cluster_arrive();
-    cluster_wait();
-  }
   for (uint32_t step = 0;; ++step) {
     const uint32_t t = t0 + step;
     const uint16_t* const in = (step & 1) ? buf1 : buf0;
@@ -145,31 +135,15 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
     if (bad) {
       atomicMin(fail, static_cast<unsigned long long>(t));
-      if constexpr (CLUSTER) {
-        // (in the last step nobody waits for the mark, and a block may have ended)
-        if (step + 1 < T) cluster_mark(&mark, step, gridDim.x);
-      } else {
-        __threadfence();
-        atomicOr(sync, kRunMark);
-      }
+      __threadfence();
+      atomicOr(sync, kRunMark);
     }
     if (step + 1 == T) break;
-    if constexpr (CLUSTER) {
-      __syncwarp();
-      cluster_arrive();
-    } else {
-      __syncthreads();
-      if (threadIdx.x == 0) run_arrive(sync);
-    }
+    __syncthreads();
+    if (threadIdx.x == 0) run_arrive(sync);
     // while the other blocks finish: the next step's words that need nothing of theirs
     keys = word_keys<NB>(a, t + 1);
     if (kAhead && (TABLES || !a.particle)) first.make(keys, a.rk, base0 + lane);
-    if constexpr (CLUSTER) {
-      cluster_wait();
-      // (a faster block may already have marked the next step)
-      if (*reinterpret_cast<volatile uint32_t*>(&mark) <= step) break;
-      continue;
-    }
     if (threadIdx.x == 0) {
       const unsigned long long v = run_wait(sync, (step + 1) * gridDim.x);
       if (v == ~0ull) {
@@ -199,36 +173,147 @@ struct RunShape {
 template <int THREADS>
 static const void* run_fn(int Q, bool tables) {
   if (Q == 3)
-    return tables ? reinterpret_cast<const void*>(step_run_kernel<3, THREADS, true, false>)
-                  : reinterpret_cast<const void*>(step_run_kernel<3, THREADS, false, false>);
+    return tables ? reinterpret_cast<const void*>(step_run_kernel<3, THREADS, true>)
+                  : reinterpret_cast<const void*>(step_run_kernel<3, THREADS, false>);
   if (Q == 5)
-    return tables ? reinterpret_cast<const void*>(step_run_kernel<5, THREADS, true, false>)
-                  : reinterpret_cast<const void*>(step_run_kernel<5, THREADS, false, false>);
+    return tables ? reinterpret_cast<const void*>(step_run_kernel<5, THREADS, true>)
+                  : reinterpret_cast<const void*>(step_run_kernel<5, THREADS, false>);
   if constexpr (THREADS <= 512)
-    return tables ? reinterpret_cast<const void*>(step_run_kernel<9, THREADS, true, false>)
-                  : reinterpret_cast<const void*>(step_run_kernel<9, THREADS, false, false>);
+    return tables ? reinterpret_cast<const void*>(step_run_kernel<9, THREADS, true>)
+                  : reinterpret_cast<const void*>(step_run_kernel<9, THREADS, false>);
   return nullptr;
 }
 
-template <int THREADS>
-static const void* cluster_fn(int Q) {
-  return Q == 3   ? reinterpret_cast<const void*>(step_run_kernel<3, THREADS, true, true>)
-         : Q == 5 ? reinterpret_cast<const void*>(step_run_kernel<5, THREADS, true, true>)
-                  : reinterpret_cast<const void*>(step_run_kernel<9, THREADS, true, true>);
+// --------------------------------------------------------------------------
+// several steps of a lattice that one cluster of blocks holds in its shared memory, a lane per
+// node: block r keeps THREADS nodes' planes (two buffers), a node's results go straight into
+// the planes of whichever blocks hold its neighbours, and the hardware's cluster barrier
+// separates the steps.  A node's destinations never change, so their addresses are made once.
+// Bound: the latency of one node's collision and of the barrier; through buffers in L2 a step
+// also waited for its stores and its loads there.  Us per step, buffers in L2 with the cluster's
+// barrier (to 4096 nodes) or the grid's / here: D1Q3 256 nodes 1.54 / 0.77, 8192 2.06 / 1.10;
+// D2Q5 96 x 40 1.72 / 0.86, 64^2 at 50 per velocity 2.37 / 1.47, 90^2 2.06 / 1.13, 90^2 at 100
+// 3.24 / 2.99; D2Q9 64^2 2.03 / 1.23, 90^2 2.34 / 1.82.  Blocks of 1024 threads (to 16384 nodes)
+// lose to all SMs with the grid barrier at 25 per velocity and more (128^2 at 50 3.45 / 2.62).
+// --------------------------------------------------------------------------
+constexpr uint32_t kClusterBlocks = 16;  // (beyond 8 a kernel opts in)
+
+template <int Q, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1)
+    step_cluster_kernel(const __grid_constant__ StepArgs a, uint16_t* buf0, uint16_t* buf1, uint32_t t0, uint32_t T,
+                        unsigned long long* fail) {
+  extern __shared__ uint4 smem4[];
+  __shared__ int stop;
+  __shared__ uint32_t mark;  // the first step of this launch that overflowed
+  uint32_t* const s = reinterpret_cast<uint32_t*>(smem4);
+  if (threadIdx.x == 0) {
+    stop = *reinterpret_cast<volatile unsigned long long*>(fail) < t0;
+    mark = ~0u;
+  }
+  constexpr uint32_t kTables = run_table_words(Q);
+  for (uint32_t i = threadIdx.x; i < kTables / 4; i += THREADS)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(uint32_t(__cvta_generic_to_shared(smem4 + i))),
+                 "l"(reinterpret_cast<const uint4*>(a.tables) + i)
+                 : "memory");
+  unsigned char* const ring = reinterpret_cast<unsigned char*>(smem4) + 4 * kTables;
+  // planes of this block's nodes, [buffer][velocity][THREADS]
+  uint16_t* const planes = reinterpret_cast<uint16_t*>(ring + kStepRing * 4 * THREADS);
+  constexpr uint32_t kBuffer = Q * THREADS;
+  const Alias8 to = Alias8::of(s, 0), tr = Alias8::of(s, 1), ta = Alias8::of(s, Q == 9 ? 2 : 1);
+  const uint32_t nodes = a.Lx * a.Ly, tid = threadIdx.x, node = blockIdx.x * THREADS + tid;
+  const bool active = node < nodes;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    planes[i * THREADS + tid] = active ? __ldcg(buf0 + (size_t(i) * nodes + node)) : 0;
+    if (!active) planes[kBuffer + i * THREADS + tid] = 0;  // nobody writes there
+  }
+  // where velocity i's results go in buffer 0 of the block that holds the neighbour
+  uint32_t dest[Q];
+  {
+    const uint32_t y = node / a.Lx, x = node - y * a.Lx;
+    const uint32_t xs[3] = {x == 0 ? a.Lx - 1 : x - 1, x, x + 1 == a.Lx ? 0 : x + 1};
+    const uint32_t ys[3] = {y == 0 ? a.Ly - 1 : y - 1, y, y + 1 == a.Ly ? 0 : y + 1};
+    // +x, -x, +y, -y, then D2Q9's (+1,+1), (-1,-1), (+1,-1), (-1,+1)
+    constexpr int dx[9] = {0, 1, -1, 0, 0, 1, -1, 1, -1}, dy[9] = {0, 0, 0, 1, -1, 1, -1, -1, 1};
+    const uint32_t own = uint32_t(__cvta_generic_to_shared(planes));
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      const uint32_t d = active ? ys[1 + dy[i]] * a.Lx + xs[1 + dx[i]] : node;
+      asm("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(dest[i]) : "r"(own + 2 * (i * THREADS + d % THREADS)), "r"(d / THREADS));
+    }
+  }
+  constexpr int NB = Q == 9 ? 4 : 2;
+  NodeKeys<NB> keys = word_keys<NB>(a, t0);
+  SlotWords<NB> words;
+  words.make(keys, a.rk, node);
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
+  __syncthreads();
+  if (stop) return;
+  // every block has started: its planes are written by other blocks from here on
+  cluster_arrive();
+  cluster_wait();
+  uint32_t step = 0;
+  for (;; ++step) {
+    const uint32_t t = t0 + step, in = (step & 1) * kBuffer, out = 2 * (kBuffer - in);
+    uint32_t m[Q], post[Q];
+    // the flip F_i(n) = n_{-i}: velocity i of the collision reads plane -i
+#pragma unroll
+    for (int i = 0; i < Q; ++i) m[i] = planes[in + (i == 0 || !a.flip ? i : (i & 1 ? i + 1 : i - 1)) * THREADS + tid];
+    collide_warp<Q, 4 * THREADS, kStepRing, true>(a, keys, to, tr, ta, ring, 4 * tid, node, m, post, &words);
+    if (active) {
+      uint32_t high = 0;
+#pragma unroll
+      for (int i = 0; i < Q; ++i) {
+        high |= post[i];
+        asm volatile("st.shared::cluster.u16 [%0], %1;\n" ::"r"(dest[i] + out), "h"(uint16_t(post[i])) : "memory");
+      }
+      if (high > 65535u) {
+        atomicMin(fail, static_cast<unsigned long long>(t));
+        cluster_mark(&mark, step, gridDim.x);
+      }
+    }
+    __syncwarp();
+    cluster_arrive();
+    if (step + 1 < T) {
+      // while the others finish: the next step's words
+      keys = word_keys<NB>(a, t + 1);
+      words.make(keys, a.rk, node);
+    }
+    cluster_wait();
+    // (a faster block may already have marked the next step)
+    if (*reinterpret_cast<volatile uint32_t*>(&mark) <= step) break;
+    if (step + 1 == T) {
+      ++step;
+      break;
+    }
+  }
+  // the state after `step` steps, into the buffer that many single steps would have left it in
+  if (active) {
+    uint16_t* const to_state = (step & 1) ? buf1 : buf0;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) to_state[size_t(i) * nodes + node] = planes[(step & 1) * kBuffer + i * THREADS + tid];
+  }
 }
 
-// Several steps of a lattice that one cluster holds, a lane per node: the cluster's barrier
-// takes a few hundred cycles where arriving at and polling a word in L2 takes two thousand.
-// Sixteen blocks of 128 or 256 threads, as few as hold the lattice (rounded to a power of two);
-// in fewer and larger blocks the steps of more warps per SM cost what the barrier gains (64^2
-// at 50 per velocity 2.84 us per step in 8 blocks of 512, 2.33 in 16 of 256, 2.58 by the grid
-// barrier).  Us per step, grid barrier / cluster: 256 nodes of D1Q3 1.75 / 1.10, D2Q5 32^2
-// 1.75 / 1.15, 96 x 40 1.88 / 1.63, D2Q9 32^2 1.97 / 1.34, 64^2 2.08 / 1.93.
-constexpr uint32_t kClusterBlocks = 16;  // (beyond 8 a kernel opts in)
-static bool cluster_shape(int Q, bool tables, uint64_t nodes, RunShape* r) {
-  if (!tables || nodes > kClusterBlocks * 256) return false;
-  *r = nodes <= kClusterBlocks * 128 ? RunShape{cluster_fn<128>(Q), 128} : RunShape{cluster_fn<256>(Q), 256};
-  return true;
+constexpr size_t cluster_smem(int Q, int threads) { return run_smem(Q, threads) + size_t(2) * Q * threads * sizeof(uint16_t); }
+
+template <int THREADS>
+static const void* cluster_fn(int Q) {
+  return Q == 3   ? reinterpret_cast<const void*>(step_cluster_kernel<3, THREADS>)
+         : Q == 5 ? reinterpret_cast<const void*>(step_cluster_kernel<5, THREADS>)
+                  : reinterpret_cast<const void*>(step_cluster_kernel<9, THREADS>);
+}
+
+static const void* cluster_fn(int Q, int threads) {
+  return threads == 128 ? cluster_fn<128>(Q) : threads == 256 ? cluster_fn<256>(Q) : cluster_fn<512>(Q);
+}
+
+// Sixteen blocks of as few threads as hold the lattice; 0: none does.
+static int cluster_threads(bool tables, uint64_t nodes) {
+  if (!tables) return 0;
+  for (int threads : {128, 256, 512})
+    if (nodes <= kClusterBlocks * uint64_t(threads)) return threads;
+  return 0;
 }
 
 static bool run_tables(int Q, const StepArgs& a) {
@@ -253,34 +338,36 @@ cudaError_t prepare_step_kernels(int Q) {
     set(run_fn<512>(Q, tables), 512);
     set(run_fn<1024>(Q, tables), 1024);
   }
-  set(cluster_fn<128>(Q), 128);
-  set(cluster_fn<256>(Q), 256);
-  for (const void* f : {cluster_fn<128>(Q), cluster_fn<256>(Q)})
+  for (int threads : {128, 256, 512}) {
+    const void* f = cluster_fn(Q, threads);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(cluster_smem(Q, threads)));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  }
   return e;
 }
 
 cudaError_t launch_step_run(int Q, const StepArgs& a, uint16_t* buf0, uint16_t* buf1, uint32_t t, uint32_t T,
                             unsigned long long* fail, unsigned long long* sync, uint32_t sms, cudaStream_t s) {
   const uint64_t nodes = uint64_t(a.Lx) * a.Ly;
-  RunShape cr;
-  if (T > 1 && cluster_shape(Q, run_tables(Q, a), nodes, &cr)) {
+  const int ct = T > 1 ? cluster_threads(run_tables(Q, a), nodes) : 0;
+  if (ct) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr = {};
     uint32_t blocks = 1;
-    while (uint64_t(blocks) * cr.threads < nodes) blocks *= 2;
+    while (uint64_t(blocks) * ct < nodes) blocks *= 2;
     attr.id = cudaLaunchAttributeClusterDimension;
     attr.val.clusterDim.x = blocks;
     attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
     cfg.gridDim = dim3(blocks);
-    cfg.blockDim = dim3(cr.threads);
-    cfg.dynamicSmemBytes = run_smem(Q, cr.threads);
+    cfg.blockDim = dim3(ct);
+    cfg.dynamicSmemBytes = cluster_smem(Q, ct);
     cfg.stream = s;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     StepArgs ca = a;
-    void* p[] = {&ca, &buf0, &buf1, &t, &T, &fail, &sync};
-    if (cudaLaunchKernelExC(&cfg, cr.fn, p) == cudaSuccess) return cudaSuccess;
+    void* p[] = {&ca, &buf0, &buf1, &t, &T, &fail};
+    if (cudaLaunchKernelExC(&cfg, cluster_fn(Q, ct), p) == cudaSuccess) return cudaSuccess;
     cudaGetLastError();  // no room for a cluster (SMs reserved elsewhere): the grid barrier instead
   }
   const RunShape r = run_shape(Q, a, nodes, sms);
