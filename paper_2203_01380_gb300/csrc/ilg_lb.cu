@@ -30,7 +30,7 @@ constexpr int kLbThreads = 256;
 __host__ __device__ constexpr int lb_run_threads(int Q, bool wide) { return !wide ? 256 : (Q == 9 ? 512 : 768); }
 constexpr uint32_t kLbMaxModes = 256;
 constexpr int kLbModeThreads = 64;     // of a projection's blocks
-constexpr int kLbClusterBlocks = 16;   // (beyond 8 a kernel opts in)
+constexpr int kLbClusterBlocks = 16;  // (beyond 8 a kernel opts in)
 constexpr uint32_t kLbCols = 32;       // columns of a block of their sums (or kLbThreads)
 constexpr uint32_t kLbFewRows = 8;
 constexpr uint32_t kLbFirstModes = 64; // passed as a kernel argument
@@ -148,11 +148,8 @@ __device__ __forceinline__ void relax(const LbCoef& k, const double (&f)[Q], dou
 
 // T steps, one node per thread: load the Q planes, relax, push.  f0 holds the state, the
 // steps alternate the buffers; a barrier of all blocks (a cooperative launch) separates them.
-// sync[0]: barrier word, sync[1]: 1 once a wait gave up.  CLUSTER: the launch is one cluster
-// (at most kLbClusterBlocks blocks, a node per thread) and its barrier the cluster's.  Us per
-// step, grid barrier / cluster: 500 nodes of D1Q3 2.0 / 1.3, D2Q5 64^2 2.5 / 2.1, D2Q9 56 x 66
-// 3.4 / 3.0 (one launch per step: 4.1).
-template <int Q, bool CLUSTER, bool WIDE>
+// sync[0]: barrier word, sync[1]: 1 once a wait gave up.
+template <int Q, bool WIDE>
 __global__ void __launch_bounds__(lb_run_threads(Q, WIDE), WIDE ? 1 : 4)
     lb_run_kernel(const __grid_constant__ LbCoef k, double* f0, double* f1, uint32_t Lx, uint32_t Ly, uint32_t T,
                   unsigned long long* sync) {
@@ -160,7 +157,7 @@ __global__ void __launch_bounds__(lb_run_threads(Q, WIDE), WIDE ? 1 : 4)
   if (threadIdx.x == 0) stop = 0;
   const uint32_t nodes = Lx * Ly;
   const size_t plane = nodes;
-  const uint32_t threads = CLUSTER ? blockDim.x : uint32_t(lb_run_threads(Q, WIDE));
+  constexpr uint32_t threads = lb_run_threads(Q, WIDE);
   const uint32_t stride = gridDim.x * threads, stride_y = stride / Lx, stride_x = stride - stride_y * Lx;
   const uint32_t first = blockIdx.x * threads + threadIdx.x;
   const uint32_t y0 = first / Lx, x0 = first - y0 * Lx;
@@ -215,12 +212,6 @@ __global__ void __launch_bounds__(lb_run_threads(Q, WIDE), WIDE ? 1 : 4)
       }
     }
     if (step + 1 == T) break;
-    if constexpr (CLUSTER) {
-      __syncwarp();
-      ilg::cluster_arrive();
-      ilg::cluster_wait();
-      continue;
-    }
     __syncthreads();
     if (threadIdx.x == 0 && ilg::run_barrier(sync, (step + 1) * gridDim.x) == ~0ull) {
       atomicExch(sync + 1, 1ull);
@@ -228,6 +219,62 @@ __global__ void __launch_bounds__(lb_run_threads(Q, WIDE), WIDE ? 1 : 4)
     }
     __syncthreads();
     if (stop) break;
+  }
+}
+
+// Several steps of a lattice that one cluster holds in its shared memory, a node per thread:
+// block r keeps blockDim.x nodes' planes (two buffers; a power of two), a node's results go
+// straight into the planes of the blocks that hold its neighbours, and the cluster's barrier
+// separates the steps.  Bound: the latency of a node's relaxation and of the barrier.  Us per
+// step, buffers in L2 with the cluster's barrier (to 4096 nodes) or the grid's / here: D1Q3 500
+// nodes 1.16 / 0.48, 16384 1.90 / 1.27; D2Q5 64^2 1.55 / 0.73, 128^2 2.10 / 1.73; D2Q9 56 x 66
+// 2.23 / 1.13, 90^2 2.61 / 1.66 (in blocks of 1024 threads 128^2 would take 3.30, on all SMs
+// 2.59).
+template <int Q, int MOST>
+__global__ void __launch_bounds__(MOST, 1)
+    lb_cluster_kernel(const __grid_constant__ LbCoef k, double* f0, double* f1, uint32_t Lx, uint32_t Ly, uint32_t T) {
+  extern __shared__ double planes[];  // [buffer][velocity][thread]
+  const uint32_t nodes = Lx * Ly, threads = blockDim.x, tid = threadIdx.x, node = blockIdx.x * threads + tid;
+  const uint32_t buffer = Q * threads;
+  const bool active = node < nodes;
+  uint32_t dest[Q];  // where velocity i's results go in buffer 0
+  {
+    const uint32_t y = node / Lx, x = node - y * Lx;
+    const uint32_t xs[3] = {x == 0 ? Lx - 1 : x - 1, x, x + 1 == Lx ? 0 : x + 1};
+    const uint32_t ys[3] = {y == 0 ? Ly - 1 : y - 1, y, y + 1 == Ly ? 0 : y + 1};
+    constexpr int dx[9] = {0, 1, -1, 0, 0, 1, -1, 1, -1}, dy[9] = {0, 0, 0, 1, -1, 1, -1, -1, 1};
+    const uint32_t own = uint32_t(__cvta_generic_to_shared(planes)), log = 31 - __clz(int(threads));
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      if (active) planes[i * threads + tid] = __ldcg(f0 + (size_t(i) * nodes + node));
+      const uint32_t d = active ? ys[1 + dy[i]] * Lx + xs[1 + dx[i]] : node;
+      asm("mapa.shared::cluster.u32 %0, %1, %2;\n"
+          : "=r"(dest[i])
+          : "r"(own + 8 * (i * threads + (d & (threads - 1)))), "r"(d >> log));
+    }
+  }
+  // every block has started: its planes are written by other blocks from here on
+  ilg::cluster_arrive();
+  ilg::cluster_wait();
+  for (uint32_t step = 0; step < T; ++step) {
+    const uint32_t in = (step & 1) * buffer, out = 8 * (buffer - in);
+    if (active) {
+      double f[Q], post[Q];
+#pragma unroll
+      for (int i = 0; i < Q; ++i) f[i] = planes[in + (i == 0 || !k.swap ? i : (i & 1 ? i + 1 : i - 1)) * threads + tid];
+      relax<Q>(k, f, post);
+#pragma unroll
+      for (int i = 0; i < Q; ++i)
+        asm volatile("st.shared::cluster.f64 [%0], %1;\n" ::"r"(dest[i] + out), "d"(post[i]) : "memory");
+    }
+    __syncwarp();
+    ilg::cluster_arrive();
+    ilg::cluster_wait();
+  }
+  double* const state = (T & 1) ? f1 : f0;
+  if (active) {
+#pragma unroll
+    for (int i = 0; i < Q; ++i) state[size_t(i) * nodes + node] = planes[(T & 1) * buffer + i * threads + tid];
   }
 }
 
@@ -562,12 +609,25 @@ int lb_grid(const ilg_lb* b) {
   return int(blocks < cap ? blocks : cap);
 }
 
-template <bool CLUSTER, bool WIDE>
+template <bool WIDE>
 const void* lb_run_of(int Q) {
-  return Q == 3   ? reinterpret_cast<const void*>(lb_run_kernel<3, CLUSTER, WIDE>)
-         : Q == 5 ? reinterpret_cast<const void*>(lb_run_kernel<5, CLUSTER, WIDE>)
-                  : reinterpret_cast<const void*>(lb_run_kernel<9, CLUSTER, WIDE>);
+  return Q == 3   ? reinterpret_cast<const void*>(lb_run_kernel<3, WIDE>)
+         : Q == 5 ? reinterpret_cast<const void*>(lb_run_kernel<5, WIDE>)
+                  : reinterpret_cast<const void*>(lb_run_kernel<9, WIDE>);
 }
+
+// most threads of a cluster's block
+int lb_cluster_threads(int Q) { return Q == 9 ? 512 : 1024; }
+
+const void* lb_cluster_fn(int Q, int threads) {
+  if (threads > 512)
+    return Q == 3 ? reinterpret_cast<const void*>(lb_cluster_kernel<3, 1024>)
+                  : reinterpret_cast<const void*>(lb_cluster_kernel<5, 1024>);
+  return Q == 3   ? reinterpret_cast<const void*>(lb_cluster_kernel<3, 512>)
+         : Q == 5 ? reinterpret_cast<const void*>(lb_cluster_kernel<5, 512>)
+                  : reinterpret_cast<const void*>(lb_cluster_kernel<9, 512>);
+}
+size_t lb_cluster_smem(int Q, int threads) { return sizeof(double) * 2 * Q * threads; }
 
 // Lattices of more nodes than this per SM: one wide block per SM, its threads' next values
 // loaded while the present ones relax.  Us per step, narrow / wide: D2Q5 350^2 3.85 / 4.09,
@@ -576,13 +636,13 @@ const void* lb_run_of(int Q) {
 constexpr size_t kLbWideNodesPerSm = 1024;
 bool lb_wide(const ilg_lb* b) { return b->nodes > kLbWideNodesPerSm * b->sms; }
 int lb_threads(const ilg_lb* b) { return lb_run_threads(b->Q, lb_wide(b)); }
-const void* lb_run_fn(const ilg_lb* b) { return lb_wide(b) ? lb_run_of<false, true>(b->Q) : lb_run_of<false, false>(b->Q); }
+const void* lb_run_fn(const ilg_lb* b) { return lb_wide(b) ? lb_run_of<true>(b->Q) : lb_run_of<false>(b->Q); }
 
-bool lb_fits_cluster(const ilg_lb* b) { return b->nodes <= size_t(kLbClusterBlocks) * kLbThreads; }
+bool lb_fits_cluster(const ilg_lb* b) { return b->nodes <= size_t(kLbClusterBlocks) * lb_cluster_threads(b->Q); }
 
 // Several steps as one cluster; false where there is no room for it (SMs reserved elsewhere).
 bool lb_launch_cluster(const ilg_lb* b, void** args) {
-  // many small blocks: the fp64 pipe of as many SMs as there are
+  // many small blocks: as many SMs as there are
   uint32_t threads = 64, blocks = 1;
   while (size_t(kLbClusterBlocks) * threads < b->nodes) threads *= 2;
   while (size_t(blocks) * threads < b->nodes) blocks *= 2;
@@ -593,10 +653,11 @@ bool lb_launch_cluster(const ilg_lb* b, void** args) {
   attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
   cfg.gridDim = dim3(blocks);
   cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = lb_cluster_smem(b->Q, int(threads));
   cfg.stream = b->stream;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  if (cudaLaunchKernelExC(&cfg, lb_run_of<true, false>(b->Q), args) == cudaSuccess) return true;
+  if (cudaLaunchKernelExC(&cfg, lb_cluster_fn(b->Q, int(threads)), args) == cudaSuccess) return true;
   cudaGetLastError();
   return false;
 }
@@ -696,8 +757,14 @@ ilg_status ilg_lb_create(const ilg_lb_params* params, void* stream, ilg_lb** out
   }
   int per_sm = 0;
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lb_run_fn(b), lb_threads(b), 0);
-  if (e == cudaSuccess && lb_fits_cluster(b))
-    e = cudaFuncSetAttribute(lb_run_of<true, false>(b->Q), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess && lb_fits_cluster(b)) {
+    for (const int threads : {512, lb_cluster_threads(b->Q)}) {
+      const void* f = lb_cluster_fn(b->Q, threads);
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(lb_cluster_smem(b->Q, threads)));
+    }
+  }
   if (e != cudaSuccess) {
     ilg_lb_destroy(b);
     return lb_cuda_fail(nullptr, e, "ilg_lb_create");

@@ -77,3 +77,23 @@ def test_one_rounding_inside(B, lattice, oj, om):
     # (D2Q9: 2^-58) of the largest value each
     units = 8 * 2.0 ** (-58 if Q == 9 else -60) * 2.0
     assert np.all(np.abs(got.astype(LD) - want) <= 2.0**-53 * 2.0 ** np.ceil(np.log2(want.astype(float))) + units)
+
+
+@pytest.mark.parametrize("lattice,Lx,Ly", [(1, 63, 1), (1, 1025, 1), (1, 4097, 1), (1, 16384, 1), (1, 16385, 1),
+                                           (2, 3, 3), (2, 65, 63), (2, 91, 90), (2, 128, 128), (2, 129, 128),
+                                           (3, 7, 9), (3, 128, 64), (3, 91, 91)])
+def test_steps_in_a_cluster(B, lattice, Lx, Ly):
+    """Many steps in one launch (lattices that a cluster's shared memory holds, and one node or row
+    more) against the same steps one call at a time, bit for bit, ending in either buffer."""
+    kw = dict(n0=30.0, amp=20.0, mode_mx=1, omega_j=1.7, omega=0.3)
+    with B.LB(lattice, Lx, Ly, **kw) as a, B.LB(lattice, Lx, Ly, **kw) as b:
+        a.init()
+        b.init()
+        for n in (2, 5):
+            a.step(n)
+            for _ in range(n):
+                b.step(1)
+            fa, ta = a.get_state()
+            fb, tb = b.get_state()
+            assert ta == tb and np.array_equal(fa, fb)
+        assert a.observables([(1, 0)])["mass"] == b.observables([(1, 0)])["mass"]
