@@ -35,6 +35,10 @@ struct ilg_ctx {
   unsigned long long* d_col = nullptr;
   unsigned long long* d_row = nullptr;
   unsigned long long* d_proj = nullptr;    // scratch of the projections
+  // mailbox of the steps that keep the planes in shared memory, and the last tag in it
+  uint32_t* d_mail = nullptr;
+  size_t mail_words = 0;
+  uint32_t mail_tag = 0;
   // pinned, written by the projections: mass, 4 per mode; after the words of h_word for up
   // to kFirstModes modes, an allocation of its own for more
   unsigned long long* h_obs = nullptr;
@@ -148,6 +152,7 @@ void free_ctx(ilg_ctx* c) {
   cudaFree(c->d_fail);
   cudaFree(c->d_mass);
   cudaFree(c->d_proj);
+  cudaFree(c->d_mail);
   if (c->mode_cap > kFirstModes) cudaFreeHost(c->h_obs);
   if (c->h_word) cudaFreeHost(c->h_word);
 }
@@ -215,6 +220,9 @@ ilg_status ilg_create(const ilg_params* params, void* stream, ilg_ctx** out) {
   c->d_row = c->d_col + c->p.Lx;
   if ((e = dev_alloc(&c->d_proj, sizeof(unsigned long long) * kProjScratchWords)) != cudaSuccess)
     return bail(e, "cudaMalloc projections");
+  c->mail_words = step_resident_mail_words(c->Q, c->p.Lx, c->nodes, uint32_t(c->sms));
+  if (c->mail_words && (e = dev_alloc(&c->d_mail, sizeof(uint32_t) * c->mail_words)) != cudaSuccess)
+    return bail(e, "cudaMalloc mailbox");
   if ((e = cudaMallocHost(&c->h_word, sizeof(unsigned long long) * (kFailWords + 1 + 4 * kFirstModes))) != cudaSuccess)
     return bail(e, "cudaMallocHost");
   c->h_obs = c->h_word + kFailWords;
@@ -230,6 +238,7 @@ ilg_status ilg_create(const ilg_params* params, void* stream, ilg_ctx** out) {
   e = cudaMemsetAsync(c->d_fail, 0xFF, sizeof(unsigned long long), c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_fail + 1, 0, 2 * sizeof(unsigned long long), c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_proj, 0, sizeof(unsigned long long) * kProjScratchWords, c->stream);
+  if (e == cudaSuccess && c->d_mail) e = cudaMemsetAsync(c->d_mail, 0, sizeof(uint32_t) * c->mail_words, c->stream);
   if (e != cudaSuccess) return bail(e, "reset flag");
   e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return bail(e, "cudaStreamSynchronize");
@@ -395,16 +404,28 @@ uint64_t vec_warps(const ilg_ctx* c) { return uint64_t(c->sms) * 3 * 8; }
 // them.  Us per step, 10 per velocity, node-parallel / 4-node / 8-node vectors: D2Q5 512^2
 // 5.4 / 5.3 / 5.7, 768^2 8.8 / 8.1 / 8.6, 1024^2 13.4 / 10.5 / 11.8, 1448^2 24.4 / 19.4 /
 // 18.1, 2048^2 45 / 33 / 30; D2Q9 (4-node) 1024^2 21 / 31, 1448^2 39 / 50, 2048^2 84 / 75.
-constexpr uint64_t kRunNodesPerSm = 2048, kRunNodesPerSm9 = 16384, kWarp4NodesPerSm = 10240;
+// With the planes in shared memory the node-parallel steps stay ahead for longer (10 per velocity,
+// omega_eff 1.8 / 1.5, node-parallel / 4-node: 640^2 5.9 / 6.1, 5.9 / 7.6; 768^2 7.76 / 7.75,
+// 7.8 / 9.6; D1Q3 2^19 5.1 / 5.7).
+constexpr uint64_t kRunNodesPerSm = 2048, kResidentNodesPerSm = 3072, kRunNodesPerSm9 = 16384, kWarp4NodesPerSm = 10240;
 
-// the kernel a step runs: the tuned one while it applies to the current state, else
+// Node-parallel steps that all SMs take with the planes in shared memory.  A launch reads the
+// planes in and writes them out again, which a few steps have to repay (us for 4 steps, buffers in
+// L2 / shared memory: 100^2 23 / 23, 400^2 48 / 41, 850^2 87 / 98; for 8 850^2 161 / 162).
+bool takes_resident(const ilg_ctx* c, const StepArgs& a, uint32_t n) {
+  return c->d_mail && n >= (c->nodes > 1024 * size_t(c->sms) ? 8u : 4u) && !a.particle && a.omega_mode == kTable &&
+         a.rest_mode == kTable && (c->Q != 9 || a.axis_mode == kTable);
+}
+
+// the kernel that n steps run: the tuned one while it applies to the current state, else
 // the default: node-parallel on small lattices; the shared-memory-staged warp kernel
 // with 4- or 8-node vectors where the rows and probabilities allow; else 8-node row tiles
 // where the rows allow; node-parallel otherwise
-int pick_kernel(const ilg_ctx* c, const StepArgs& a) {
+int pick_kernel(const ilg_ctx* c, const StepArgs& a, uint32_t n) {
   if (c->kernel_choice >= 0 && kernel_applies(c, a, c->kernel_choice)) return c->kernel_choice;
   const uint64_t sms = uint64_t(c->sms);
-  if (c->nodes <= (c->Q == 9 ? kRunNodesPerSm9 : kRunNodesPerSm) * sms) return kKernelNode;
+  const uint64_t run = c->Q == 9 ? kRunNodesPerSm9 : (takes_resident(c, a, n) ? kResidentNodesPerSm : kRunNodesPerSm);
+  if (c->nodes <= run * sms) return kKernelNode;
   const bool w4 = kernel_applies(c, a, kKernelWarp4);
   if (c->Q != 9 && w4 && c->nodes <= kWarp4NodesPerSm * sms) return kKernelWarp4;
   if (kernel_applies(c, a, kKernelWarp8)) return kKernelWarp8;
@@ -434,16 +455,37 @@ cudaError_t launch_steps(const ilg_ctx* c, int kind, const StepArgs& a, uint16_t
   return launch_step_run(c->Q, a, b0, b1, uint32_t(t), T, fail_word, fail_word + 1, sms, c->stream);
 }
 
-// T single steps from step t (the state in bufs[cur], the steps alternate the buffers), in
-// few launches of several steps each where the kernel takes them
-cudaError_t launch_singles(const ilg_ctx* c, int kind, const StepArgs& a, uint16_t* const* bufs, int cur, uint64_t t,
-                           uint32_t T, unsigned long long* fail_word) {
+// A launch of single steps: n from step t, the state in buffer cur.
+struct StepLaunch {
+  uint64_t t;
+  uint32_t n;
+  int cur;
+  bool resident;  // leaves its input as it was and its result in the other buffer
+};
+
+// T single steps from step t (the state in bufs[cur]; cur: afterwards), in few launches of
+// several steps each where the kernel takes them.  done (or NULL): what was launched.
+cudaError_t launch_singles(ilg_ctx* c, int kind, const StepArgs& a, uint16_t* const* bufs, int& cur, uint64_t t, uint32_t T,
+                           unsigned long long* fail_word, std::vector<StepLaunch>* done = nullptr) {
   constexpr uint32_t kRunSteps = 4096;         // per launch
   constexpr uint64_t kRunNodes = 1ull << 26;  // beyond: a step takes half a millisecond and more, a launch nothing of it
+  constexpr uint32_t kTags = 1u << 16;
   bool run = takes_runs(kind) && (kind == kKernelNode || c->nodes < kRunNodes);
   for (uint32_t k = 0; k < T;) {
     const uint32_t n = run ? std::min(T - k, kRunSteps) : 1;
-    const cudaError_t e = launch_steps(c, kind, a, bufs[cur], bufs[cur ^ 1], t + k, n, fail_word);
+    const bool resident = run && kind == kKernelNode && takes_resident(c, a, n);
+    cudaError_t e;
+    if (resident) {
+      if (c->mail_tag + n >= kTags) {
+        if ((e = cudaMemsetAsync(c->d_mail, 0, sizeof(uint32_t) * c->mail_words, c->stream)) != cudaSuccess) return e;
+        c->mail_tag = 0;
+      }
+      e = launch_step_resident(c->Q, a, bufs[cur], bufs[cur ^ 1], uint32_t(t + k), n, fail_word, fail_word + 1, c->d_mail,
+                               c->mail_tag + 1, uint32_t(c->sms), c->stream);
+      if (e == cudaSuccess) c->mail_tag += n;
+    } else {
+      e = launch_steps(c, kind, a, bufs[cur], bufs[cur ^ 1], t + k, n, fail_word);
+    }
     if (e == cudaErrorCooperativeLaunchTooLarge && n > 1) {
       // the device cannot hold all blocks at once (SMs reserved elsewhere): step by step
       cudaGetLastError();
@@ -451,8 +493,9 @@ cudaError_t launch_singles(const ilg_ctx* c, int kind, const StepArgs& a, uint16
       continue;
     }
     if (e != cudaSuccess) return e;
+    if (done) done->push_back({t + k, n, cur, resident});
     k += n;
-    cur ^= int(n & 1u);
+    cur ^= resident ? 1 : int(n & 1u);
   }
   return cudaSuccess;
 }
@@ -474,7 +517,7 @@ ilg_status ilg_step(ilg_ctx* c, uint32_t T) {
   const StepArgs a = step_args(c);
   // high occupations and the particle sampler go straight to the general collision
   // (node-parallel kernel)
-  const int kind = pick_kernel(c, a);
+  const int kind = pick_kernel(c, a, T);
   const int cur0 = c->cur;
   const uint64_t t0 = c->t;
   // blocks of tb_depth steps (temporal blocking), then single steps; a block or step k
@@ -493,11 +536,10 @@ ilg_status ilg_step(ilg_ctx* c, uint32_t T) {
     }
   }
   const uint64_t t_single = t;  // single steps from here
-  const uint64_t blocks = tb >= 2 ? (t - t0) / tb : 0;
+  std::vector<StepLaunch> singles;
   if (const uint32_t n = uint32_t(t0 + T - t)) {
-    const cudaError_t e = launch_singles(c, kind, a, c->buf, cur, t, n, c->d_fail);
+    const cudaError_t e = launch_singles(c, kind, a, c->buf, cur, t, n, c->d_fail, &singles);
     if (e != cudaSuccess) return cuda_fail(c, e, "step kernel");
-    cur ^= int(n & 1u);
   }
   ILG_CUDA(c, cudaMemcpyAsync(c->h_word, c->d_fail, sizeof(unsigned long long) * kFailWords, cudaMemcpyDeviceToHost,
                               c->stream),
@@ -514,12 +556,24 @@ ilg_status ilg_step(ilg_ctx* c, uint32_t T) {
     return fail(c, ILG_E_TIMEOUT, "a wait between the blocks of a several-step launch gave up: the state is lost");
   }
   if (f != ~0ull) {
-    // the block or step that started at step f failed: its input buffer still holds the
-    // state at f
-    const uint64_t k = f < t_single ? (f - t0) / tb : blocks + (f - t_single);
-    c->cur = cur0 ^ int(k & 1u);
-    c->t = f;
     ILG_CUDA(c, cudaMemsetAsync(c->d_fail, 0xFF, sizeof(unsigned long long), c->stream), "reset flag");
+    if (f < t_single) {
+      // the block that started at step f failed: its input buffer still holds the state at f
+      c->cur = cur0 ^ int((f - t0) / tb & 1u);
+    } else {
+      // the launch that step f belongs to: its input buffer still holds the state at f, or, with
+      // the planes in shared memory, the state that the launch started from
+      size_t j = 0;
+      while (j + 1 < singles.size() && singles[j + 1].t <= f) ++j;
+      const StepLaunch& l = singles[j];
+      const uint32_t ahead = uint32_t(f - l.t);
+      if (l.resident && ahead)
+        ILG_CUDA(c, launch_step_run(c->Q, a, c->buf[l.cur], c->buf[l.cur ^ 1], uint32_t(l.t), ahead, c->d_fail, c->d_fail + 1,
+                                    uint32_t(c->sms), c->stream),
+                 "steps before the overflow");
+      c->cur = l.cur ^ int(ahead & 1u);
+    }
+    c->t = f;
     ILG_CUDA(c, cudaStreamSynchronize(c->stream), "reset flag");
     char buf[160];
     std::snprintf(buf, sizeof(buf), "occupation above 65535 in the launch from step %llu; state kept at t = %llu", f, f);
@@ -584,7 +638,6 @@ ilg_status ilg_autotune(ilg_ctx* c, uint32_t trial_steps, ilg_tuning* out) {
       cudaError_t r = cudaSuccess;
       if (depth == 1) {
         r = launch_singles(c, cand, a, s, cur, t, n, fw);
-        cur ^= int(n & 1u);
       } else {
         for (uint32_t k = 0; k < n && r == cudaSuccess; ++k) {
           r = launch_step_tb(a, s[cur], s[cur ^ 1], uint32_t(t) + k * depth, depth, tb_tile(depth), fw, tb_grid(c, depth),

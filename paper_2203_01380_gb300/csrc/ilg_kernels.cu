@@ -320,11 +320,250 @@ static bool run_tables(int Q, const StepArgs& a) {
   return !a.particle && a.omega_mode == kTable && a.rest_mode == kTable && (Q != 9 || a.axis_mode == kTable);
 }
 
+// --------------------------------------------------------------------------
+// several steps of a lattice whose planes all SMs together hold in shared memory: block b keeps
+// an equal share of the nodes' runs of 32 (row-major), and a result for a node of another share
+// goes there as a word of a mailbox in L2 that carries the step's tag beside the value; whoever
+// needs it polls that word, so no barrier of all blocks and no fence stands between the steps.
+// Runs whose neighbours lie in other shares come first in a step: their words are on the way
+// while the rest collides.  A mailbox word of one parity is written again only by a node that
+// has had, as an input, a result of the node that read it.
+// buf0 is only read: should a step overflow, the caller takes the steps before it again from
+// there, since the shares may be steps apart by then.
+// Bound: integer issue; with few nodes per SM a word's way to L2 and back.  Us per step, buffers
+// in L2 and a barrier of all blocks / here: D2Q5 100^2 at 12 per velocity 2.09 / 1.43, 301 x 200
+// 2.58 / 1.88, 400^2 at 50 8.01 / 5.72, 512^2 at 50 8.13 / 7.25, 850^2 at 50 18.3 / 17.9; D1Q3
+// 65000 nodes at 30 2.46 / 1.54, 2^18 4.75 / 3.62, 2^20 13.3 / 12.0; D2Q9 200^2 3.15 / 2.45.
+// Packed tables and shorter rings of extension words, which would let the planes of 1024^2 fit,
+// cost there what the barrier takes (at 50 per velocity 24.9 / 25.7).  A pause between polls costs
+// more than the polls (301 x 200 at 50 per velocity 2.79, 3.9 with 20 ns).
+// --------------------------------------------------------------------------
+struct ResidentArgs {
+  uint32_t* mail;        // [parity][velocity - 1][node]: tag << 16 | value
+  uint32_t tag;          // of the first step's results; below 2^16 for all steps
+  uint32_t stride;       // nodes of the largest share
+  unsigned long long* gave_up;  // set to 1 when a poll gave up
+};
+constexpr uint32_t kMailPolls = 1u << 21;  // seconds
+
+__device__ __forceinline__ uint32_t mail_load(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void mail_store(uint32_t* p, uint32_t v) {
+  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;\n" ::"l"(p), "r"(v) : "memory");
+}
+
+template <int Q, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1)
+    step_resident_kernel(const __grid_constant__ StepArgs a, const uint16_t* buf0, uint16_t* buf1, uint32_t t0, uint32_t T,
+                         unsigned long long* fail, const __grid_constant__ ResidentArgs ra) {
+  constexpr uint32_t kTables = run_table_words(Q);
+  extern __shared__ uint4 smem4[];
+  __shared__ int stop;
+  uint32_t* const s = reinterpret_cast<uint32_t*>(smem4);
+  if (threadIdx.x == 0) stop = *reinterpret_cast<volatile unsigned long long*>(fail) < t0;
+  for (uint32_t i = threadIdx.x; i < kTables / 4; i += blockDim.x)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(uint32_t(__cvta_generic_to_shared(smem4 + i))),
+                 "l"(reinterpret_cast<const uint4*>(a.tables) + i)
+                 : "memory");
+  unsigned char* const words = reinterpret_cast<unsigned char*>(smem4) + 4 * kTables;
+  uint16_t* const planes = reinterpret_cast<uint16_t*>(words + kStepRing * 4 * THREADS);  // [buffer][velocity][stride]
+  const Alias8 to = Alias8::of(s, 0), tr = Alias8::of(s, 1), ta = Alias8::of(s, Q == 9 ? 2 : 1);
+
+  const uint32_t nodes = a.Lx * a.Ly, lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  const uint32_t runs = (nodes + 31) >> 5;
+  // runs [r0, r0 + n) of the lattice, nodes [a0, a0 + P)
+  const uint32_t r0 = uint32_t(uint64_t(blockIdx.x) * runs / gridDim.x);
+  const uint32_t n = uint32_t(uint64_t(blockIdx.x + 1) * runs / gridDim.x) - r0;
+  const uint32_t a0 = r0 * 32, P = min(n * 32, nodes - a0);
+  // how far a node's neighbours lie, wraps from the last row to the first aside (D2Q9: up to
+  // two rows from a row's ends)
+  const uint32_t near = Q == 3 ? 1 : (Q == 5 ? a.Lx : a.Lx + 1);
+  const uint32_t edge = min((near + 31) / 32 + 1, (n + 1) / 2);  // runs at either end that come first
+  const uint32_t stride = ra.stride, buffer = Q * stride;
+  for (uint32_t l = threadIdx.x; l < P; l += blockDim.x)
+#pragma unroll
+    for (int i = 0; i < Q; ++i) planes[i * stride + l] = __ldcg(buf0 + (size_t(i) * nodes + a0 + l));
+  uint32_t* const xs = reinterpret_cast<uint32_t*>(planes + 2 * buffer);  // x of each run's first node
+  for (uint32_t r = threadIdx.x; r < n; r += blockDim.x) xs[r] = (a0 + 32 * r) % a.Lx;
+  constexpr int NB = Q == 9 ? 4 : 2;
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
+  __syncthreads();
+  if (stop) return;
+
+  // the j-th run of a step: the ends of the share first
+  const auto run_of = [&](uint32_t j) { return j >= 2 * edge ? j - edge : (j & 1 ? n - 1 - j / 2 : j / 2); };
+  // a node's neighbours in its row and beside it (wrapped), and whether they lie in this share
+  struct Around {
+    uint32_t right, left, dy_up, dy_down;  // (what to add to a node to move a row up / down)
+  };
+  const auto around = [&](uint32_t node, uint32_t x) {
+    Around o;
+    o.right = x + 1 == a.Lx ? node + 1 - a.Lx : node + 1;
+    o.left = x == 0 ? node + a.Lx - 1 : node - 1;
+    o.dy_up = node + a.Lx >= nodes ? a.Lx - nodes : a.Lx;
+    o.dy_down = node < a.Lx ? nodes - a.Lx : 0u - a.Lx;
+    return o;
+  };
+  // neighbour of velocity i (+x, -x, +y, -y, then D2Q9's (+1,+1), (-1,-1), (+1,-1), (-1,+1))
+  const auto neighbour = [&](const Around& o, uint32_t node, int i) {
+    constexpr int dx[9] = {0, 1, -1, 0, 0, 1, -1, 1, -1}, dy[9] = {0, 0, 0, 1, -1, 1, -1, -1, 1};
+    const uint32_t in_row = dx[i] > 0 ? o.right : (dx[i] < 0 ? o.left : node);
+    return dy[i] > 0 ? in_row + o.dy_up : (dy[i] < 0 ? in_row + o.dy_down : in_row);
+  };
+  const auto opposite = [](int i) { return i == 0 ? 0 : (i & 1 ? i + 1 : i - 1); };
+  // the words of plane p for this share's nodes whose plane-p value comes from elsewhere, of the
+  // state that tag stands for (parity: of its step)
+  const auto take_mail = [&](const Around& o, uint32_t node, bool active, uint32_t tag, uint32_t parity, uint32_t (&v)[Q]) {
+    const uint32_t* const box = ra.mail + size_t(parity) * (Q - 1) * nodes + node;
+    uint32_t w[Q];
+    bool cross[Q];
+    bool missing = false;
+#pragma unroll
+    for (int p = 1; p < Q; ++p) {
+      cross[p] = active && neighbour(o, node, opposite(p)) - a0 >= P;
+      w[p] = cross[p] ? mail_load(box + size_t(p - 1) * nodes) : 0u;
+    }
+#pragma unroll
+    for (int p = 1; p < Q; ++p) missing |= cross[p] && (w[p] >> 16) != tag;
+    for (uint32_t polls = 0; missing; ++polls) {
+      if (polls == kMailPolls || *reinterpret_cast<volatile int*>(&stop)) {
+        atomicExch(ra.gave_up, 1ull);
+        *reinterpret_cast<volatile int*>(&stop) = 1;
+        break;
+      }
+      missing = false;
+#pragma unroll
+      for (int p = 1; p < Q; ++p)
+        if (cross[p] && (w[p] >> 16) != tag) {
+          w[p] = mail_load(box + size_t(p - 1) * nodes);
+          missing |= (w[p] >> 16) != tag;
+        }
+    }
+#pragma unroll
+    for (int p = 1; p < Q; ++p)
+      if (cross[p]) v[p] = w[p] & 0xFFFFu;
+  };
+
+  NodeKeys<NB> keys = word_keys<NB>(a, t0);
+  for (uint32_t step = 0;; ++step) {
+    const uint32_t t = t0 + step, in = (step & 1) * buffer, out = buffer - in;
+    bool bad = false;
+    for (uint32_t j = warp; j < n; j += warps) {
+      const uint32_t r = run_of(j), l = 32 * r + lane, node = a0 + l;
+      const bool active = l < P;
+      const uint32_t x0 = xs[r];
+      uint32_t x = x0 + lane;
+      if (x >= a.Lx) x -= a.Lx;
+      const uint32_t reach = Q == 9 && (x0 == 0 || x0 + 32 >= a.Lx) ? 2 * a.Lx : near;
+      // every neighbour of the run's nodes in this share
+      const bool inner = 32 * r >= reach && 32 * r + 31 + reach < P && 32 * r + a0 >= reach && 32 * r + a0 + 31 + reach < nodes;
+      uint32_t v[Q], m[Q], post[Q];
+#pragma unroll
+      for (int i = 0; i < Q; ++i) v[i] = active ? planes[in + i * stride + l] : 0u;
+      Around o = around(node, x);
+      if (!inner && step > 0) take_mail(o, node, active, ra.tag + step - 1, step & 1, v);
+      // the flip F_i(n) = n_{-i}: velocity i of the collision reads plane -i
+#pragma unroll
+      for (int i = 0; i < Q; ++i) m[i] = a.flip ? v[opposite(i)] : v[i];
+      collide_warp<Q, 4 * THREADS, kStepRing, true>(a, keys, to, tr, ta, words, 4 * threadIdx.x, node, m, post);
+      if (active) {
+        uint32_t high = 0;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) high |= post[i];
+        bad |= high > 65535u;
+        planes[out + l] = uint16_t(post[0]);
+        if (inner) {
+#pragma unroll
+          for (int i = 1; i < Q; ++i) planes[out + i * stride + (neighbour(o, node, i) - a0)] = uint16_t(post[i]);
+        } else {
+          uint32_t* const box = ra.mail + size_t((step + 1) & 1) * (Q - 1) * nodes;
+          const uint32_t tag = (ra.tag + step) << 16;
+#pragma unroll
+          for (int i = 1; i < Q; ++i) {
+            const uint32_t d = neighbour(o, node, i);
+            if (d - a0 < P) planes[out + i * stride + (d - a0)] = uint16_t(post[i]);
+            else mail_store(box + (size_t(i - 1) * nodes + d), tag | (post[i] & 0xFFFFu));
+          }
+        }
+      }
+    }
+    if (bad) atomicMin(fail, static_cast<unsigned long long>(t));
+    keys = word_keys<NB>(a, t + 1);
+    __syncthreads();
+    if (stop || step + 1 == T) break;
+  }
+  if (stop) return;
+  for (uint32_t r = warp; r < n; r += warps) {
+    const uint32_t l = 32 * r + lane, node = a0 + l;
+    const bool active = l < P;
+    uint32_t x = xs[r] + lane, v[Q];
+    if (x >= a.Lx) x -= a.Lx;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) v[i] = active ? planes[(T & 1) * buffer + i * stride + l] : 0u;
+    take_mail(around(node, x), node, active, ra.tag + T - 1, T & 1, v);
+    if (active)
+#pragma unroll
+      for (int i = 0; i < Q; ++i) buf1[size_t(i) * nodes + node] = uint16_t(v[i]);
+  }
+}
+
 static RunShape run_shape(int Q, const StepArgs& a, uint64_t nodes, uint32_t sms) {
   const bool tables = run_tables(Q, a);
   if (nodes <= uint64_t(sms) * 128) return {run_fn<128>(Q, tables), 128};
   if (Q == 9 || nodes <= uint64_t(sms) * 512) return {run_fn<512>(Q, tables), 512};
   return {run_fn<1024>(Q, tables), 1024};
+}
+
+template <int THREADS>
+static const void* resident_fn(int Q) {
+  if (Q == 3) return reinterpret_cast<const void*>(step_resident_kernel<3, THREADS>);
+  if (Q == 5) return reinterpret_cast<const void*>(step_resident_kernel<5, THREADS>);
+  if constexpr (THREADS <= 512) return reinterpret_cast<const void*>(step_resident_kernel<9, THREADS>);
+  return nullptr;
+}
+
+struct ResidentShape {
+  const void* fn;
+  int threads;            // of the instantiation; a block has no more warps than runs
+  uint32_t blocks, runs;  // runs of the largest share
+  size_t smem;
+};
+constexpr size_t kResidentSmem = 227 * 1024 - 256;
+
+// One share per SM, in blocks of as few threads as give every node a lane (as run_shape); false:
+// the planes do not fit, the lattice is a cluster's, a run may span more than two rows, or a
+// D2Q9 block would have more than one run per warp (its eight words per node then cost more than
+// the barrier: 512^2 8.5 us per step / 7.5).
+static bool resident_shape(int Q, uint32_t Lx, uint64_t nodes, uint32_t sms, ResidentShape* r) {
+  if (Lx < 32 || nodes <= uint64_t(kClusterBlocks) * 512 || nodes >= (1u << 30)) return false;
+  const uint32_t runs = uint32_t((nodes + 31) / 32);
+  r->blocks = std::min(runs, sms);
+  r->runs = (runs + r->blocks - 1) / r->blocks;
+  if (Q == 9 && r->runs > 16) return false;
+  r->threads = r->runs <= 4 ? 128 : (r->runs <= 16 ? 512 : 1024);
+  r->fn = r->threads == 128 ? resident_fn<128>(Q) : r->threads == 512 ? resident_fn<512>(Q) : resident_fn<1024>(Q);
+  r->smem = sizeof(uint32_t) * (run_table_words(Q) + size_t(kStepRing) * r->threads + r->runs) +
+            sizeof(uint16_t) * 2 * Q * 32 * size_t(r->runs);
+  return r->smem <= kResidentSmem;
+}
+
+size_t step_resident_mail_words(int Q, uint32_t Lx, uint64_t nodes, uint32_t sms) {
+  ResidentShape r;
+  return resident_shape(Q, Lx, nodes, sms, &r) ? 2 * size_t(Q - 1) * nodes : 0;
+}
+
+cudaError_t launch_step_resident(int Q, const StepArgs& a, const uint16_t* buf0, uint16_t* buf1, uint32_t t, uint32_t T,
+                                 unsigned long long* fail, unsigned long long* sync, uint32_t* mail, uint32_t tag,
+                                 uint32_t sms, cudaStream_t s) {
+  ResidentShape r;
+  if (!run_tables(Q, a) || !resident_shape(Q, a.Lx, uint64_t(a.Lx) * a.Ly, sms, &r)) return cudaErrorNotSupported;
+  StepArgs args = a;
+  ResidentArgs ra{mail, tag, 32 * r.runs, sync + 1};
+  void* p[] = {&args, &buf0, &buf1, &t, &T, &fail, &ra};
+  return cudaLaunchCooperativeKernel(r.fn, dim3(r.blocks), dim3(std::min<uint32_t>(r.threads, 32 * r.runs)), p, r.smem, s);
 }
 
 cudaError_t prepare_step_kernels(int Q) {
@@ -338,6 +577,9 @@ cudaError_t prepare_step_kernels(int Q) {
     set(run_fn<512>(Q, tables), 512);
     set(run_fn<1024>(Q, tables), 1024);
   }
+  for (const void* f : {resident_fn<128>(Q), resident_fn<512>(Q), resident_fn<1024>(Q)})
+    if (f && e == cudaSuccess)
+      e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kResidentSmem));
   for (int threads : {128, 256, 512}) {
     const void* f = cluster_fn(Q, threads);
     if (e == cudaSuccess)

@@ -28,6 +28,15 @@ cudaError_t prepare_step_kernels(int Q);  // opt in to the table block's shared 
 // a wait between blocks gave up
 cudaError_t launch_step_run(int Q, const StepArgs& a, uint16_t* buf0, uint16_t* buf1, uint32_t t, uint32_t T,
                             unsigned long long* fail, unsigned long long* sync, uint32_t sms, cudaStream_t s);
+// The same where all SMs hold the lattice's planes in shared memory: T steps (2 at least) from
+// step t, the state in buf0 (only read), the state after them in buf1, whatever T.  mail:
+// step_resident_mail_words words (0: the lattice does not fit), zeroed, in which no tag of
+// [tag, tag + T) stands yet; tag at least 1, tag + T at most 2^16.  sync as launch_step_run.
+// Should a step overflow, *fail is the first that does and buf1 holds nothing.
+size_t step_resident_mail_words(int Q, uint32_t Lx, uint64_t nodes, uint32_t sms);
+cudaError_t launch_step_resident(int Q, const StepArgs& a, const uint16_t* buf0, uint16_t* buf1, uint32_t t, uint32_t T,
+                                 unsigned long long* fail, unsigned long long* sync, uint32_t* mail, uint32_t tag,
+                                 uint32_t sms, cudaStream_t s);
 cudaError_t prepare_step_vec_kernels();
 uint32_t step_vec_width();  // nodes per thread of the default row-tiled step (rows must be a multiple)
 uint32_t step_vec_blocks_per_sm(int npt);
