@@ -48,6 +48,9 @@ struct ilg_ctx {
   int kernel_choice = -1;                  // single-step kernel chosen by ilg_autotune (-1: default)
   double omega_star = 0;
   unsigned long long* h_word = nullptr;    // pinned readback, kFailWords words
+  volatile uint32_t* h_mark = nullptr;     // pinned: StepArgs::mark
+  uint32_t* d_init = nullptr;              // tables of the initial state
+  size_t init_words = 0;
   std::string err;
 };
 
@@ -141,6 +144,7 @@ StepArgs step_args(const ilg_ctx* c) {
   a.key1 = uint32_t(c->p.seed >> 32);
   a.replica = c->p.replica;
   a.tables = c->d_tables;
+  a.mark = const_cast<uint32_t*>(c->h_mark);
   ilg::round_keys(c->p.seed, a.rk);
   return a;
 }
@@ -153,6 +157,7 @@ void free_ctx(ilg_ctx* c) {
   cudaFree(c->d_mass);
   cudaFree(c->d_proj);
   cudaFree(c->d_mail);
+  cudaFree(c->d_init);
   if (c->mode_cap > kFirstModes) cudaFreeHost(c->h_obs);
   if (c->h_word) cudaFreeHost(c->h_word);
 }
@@ -223,9 +228,13 @@ ilg_status ilg_create(const ilg_params* params, void* stream, ilg_ctx** out) {
   c->mail_words = step_resident_mail_words(c->Q, c->p.Lx, c->nodes, uint32_t(c->sms));
   if (c->mail_words && (e = dev_alloc(&c->d_mail, sizeof(uint32_t) * c->mail_words)) != cudaSuccess)
     return bail(e, "cudaMalloc mailbox");
-  if ((e = cudaMallocHost(&c->h_word, sizeof(unsigned long long) * (kFailWords + 1 + 4 * kFirstModes))) != cudaSuccess)
+  // the words of a failed step | mass and modes | the mark
+  const size_t host_words = kFailWords + 1 + 4 * kFirstModes;
+  if ((e = cudaMallocHost(&c->h_word, sizeof(unsigned long long) * (host_words + 1))) != cudaSuccess)
     return bail(e, "cudaMallocHost");
   c->h_obs = c->h_word + kFailWords;
+  c->h_mark = reinterpret_cast<uint32_t*>(c->h_word + host_words);
+  *c->h_mark = 0;
   c->mode_cap = kFirstModes;
 
   std::vector<uint32_t> tables(block_words, 0u);
@@ -259,25 +268,26 @@ ilg_status ilg_init(ilg_ctx* c) {
   InitTables it;
   std::string msg;
   if (!build_init_tables(c->p, c->Q, &it, &msg)) return fail(c, ILG_E_INVALID, msg);
-  uint32_t *d_off = nullptr, *d_cnt = nullptr, *d_tab = nullptr;
-  auto cleanup = [&]() {
-    cudaFree(d_off);
-    cudaFree(d_cnt);
-    cudaFree(d_tab);
-  };
-  cudaError_t e;
-  if ((e = dev_alloc(&d_off, sizeof(uint32_t) * it.offset.size())) != cudaSuccess ||
-      (e = dev_alloc(&d_cnt, sizeof(uint32_t) * it.count.size())) != cudaSuccess ||
-      (e = dev_alloc(&d_tab, sizeof(uint32_t) * it.table.size())) != cudaSuccess) {
-    cleanup();
-    return cuda_fail(c, e, "cudaMalloc init tables");
+  // offsets | counts | tables, in one array that the context keeps (its size follows from the
+  // parameters) and one copy
+  const size_t cells = it.offset.size();
+  std::vector<uint32_t> all;
+  all.reserve(2 * cells + it.table.size());
+  all.insert(all.end(), it.offset.begin(), it.offset.end());
+  all.insert(all.end(), it.count.begin(), it.count.end());
+  all.insert(all.end(), it.table.begin(), it.table.end());
+  cudaError_t e = cudaSuccess;
+  if (c->init_words < all.size()) {
+    cudaFree(c->d_init);
+    c->d_init = nullptr;
+    c->init_words = 0;
+    if ((e = dev_alloc(&c->d_init, sizeof(uint32_t) * all.size())) != cudaSuccess)
+      return cuda_fail(c, e, "cudaMalloc init tables");
+    c->init_words = all.size();
   }
-  if ((e = cudaMemcpyAsync(d_off, it.offset.data(), sizeof(uint32_t) * it.offset.size(), cudaMemcpyHostToDevice, c->stream)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(d_cnt, it.count.data(), sizeof(uint32_t) * it.count.size(), cudaMemcpyHostToDevice, c->stream)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(d_tab, it.table.data(), sizeof(uint32_t) * it.table.size(), cudaMemcpyHostToDevice, c->stream)) != cudaSuccess) {
-    cleanup();
+  const uint32_t *d_off = c->d_init, *d_cnt = d_off + cells, *d_tab = d_cnt + cells;
+  if ((e = cudaMemcpyAsync(c->d_init, all.data(), sizeof(uint32_t) * all.size(), cudaMemcpyHostToDevice, c->stream)) != cudaSuccess)
     return cuda_fail(c, e, "copy init tables");
-  }
   InitArgs a{};
   a.Lx = c->p.Lx;
   a.Ly = c->p.Ly;
@@ -298,12 +308,9 @@ ilg_status ilg_init(ilg_ctx* c) {
   a.offset = d_off;
   a.count = d_cnt;
   a.table = d_tab;
-  if ((e = launch_init(c->Q, a, uint32_t(it.table.size()), c->buf[c->cur], uint32_t(c->sms), c->stream)) != cudaSuccess) {
-    cleanup();
+  if ((e = launch_init(c->Q, a, uint32_t(it.table.size()), c->buf[c->cur], uint32_t(c->sms), c->stream)) != cudaSuccess)
     return cuda_fail(c, e, "init kernel");
-  }
   e = cudaStreamSynchronize(c->stream);
-  cleanup();
   if (e != cudaSuccess) return cuda_fail(c, e, "init kernel");
   c->t = 0;
   c->has_state = true;
@@ -541,6 +548,14 @@ ilg_status ilg_step(ilg_ctx* c, uint32_t T) {
     const cudaError_t e = launch_singles(c, kind, a, c->buf, cur, t, n, c->d_fail, &singles);
     if (e != cudaSuccess) return cuda_fail(c, e, "step kernel");
   }
+  ILG_CUDA(c, cudaStreamSynchronize(c->stream), "step");
+  if (*c->h_mark == 0) {
+    c->cur = cur;
+    c->t = t0 + T;
+    return ILG_OK;
+  }
+  // a step overflowed, or a wait gave up
+  *c->h_mark = 0;
   ILG_CUDA(c, cudaMemcpyAsync(c->h_word, c->d_fail, sizeof(unsigned long long) * kFailWords, cudaMemcpyDeviceToHost,
                               c->stream),
            "read overflow word");
@@ -672,6 +687,7 @@ ilg_status ilg_autotune(ilg_ctx* c, uint32_t trial_steps, ilg_tuning* out) {
     e = trial(cand, &res.ms_per_step[cand]);
   }
   release();
+  *c->h_mark = 0;  // (a trial may have overflowed)
   if (e != cudaSuccess) return cuda_fail(c, e, "autotune trial");
   int best = -1;
   for (int k = 0; k < kCandidates; ++k)

@@ -43,7 +43,22 @@ struct StepArgs {
   uint32_t replica;
   const uint32_t* tables;   // device, kDevBlockWords words (layout above)
   uint32_t rk[20];          // round keys (key0 + r W0, key1 + r W1), r = 0..9
+  uint32_t* mark;           // a context's steps: mapped host word, set when a step overflows or a
+                            //    wait gives up (the host then reads which), so that no copy has
+                            //    to follow: behind a kernel the copy engine looks only every 12 us
+                            //    whether it is done (us per call, copy / mark: 300 x 200, 1 step
+                            //    24 / 14, 2 24.6 / 17)
 };
+
+// The step t of a context overflows.
+__device__ __forceinline__ void note_overflow(const StepArgs& a, unsigned long long* fail, uint32_t t) {
+  atomicMin(fail, static_cast<unsigned long long>(t));
+  *const_cast<volatile uint32_t*>(a.mark) = 1;
+}
+__device__ __forceinline__ void note_gave_up(const StepArgs& a, unsigned long long* word) {
+  atomicExch(word, 1ull);
+  *const_cast<volatile uint32_t*>(a.mark) = 1;
+}
 
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11): ten rounds of two 32x32->64
 // multiplies, the high halves xored with the other counter words and the round key,

@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       base += stride;
     }
     if (bad) {
-      atomicMin(fail, static_cast<unsigned long long>(t));
+      note_overflow(a, fail, t);
       __threadfence();
       atomicOr(sync, kRunMark);
     }
@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     if (threadIdx.x == 0) {
       const unsigned long long v = run_wait(sync, (step + 1) * gridDim.x);
       if (v == ~0ull) {
-        atomicExch(sync + 1, 1ull);
+        note_gave_up(a, sync + 1);
         stop = 1;
       } else if (v >= kRunMark) {
         // a step overflowed: this one, or already the next one (a faster block's)
@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         asm volatile("st.shared::cluster.u16 [%0], %1;\n" ::"r"(dest[i] + out), "h"(uint16_t(post[i])) : "memory");
       }
       if (high > 65535u) {
-        atomicMin(fail, static_cast<unsigned long long>(t));
+        note_overflow(a, fail, t);
         cluster_mark(&mark, step, gridDim.x);
       }
     }
@@ -430,7 +430,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     for (int p = 1; p < Q; ++p) missing |= cross[p] && (w[p] >> 16) != tag;
     for (uint32_t polls = 0; missing; ++polls) {
       if (polls == kMailPolls || *reinterpret_cast<volatile int*>(&stop)) {
-        atomicExch(ra.gave_up, 1ull);
+        note_gave_up(a, ra.gave_up);
         *reinterpret_cast<volatile int*>(&stop) = 1;
         break;
       }
@@ -490,7 +490,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
       }
     }
-    if (bad) atomicMin(fail, static_cast<unsigned long long>(t));
+    if (bad) note_overflow(a, fail, t);
     keys = word_keys<NB>(a, t + 1);
     __syncthreads();
     if (stop || step + 1 == T) break;

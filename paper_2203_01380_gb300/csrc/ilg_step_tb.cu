@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(kTbThreads, 2) step_tb_kernel(StepArgs a, cons
     }
     __syncthreads();
   }
-  if (bad) atomicMin(fail, static_cast<unsigned long long>(t0));
+  if (bad) note_overflow(a, fail, t0);
 }
 
 }  // namespace

@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(kVecThreads, MINB)
       }
     }
   }
-  if (bad) atomicMin(fail, static_cast<unsigned long long>(t));
+  if (bad) note_overflow(a, fail, t);
 }
 
 // Warp-segment form of the same step: no block-wide exchange.  Each warp takes
@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(kVecThreads, MINB)
       }
     }
   }
-  if (bad) atomicMin(fail, static_cast<unsigned long long>(t));
+  if (bad) note_overflow(a, fail, t);
 }
 
 constexpr size_t kVecSmem = sizeof(uint32_t) * kDevStagedWords;

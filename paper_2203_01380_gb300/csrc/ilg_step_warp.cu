@@ -524,7 +524,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   cp_async_wait_all();  // the last (empty) group: nothing lands after the warp exits
   }
   if (bad) {
-    atomicMin(fail, static_cast<unsigned long long>(t));
+    note_overflow(a, fail, t);
     __threadfence();
     atomicOr(sync, kRunMark);
   }
@@ -533,7 +533,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   if (threadIdx.x == 0) {
     const unsigned long long v = run_barrier(sync, (step + 1) * gridDim.x);
     if (v == ~0ull) {
-      atomicExch(sync + 1, 1ull);
+      note_gave_up(a, sync + 1);
       stop = 1;
     } else if (v >= kRunMark) {
       // a step overflowed: this one, or already the next one (a faster block's)

