@@ -802,6 +802,7 @@ __global__ void __launch_bounds__(32 * kSumGroups) sums_kernel(const uint16_t* _
                                                                unsigned long long* __restrict__ mass, int want_rows) {
   __shared__ uint32_t red[kSumGroups][32 * VEC];
   __shared__ unsigned long long total[kSumGroups];
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (they wait for this kernel's end themselves)
   const uint32_t tx = threadIdx.x & 31u, ty = threadIdx.x >> 5;
   const uint64_t x = (uint64_t(blockIdx.x) * 32 + tx) * VEC;
   const size_t plane = size_t(Lx) * Ly;
@@ -1036,19 +1037,25 @@ __device__ __forceinline__ void block_sums(Sums& v, unsigned long long (*sw)[kPr
   }
 }
 
+// Cosine and sine of 2 pi m x / L.
+__device__ __forceinline__ void mode_at(uint32_t L, uint32_t m, uint64_t x, double& cs, double& sn) {
+  // (m, x < L)
+  const uint32_t r = L <= 65536u ? (m * uint32_t(x)) % L : uint32_t((uint64_t(m) * x) % L);
+  sincospi(2.0 * double(r) / double(L), &sn, &cs);
+}
+
+// cs, sn: the first entry's of this thread
 template <class Sums>
 __device__ __forceinline__ void project_chunk(const ProjArgs& a, const unsigned long long* S, uint32_t L, uint32_t m,
-                                              long long M, unsigned long long (*sw)[kProjWords], bool* last) {
+                                              long long M, double cs, double sn, unsigned long long (*sw)[kProjWords],
+                                              bool* last) {
   const uint32_t mi = blockIdx.y, P = gridDim.x;
   const uint32_t x0 = uint32_t(uint64_t(L) * blockIdx.x / P), x1 = uint32_t(uint64_t(L) * (blockIdx.x + 1) / P);
   Sums v;
-  for (uint64_t x = uint64_t(x0) + threadIdx.x; x < x1; x += kProjThreads) {
-    const long long D = static_cast<long long>(L) * static_cast<long long>(S[x]) - M;
-    // (m, x < L)
-    const uint32_t r = L <= 65536u ? (m * uint32_t(x)) % L : uint32_t((uint64_t(m) * x) % L);
-    double sn, cs;
-    sincospi(2.0 * double(r) / double(L), &sn, &cs);
-    v.add(cs, sn, D);
+  for (uint64_t x = uint64_t(x0) + threadIdx.x; x < x1;) {
+    v.add(cs, sn, static_cast<long long>(L) * static_cast<long long>(S[x]) - M);
+    x += kProjThreads;
+    if (x < x1) mode_at(L, m, x, cs, sn);
   }
   block_sums(v, sw);
   if (P > 1) {
@@ -1100,10 +1107,14 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(const __grid_cons
   const bool along_x = !((a.along_y[blockIdx.y / 32] >> (blockIdx.y % 32)) & 1u);
   const unsigned long long* S = along_x ? a.colsum : a.rowsum;
   const uint32_t L = along_x ? a.Lx : a.Ly, m = a.modes[blockIdx.y];
+  double cs, sn;
+  mode_at(L, m, min(uint64_t(L) * blockIdx.x / gridDim.x + threadIdx.x, uint64_t(L) - 1), cs, sn);
+  // (launched while the sums' kernel runs: from here on what it wrote is there)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const long long M = static_cast<long long>(*a.mass_in);
   // sum |D| <= 2 L M
-  if (__umul64hi(L, (unsigned long long)M) == 0) project_chunk<FixedSums>(a, S, L, m, M, sw, &last);
-  else project_chunk<DoubleSums>(a, S, L, m, M, sw, &last);
+  if (__umul64hi(L, (unsigned long long)M) == 0) project_chunk<FixedSums>(a, S, L, m, M, cs, sn, sw, &last);
+  else project_chunk<DoubleSums>(a, S, L, m, M, cs, sn, sw, &last);
 }
 
 cudaError_t launch_project(const ProjWork& w, uint32_t Lx, uint32_t Ly, const int32_t* modes, uint32_t nmodes,
@@ -1131,9 +1142,20 @@ cudaError_t launch_project(const ProjWork& w, uint32_t Lx, uint32_t Ly, const in
     }
     const uint32_t P = uint32_t(std::min<uint64_t>(std::max<uint32_t>(1, kProjBlocks / a.nmodes),
                                                    (uint64_t(L) + kProjThreads - 1) / kProjThreads));
-    project_kernel<<<dim3(P, a.nmodes), kProjThreads, 0, s>>>(a);
+    // the first launch begins, and makes its first sines and cosines, while the sums' kernel runs
+    // (us per call of the observables: 1024^2 33.6 -> 28.7, 256 nodes 27.6 -> 25.6)
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3(P, a.nmodes);
+    cfg.blockDim = dim3(kProjThreads);
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = k == 0 ? 1 : 0;
+    if (const cudaError_t e = cudaLaunchKernelEx(&cfg, project_kernel, a); e != cudaSuccess) return e;
   }
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 // --------------------------------------------------------------------------
