@@ -7,12 +7,14 @@
 // block ran it or on the other replicas of the batch.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "ilg_batch.h"
 #include "ilg_collide.cuh"
 #include "ilg_device.cuh"
 #include "ilg_fixed.cuh"
+#include "ilg_sync.cuh"
 
 namespace ilg {
 
@@ -375,6 +377,313 @@ __global__ void __launch_bounds__(REC || STATES ? BatchShape<THREADS>::kMost : T
   }
 }
 
+// --- a ring split between the blocks of a cluster ----------------------------
+//
+// Where there are fewer rings than half of the SMs, a ring's nodes are split between the
+// blocks of a cluster, one block per SM.  A block keeps its own nodes and a halo of 8 to 23
+// nodes on both sides, which it advances as well (a node's random words depend on the node
+// and the step alone); with every step the outermost nodes of the halo lapse, and when it is
+// used up the neighbours' nodes come through the cluster's shared memory.  So the blocks
+// meet once in 8 to 23 steps and not in each: occupations sent to the neighbour in every
+// step, as words with the step's tag, cost 0.4 us per step (rings of 64 nodes 1.09 us per
+// step instead of 0.69).
+// Bound as before by integer issue for long shares and a node's chain of draws for short
+// ones.  Us per step, one block per ring / split: one ring of 8192 nodes at 50 per velocity
+// 15.1 / 1.8, 18 rings of up to 8192 15.1 / 3.6, 38 of 4000 6.2 / 2.9, 76 of 1000 1.9 / 1.4;
+// with statistics 12 rings of 1000 2.58 / 1.16, 70 of 320 1.03 / 0.93; one ring of 256 with
+// its states 1.01 / 0.89.  Rings below 256 nodes gain nothing (128: 0.90 / 0.92, 64: 0.81 /
+// 0.89) and stay in one block.
+
+constexpr uint32_t kSplitFrom = 256;  // nodes of the batch's longest ring
+constexpr uint32_t kMostHalo = 24;
+
+struct ShareShared {
+  uint32_t fail;  // first step that would overflow
+  unsigned long long mass;
+  long long c[4];                        // sums of the mode's trigonometric values
+  // nodes that came from the left, from the right neighbour, by the exchange's parity: a
+  // neighbour writes one again after the next exchange, which all reach behind their reading
+  uint16_t mail[2][2][3 * kMostHalo];
+  BatchStepKeys keys[2][32];
+};
+
+__device__ __forceinline__ uint32_t mapa(const void* p, uint32_t rank) {
+  uint32_t at;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(at) : "r"(uint32_t(__cvta_generic_to_shared(p))), "r"(rank));
+  return at;
+}
+
+// A block's part of a ring: its own nodes lo .. lo + n - 1 and `halo` nodes on both sides,
+// local nodes 0 .. n + 2 halo - 1 of planes of `stride` nodes.
+struct Share {
+  uint32_t lo, n, halo, stride;
+  uint32_t left, right;  // the neighbours' ranks
+};
+
+// The neighbours' nodes beside the block's own.
+// (threads: those that work on the share; none in a block without nodes)
+__device__ __forceinline__ void exchange(const Share& h, uint16_t* src, ShareShared& sh, uint32_t parity, uint32_t threads) {
+  const uint32_t H = h.halo, items = threadIdx.x < threads ? 6 * H : 0;
+  for (uint32_t j = threadIdx.x; j < items; j += threads) {
+    const uint32_t side = j >= 3 * H, q = j - side * 3 * H, v = q / H, c = q - v * H;  // the first nodes go left, the last right
+    const uint32_t at = mapa(&sh.mail[parity][side ^ 1][q], side ? h.right : h.left);
+    asm volatile("st.shared::cluster.u16 [%0], %1;\n" ::"r"(at), "h"(src[v * h.stride + c + (side ? h.n : H)]) : "memory");
+  }
+  cluster_arrive();
+  cluster_wait();
+  for (uint32_t j = threadIdx.x; j < items; j += threads) {
+    const uint32_t side = j >= 3 * H, q = j - side * 3 * H, v = q / H, c = q - v * H;
+    src[v * h.stride + c + (side ? H + h.n : 0)] = sh.mail[parity][side][q];
+  }
+  __syncthreads();
+}
+
+// T steps of a share (see run_ring); src holds the state of its own nodes afterwards.  A
+// step that would overflow is marked and the share goes on with occupations cut to 16 bits:
+// the ring's blocks then start again and stop before that step.  The recording warps add
+// their sums of a state to the record in memory (parts as in ModeSums; zero at the start).
+template <bool REC, bool STATES, bool TABLES, class Tab>
+__device__ __forceinline__ void run_share(const BatchArgs& b, const StepArgs& a, const ReplicaDesc& d, uint32_t r,
+                                          const Share& h, uint32_t T, const uint32_t* tables, const Tab& to, const Tab& tr,
+                                          unsigned char* words, ShareShared& sh, uint16_t*& src, uint16_t* dst,
+                                          uint32_t colliders, uint32_t recorders) {
+  constexpr uint32_t S = 4 * 1024;
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+  const uint32_t H = h.halo, n = h.n, P = h.stride, N = n + 2 * H, L = d.L;
+  const auto bar = [&]() { asm volatile("bar.sync 1, %0;" ::"r"((colliders + recorders) * 32) : "memory"); };
+  uint32_t s = 0, since = 0, parity = 0;  // steps since the last exchange
+  const auto meet = [&]() {
+    if (since == H && H) {
+      exchange(h, src, sh, parity, (colliders + recorders) * 32);
+      parity ^= 1;
+      since = 0;
+    }
+  };
+  const auto turn = [&]() {
+    uint16_t* tmp = src;
+    src = dst;
+    dst = tmp;
+    since += 1;
+  };
+  if (warp >= colliders + recorders) {
+    // nothing to do but the exchanges
+    for (; s < T; ++s) {
+      meet();
+      turn();
+    }
+    return;
+  }
+  if constexpr (REC || STATES) {
+    if (warp >= colliders) {
+      const longlong2* trig = REC ? b.trig + d.state_off / 3 + h.lo : nullptr;
+      unsigned long long* const rec =
+          REC ? reinterpret_cast<unsigned long long*>(b.record) + size_t(r) * (size_t(b.T) + 1) * 4 : nullptr;
+      for (;; ++s) {
+        if (s < T) meet();
+        ModeSums ms;
+        if constexpr (REC) ms.clear();
+        uint16_t* const rs = STATES && s > 0 ? b.states + d.state_off * b.T + size_t(s - 1) * 3 * L + h.lo : nullptr;
+#pragma unroll 4
+        for (uint32_t i = 32 * (warp - colliders) + lane; i < n; i += 32 * recorders) {
+          const uint32_t m0 = src[H + i], m1 = src[P + H + i], m2 = src[2 * P + H + i];
+          if constexpr (REC) ms.add(trig[i], m0 + m1 + m2);
+          if constexpr (STATES) {
+            if (s > 0) {
+              rs[i] = uint16_t(m0);
+              rs[L + i] = uint16_t(m1);
+              rs[2 * L + i] = uint16_t(m2);
+            }
+          }
+        }
+        if constexpr (REC) {
+          const long long v = ms.warp_sum(lane);
+          if ((lane & 7) == 0) atomicAdd(rec + 4 * size_t(s) + (lane >> 3), (unsigned long long)v);
+        }
+        if (s == T) return;
+        bar();
+        turn();
+      }
+    }
+  }
+  WordKeys k;
+  k.slot.A = uint32_t((uint64_t(0xCD9E8D57u) * a.replica) >> 32) ^ a.rk[0];
+  k.ext_e = uint32_t(uint64_t(0xCD9E8D57u) * a.replica) ^ a.rk[2];
+  // the flip F_i(n) = n_{-i}: velocity i of the collision reads plane -i
+  const uint32_t p1 = d.flip ? 2 * P : P, p2 = d.flip ? P : 2 * P;
+  const uint32_t past = H ? P - 1 : 0, before = H ? P - 1 : N - 1;  // a spare node, or the ring's other end
+  for (; s < T; ++s) {
+    meet();
+    {
+      const uint4* q = reinterpret_cast<const uint4*>(&sh.keys[(s >> 5) & 1][s & 31]);
+      const uint4 k0 = q[0], k1 = q[1];
+      k.slot.G = k0.x;
+      k.slot.H[0] = k0.y;
+      k.slot.I[0] = k0.z;
+      k.slot.J[0] = k0.w;
+      k.slot.H[1] = k1.x;
+      k.slot.I[1] = k1.y;
+      k.slot.J[1] = k1.z;
+      k.ext_c = k1.w;
+    }
+    bool bad = false;
+    // without the `since` outermost nodes, whose neighbours' particles have not come
+    const uint32_t valid = H ? N - 2 * since : N;
+    for (uint32_t i0 = warp * 32; i0 < N; i0 += colliders * 32) {
+      const uint32_t i = i0 + lane;
+      const bool active = i - (H ? since : 0u) < valid;
+      uint32_t x = h.lo + i + (i < H && h.lo + i < H ? L : 0) - H;  // modulo L
+      x -= x >= L ? L : 0;
+      uint32_t m[3], post[3];
+      m[0] = active ? src[i] : 0u;
+      m[1] = active ? src[p1 + i] : 0u;
+      m[2] = active ? src[p2 + i] : 0u;
+      if (!TABLES && a.particle) collide_particle<3>(a, tables, x, d.t + s, m, post);
+      else collide_warp<3, S, kBatchExtWords, TABLES>(a, k, to, tr, tr, words, 4 * tid, x, m, post);
+      if (active) {
+        bad |= (post[0] | post[1] | post[2]) > 65535u && i - H < n;
+        dst[i] = uint16_t(post[0]);
+        dst[P + (i + 1 == N ? past : i + 1)] = uint16_t(post[1]);
+        dst[2 * P + (i == 0 ? before : i - 1)] = uint16_t(post[2]);
+      }
+    }
+    if (bad) atomicMin(&sh.fail, s);
+    bar();
+    if (warp == 0 && (s & 31) == 31) make_step_keys(a, d.t, s + 33, sh.keys);
+    turn();
+  }
+}
+
+// How a ring of L nodes lies in a cluster: parts of at least 32 nodes, and as many nodes
+// beside them as fill the last warp (8 to 23).  One part: no halo.
+struct RingSplit {
+  uint32_t parts, most, halo, tiles;
+};
+__host__ __device__ constexpr RingSplit ring_split(uint32_t L, uint32_t blocks) {
+  RingSplit q{L / 32 < blocks ? L / 32 : blocks, 0, 0, 0};
+  if (q.parts < 2) q.parts = 1;
+  q.most = (L + q.parts - 1) / q.parts;
+  q.tiles = (q.most + (q.parts > 1 ? 16 : 0) + 31) / 32;
+  q.halo = q.parts > 1 ? (32 * q.tiles - q.most) / 2 : 0;
+  return q;
+}
+
+// A cluster of `blocks` per ring.
+template <bool REC, bool STATES>
+__global__ void __launch_bounds__(1024, 1)
+    batch_cluster_kernel(const __grid_constant__ BatchArgs b, const __grid_constant__ StepArgs common, uint32_t blocks,
+                         uint32_t recorders) {
+  extern __shared__ uint4 smem4[];
+  uint32_t* tables = reinterpret_cast<uint32_t*>(smem4);
+  unsigned char* const words = reinterpret_cast<unsigned char*>(tables + kDevStagedWords);
+  uint16_t* const ring = reinterpret_cast<uint16_t*>(words + kBatchExtWords * 4 * 1024);  // 2 x 3 x stride
+  __shared__ ShareShared sh;
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, threads = blockDim.x;
+  const uint32_t r = blockIdx.x / blocks, rank = blockIdx.x % blocks;
+  const ReplicaDesc d = b.desc[r];
+  const uint32_t L = d.L;
+  StepArgs a = common;
+  a.omega_mode = d.omega_mode;
+  a.rest_mode = d.rest_mode;
+  a.replica = d.replica;
+  a.particle = d.particle;
+  const RingSplit q = ring_split(L, blocks);
+  Share h;
+  h.halo = q.halo;
+  h.stride = q.most + 2 * q.halo + 1;
+  h.lo = min(rank, q.parts) * L / q.parts;
+  h.n = min(rank + 1, q.parts) * L / q.parts - h.lo;
+  h.right = rank + 1 >= q.parts ? 0 : rank + 1;
+  h.left = rank == 0 ? q.parts - 1 : rank - 1;
+  const uint32_t N = h.n ? h.n + 2 * h.halo : 0;
+  if (tid == 0) {
+    sh.mass = 0ull;
+    sh.c[0] = sh.c[1] = sh.c[2] = sh.c[3] = 0;
+  }
+  {
+    const uint4* g4 = reinterpret_cast<const uint4*>(b.tables + size_t(r) * kDevBlockWords);
+#pragma unroll 8
+    for (uint32_t i = tid; i < kDevStagedWords / 4; i += threads) smem4[i] = g4[i];
+  }
+  uint16_t* const gs = b.state + d.state_off;
+  unsigned long long* const rec =
+      REC ? reinterpret_cast<unsigned long long*>(b.record) + size_t(r) * (size_t(b.T) + 1) * 4 : nullptr;
+  __syncthreads();
+  if constexpr (REC) {
+    // the whole ring's mass and the sums of the mode's values
+    const longlong2* trig = b.trig + d.state_off / 3;
+    unsigned long long part = 0;
+    ModeSums ms;
+    ms.clear();
+    for (uint32_t x = tid; x < L; x += threads) {
+      part += uint32_t(gs[x]) + gs[L + x] + gs[2 * L + x];
+      ms.add(trig[x], 1u);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(kFullWarp, part, o);
+    if (lane == 0 && part) atomicAdd(&sh.mass, part);
+    const long long v = ms.warp_sum(lane);
+    if ((lane & 7) == 0) atomicAdd(reinterpret_cast<unsigned long long*>(&sh.c[lane >> 3]), (unsigned long long)v);
+  }
+  const Alias8 to = Alias8::of(tables, 0), tr = Alias8::of(tables, 1);
+  const uint32_t colliders = min((N + 31) >> 5, threads / 32 - recorders);
+  uint32_t T = b.T;
+  uint16_t* src;
+  bool over = false;
+  for (;;) {
+    src = ring;
+    for (uint32_t i = tid; i < N; i += threads) {
+      const uint32_t x = (h.lo + i + L - h.halo) % L;
+#pragma unroll
+      for (uint32_t v = 0; v < 3; ++v) ring[v * h.stride + i] = gs[v * L + x];
+    }
+    if (tid == 0) sh.fail = ~0u;
+    if (warp == 0) {
+      make_step_keys(a, d.t, 0, sh.keys);
+      make_step_keys(a, d.t, 32, sh.keys);
+    }
+    if constexpr (REC)
+      for (size_t i = rank * threads + tid; i < (size_t(b.T) + 1) * 4; i += blocks * threads) rec[i] = 0ull;
+    cluster_arrive();
+    cluster_wait();
+    const bool plain = !a.particle && a.omega_mode == kTable && a.rest_mode == kTable;
+    if (plain) run_share<REC, STATES, true>(b, a, d, r, h, T, tables, to, tr, words, sh, src, ring + 3 * h.stride, colliders, h.n ? recorders : 0);
+    else run_share<REC, STATES, false>(b, a, d, r, h, T, tables, to, tr, words, sh, src, ring + 3 * h.stride, colliders, h.n ? recorders : 0);
+    cluster_arrive();
+    cluster_wait();
+    uint32_t fail = ~0u;
+    if (lane < blocks) asm volatile("ld.shared::cluster.u32 %0, [%1];\n" : "=r"(fail) : "r"(mapa(&sh.fail, lane)) : "memory");
+    fail = __reduce_min_sync(kFullWarp, fail);
+    if (fail == ~0u) break;
+    // once more from the start, as far as the ring goes
+    over = true;
+    T = fail;
+    cluster_arrive();  // all have read `fail`
+    cluster_wait();
+  }
+  for (uint32_t i = tid; i < h.n; i += threads) {
+#pragma unroll
+    for (uint32_t v = 0; v < 3; ++v) gs[v * L + h.lo + i] = src[v * h.stride + h.halo + i];
+  }
+  if constexpr (REC) {
+    // the parts' sums into the states' 128-bit sums, as write_sums
+    const __int128 M = (long long)sh.mass;
+    for (size_t i = rank * threads + tid; i < 2 * (size_t(T) + 1); i += blocks * threads) {
+      const uint32_t k = 2 * (i & 1);
+      const long long low = (long long)__ldcg(rec + 2 * i), high = (long long)__ldcg(rec + 2 * i + 1);
+      const __int128 S = (__int128(high) << 32) + low, Z = (__int128(sh.c[k + 1]) << 32) + sh.c[k];
+      const __int128 v = S * __int128(L) - Z * M;
+      rec[2 * i] = (unsigned long long)v;
+      rec[2 * i + 1] = (unsigned long long)(v >> 64);
+    }
+  }
+  if (rank == 0 && tid == 0) {
+    b.desc[r].t = d.t + T;
+    if (over) b.failed[r] = 1u;
+  }
+  cluster_arrive();  // no block leaves while another may read from it
+  cluster_wait();
+}
+
 // The instantiation for a shape and what it records.
 const void* batch_fn(int threads, bool rec, bool states) {
   auto pick = [&](auto shape) {
@@ -396,6 +705,13 @@ const void* batch_fn(int threads, bool rec, bool states) {
 // 1024-thread block per SM.  The autotuner (ilg_batch_autotune) may pick 256, 512 or 1024
 // threads instead.
 constexpr uint32_t kBatchSmallL = 1024;
+
+static const void* share_fn(bool rec, bool states) {
+  if (rec) return states ? reinterpret_cast<const void*>(batch_cluster_kernel<true, true>)
+                         : reinterpret_cast<const void*>(batch_cluster_kernel<true, false>);
+  return states ? reinterpret_cast<const void*>(batch_cluster_kernel<false, true>)
+                : reinterpret_cast<const void*>(batch_cluster_kernel<false, false>);
+}
 
 size_t batch_smem_bytes(uint32_t Lmax, int threads) {
   const uint32_t table = threads == 1024 ? BatchShape<1024>::kTableWords : BatchShape<256>::kTableWords;
@@ -420,8 +736,54 @@ cudaError_t prepare_batch_kernel(uint32_t Lmax, int threads) {
       const cudaError_t e = cudaFuncSetAttribute(batch_fn(threads, rec, states), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  int(kBatchSmemCap));
       if (e != cudaSuccess) return e;
+      const cudaError_t f = cudaFuncSetAttribute(share_fn(rec, states), cudaFuncAttributeMaxDynamicSharedMemorySize, int(kBatchSmemCap));
+      if (f != cudaSuccess) return f;
+      const cudaError_t g = cudaFuncSetAttribute(share_fn(rec, states), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (g != cudaSuccess) return g;
     }
   return cudaSuccess;
+}
+
+// (more than half of an SM's: a block has an SM to itself)
+static size_t share_smem(uint32_t Lmax, uint32_t blocks) {
+  const size_t n = sizeof(uint32_t) * (kDevStagedWords + size_t(kBatchExtWords) * 1024) +
+                   2 * 3 * sizeof(uint16_t) * (ring_split(Lmax, blocks).most + 2 * kMostHalo + 1);
+  return std::max<size_t>(n, 116 * 1024);
+}
+
+// The split form, where it is the better one and fits: the largest clusters (any number of
+// blocks up to 16) that are resident at the same time for all rings.  At least 256 threads
+// (they stage the tables); one recording warp for four colliding ones, at most 8: 9 rings of
+// up to 1000 nodes with states 1.52 us per step, with twice as many 1.53, with all 1.58.
+static bool launch_split(const BatchArgs& b, const StepArgs& common, int sms, cudaStream_t s) {
+  if (b.Lmax < kSplitFrom) return false;
+  const bool rec = b.record || b.states;
+  const void* fn = share_fn(b.record != nullptr, b.states != nullptr);
+  for (uint32_t blocks = std::min({16u, uint32_t(sms) / b.n, b.Lmax / 32}); blocks >= 2; --blocks) {
+    const uint32_t tiles = ring_split(b.Lmax, blocks).tiles;
+    uint32_t recorders = rec ? std::clamp((tiles + 1) / 4, 1u, 8u) : 0u;
+    const uint32_t rounds = (tiles + 31 - recorders) / (32 - recorders);
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = blocks;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(b.n * blocks);
+    cfg.blockDim = dim3(std::max(256u, ((tiles + rounds - 1) / rounds + recorders) * 32));
+    cfg.dynamicSmemBytes = share_smem(b.Lmax, blocks);
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int fit = 0;
+    if (cudaOccupancyMaxActiveClusters(&fit, fn, &cfg) == cudaSuccess && uint32_t(fit) >= b.n) {
+      BatchArgs ba = b;
+      StepArgs ca = common;
+      void* p[] = {&ba, &ca, &blocks, &recorders};
+      if (cudaLaunchKernelExC(&cfg, fn, p) == cudaSuccess) return true;
+    }
+    cudaGetLastError();
+  }
+  return false;
 }
 
 // Persistent grid: as many blocks as fit on every SM (shared memory and registers
@@ -429,6 +791,7 @@ cudaError_t prepare_batch_kernel(uint32_t Lmax, int threads) {
 // ring keeps equally busy (320 nodes on the 256-thread shape: 160 threads, two nodes each),
 // and the recording warps.
 cudaError_t launch_batch(const BatchArgs& b, const StepArgs& common, int sms, cudaStream_t s, int shape) {
+  if (launch_split(b, common, sms, s)) return cudaSuccess;
   const size_t smem = batch_smem_bytes(b.Lmax, shape);
   const bool rec = b.record != nullptr || b.states != nullptr;
   const uint32_t most = uint32_t(shape) / 32, tiles = (b.Lmax + 31) / 32;
