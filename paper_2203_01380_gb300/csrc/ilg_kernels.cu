@@ -26,8 +26,8 @@ namespace ilg {
 // once, in the 64-bit form whose draw takes two instructions fewer than the packed one
 // (29.1 against 31.0 us per step for two blocks of 512, 33 with packed tables).  Us per
 // step against one launch per step with a collision that loops per lane: 1024^2 at 50 per
-// velocity 25.0 / 37.3 (omega* 0.5), 15.7 / 26.8 (0.1); 1501 x 777 at 100 per velocity
-// 44.5 / 66; 1024^2 at 200 per velocity, omega* = 1, 83 / 241; 96 x 40 1.6 / 18.7.
+// velocity 24.3 / 37.3 (omega* 0.5), 15.25 / 26.8 (0.1); 1501 x 777 at 100 per velocity
+// 42.2 / 66; 1024^2 at 200 per velocity, omega* = 1, 80.5 / 241; 96 x 40 1.6 / 18.7.
 // --------------------------------------------------------------------------
 constexpr uint32_t kStepRing = 16;  // extension words per lane
 
@@ -60,7 +60,11 @@ __global__ void __launch_bounds__(THREADS, 1)
   const uint32_t stride = gridDim.x * THREADS;
   const uint32_t stride_y = stride / a.Lx, stride_x = stride - stride_y * a.Lx;
   const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t base0 = blockIdx.x * THREADS + (threadIdx.x - lane);  // the warp's first node
+  // the warp's first node: runs of 32 go to the blocks in turn, so that what is left for the
+  // last pass lies on all SMs and not on some with all their warps (1024^2 at 50 per velocity
+  // 24.3 instead of 25.0 us per step, 15.25 / 15.75 at omega* = 0.1; 1501 x 777 at 100 42.2 /
+  // 44.5; 2^20 nodes of D1Q3 23.7 / 25.3)
+  const uint32_t base0 = ((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32;
   const uint32_t y0 = (base0 + lane) / a.Lx, x0 = base0 + lane - y0 * a.Lx;
   // the launch-wide Philox rounds of a step, and the first node's words: made for the next
   // step between a block's arrival at the barrier and its wait there (1024^2 at 50 per
