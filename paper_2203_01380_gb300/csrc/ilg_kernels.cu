@@ -26,16 +26,19 @@ namespace ilg {
 // once, in the 64-bit form whose draw takes two instructions fewer than the packed one
 // (29.1 against 31.0 us per step for two blocks of 512, 33 with packed tables).  Us per
 // step against one launch per step with a collision that loops per lane: 1024^2 at 50 per
-// velocity 24.3 / 37.3 (omega* 0.5), 15.25 / 26.8 (0.1); 1501 x 777 at 100 per velocity
-// 42.2 / 66; 1024^2 at 200 per velocity, omega* = 1, 80.5 / 241; 96 x 40 1.6 / 18.7.
+// velocity 24.0 / 37.3 (omega* 0.5), 15.0 / 26.8 (0.1); 1501 x 777 at 100 per velocity
+// 41.8 / 66; 1024^2 at 200 per velocity, omega* = 1, 80.5 / 241; 96 x 40 1.6 / 18.7.
 // --------------------------------------------------------------------------
 constexpr uint32_t kStepRing = 16;  // extension words per lane
 
 __host__ __device__ constexpr uint32_t run_table_words(int Q) { return Q == 9 ? kDevBlockWords9 : kDevStagedWords; }
 
 // sync[0]: the barrier word, sync[1]: set to 1 when a wait gave up.  TABLES: the binomial
-// sampler with both probabilities strictly between 0 and 1; false: anything else.
-template <int Q, int THREADS, bool TABLES>
+// sampler with both probabilities strictly between 0 and 1; false: anything else.  Off: type
+// of a byte's place in a plane, 32 bits where that is enough (an add each for the five loads
+// and stores instead of two: 1024^2 at 50 per velocity 24.0 / 24.3 us per step, 15.0 / 15.25
+// at omega* = 0.1).
+template <int Q, int THREADS, bool TABLES, class Off>
 __global__ void __launch_bounds__(THREADS, 1)
     step_run_kernel(const __grid_constant__ StepArgs a, uint16_t* buf0, uint16_t* buf1, uint32_t t0, uint32_t T,
                     unsigned long long* fail, unsigned long long* sync) {
@@ -87,16 +90,21 @@ __global__ void __launch_bounds__(THREADS, 1)
     // nodes) with a carry instead of a division per node
     uint32_t base = base0, x = x0, y = y0;
     // the flip F_i(n) = n_{-i}: velocity i of the collision reads plane -i
-    const uint16_t* from[Q];
+    const unsigned char* from[Q];
+    unsigned char* to_plane[Q];
 #pragma unroll
-    for (int i = 0; i < Q; ++i) from[i] = in + (i == 0 || !a.flip ? i : (i & 1 ? i + 1 : i - 1)) * plane;
+    for (int i = 0; i < Q; ++i) {
+      from[i] = reinterpret_cast<const unsigned char*>(in + (i == 0 || !a.flip ? i : (i & 1 ? i + 1 : i - 1)) * plane);
+      to_plane[i] = reinterpret_cast<unsigned char*>(out + i * plane);
+    }
     while (base < nodes) {
       const uint32_t node = base + lane;
       const bool active = node < nodes && node >= base;
+      const Off off = Off(node) * 2;
       uint32_t m[Q], post[Q];
       // (through L2 only: another SM wrote these lines in the step before)
 #pragma unroll
-      for (int i = 0; i < Q; ++i) m[i] = active ? __ldcg(from[i] + node) : 0u;
+      for (int i = 0; i < Q; ++i) m[i] = active ? __ldcg(reinterpret_cast<const uint16_t*>(from[i] + off)) : 0u;
       if (!TABLES && a.particle) collide_particle<Q>(a, s, node, t, m, post);
       else if constexpr (kAhead) {
         SlotWords<NB> w = first;
@@ -110,21 +118,22 @@ __global__ void __launch_bounds__(THREADS, 1)
 #pragma unroll
         for (int i = 0; i < Q; ++i) high |= post[i];
         bad |= high > 65535u;
-        uint16_t* const o = out + node;  // row y starts at node - x
-        o[0] = uint16_t(post[0]);
-        const int64_t right = x + 1 == a.Lx ? -int64_t(x) : 1, left = x == 0 ? int64_t(a.Lx) - 1 : -1;
-        (o + plane)[right] = uint16_t(post[1]);
-        (o + 2 * plane)[left] = uint16_t(post[2]);
+        const auto put = [&](int i, Off at) { *reinterpret_cast<uint16_t*>(to_plane[i] + at) = uint16_t(post[i]); };
+        // (offsets modulo 2^32: row y starts at node - x)
+        const Off right = x + 1 == a.Lx ? Off(2) - Off(a.Lx) * 2 : Off(2), left = x == 0 ? Off(a.Lx) * 2 - 2 : Off(0) - 2;
+        put(0, off);
+        put(1, off + right);
+        put(2, off + left);
         if constexpr (Q >= 5) {
-          uint16_t* const up = out + (size_t(y + 1 == a.Ly ? 0 : y + 1) * a.Lx + x);
-          uint16_t* const down = out + (size_t(y == 0 ? a.Ly - 1 : y - 1) * a.Lx + x);
-          up[3 * plane] = uint16_t(post[3]);
-          down[4 * plane] = uint16_t(post[4]);
+          const Off row = Off(a.Lx) * 2, rows = Off(nodes) * 2;
+          const Off up = y + 1 == a.Ly ? off + row - rows : off + row, down = y == 0 ? off + rows - row : off - row;
+          put(3, up);
+          put(4, down);
           if constexpr (Q == 9) {
-            (up + 5 * plane)[right] = uint16_t(post[5]);
-            (down + 6 * plane)[left] = uint16_t(post[6]);
-            (down + 7 * plane)[right] = uint16_t(post[7]);
-            (up + 8 * plane)[left] = uint16_t(post[8]);
+            put(5, up + right);
+            put(6, down + left);
+            put(7, down + right);
+            put(8, up + left);
           }
         }
       }
@@ -174,17 +183,22 @@ struct RunShape {
   int threads;
 };
 
+template <int Q, int THREADS>
+static const void* run_of(bool tables, bool far) {
+  if constexpr (THREADS == (Q == 9 ? 512 : 1024)) {
+    if (far) return tables ? reinterpret_cast<const void*>(step_run_kernel<Q, THREADS, true, uint64_t>)
+                           : reinterpret_cast<const void*>(step_run_kernel<Q, THREADS, false, uint64_t>);
+  }
+  return tables ? reinterpret_cast<const void*>(step_run_kernel<Q, THREADS, true, uint32_t>)
+                : reinterpret_cast<const void*>(step_run_kernel<Q, THREADS, false, uint32_t>);
+}
+
+// far: planes of more than 2^32 bytes (the largest blocks only).
 template <int THREADS>
-static const void* run_fn(int Q, bool tables) {
-  if (Q == 3)
-    return tables ? reinterpret_cast<const void*>(step_run_kernel<3, THREADS, true>)
-                  : reinterpret_cast<const void*>(step_run_kernel<3, THREADS, false>);
-  if (Q == 5)
-    return tables ? reinterpret_cast<const void*>(step_run_kernel<5, THREADS, true>)
-                  : reinterpret_cast<const void*>(step_run_kernel<5, THREADS, false>);
-  if constexpr (THREADS <= 512)
-    return tables ? reinterpret_cast<const void*>(step_run_kernel<9, THREADS, true>)
-                  : reinterpret_cast<const void*>(step_run_kernel<9, THREADS, false>);
+static const void* run_fn(int Q, bool tables, bool far = false) {
+  if (Q == 3) return run_of<3, THREADS>(tables, far);
+  if (Q == 5) return run_of<5, THREADS>(tables, far);
+  if constexpr (THREADS <= 512) return run_of<9, THREADS>(tables, far);
   return nullptr;
 }
 
@@ -517,8 +531,9 @@ __global__ void __launch_bounds__(THREADS, 1)
 static RunShape run_shape(int Q, const StepArgs& a, uint64_t nodes, uint32_t sms) {
   const bool tables = run_tables(Q, a);
   if (nodes <= uint64_t(sms) * 128) return {run_fn<128>(Q, tables), 128};
-  if (Q == 9 || nodes <= uint64_t(sms) * 512) return {run_fn<512>(Q, tables), 512};
-  return {run_fn<1024>(Q, tables), 1024};
+  const bool far = nodes > (uint64_t(1) << 31);
+  if (Q == 9 || nodes <= uint64_t(sms) * 512) return {run_fn<512>(Q, tables, far), 512};
+  return {run_fn<1024>(Q, tables, far), 1024};
 }
 
 template <int THREADS>
@@ -580,6 +595,7 @@ cudaError_t prepare_step_kernels(int Q) {
     set(run_fn<128>(Q, tables), 128);
     set(run_fn<512>(Q, tables), 512);
     set(run_fn<1024>(Q, tables), 1024);
+    set(Q == 9 ? run_fn<512>(Q, tables, true) : run_fn<1024>(Q, tables, true), Q == 9 ? 512 : 1024);
   }
   for (const void* f : {resident_fn<128>(Q), resident_fn<512>(Q), resident_fn<1024>(Q)})
     if (f && e == cudaSuccess)
