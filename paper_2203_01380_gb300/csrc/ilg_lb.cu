@@ -159,7 +159,11 @@ __global__ void __launch_bounds__(lb_run_threads(Q, WIDE), WIDE ? 1 : 4)
   const size_t plane = nodes;
   constexpr uint32_t threads = lb_run_threads(Q, WIDE);
   const uint32_t stride = gridDim.x * threads, stride_y = stride / Lx, stride_x = stride - stride_y * Lx;
-  const uint32_t first = blockIdx.x * threads + threadIdx.x;
+  // Runs of 32 nodes go to the blocks in turn (wide blocks): what is left for the last pass then
+  // lies on all SMs (700^2 7.0 instead of 7.7 us per step, 1024^2 12.2 / 12.3; D2Q9 500^2 6.8 /
+  // 7.5).  With several narrow blocks on an SM it lies there anyway (300 x 200 2.68 / 2.63).
+  const uint32_t lane = threadIdx.x & 31u, run = WIDE ? (threadIdx.x >> 5) * gridDim.x + blockIdx.x : (blockIdx.x * threads + threadIdx.x) >> 5;
+  const uint32_t first = run * 32 + lane;
   const uint32_t y0 = first / Lx, x0 = first - y0 * Lx;
   for (uint32_t step = 0;; ++step) {
     const double* const in = (step & 1) ? f1 : f0;
