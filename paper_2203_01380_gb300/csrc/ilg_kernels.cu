@@ -64,10 +64,13 @@ __global__ void __launch_bounds__(THREADS, 1)
   const uint32_t stride_y = stride / a.Lx, stride_x = stride - stride_y * a.Lx;
   const uint32_t lane = threadIdx.x & 31u;
   // the warp's first node: runs of 32 go to the blocks in turn, so that what is left for the
-  // last pass lies on all SMs and not on some with all their warps (1024^2 at 50 per velocity
-  // 24.3 instead of 25.0 us per step, 15.25 / 15.75 at omega* = 0.1; 1501 x 777 at 100 42.2 /
-  // 44.5; 2^20 nodes of D1Q3 23.7 / 25.3)
-  const uint32_t base0 = ((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32;
+  // last pass lies on all SMs and not on some with all their warps (1501 x 777 at 100 per velocity
+  // 42.2 instead of 44.5 us per step, 2^20 nodes of D1Q3 23.7 / 25.3).  Four warps in a row take
+  // theirs in another order than the four before: with the same one a sub-partition meets the
+  // same part of a row each time, the crowded one of a sine (1024^2 at 50 +- 20, omega* = 0.5:
+  // 24.8 us per step, here 24.0; 15.6, here 15.3 at 0.1; 1024 nodes in a row per block 24.85, 16.0)
+  const uint32_t warp = threadIdx.x >> 5, place = (warp & ~3u) | ((warp + (warp >> 2)) & 3u);
+  const uint32_t base0 = (place * gridDim.x + blockIdx.x) * 32;
   const uint32_t y0 = (base0 + lane) / a.Lx, x0 = base0 + lane - y0 * a.Lx;
   // the launch-wide Philox rounds of a step, and the first node's words: made for the next
   // step between a block's arrival at the barrier and its wait there (1024^2 at 50 per
