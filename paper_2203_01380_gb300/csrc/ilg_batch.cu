@@ -134,6 +134,14 @@ __device__ __forceinline__ void make_step_keys(const StepArgs& a, uint32_t t0, u
   keys[(s0 >> 5) & 1][j] = BatchStepKeys{k.slot.G,    k.slot.H[0], k.slot.I[0], k.slot.J[0],
                                          k.slot.H[1], k.slot.I[1], k.slot.J[1], k.ext_c};
 }
+__device__ __forceinline__ void make_step_keys(const StepArgs& a, uint32_t t0, uint32_t s0, WordKeys (&keys)[2][32]) {
+  const uint32_t j = threadIdx.x & 31u;
+  keys[(s0 >> 5) & 1][j] = word_keys(a, t0 + s0 + j);
+}
+
+// The words a node is collided with: those in shared memory, or those held in registers.
+__device__ __forceinline__ const volatile WordKeys& step_words(const WordKeys& shared, const WordKeys&) { return shared; }
+__device__ __forceinline__ const WordKeys& step_words(const BatchStepKeys&, const WordKeys& held) { return held; }
 
 // Rings of a block: shared memory, the block's threads and how its words are kept.  Bound:
 // integer issue for long rings (see collide_warp), the latency of a step (its node's
@@ -163,8 +171,13 @@ struct BatchShape {
   static constexpr int kMost = THREADS + (THREADS == 256 ? 64 : 0);
 };
 
-// The shared memory of a batch block beside its dynamic part.
-template <int THREADS>
+// The shared memory of a batch block beside its dynamic part.  ALONE: a 256-thread block that
+// has an SM to itself (no more rings than SMs).  A step's launch-wide words are then read where
+// they are used: with few warps that is off the step's chain (one ring of 64 nodes with its
+// states 0.77 instead of 0.81 us per step, of 128 0.86 / 0.90); where warps keep the issue busy
+// the loads cost more than the registers (512 rings of 320 nodes 6.40 / 6.20 ms, 152 rings of
+// 8192 at 100 per velocity 22.8 / 21.7 us per step).
+template <int THREADS, bool ALONE>
 struct BatchShared {
   // states whose partial sums are written out together, and room for as many again
   static constexpr uint32_t kGroup = 8, kSlots = 2 * kGroup;
@@ -173,7 +186,7 @@ struct BatchShared {
   unsigned long long mass;
   long long c[4];  // sums of the mode's trigonometric values
   long long red[kSlots][4 * BatchShape<THREADS>::kRecorders];  // partial sums of the last states
-  BatchStepKeys keys[2][32];                                   // of 64 steps
+  std::conditional_t<ALONE, WordKeys, BatchStepKeys> keys[2][32];  // of 64 steps
 };
 
 // All steps of one ring that lies in src (3 planes of L; dst: the other buffer): the first
@@ -181,13 +194,13 @@ struct BatchShared {
 // state; STATES: every state to b.states) follow them and see a state's planes in the step
 // that reads them.  TABLES: see collide_warp (and the binomial sampler).  Returns the steps
 // done; src is the buffer that holds the state.
-template <int THREADS, bool REC, bool STATES, bool TABLES, class Tab>
+template <int THREADS, bool ALONE, bool REC, bool STATES, bool TABLES, class Tab>
 __device__ __forceinline__ uint32_t run_ring(const BatchArgs& b, const StepArgs& a, const ReplicaDesc& d, uint32_t r,
                                              const uint32_t* tables, const Tab& to, const Tab& tr, unsigned char* words,
-                                             BatchShared<THREADS>& sh, uint16_t*& src, uint16_t* dst, uint32_t colliders) {
+                                             BatchShared<THREADS, ALONE>& sh, uint16_t*& src, uint16_t* dst, uint32_t colliders) {
   constexpr uint32_t S = 4 * THREADS;
   constexpr uint32_t R = REC || STATES ? BatchShape<THREADS>::kRecorders : 0;
-  constexpr uint32_t kGroup = BatchShared<THREADS>::kGroup, kSlots = BatchShared<THREADS>::kSlots;
+  constexpr uint32_t kGroup = BatchShared<THREADS, ALONE>::kGroup, kSlots = BatchShared<THREADS, ALONE>::kSlots;
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   const uint32_t L = d.L, T = b.T;
   const uint64_t mass = sh.mass;
@@ -245,22 +258,23 @@ __device__ __forceinline__ uint32_t run_ring(const BatchArgs& b, const StepArgs&
       return s;
     }
   }
-  WordKeys k;
-  k.slot.A = uint32_t((uint64_t(0xCD9E8D57u) * a.replica) >> 32) ^ a.rk[0];
-  k.ext_e = uint32_t(uint64_t(0xCD9E8D57u) * a.replica) ^ a.rk[2];
+  WordKeys held;
+  held.slot.A = uint32_t((uint64_t(0xCD9E8D57u) * a.replica) >> 32) ^ a.rk[0];
+  held.ext_e = uint32_t(uint64_t(0xCD9E8D57u) * a.replica) ^ a.rk[2];
   for (; s < T; ++s) {
-    {
+    if constexpr (!ALONE) {
       const uint4* q = reinterpret_cast<const uint4*>(&sh.keys[(s >> 5) & 1][s & 31]);
       const uint4 k0 = q[0], k1 = q[1];
-      k.slot.G = k0.x;
-      k.slot.H[0] = k0.y;
-      k.slot.I[0] = k0.z;
-      k.slot.J[0] = k0.w;
-      k.slot.H[1] = k1.x;
-      k.slot.I[1] = k1.y;
-      k.slot.J[1] = k1.z;
-      k.ext_c = k1.w;
+      held.slot.G = k0.x;
+      held.slot.H[0] = k0.y;
+      held.slot.I[0] = k0.z;
+      held.slot.J[0] = k0.w;
+      held.slot.H[1] = k1.x;
+      held.slot.I[1] = k1.y;
+      held.slot.J[1] = k1.z;
+      held.ext_c = k1.w;
     }
+    const auto& k = step_words(sh.keys[(s >> 5) & 1][s & 31], held);
     bool bad = false;
     for (uint32_t x0 = warp * 32; x0 < L; x0 += colliders * 32) {
       const uint32_t x = x0 + lane;
@@ -291,7 +305,7 @@ __device__ __forceinline__ uint32_t run_ring(const BatchArgs& b, const StepArgs&
   return s;
 }
 
-template <int THREADS, bool REC, bool STATES>
+template <int THREADS, bool REC, bool STATES, bool ALONE = false>
 __global__ void __launch_bounds__(REC || STATES ? BatchShape<THREADS>::kMost : THREADS,
                                   REC || STATES ? 65536 / (64 * BatchShape<THREADS>::kMost) : BatchShape<THREADS>::kPerSm)
     batch_d1q3_kernel(const __grid_constant__ BatchArgs b, const __grid_constant__ StepArgs common) {
@@ -301,7 +315,7 @@ __global__ void __launch_bounds__(REC || STATES ? BatchShape<THREADS>::kMost : T
   uint32_t* tables = reinterpret_cast<uint32_t*>(smem4);
   unsigned char* const words = reinterpret_cast<unsigned char*>(tables + Shape::kTableWords);
   uint16_t* ring = reinterpret_cast<uint16_t*>(words + Shape::kRing * 4 * THREADS);  // 2 x 3 x Lmax
-  __shared__ BatchShared<THREADS> sh;
+  __shared__ BatchShared<THREADS, ALONE> sh;
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
   const uint32_t threads = blockDim.x;
 
@@ -364,8 +378,8 @@ __global__ void __launch_bounds__(REC || STATES ? BatchShape<THREADS>::kMost : T
       uint16_t* src = ring;
       const bool plain = !a.particle && a.omega_mode == kTable && a.rest_mode == kTable;
       const uint32_t done =
-          plain ? run_ring<THREADS, REC, STATES, true>(b, a, d, r, tables, to, tr, words, sh, src, ring + 3 * L, colliders)
-                : run_ring<THREADS, REC, STATES, false>(b, a, d, r, tables, to, tr, words, sh, src, ring + 3 * L, colliders);
+          plain ? run_ring<THREADS, ALONE, REC, STATES, true>(b, a, d, r, tables, to, tr, words, sh, src, ring + 3 * L, colliders)
+                : run_ring<THREADS, ALONE, REC, STATES, false>(b, a, d, r, tables, to, tr, words, sh, src, ring + 3 * L, colliders);
       // ring back to global memory; the replica's step counter moves on
       for (uint32_t i = tid; i < 3 * L; i += (colliders + R) * 32) gs[i] = src[i];
       if (tid == 0) {
@@ -390,8 +404,8 @@ __global__ void __launch_bounds__(REC || STATES ? BatchShape<THREADS>::kMost : T
 // Bound as before by integer issue for long shares and a node's chain of draws for short
 // ones.  Us per step, one block per ring / split: one ring of 8192 nodes at 50 per velocity
 // 15.1 / 1.8, 18 rings of up to 8192 15.1 / 3.6, 38 of 4000 6.2 / 2.9, 76 of 1000 1.9 / 1.4;
-// with statistics 12 rings of 1000 2.58 / 1.16, 70 of 320 1.03 / 0.93; one ring of 256 with
-// its states 1.01 / 0.89.  Rings below 256 nodes gain nothing (128: 0.90 / 0.92, 64: 0.81 /
+// with statistics 12 rings of 1000 2.58 / 1.11, 70 of 320 1.03 / 0.91; one ring of 256 with
+// its states 1.01 / 0.88.  Rings below 256 nodes gain nothing (128: 0.90 / 0.92, 64: 0.81 /
 // 0.89) and stay in one block.
 
 constexpr uint32_t kSplitFrom = 256;  // nodes of the batch's longest ring
@@ -404,7 +418,7 @@ struct ShareShared {
   // nodes that came from the left, from the right neighbour, by the exchange's parity: a
   // neighbour writes one again after the next exchange, which all reach behind their reading
   uint16_t mail[2][2][3 * kMostHalo];
-  BatchStepKeys keys[2][32];
+  WordKeys keys[2][32];
 };
 
 __device__ __forceinline__ uint32_t mapa(const void* p, uint32_t rank) {
@@ -505,26 +519,14 @@ __device__ __forceinline__ void run_share(const BatchArgs& b, const StepArgs& a,
       }
     }
   }
-  WordKeys k;
-  k.slot.A = uint32_t((uint64_t(0xCD9E8D57u) * a.replica) >> 32) ^ a.rk[0];
-  k.ext_e = uint32_t(uint64_t(0xCD9E8D57u) * a.replica) ^ a.rk[2];
   // the flip F_i(n) = n_{-i}: velocity i of the collision reads plane -i
   const uint32_t p1 = d.flip ? 2 * P : P, p2 = d.flip ? P : 2 * P;
   const uint32_t past = H ? P - 1 : 0, before = H ? P - 1 : N - 1;  // a spare node, or the ring's other end
   for (; s < T; ++s) {
     meet();
-    {
-      const uint4* q = reinterpret_cast<const uint4*>(&sh.keys[(s >> 5) & 1][s & 31]);
-      const uint4 k0 = q[0], k1 = q[1];
-      k.slot.G = k0.x;
-      k.slot.H[0] = k0.y;
-      k.slot.I[0] = k0.z;
-      k.slot.J[0] = k0.w;
-      k.slot.H[1] = k1.x;
-      k.slot.I[1] = k1.y;
-      k.slot.J[1] = k1.z;
-      k.ext_c = k1.w;
-    }
+    // (read where they are used: 0.93 instead of 0.98 us per step for 5 rings of 3000; in run_ring,
+    // whose shares keep the issue busy, 22.8 instead of 21.7 for 152 rings of 8192)
+    const volatile WordKeys& k = sh.keys[(s >> 5) & 1][s & 31];
     bool bad = false;
     // without the `since` outermost nodes, whose neighbours' particles have not come
     const uint32_t valid = H ? N - 2 * since : N;
@@ -685,17 +687,19 @@ __global__ void __launch_bounds__(1024, 1)
 }
 
 // The instantiation for a shape and what it records.
-const void* batch_fn(int threads, bool rec, bool states) {
-  auto pick = [&](auto shape) {
+const void* batch_fn(int threads, bool rec, bool states, bool alone) {
+  auto pick = [&](auto shape, auto own) {
     constexpr int N = decltype(shape)::value;
-    if (rec) return states ? reinterpret_cast<const void*>(batch_d1q3_kernel<N, true, true>)
-                           : reinterpret_cast<const void*>(batch_d1q3_kernel<N, true, false>);
-    return states ? reinterpret_cast<const void*>(batch_d1q3_kernel<N, false, true>)
-                  : reinterpret_cast<const void*>(batch_d1q3_kernel<N, false, false>);
+    constexpr bool A = decltype(own)::value;
+    if (rec) return states ? reinterpret_cast<const void*>(batch_d1q3_kernel<N, true, true, A>)
+                           : reinterpret_cast<const void*>(batch_d1q3_kernel<N, true, false, A>);
+    return states ? reinterpret_cast<const void*>(batch_d1q3_kernel<N, false, true, A>)
+                  : reinterpret_cast<const void*>(batch_d1q3_kernel<N, false, false, A>);
   };
-  if (threads == 256) return pick(std::integral_constant<int, 256>{});
-  if (threads == 512) return pick(std::integral_constant<int, 512>{});
-  return pick(std::integral_constant<int, 1024>{});
+  if (threads == 256)
+    return alone ? pick(std::integral_constant<int, 256>{}, std::true_type{}) : pick(std::integral_constant<int, 256>{}, std::false_type{});
+  if (threads == 512) return pick(std::integral_constant<int, 512>{}, std::false_type{});
+  return pick(std::integral_constant<int, 1024>{}, std::false_type{});
 }
 
 }  // namespace
@@ -733,9 +737,11 @@ cudaError_t prepare_batch_kernel(uint32_t Lmax, int threads) {
   if (!batch_shape_fits(Lmax, threads)) return cudaErrorInvalidValue;
   for (bool rec : {false, true})
     for (bool states : {false, true}) {
-      const cudaError_t e = cudaFuncSetAttribute(batch_fn(threads, rec, states), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 int(kBatchSmemCap));
-      if (e != cudaSuccess) return e;
+      for (bool alone : {false, true}) {
+        const cudaError_t e = cudaFuncSetAttribute(batch_fn(threads, rec, states, alone),
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, int(kBatchSmemCap));
+        if (e != cudaSuccess) return e;
+      }
       const cudaError_t f = cudaFuncSetAttribute(share_fn(rec, states), cudaFuncAttributeMaxDynamicSharedMemorySize, int(kBatchSmemCap));
       if (f != cudaSuccess) return f;
       const cudaError_t g = cudaFuncSetAttribute(share_fn(rec, states), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -802,7 +808,7 @@ cudaError_t launch_batch(const BatchArgs& b, const StepArgs& common, int sms, cu
   const uint32_t room = shape == 256 && b.n <= uint32_t(sms) ? most : most - recorders;
   const uint32_t rounds = (tiles + room - 1) / room;
   const int threads = int(((tiles + rounds - 1) / rounds + recorders) * 32);
-  const void* fn = batch_fn(shape, b.record != nullptr, b.states != nullptr);
+  const void* fn = batch_fn(shape, b.record != nullptr, b.states != nullptr, b.n <= uint32_t(sms));
   int per_sm = 1;
   const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem);
   if (e != cudaSuccess) return e;

@@ -5,7 +5,7 @@
 // and a barrier of all blocks separates the steps.  Each lattice keeps its own step counter,
 // replica word and two buffers, so its result is the one it would have had alone.
 // Bound: integer issue (see collide_warp; 70 % of it while many lattices run).  24 requests of
-// 64 to 1024 a side at 5 to 100 per velocity: 51.4 ms in these launches.  What a step's nodes
+// 64 to 1024 a side at 5 to 100 per velocity: 52 ms in these launches.  What a step's nodes
 // have in common (ten Philox words, ten planes) is read from shared memory where it is used:
 // those loads cost next to nothing beside the collision, while some 30 registers for them left it
 // short (55.2 ms; one lattice of 1024^2 at 50 per velocity 27.7 / 24.9 us per step, 17.9 / 15.4 at
