@@ -353,8 +353,8 @@ static bool run_tables(int Q, const StepArgs& a) {
 // there, since the shares may be steps apart by then.
 // Bound: integer issue; with few nodes per SM a word's way to L2 and back.  Us per step, buffers
 // in L2 and a barrier of all blocks / here: D2Q5 100^2 at 12 per velocity 2.09 / 1.43, 301 x 200
-// 2.58 / 1.88, 400^2 at 50 8.01 / 5.72, 512^2 at 50 8.13 / 7.25, 850^2 at 50 18.3 / 17.9; D1Q3
-// 65000 nodes at 30 2.46 / 1.54, 2^18 4.75 / 3.62, 2^20 13.3 / 12.0; D2Q9 200^2 3.15 / 2.45.
+// 2.58 / 1.78, 400^2 at 50 8.01 / 5.61, 512^2 at 50 8.13 / 7.00, 850^2 at 50 18.3 / 17.5; D1Q3
+// 65000 nodes at 30 2.46 / 1.46, 2^18 4.75 / 3.50, 2^20 13.3 / 12.0; D2Q9 200^2 3.15 / 2.43.
 // Packed tables and shorter rings of extension words, which would let the planes of 1024^2 fit,
 // cost there what the barrier takes (at 50 per velocity 24.9 / 25.7).  A pause between polls costs
 // more than the polls (301 x 200 at 50 per velocity 2.79, 3.9 with 20 ns).
@@ -468,9 +468,20 @@ __global__ void __launch_bounds__(THREADS, 1)
       if (cross[p]) v[p] = w[p] & 0xFFFFu;
   };
 
-  NodeKeys<NB> keys = word_keys<NB>(a, t0);
+  // A step's launch-wide Philox words: shares of several runs per warp (or nearly so) read them
+  // from shared memory, made there by one thread a step ahead, and have the registers for the
+  // collision (us per step: 513 x 512 at 12 per velocity 4.30 / 4.54 in registers, 768^2 at 10
+  // 7.4 / 7.8, 850^2 at 50 17.5 / 17.9); where a step is one node's chain they stay in registers
+  // (100^2 1.44 / 1.38; D2Q9 200^2 2.50 / 2.44).
+  constexpr bool kSharedWords = THREADS >= 512 && Q != 9;
+  __shared__ NodeKeys<NB> step_words[2];
+  NodeKeys<NB> held = word_keys<NB>(a, t0);
+  const bool maker = kSharedWords && threadIdx.x == blockDim.x - 1;
+  if (maker) step_words[0] = held;
+  if (kSharedWords) __syncthreads();
   for (uint32_t step = 0;; ++step) {
     const uint32_t t = t0 + step, in = (step & 1) * buffer, out = buffer - in;
+    if (maker) step_words[(step + 1) & 1] = word_keys<NB>(a, t + 1);
     bool bad = false;
     for (uint32_t j = warp; j < n; j += warps) {
       const uint32_t r = run_of(j), l = 32 * r + lane, node = a0 + l;
@@ -489,7 +500,12 @@ __global__ void __launch_bounds__(THREADS, 1)
       // the flip F_i(n) = n_{-i}: velocity i of the collision reads plane -i
 #pragma unroll
       for (int i = 0; i < Q; ++i) m[i] = a.flip ? v[opposite(i)] : v[i];
-      collide_warp<Q, 4 * THREADS, kStepRing, true>(a, keys, to, tr, ta, words, 4 * threadIdx.x, node, m, post);
+      if constexpr (kSharedWords) {
+        const volatile NodeKeys<NB>& shared = step_words[step & 1];
+        collide_warp<Q, 4 * THREADS, kStepRing, true>(a, shared, to, tr, ta, words, 4 * threadIdx.x, node, m, post);
+      } else {
+        collide_warp<Q, 4 * THREADS, kStepRing, true>(a, held, to, tr, ta, words, 4 * threadIdx.x, node, m, post);
+      }
       if (active) {
         uint32_t high = 0;
 #pragma unroll
@@ -512,7 +528,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       }
     }
     if (bad) note_overflow(a, fail, t);
-    keys = word_keys<NB>(a, t + 1);
+    if (!kSharedWords) held = word_keys<NB>(a, t + 1);
     __syncthreads();
     if (stop || step + 1 == T) break;
   }
