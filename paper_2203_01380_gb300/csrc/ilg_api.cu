@@ -412,9 +412,9 @@ uint64_t vec_warps(const ilg_ctx* c) { return uint64_t(c->sms) * 3 * 8; }
 // 5.4 / 5.3 / 5.7, 768^2 8.8 / 8.1 / 8.6, 1024^2 13.4 / 10.5 / 11.8, 1448^2 24.4 / 19.4 /
 // 18.1, 2048^2 45 / 33 / 30; D2Q9 (4-node) 1024^2 21 / 31, 1448^2 39 / 50, 2048^2 84 / 75.
 // With the planes in shared memory the node-parallel steps stay ahead for longer (10 per velocity,
-// omega_eff 1.8 / 1.5, node-parallel / 4-node: 640^2 5.9 / 6.1, 5.9 / 7.6; 768^2 7.76 / 7.75,
-// 7.8 / 9.6; D1Q3 2^19 5.1 / 5.7).
-constexpr uint64_t kRunNodesPerSm = 2048, kResidentNodesPerSm = 3072, kRunNodesPerSm9 = 16384, kWarp4NodesPerSm = 10240;
+// omega_eff 1.8 / 1.5, node-parallel / 4-node: 640^2 5.4 / 6.1, 5.4 / 7.6; 768^2 7.3 / 7.7,
+// 7.4 / 9.5; 864^2 8.9 / 7.8; D1Q3 2^19 4.8 / 5.6, 2^20 8.9 / 8.3).
+constexpr uint64_t kRunNodesPerSm = 2048, kResidentNodesPerSm = 4096, kRunNodesPerSm9 = 16384, kWarp4NodesPerSm = 10240;
 
 // Node-parallel steps that all SMs take with the planes in shared memory.  A launch reads the
 // planes in and writes them out again, which a few steps have to repay (us for 4 steps, buffers in
