@@ -736,10 +736,16 @@ ilg_status ilg_observables(ilg_ctx* c, const int32_t* modes, uint32_t nmodes, ui
     c->mode_cap = nmodes;
   }
   const uint32_t Lx = c->p.Lx, Ly = c->p.Ly;
-  const ilg_status st = queue_sums(c, want_rows);
-  if (st != ILG_OK) return st;
   const double* const res = reinterpret_cast<const double*>(c->h_obs + 1);
-  if (nmodes)
+  const bool small = nmodes && !col_sums && !row_sums && takes_small_project(Lx, Ly, nmodes);
+  if (!small) {
+    const ilg_status st = queue_sums(c, want_rows);
+    if (st != ILG_OK) return st;
+  }
+  if (small)
+    ILG_CUDA(c, launch_small_project(c->Q, c->buf[c->cur], Lx, Ly, modes, nmodes, const_cast<double*>(res), c->h_obs, c->stream),
+             "projection kernel");
+  else if (nmodes)
     ILG_CUDA(c, launch_project(ProjWork{c->d_col, c->d_row, c->d_mass, c->d_proj}, Lx, Ly, modes, nmodes,
                                const_cast<double*>(res), c->h_obs, c->stream),
              "projection kernel");

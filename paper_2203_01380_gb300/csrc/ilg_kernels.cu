@@ -1083,6 +1083,25 @@ __device__ __forceinline__ void mode_at(uint32_t L, uint32_t m, uint64_t x, doub
   sincospi(2.0 * double(r) / double(L), &sn, &cs);
 }
 
+// One warp: a mode's results from its sums (in lane 0).  Lane 0 takes the real part, lane 1 the
+// imaginary one: two divisions one after the other, not four.
+template <class Sums>
+__device__ __forceinline__ void write_mode(const ProjArgs& a, uint32_t mi, uint32_t L, const Sums& v) {
+  unsigned long long w[kProjWords];
+  v.pack(w);
+#pragma unroll
+  for (int i = 0; i < kProjWords; ++i) w[i] = __shfl_sync(0xFFFFFFFFu, w[i], 0);
+  const bool first = threadIdx.x == 0;
+  const double q = Sums::value(first ? w[0] : w[2], first ? w[1] : w[3]) / double(L);
+  const double re = __shfl_sync(0xFFFFFFFFu, q, 0), im = __shfl_sync(0xFFFFFFFFu, q, 1);
+  const double K = double(a.Lx) * double(a.Ly);
+  const double p = (first ? re * re + im * im : im) / (first ? K : K / 2.0);
+  if (threadIdx.x < 2) {
+    a.res[4 * mi + threadIdx.x] = q;
+    a.res[4 * mi + 3 - threadIdx.x] = p;  // S(k), amplitude
+  }
+}
+
 // cs, sn: the first entry's of this thread
 template <class Sums>
 __device__ __forceinline__ void project_chunk(const ProjArgs& a, const unsigned long long* S, uint32_t L, uint32_t m,
@@ -1118,22 +1137,9 @@ __device__ __forceinline__ void project_chunk(const ProjArgs& a, const unsigned 
     }
     block_sums(v, sw);
   }
-  // lane 0 the real part, lane 1 the imaginary one: two divisions one after the other, not four
   if (threadIdx.x < 32) {
-    unsigned long long w[kProjWords];
-    v.pack(w);
-#pragma unroll
-    for (int i = 0; i < kProjWords; ++i) w[i] = __shfl_sync(0xFFFFFFFFu, w[i], 0);
-    const bool first = threadIdx.x == 0;
-    const double q = Sums::value(first ? w[0] : w[2], first ? w[1] : w[3]) / double(L);
-    const double re = __shfl_sync(0xFFFFFFFFu, q, 0), im = __shfl_sync(0xFFFFFFFFu, q, 1);
-    const double K = double(a.Lx) * double(a.Ly);
-    const double p = (first ? re * re + im * im : im) / (first ? K : K / 2.0);
-    if (threadIdx.x < 2) {
-      a.res[4 * mi + threadIdx.x] = q;
-      a.res[4 * mi + 3 - threadIdx.x] = p;  // S(k), amplitude
-    }
-    if (first) {
+    write_mode(a, mi, L, v);
+    if (threadIdx.x == 0) {
       if (P > 1) a.ticket[mi] = 0;
       if (mi == 0) *a.mass_out = static_cast<unsigned long long>(M);
     }
@@ -1156,6 +1162,149 @@ __global__ void __launch_bounds__(kProjThreads) project_kernel(const __grid_cons
   else project_chunk<DoubleSums>(a, S, L, m, M, cs, sn, sw, &last);
 }
 
+// A launch's modes, modulo their sides' lengths; returns the longest side among them.
+static uint32_t set_modes(ProjArgs& a, const int32_t* modes) {
+  std::memset(a.along_y, 0, sizeof a.along_y);
+  uint32_t L = 0;
+  for (uint32_t j = 0; j < a.nmodes; ++j) {
+    const int32_t mx = modes[2 * j], my = modes[2 * j + 1];
+    const int64_t side = my == 0 ? a.Lx : a.Ly, m = my == 0 ? mx : my;
+    a.modes[j] = uint32_t((m % side + side) % side);
+    if (my != 0) a.along_y[j / 32] |= 1u << (j % 32);
+    L = std::max(L, uint32_t(side));
+  }
+  return L;
+}
+
+// --------------------------------------------------------------------------
+// a small lattice's mass and projections in one launch: a cluster of eight blocks per mode, each
+// with an eighth of the mode's side.  A block adds its nodes up in shared memory while its first
+// sines are made; with D(x) = L N(x) - M, the sums of c D are L S - M C (S = sum c N, C = sum c,
+// exact as the other form's), so the mass has to be known only in the end.
+// Bound: latency (a launch, the sines' double precision, a reduction, two divisions): a call
+// takes 23.0 us for 256 nodes where the two launches took 24.8 to 25.6.
+// --------------------------------------------------------------------------
+constexpr uint32_t kSmallProjBlocks = 8, kSmallProjThreads = 256, kSmallProjNodes = 16384, kSmallProjModes = 32;
+constexpr uint32_t kSmallProjSide = kSmallProjBlocks * kSmallProjThreads;  // at most one entry per thread
+
+struct SmallSums {
+  unsigned long long w[9];  // S, C (real, imaginary: low, high word each), mass
+  __device__ void add(const SmallSums& o) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const unsigned __int128 v = ((unsigned __int128)w[2 * k + 1] << 64 | w[2 * k]) +
+                                  ((unsigned __int128)o.w[2 * k + 1] << 64 | o.w[2 * k]);
+      w[2 * k] = (unsigned long long)v;
+      w[2 * k + 1] = (unsigned long long)(v >> 64);
+    }
+    w[8] += o.w[8];
+  }
+  __device__ void warp_sum() {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      SmallSums other;
+#pragma unroll
+      for (int i = 0; i < 9; ++i) other.w[i] = __shfl_down_sync(0xFFFFFFFFu, w[i], o);
+      add(other);
+    }
+  }
+  __device__ __int128 value(int k) const { return (__int128)((unsigned __int128)w[2 * k + 1] << 64 | w[2 * k]); }
+};
+
+template <int Q>
+__global__ void __launch_bounds__(kSmallProjThreads) small_project_kernel(const __grid_constant__ ProjArgs a,
+                                                                          const uint16_t* __restrict__ state) {
+  constexpr uint32_t kWarps = kSmallProjThreads / 32;
+  __shared__ uint32_t count[kSmallProjThreads];  // (at most 2048 nodes of a column: below 2^32)
+  __shared__ SmallSums parts[kSmallProjBlocks * kWarps];              // the first block's: all warps' sums
+  const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, mi = blockIdx.y, rank = blockIdx.x;
+  cluster_arrive();
+  const bool along_x = !((a.along_y[mi / 32] >> (mi % 32)) & 1u);
+  const uint32_t L = along_x ? a.Lx : a.Ly, m = a.modes[mi], nodes = a.Lx * a.Ly;
+  const uint32_t x0 = L * rank / kSmallProjBlocks, n = L * (rank + 1) / kSmallProjBlocks - x0;
+  count[tid] = 0;
+  // an entry's sine is made by the last threads first: other warps load meanwhile (23.0 / 23.9 us)
+  const uint32_t e0 = kSmallProjThreads - 1 - tid;
+  __syncthreads();
+  double cs = 0.0, sn = 0.0;
+  if (e0 < n) mode_at(L, m, x0 + e0, cs, sn);
+  const uint32_t items = along_x ? n * a.Ly : n * a.Lx;
+  for (uint32_t j = tid; j < items; j += kSmallProjThreads) {
+    const uint32_t row = j / (along_x ? n : a.Lx), at = j - row * (along_x ? n : a.Lx);
+    const uint32_t node = along_x ? row * a.Lx + x0 + at : x0 * a.Lx + j;
+    uint32_t v = 0;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) v += __ldcg(state + size_t(i) * nodes + node);
+    atomicAdd(&count[along_x ? at : row], v);
+  }
+  __syncthreads();
+  SmallSums v{};
+  const uint32_t N = e0 < n ? count[e0] : 0;
+  const long long c = fixed62(cs), sine = fixed62(sn);
+  v.w[8] = N;
+  const __int128 sums[4] = {__int128(c) * N, __int128(sine) * N, c, sine};
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    v.w[2 * k] = (unsigned long long)sums[k];
+    v.w[2 * k + 1] = (unsigned long long)(sums[k] >> 64);
+  }
+  v.warp_sum();
+  cluster_wait();  // the first block has started
+  {
+    uint32_t at;
+    asm("mapa.shared::cluster.u32 %0, %1, 0;\n" : "=r"(at) : "r"(uint32_t(__cvta_generic_to_shared(&parts[rank * kWarps + warp]))));
+    if (lane == 0)
+#pragma unroll
+      for (int i = 0; i < 9; ++i) asm volatile("st.shared::cluster.u64 [%0], %1;\n" ::"r"(at + 8 * i), "l"(v.w[i]) : "memory");
+  }
+  __syncwarp();
+  cluster_arrive();
+  cluster_wait();
+  if (rank != 0 || warp != 0) return;
+  v = parts[lane];
+  for (uint32_t k = lane + 32; k < kSmallProjBlocks * kWarps; k += 32) v.add(parts[k]);
+  v.warp_sum();
+  const __int128 M = (__int128)v.w[8];
+  FixedSums r;
+  r.re = v.value(0) * L - v.value(2) * M;
+  r.im = v.value(1) * L - v.value(3) * M;
+  write_mode(a, mi, L, r);
+  if (lane == 0 && mi == 0) *a.mass_out = v.w[8];
+}
+
+// (us per call, one launch / two: 256 nodes and one mode 23.0 / 24.8, 96 x 40 23.2 / 26.1, 128^2
+// 24.2 / 26.0, 16 modes 27.1 / 28.9, 60 35.5 / 35.6, 200 67 / 57; a side of 2000 25.2 / 28.0, of
+// 4096 28.4 / 27.4, of 5400 31.0 / 28.3)
+bool takes_small_project(uint32_t Lx, uint32_t Ly, uint32_t nmodes) {
+  return std::max(Lx, Ly) <= kSmallProjSide && uint64_t(Lx) * Ly <= kSmallProjNodes && nmodes <= kSmallProjModes;
+}
+
+cudaError_t launch_small_project(int Q, const uint16_t* state, uint32_t Lx, uint32_t Ly, const int32_t* modes,
+                                 uint32_t nmodes, double* res, unsigned long long* mass, cudaStream_t s) {
+  ProjArgs a{};
+  a.Lx = Lx;
+  a.Ly = Ly;
+  a.mass_out = mass;
+  const void* fn = Q == 3   ? reinterpret_cast<const void*>(small_project_kernel<3>)
+                   : Q == 5 ? reinterpret_cast<const void*>(small_project_kernel<5>)
+                            : reinterpret_cast<const void*>(small_project_kernel<9>);
+  a.nmodes = nmodes;
+  a.res = res;
+  set_modes(a, modes);
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = kSmallProjBlocks;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(kSmallProjBlocks, nmodes);
+  cfg.blockDim = dim3(kSmallProjThreads);
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  void* p[] = {&a, &state};
+  return cudaLaunchKernelExC(&cfg, fn, p);
+}
+
 cudaError_t launch_project(const ProjWork& w, uint32_t Lx, uint32_t Ly, const int32_t* modes, uint32_t nmodes,
                            double* res, unsigned long long* mass, cudaStream_t s) {
   ProjArgs a{};
@@ -1170,15 +1319,7 @@ cudaError_t launch_project(const ProjWork& w, uint32_t Lx, uint32_t Ly, const in
   for (uint32_t k = 0; k < nmodes; k += kProjModes) {
     a.nmodes = std::min(nmodes - k, kProjModes);
     a.res = res + size_t(4) * k;
-    std::memset(a.along_y, 0, sizeof a.along_y);
-    uint32_t L = 0;
-    for (uint32_t j = 0; j < a.nmodes; ++j) {
-      const int32_t mx = modes[2 * (k + j)], my = modes[2 * (k + j) + 1];
-      const int64_t side = my == 0 ? Lx : Ly, m = my == 0 ? mx : my;
-      a.modes[j] = uint32_t((m % side + side) % side);
-      if (my != 0) a.along_y[j / 32] |= 1u << (j % 32);
-      L = std::max(L, uint32_t(side));
-    }
+    const uint32_t L = set_modes(a, modes + 2 * size_t(k));
     const uint32_t P = uint32_t(std::min<uint64_t>(std::max<uint32_t>(1, kProjBlocks / a.nmodes),
                                                    (uint64_t(L) + kProjThreads - 1) / kProjThreads));
     // the first launch begins, and makes its first sines and cosines, while the sums' kernel runs
