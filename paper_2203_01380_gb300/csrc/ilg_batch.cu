@@ -8,7 +8,10 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <functional>
+#include <queue>
 #include <type_traits>
+#include <vector>
 
 #include "ilg_batch.h"
 #include "ilg_collide.cuh"
@@ -393,8 +396,8 @@ __global__ void __launch_bounds__(REC || STATES ? BatchShape<THREADS>::kMost : T
 
 // --- a ring split between the blocks of a cluster ----------------------------
 //
-// Where there are fewer rings than half of the SMs, a ring's nodes are split between the
-// blocks of a cluster, one block per SM.  A block keeps its own nodes and a halo of 8 to 23
+// Where a ring per block would leave SMs idle (few rings, or rings of unlike length), a ring's
+// nodes are split between the blocks of a cluster, one block per SM.  A block keeps its own nodes and a halo of 8 to 23
 // nodes on both sides, which it advances as well (a node's random words depend on the node
 // and the step alone); with every step the outermost nodes of the halo lapse, and when it is
 // used up the neighbours' nodes come through the cluster's shared memory.  So the blocks
@@ -403,7 +406,7 @@ __global__ void __launch_bounds__(REC || STATES ? BatchShape<THREADS>::kMost : T
 // step instead of 0.69).
 // Bound as before by integer issue for long shares and a node's chain of draws for short
 // ones.  Us per step, one block per ring / split: one ring of 8192 nodes at 50 per velocity
-// 15.1 / 1.8, 18 rings of up to 8192 15.1 / 3.6, 38 of 4000 6.2 / 2.9, 76 of 1000 1.9 / 1.4;
+// 15.1 / 1.75, 18 rings of up to 8192 15.1 / 2.5, 38 of 4000 6.2 / 2.9, 76 of 1000 1.9 / 1.4;
 // with statistics 12 rings of 1000 2.58 / 1.11, 70 of 320 1.03 / 0.91; one ring of 256 with
 // its states 1.01 / 0.88.  Rings below 256 nodes gain nothing (128: 0.90 / 0.92, 64: 0.81 /
 // 0.89) and stay in one block.
@@ -569,18 +572,23 @@ __host__ __device__ constexpr RingSplit ring_split(uint32_t L, uint32_t blocks) 
   return q;
 }
 
-// A cluster of `blocks` per ring.
-template <bool REC, bool STATES>
-__global__ void __launch_bounds__(1024, 1)
-    batch_cluster_kernel(const __grid_constant__ BatchArgs b, const __grid_constant__ StepArgs common, uint32_t blocks,
-                         uint32_t recorders) {
-  extern __shared__ uint4 smem4[];
+// One ring by `blocks` blocks of a cluster, of which this is number `rank`; ALONE: by one block
+// where blocks = 1.
+template <bool REC, bool STATES, bool ALONE>
+__device__ __forceinline__ void run_split(const BatchArgs& b, const StepArgs& common, uint32_t r, uint32_t blocks,
+                                          uint32_t rank, uint32_t recorders, uint4* smem4, ShareShared& sh) {
   uint32_t* tables = reinterpret_cast<uint32_t*>(smem4);
   unsigned char* const words = reinterpret_cast<unsigned char*>(tables + kDevStagedWords);
   uint16_t* const ring = reinterpret_cast<uint16_t*>(words + kBatchExtWords * 4 * 1024);  // 2 x 3 x stride
-  __shared__ ShareShared sh;
   const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, threads = blockDim.x;
-  const uint32_t r = blockIdx.x / blocks, rank = blockIdx.x % blocks;
+  const auto meet = [&] {
+    if (ALONE && blocks == 1) {
+      __syncthreads();
+    } else {
+      cluster_arrive();
+      cluster_wait();
+    }
+  };
   const ReplicaDesc d = b.desc[r];
   const uint32_t L = d.L;
   StepArgs a = common;
@@ -645,22 +653,20 @@ __global__ void __launch_bounds__(1024, 1)
     }
     if constexpr (REC)
       for (size_t i = rank * threads + tid; i < (size_t(b.T) + 1) * 4; i += blocks * threads) rec[i] = 0ull;
-    cluster_arrive();
-    cluster_wait();
+    meet();
     const bool plain = !a.particle && a.omega_mode == kTable && a.rest_mode == kTable;
     if (plain) run_share<REC, STATES, true>(b, a, d, r, h, T, tables, to, tr, words, sh, src, ring + 3 * h.stride, colliders, h.n ? recorders : 0);
     else run_share<REC, STATES, false>(b, a, d, r, h, T, tables, to, tr, words, sh, src, ring + 3 * h.stride, colliders, h.n ? recorders : 0);
-    cluster_arrive();
-    cluster_wait();
+    meet();
     uint32_t fail = ~0u;
-    if (lane < blocks) asm volatile("ld.shared::cluster.u32 %0, [%1];\n" : "=r"(fail) : "r"(mapa(&sh.fail, lane)) : "memory");
+    if (ALONE && blocks == 1) fail = sh.fail;
+    else if (lane < blocks) asm volatile("ld.shared::cluster.u32 %0, [%1];\n" : "=r"(fail) : "r"(mapa(&sh.fail, lane)) : "memory");
     fail = __reduce_min_sync(kFullWarp, fail);
     if (fail == ~0u) break;
     // once more from the start, as far as the ring goes
     over = true;
     T = fail;
-    cluster_arrive();  // all have read `fail`
-    cluster_wait();
+    meet();  // all have read `fail`
   }
   for (uint32_t i = tid; i < h.n; i += threads) {
 #pragma unroll
@@ -682,8 +688,45 @@ __global__ void __launch_bounds__(1024, 1)
     b.desc[r].t = d.t + T;
     if (over) b.failed[r] = 1u;
   }
-  cluster_arrive();  // no block leaves while another may read from it
-  cluster_wait();
+}
+
+// PULL: clusters of `blocks` pull the `split` longest rings one by one, then the others `blocks`
+// at a time, one per block.  Else every ring has a cluster.
+template <bool REC, bool STATES, bool PULL>
+__global__ void __launch_bounds__(1024, 1)
+    batch_cluster_kernel(const __grid_constant__ BatchArgs b, const __grid_constant__ StepArgs common, uint32_t blocks,
+                         uint32_t recorders, uint32_t split) {
+  extern __shared__ uint4 smem4[];
+  __shared__ ShareShared sh;
+  const uint32_t rank = blockIdx.x % blocks;
+  const auto meet = [] {
+    cluster_arrive();
+    cluster_wait();
+  };
+  if constexpr (!PULL) {
+    run_split<REC, STATES, false>(b, common, b.order[blockIdx.x / blocks], blocks, rank, recorders, smem4, sh);
+    meet();  // no block leaves while another may read from it
+  } else {
+    __shared__ uint32_t tasks[2];
+    meet();  // all blocks have started
+    for (uint32_t turn = 0;; turn ^= 1) {
+      if (rank == 0 && threadIdx.x < 32) {
+        const uint32_t lane = threadIdx.x;
+        uint32_t next = 0;
+        if (lane == 0) next = atomicAdd(b.counter, 1u);
+        next = __shfl_sync(kFullWarp, next, 0);
+        if (lane < blocks)
+          asm volatile("st.shared::cluster.u32 [%0], %1;\n" ::"r"(mapa(&tasks[turn], lane)), "r"(next) : "memory");
+      }
+      meet();  // (and all are done with the last task)
+      const uint32_t task = tasks[turn];
+      const bool alone = task >= split;
+      const uint64_t first = alone ? split + uint64_t(task - split) * blocks : task, at = first + (alone ? rank : 0);
+      if (first >= b.n) return;  // no block reads from another after this
+      if (at < b.n)
+        run_split<REC, STATES, true>(b, common, b.order[at], alone ? 1 : blocks, alone ? 0 : rank, recorders, smem4, sh);
+    }
+  }
 }
 
 // The instantiation for a shape and what it records.
@@ -710,11 +753,12 @@ const void* batch_fn(int threads, bool rec, bool states, bool alone) {
 // threads instead.
 constexpr uint32_t kBatchSmallL = 1024;
 
+template <bool PULL>
 static const void* share_fn(bool rec, bool states) {
-  if (rec) return states ? reinterpret_cast<const void*>(batch_cluster_kernel<true, true>)
-                         : reinterpret_cast<const void*>(batch_cluster_kernel<true, false>);
-  return states ? reinterpret_cast<const void*>(batch_cluster_kernel<false, true>)
-                : reinterpret_cast<const void*>(batch_cluster_kernel<false, false>);
+  if (rec) return states ? reinterpret_cast<const void*>(batch_cluster_kernel<true, true, PULL>)
+                         : reinterpret_cast<const void*>(batch_cluster_kernel<true, false, PULL>);
+  return states ? reinterpret_cast<const void*>(batch_cluster_kernel<false, true, PULL>)
+                : reinterpret_cast<const void*>(batch_cluster_kernel<false, false, PULL>);
 }
 
 size_t batch_smem_bytes(uint32_t Lmax, int threads) {
@@ -742,10 +786,11 @@ cudaError_t prepare_batch_kernel(uint32_t Lmax, int threads) {
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, int(kBatchSmemCap));
         if (e != cudaSuccess) return e;
       }
-      const cudaError_t f = cudaFuncSetAttribute(share_fn(rec, states), cudaFuncAttributeMaxDynamicSharedMemorySize, int(kBatchSmemCap));
-      if (f != cudaSuccess) return f;
-      const cudaError_t g = cudaFuncSetAttribute(share_fn(rec, states), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-      if (g != cudaSuccess) return g;
+      for (const void* fn : {share_fn<false>(rec, states), share_fn<true>(rec, states)}) {
+        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kBatchSmemCap));
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return e;
+      }
     }
   return cudaSuccess;
 }
@@ -753,42 +798,100 @@ cudaError_t prepare_batch_kernel(uint32_t Lmax, int threads) {
 // (more than half of an SM's: a block has an SM to itself)
 static size_t share_smem(uint32_t Lmax, uint32_t blocks) {
   const size_t n = sizeof(uint32_t) * (kDevStagedWords + size_t(kBatchExtWords) * 1024) +
-                   2 * 3 * sizeof(uint16_t) * (ring_split(Lmax, blocks).most + 2 * kMostHalo + 1);
+                   2 * 3 * sizeof(uint16_t) * std::max(ring_split(Lmax, blocks).most + 2 * kMostHalo + 1, kSplitFrom);
   return std::max<size_t>(n, 116 * 1024);
 }
 
-// The split form, where it is the better one and fits: the largest clusters (any number of
-// blocks up to 16) that are resident at the same time for all rings.  At least 256 threads
-// (they stage the tables); one recording warp for four colliding ones, at most 8: 9 rings of
-// up to 1000 nodes with states 1.52 us per step, with twice as many 1.53, with all 1.58.
-static bool launch_split(const BatchArgs& b, const StepArgs& common, int sms, cudaStream_t s) {
-  if (b.Lmax < kSplitFrom) return false;
+// What a step costs, in us at 30 per velocity: a ring of one block, a part of a ring.
+static double ring_cost(double nodes) { return std::max(0.65 + 0.7e-3 * nodes, 0.4 + 1.45e-3 * nodes); }
+static double part_cost(double nodes) { return std::max(0.72 + 0.8e-3 * nodes, 0.55 + 1.6e-3 * nodes); }
+
+// When pieces of work, the longest first, are done by workers that pull them.
+template <class Cost>
+static double makespan(uint32_t pieces, uint32_t workers, const Cost& cost) {
+  if (pieces <= workers) return cost(0);
+  std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
+  double end = 0;
+  for (uint32_t i = 0; i < pieces; ++i) {
+    double t = cost(i);
+    if (i >= workers) {
+      t += free_at.top();
+      free_at.pop();
+    }
+    free_at.push(t);
+    end = std::max(end, t);
+  }
+  return end;
+}
+
+// The split form, where it is expected to be faster than a ring per block: the size of cluster
+// with which the rings are done first (a tenth allowed for what pulling costs).  Us per step, a
+// ring per block / split: 100 rings of 64 to 8192 nodes at 30 per velocity 11.9 / 4.3, 200 12.0 /
+// 6.5, 400 at 50 15.2 / 13.2; 150 of 64 to 2000 3.3 / 2.2.  At least 256 threads (they stage the
+// tables); one recording warp for four colliding ones, at most 8: 9 rings of up to 1000 nodes with
+// states 1.52 us per step, with twice as many 1.53, with all 1.58.
+static bool launch_split(const BatchArgs& b, const uint32_t* lengths, const StepArgs& common, int sms, cudaStream_t s) {
+  const uint32_t N = uint32_t(sms), n = b.n;
+  // more than eight rings per SM keep all SMs busy to the end
+  if (b.Lmax < kSplitFrom || n > 8 * N) return false;
   const bool rec = b.record || b.states;
-  const void* fn = share_fn(b.record != nullptr, b.states != nullptr);
-  for (uint32_t blocks = std::min({16u, uint32_t(sms) / b.n, b.Lmax / 32}); blocks >= 2; --blocks) {
-    const uint32_t tiles = ring_split(b.Lmax, blocks).tiles;
-    uint32_t recorders = rec ? std::clamp((tiles + 1) / 4, 1u, 8u) : 0u;
+  const uint32_t split = uint32_t(std::partition_point(lengths, lengths + n, [](uint32_t L) { return L >= kSplitFrom; }) - lengths);
+  // (rings of up to kBatchSmallL nodes in larger numbers: several blocks on an SM)
+  const bool several = b.Lmax <= kBatchSmallL && n > N;
+  double nodes = 0;
+  for (uint32_t i = 0; i < n; ++i) nodes += lengths[i];
+  const auto whole = [&](uint32_t i) { return ring_cost(lengths[i]); };
+  double least = several ? std::max(whole(0), 1.45e-3 * nodes / N) : makespan(n, N, whole);
+  uint32_t best = 0, clusters = 0;
+  bool pull = false;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  uint32_t recorders = 0;
+  const auto shape = [&](uint32_t blocks) {
+    const uint32_t tiles = std::max(ring_split(b.Lmax, blocks).tiles, split < n ? kSplitFrom / 32 : 1u);
+    recorders = rec ? std::clamp((tiles + 1) / 4, 1u, 8u) : 0u;
     const uint32_t rounds = (tiles + 31 - recorders) / (32 - recorders);
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
     attr.val.clusterDim.x = blocks;
-    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(b.n * blocks);
     cfg.blockDim = dim3(std::max(256u, ((tiles + rounds - 1) / rounds + recorders) * 32));
     cfg.dynamicSmemBytes = share_smem(b.Lmax, blocks);
-    cfg.stream = s;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.gridDim = dim3(blocks);
+  };
+  for (uint32_t blocks = std::min(16u, b.Lmax / 32); blocks >= 2; --blocks) {
+    const uint32_t pieces = split + (n - split + blocks - 1) / blocks;
+    const auto piece = [&](uint32_t i) {
+      return i < split ? part_cost(double(lengths[i]) / blocks) : ring_cost(lengths[split + (i - split) * blocks]);
+    };
+    const auto time = [&](uint32_t room) { return n <= room ? part_cost(double(b.Lmax) / blocks) : 1.1 * makespan(pieces, room, piece); };
+    if (time(N / blocks) >= least) continue;
+    shape(blocks);
     int fit = 0;
-    if (cudaOccupancyMaxActiveClusters(&fit, fn, &cfg) == cudaSuccess && uint32_t(fit) >= b.n) {
-      BatchArgs ba = b;
-      StepArgs ca = common;
-      void* p[] = {&ba, &ca, &blocks, &recorders};
-      if (cudaLaunchKernelExC(&cfg, fn, p) == cudaSuccess) return true;
+    if (cudaOccupancyMaxActiveClusters(&fit, share_fn<true>(b.record != nullptr, b.states != nullptr), &cfg) != cudaSuccess || fit < 1) {
+      cudaGetLastError();
+      continue;
     }
-    cudaGetLastError();
+    const double t = time(uint32_t(fit));
+    if (t >= least) continue;
+    least = t;
+    best = blocks;
+    pull = n > uint32_t(fit);
+    clusters = pull ? std::min(pieces, uint32_t(fit)) : n;
   }
+  if (!best) return false;
+  shape(best);
+  cfg.gridDim = dim3(clusters * best);
+  BatchArgs ba = b;
+  StepArgs ca = common;
+  uint32_t whole_from = split;
+  void* p[] = {&ba, &ca, &best, &recorders, &whole_from};
+  const void* fn = pull ? share_fn<true>(b.record != nullptr, b.states != nullptr)
+                        : share_fn<false>(b.record != nullptr, b.states != nullptr);
+  if (cudaLaunchKernelExC(&cfg, fn, p) == cudaSuccess) return true;
+  cudaGetLastError();
   return false;
 }
 
@@ -796,8 +899,8 @@ static bool launch_split(const BatchArgs& b, const StepArgs& common, int sms, cu
 // decide), at most one per ring.  A block has as many of its shape's threads as the longest
 // ring keeps equally busy (320 nodes on the 256-thread shape: 160 threads, two nodes each),
 // and the recording warps.
-cudaError_t launch_batch(const BatchArgs& b, const StepArgs& common, int sms, cudaStream_t s, int shape) {
-  if (launch_split(b, common, sms, s)) return cudaSuccess;
+cudaError_t launch_batch(const BatchArgs& b, const uint32_t* lengths, const StepArgs& common, int sms, cudaStream_t s, int shape) {
+  if (launch_split(b, lengths, common, sms, s)) return cudaSuccess;
   const size_t smem = batch_smem_bytes(b.Lmax, shape);
   const bool rec = b.record != nullptr || b.states != nullptr;
   const uint32_t most = uint32_t(shape) / 32, tiles = (b.Lmax + 31) / 32;

@@ -20,6 +20,7 @@ struct ilg_batch {
   uint32_t n = 0;
   std::vector<ilg_params> p;
   std::vector<ReplicaDesc> desc;      // host mirror (t updated after each run)
+  std::vector<uint32_t> lengths;      // longest first
   cudaStream_t stream = nullptr;
   bool own_stream = false;            // created here: a capture needs a non-legacy stream
   int sms = 0;
@@ -160,6 +161,7 @@ ilg_status ilg_batch_create(const ilg_params* params, uint32_t n, void* stream, 
   std::vector<uint32_t> order(n);
   std::iota(order.begin(), order.end(), 0u);
   std::stable_sort(order.begin(), order.end(), [&](uint32_t x, uint32_t y) { return b->desc[x].L > b->desc[y].L; });
+  for (uint32_t i : order) b->lengths.push_back(b->desc[i].L);
 
   if ((e = dev_alloc(&b->d_state, sizeof(uint16_t) * b->total)) != cudaSuccess) return bail(e, "cudaMalloc state");
   if ((e = dev_alloc(&b->d_desc, sizeof(ReplicaDesc) * n)) != cudaSuccess) return bail(e, "cudaMalloc desc");
@@ -332,7 +334,7 @@ ilg_status batch_launch(ilg_batch* b, uint32_t T, int32_t record_mode, bool rec,
     BCUDA(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal), "begin capture");
     cudaError_t e = cudaMemsetAsync(b->d_counter, 0, sizeof(unsigned int), b->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_failed, 0, sizeof(uint32_t) * b->n, b->stream);
-    if (e == cudaSuccess) e = launch_batch(a, b->common, b->sms, b->stream, b->threads);
+    if (e == cudaSuccess) e = launch_batch(a, b->lengths.data(), b->common, b->sms, b->stream, b->threads);
     cudaError_t e2 = cudaStreamEndCapture(b->stream, &g);
     if (e != cudaSuccess || e2 != cudaSuccess) {
       if (g) cudaGraphDestroy(g);
@@ -502,7 +504,7 @@ ilg_status ilg_batch_autotune(ilg_batch* b, uint32_t trial_steps, ilg_tuning* ou
       e = cudaMemsetAsync(s_counter, 0, sizeof(unsigned int), b->stream);
       if (e == cudaSuccess) e = cudaMemsetAsync(s_failed, 0, sizeof(uint32_t) * b->n, b->stream);
       if (e == cudaSuccess) e = cudaEventRecord(e0, b->stream);
-      if (e == cudaSuccess) e = launch_batch(a, b->common, b->sms, b->stream, threads);
+      if (e == cudaSuccess) e = launch_batch(a, b->lengths.data(), b->common, b->sms, b->stream, threads);
       if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
       if (e == cudaSuccess) e = cudaEventSynchronize(e1);
       if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);

@@ -2,8 +2,9 @@
 the shortest that is split, that leave parts of unlike size, rings too short to be split
 beside long ones (down to three nodes), the longest ring, every number of rings per cluster
 size; steps beyond several exchanges of the halos and the 64 steps whose words are made
-ahead; both samplers and probabilities that are never or always; a ring that overflows after
-its beams have crossed the border of two parts.  States bit for bit; amplitudes as for the
+ahead; more rings than clusters, which pull them, the short ones one per block; both samplers and
+probabilities that are never or always; a ring that overflows after its beams have crossed the
+border of two parts, and one of a block of its own.  States bit for bit; amplitudes as for the
 unsplit rings (1e-12 of the sum of magnitudes, 2^-62 fixed point against extended precision)."""
 import numpy as np
 import pytest
@@ -26,6 +27,7 @@ def rings(Ls, **kw):
 
 CASES = [([256], 90, {}), ([257, 3, 5, 31, 63, 64, 95], 75, {}), ([1000] * 16 + [97], 40, dict(n0=90.0)),
          ([10240], 30, {}), ([4099, 300, 8192], 35, dict(omega_eff=0.6)), ([700] * 50, 25, {}), ([511] * 76, 25, {}),
+         ([2500] * 12 + [700] * 40 + list(range(3, 74)), 30, {}), ([2000] * 5 + [130, 255, 256, 77] * 30, 30, dict(sampler=1)),
          ([600, 40], 30, dict(sampler=1)), ([333], 30, dict(omega_eff=2.0)), ([333], 30, dict(omega_eff=1.0, n0=150.0))]
 
 
@@ -51,10 +53,11 @@ def test_split_rings(B, Ls, T, kw):
             assert np.array_equal(a.get_state(i)[0], s) and np.array_equal(b.get_state(i)[0], s)
 
 
-def test_split_ring_overflows(B):
+@pytest.mark.parametrize("L,more", [(300, []), (300, [2500] * 12 + [90] * 120), (200, [2500] * 12 + [90] * 120)])
+def test_split_ring_overflows(B, L, more):
     # two beams meet at a crowded node between two parts
-    reps = rings([300, 300], omega_eff=0.02, theta=0.01, amp=0.0)
-    s0 = np.full((3, 1, 300), 5, np.uint16)
+    reps = rings([L, L] + more, omega_eff=0.02, theta=0.01, amp=0.0)
+    s0 = np.full((3, 1, L), 5, np.uint16)
     s0[0, 0, 100], s0[1, 0, 80], s0[2, 0, 120] = 65400, 48000, 48000
     ref = O.Lattice(**reps[0])
     s, t = s0, 3
