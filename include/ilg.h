@@ -257,8 +257,9 @@ ilg_status ilg_batch_ensemble(ilg_batch* b, uint32_t T, int32_t mode, double* st
 /* Batch autotuner: times the block shapes 256, 512 and 1024 threads (candidates 0-2;
  * ceil(L / threads) nodes of a ring per thread and step, as many blocks per SM as
  * shared memory allows) for trial_steps steps (0: 50; at most 10000) on copies of all
- * rings, and keeps the fastest for later runs.  States, step counters and results are
- * unchanged.  out may be NULL.  Synchronous. */
+ * rings, and keeps the fastest for later runs.  Few rings, and rings of unlike length, are
+ * split between SMs whatever the shape, and all candidates then take the same time.  States,
+ * step counters and results are unchanged.  out may be NULL.  Synchronous. */
 ilg_status ilg_batch_autotune(ilg_batch* b, uint32_t trial_steps, ilg_tuning* out);
 
 /* ---------------------------------------------------------------------------

@@ -78,12 +78,12 @@ struct ProjWork {
   unsigned long long* scratch;
 };
 // modes: host, nmodes > 0 pairs; res (4 doubles per mode) and mass: device or mapped host memory
+cudaError_t launch_project(const ProjWork& w, uint32_t Lx, uint32_t Ly, const int32_t* modes, uint32_t nmodes,
+                           double* res, unsigned long long* mass, cudaStream_t s);
 // the same with the sums in one launch, for small lattices
 bool takes_small_project(uint32_t Lx, uint32_t Ly, uint32_t nmodes);  // nmodes > 0
 cudaError_t launch_small_project(int Q, const uint16_t* state, uint32_t Lx, uint32_t Ly, const int32_t* modes,
                                  uint32_t nmodes, double* res, unsigned long long* mass, cudaStream_t s);
-cudaError_t launch_project(const ProjWork& w, uint32_t Lx, uint32_t Ly, const int32_t* modes, uint32_t nmodes,
-                           double* res, unsigned long long* mass, cudaStream_t s);
 cudaError_t launch_philox(const uint32_t* ctr, uint32_t k0, uint32_t k1, uint32_t* out, size_t n,
                           cudaStream_t s);
 
