@@ -352,11 +352,11 @@ cudaError_t queue_results(ilg_server* s, const std::vector<Resident>& out) {
 }
 
 // ... then, with the next round already queued, the states are copied out on a stream of
-// their own (the round that wrote them has completed), the memory goes back to the arena and
-// the results to the result queue.
+// their own, the memory goes back to the arena and the results to the result queue.
 cudaError_t deliver(ilg_server* s, std::vector<Resident>& out) {
   if (out.empty()) return cudaSuccess;
-  cudaError_t e = cudaSuccess;
+  // behind the last round and the initial states: a request of no steps takes part in no round
+  cudaError_t e = cudaStreamWaitEvent(s->out_stream, s->out_ev, 0);
   for (size_t i = 0; i < out.size() && e == cudaSuccess; ++i)
     if (has_result(out[i]) && out[i].rq.final_state)
       e = cudaMemcpyAsync(out[i].rq.final_state, state_of(s, out[i]), out[i].state_bytes, cudaMemcpyDeviceToHost,
