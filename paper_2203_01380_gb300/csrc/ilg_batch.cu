@@ -9,9 +9,7 @@
 
 #include <algorithm>
 #include <functional>
-#include <queue>
 #include <type_traits>
-#include <vector>
 
 #include "ilg_batch.h"
 #include "ilg_collide.cuh"
@@ -397,12 +395,12 @@ __global__ void __launch_bounds__(REC || STATES ? BatchShape<THREADS>::kMost : T
 // --- a ring split between the blocks of a cluster ----------------------------
 //
 // Where a ring per block would leave SMs idle (few rings, or rings of unlike length), a ring's
-// nodes are split between the blocks of a cluster, one block per SM.  A block keeps its own nodes and a halo of 8 to 23
-// nodes on both sides, which it advances as well (a node's random words depend on the node
-// and the step alone); with every step the outermost nodes of the halo lapse, and when it is
-// used up the neighbours' nodes come through the cluster's shared memory.  So the blocks
-// meet once in 8 to 23 steps and not in each: occupations sent to the neighbour in every
-// step, as words with the step's tag, cost 0.4 us per step (rings of 64 nodes 1.09 us per
+// nodes are split between the blocks of a cluster, one block per SM.  A block keeps its own
+// nodes and a halo of 8 to 23 nodes on both sides, which it advances as well (a node's random
+// words depend on the node and the step alone); with every step the outermost nodes of the halo
+// lapse, and when it is used up the neighbours' nodes come through the cluster's shared memory.
+// So the blocks meet once in 8 to 23 steps and not in each: occupations sent to the neighbour in
+// every step, as words with the step's tag, cost 0.4 us per step (rings of 64 nodes 1.09 us per
 // step instead of 0.69).
 // Bound as before by integer issue for long shares and a node's chain of draws for short
 // ones.  Us per step, one block per ring / split: one ring of 8192 nodes at 50 per velocity
@@ -442,7 +440,7 @@ struct Share {
 __device__ __forceinline__ void exchange(const Share& h, uint16_t* src, ShareShared& sh, uint32_t parity, uint32_t threads) {
   const uint32_t H = h.halo, items = threadIdx.x < threads ? 6 * H : 0;
   for (uint32_t j = threadIdx.x; j < items; j += threads) {
-    const uint32_t side = j >= 3 * H, q = j - side * 3 * H, v = q / H, c = q - v * H;  // the first nodes go left, the last right
+    const uint32_t side = j >= 3 * H, q = j - side * 3 * H, v = q / H, c = q - v * H;  // first nodes left, last right
     const uint32_t at = mapa(&sh.mail[parity][side ^ 1][q], side ? h.right : h.left);
     asm volatile("st.shared::cluster.u16 [%0], %1;\n" ::"r"(at), "h"(src[v * h.stride + c + (side ? h.n : H)]) : "memory");
   }
@@ -655,12 +653,17 @@ __device__ __forceinline__ void run_split(const BatchArgs& b, const StepArgs& co
       for (size_t i = rank * threads + tid; i < (size_t(b.T) + 1) * 4; i += blocks * threads) rec[i] = 0ull;
     meet();
     const bool plain = !a.particle && a.omega_mode == kTable && a.rest_mode == kTable;
-    if (plain) run_share<REC, STATES, true>(b, a, d, r, h, T, tables, to, tr, words, sh, src, ring + 3 * h.stride, colliders, h.n ? recorders : 0);
-    else run_share<REC, STATES, false>(b, a, d, r, h, T, tables, to, tr, words, sh, src, ring + 3 * h.stride, colliders, h.n ? recorders : 0);
+    const uint32_t R = h.n ? recorders : 0;
+    uint16_t* const other = ring + 3 * h.stride;
+    if (plain)
+      run_share<REC, STATES, true>(b, a, d, r, h, T, tables, to, tr, words, sh, src, other, colliders, R);
+    else
+      run_share<REC, STATES, false>(b, a, d, r, h, T, tables, to, tr, words, sh, src, other, colliders, R);
     meet();
     uint32_t fail = ~0u;
     if (ALONE && blocks == 1) fail = sh.fail;
-    else if (lane < blocks) asm volatile("ld.shared::cluster.u32 %0, [%1];\n" : "=r"(fail) : "r"(mapa(&sh.fail, lane)) : "memory");
+    else if (lane < blocks)
+      asm volatile("ld.shared::cluster.u32 %0, [%1];\n" : "=r"(fail) : "r"(mapa(&sh.fail, lane)) : "memory");
     fail = __reduce_min_sync(kFullWarp, fail);
     if (fail == ~0u) break;
     // once more from the start, as far as the ring goes
@@ -740,7 +743,8 @@ const void* batch_fn(int threads, bool rec, bool states, bool alone) {
                   : reinterpret_cast<const void*>(batch_d1q3_kernel<N, false, false, A>);
   };
   if (threads == 256)
-    return alone ? pick(std::integral_constant<int, 256>{}, std::true_type{}) : pick(std::integral_constant<int, 256>{}, std::false_type{});
+    return alone ? pick(std::integral_constant<int, 256>{}, std::true_type{})
+                 : pick(std::integral_constant<int, 256>{}, std::false_type{});
   if (threads == 512) return pick(std::integral_constant<int, 512>{}, std::false_type{});
   return pick(std::integral_constant<int, 1024>{}, std::false_type{});
 }
@@ -806,19 +810,30 @@ static size_t share_smem(uint32_t Lmax, uint32_t blocks) {
 static double ring_cost(double nodes) { return std::max(0.65 + 0.7e-3 * nodes, 0.4 + 1.45e-3 * nodes); }
 static double part_cost(double nodes) { return std::max(0.72 + 0.8e-3 * nodes, 0.55 + 1.6e-3 * nodes); }
 
-// When pieces of work, the longest first, are done by workers that pull them.
+// When pieces of work, the longest first, are done by workers that pull them: at the earliest
+// (all busy to the end), and one piece after the other.
+template <class Cost>
+static double work_bound(uint32_t pieces, uint32_t workers, const Cost& cost) {
+  double sum = 0;
+  for (uint32_t i = 0; i < pieces; ++i) sum += cost(i);
+  return std::max(cost(0), sum / workers);
+}
 template <class Cost>
 static double makespan(uint32_t pieces, uint32_t workers, const Cost& cost) {
+  constexpr uint32_t kMost = 512;
   if (pieces <= workers) return cost(0);
-  std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
-  double end = 0;
+  if (workers > kMost) return work_bound(pieces, workers, cost);
+  double free_at[kMost], end = 0;  // a heap, the earliest first
   for (uint32_t i = 0; i < pieces; ++i) {
     double t = cost(i);
+    uint32_t held = i;
     if (i >= workers) {
-      t += free_at.top();
-      free_at.pop();
+      std::pop_heap(free_at, free_at + workers, std::greater<double>());
+      held = workers - 1;
+      t += free_at[held];
     }
-    free_at.push(t);
+    free_at[held] = t;
+    std::push_heap(free_at, free_at + held + 1, std::greater<double>());
     end = std::max(end, t);
   }
   return end;
@@ -835,7 +850,8 @@ static bool launch_split(const BatchArgs& b, const uint32_t* lengths, const Step
   // more than eight rings per SM keep all SMs busy to the end
   if (b.Lmax < kSplitFrom || n > 8 * N) return false;
   const bool rec = b.record || b.states;
-  const uint32_t split = uint32_t(std::partition_point(lengths, lengths + n, [](uint32_t L) { return L >= kSplitFrom; }) - lengths);
+  const auto is_long = [](uint32_t L) { return L >= kSplitFrom; };
+  const uint32_t split = uint32_t(std::partition_point(lengths, lengths + n, is_long) - lengths);
   // (rings of up to kBatchSmallL nodes in larger numbers: several blocks on an SM)
   const bool several = b.Lmax <= kBatchSmallL && n > N;
   double nodes = 0;
@@ -866,15 +882,17 @@ static bool launch_split(const BatchArgs& b, const uint32_t* lengths, const Step
     const auto piece = [&](uint32_t i) {
       return i < split ? part_cost(double(lengths[i]) / blocks) : ring_cost(lengths[split + (i - split) * blocks]);
     };
-    const auto time = [&](uint32_t room) { return n <= room ? part_cost(double(b.Lmax) / blocks) : 1.1 * makespan(pieces, room, piece); };
-    if (time(N / blocks) >= least) continue;
+    const bool own = n <= N / blocks;  // perhaps a cluster for every ring
+    const double longest = part_cost(double(b.Lmax) / blocks);
+    if ((own ? longest : 1.1 * work_bound(pieces, N / blocks, piece)) >= least) continue;
     shape(blocks);
     int fit = 0;
-    if (cudaOccupancyMaxActiveClusters(&fit, share_fn<true>(b.record != nullptr, b.states != nullptr), &cfg) != cudaSuccess || fit < 1) {
+    const void* fn = share_fn<true>(b.record != nullptr, b.states != nullptr);
+    if (cudaOccupancyMaxActiveClusters(&fit, fn, &cfg) != cudaSuccess || fit < 1) {
       cudaGetLastError();
       continue;
     }
-    const double t = time(uint32_t(fit));
+    const double t = n <= uint32_t(fit) ? longest : 1.1 * makespan(pieces, uint32_t(fit), piece);
     if (t >= least) continue;
     least = t;
     best = blocks;
@@ -899,7 +917,8 @@ static bool launch_split(const BatchArgs& b, const uint32_t* lengths, const Step
 // decide), at most one per ring.  A block has as many of its shape's threads as the longest
 // ring keeps equally busy (320 nodes on the 256-thread shape: 160 threads, two nodes each),
 // and the recording warps.
-cudaError_t launch_batch(const BatchArgs& b, const uint32_t* lengths, const StepArgs& common, int sms, cudaStream_t s, int shape) {
+cudaError_t launch_batch(const BatchArgs& b, const uint32_t* lengths, const StepArgs& common, int sms, cudaStream_t s,
+                         int shape) {
   if (launch_split(b, lengths, common, sms, s)) return cudaSuccess;
   const size_t smem = batch_smem_bytes(b.Lmax, shape);
   const bool rec = b.record != nullptr || b.states != nullptr;

@@ -53,7 +53,8 @@ uint32_t batch_default_threads(uint32_t Lmax, uint32_t n, uint32_t sms);
 cudaError_t prepare_batch_kernel(uint32_t Lmax, int threads);
 // lengths: the rings' (host), longest first.  (Not in BatchArgs: with the kernels' arguments eight
 // bytes further on 512 rings of 320 nodes take 6.41 instead of 6.20 ms.)
-cudaError_t launch_batch(const BatchArgs& b, const uint32_t* lengths, const StepArgs& common, int sms, cudaStream_t s, int shape);
+cudaError_t launch_batch(const BatchArgs& b, const uint32_t* lengths, const StepArgs& common, int sms, cudaStream_t s,
+                         int shape);
 cudaError_t launch_batch_obs(const ReplicaDesc* desc, const uint16_t* state, uint32_t n, int32_t mode,
                              unsigned long long* mass, double* amp, cudaStream_t s);
 cudaError_t launch_batch_amp(const ReplicaDesc* desc, const double* record, uint32_t n, uint32_t T, double* amp,
