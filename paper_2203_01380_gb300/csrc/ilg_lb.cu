@@ -690,6 +690,14 @@ ilg_status lb_gave_up(ilg_lb* b) {
   return lb_fail(b, ILG_E_TIMEOUT, "a wait between the blocks of a several-step launch gave up: the state is lost");
 }
 
+// A fresh state: a wait that gave up in earlier steps, not read back yet, does not concern it.
+cudaError_t lb_forget_waits(ilg_lb* b) {
+  b->h_sync = 0;
+  if (!b->waits) return cudaSuccess;
+  b->waits = false;
+  return cudaMemsetAsync(b->d_sync, 0, 2 * sizeof(unsigned long long), b->stream);  // behind those steps
+}
+
 }  // namespace
 
 extern "C" {
@@ -826,6 +834,7 @@ ilg_status ilg_lb_init(ilg_lb* b) {
     axis = along_x ? 1 : 2;
     mode = uint32_t(((m % L) + L) % L);
   }
+  LB_CUDA(b, lb_forget_waits(b), "lattice Boltzmann init");
   double* d_lam = nullptr;
   LB_CUDA(b, ilg::dev_alloc(&d_lam, sizeof(double) * lam.size()), "cudaMalloc");
   cudaError_t e = cudaMemcpyAsync(d_lam, lam.data(), sizeof(double) * lam.size(), cudaMemcpyHostToDevice, b->stream);
@@ -852,6 +861,7 @@ ilg_status ilg_lb_init(ilg_lb* b) {
 ilg_status ilg_lb_set_state(ilg_lb* b, const double* host, size_t n, uint64_t t) {
   if (!b) return ILG_E_INVALID;
   if (!host || n != size_t(b->Q) * b->nodes) return lb_fail(b, ILG_E_INVALID, "state must hold Q*Lx*Ly doubles");
+  LB_CUDA(b, lb_forget_waits(b), "copy in");
   LB_CUDA(b, cudaMemcpyAsync(b->f[b->cur], host, sizeof(double) * n, cudaMemcpyHostToDevice, b->stream), "copy in");
   LB_CUDA(b, cudaStreamSynchronize(b->stream), "copy in");
   b->t = t;
