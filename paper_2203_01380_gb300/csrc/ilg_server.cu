@@ -520,6 +520,11 @@ void worker_main(ilg_server* s) {
     }
     if (!lat.empty() && q > 0) {
       share_out(cost, lat, uint32_t(s->sms), &shares, &first, &part);
+      // (the cuts add one share per block at most: see share_out)
+      if (shares.size() > size_t(s->sms) + s->max_slots) {
+        e = cudaErrorInvalidValue;
+        break;
+      }
       const size_t n = lat.size(), blocks = first.size() - 1;
       unsigned long long* const d_cycles = s->d_round + 1;
       uint32_t* const d_fail = reinterpret_cast<uint32_t*>(d_cycles + s->sms);
