@@ -69,10 +69,14 @@ __device__ __forceinline__ longlong2 trig_fixed(uint32_t r, uint32_t L) {
 //   re = sum_x cos(2 pi r / L) D(x) / L,  im = sum_x sin(2 pi r / L) D(x) / L.
 // The trigonometric values enter as 2^-62 fixed-point integers and the sums are exact, so
 // they do not depend on the summation order.  A step adds only
-//   sum_x c(x) N(x),  c = c1 2^32 + c0:  N c0 < 2^50 and |N c1| < 2^48 per node, below 2^63
-// over a ring (four wide multiply-adds per node, against two 64 x 64 -> 128 products);
+//   sum_x c(x) N(x),  c = c1 2^32 + c0:  N c0 < 3 65535 2^32 and |N c1| < 2^48 per node, below
+// 2^63 over the longest ring (four wide multiply-adds per node, against two 64 x 64 -> 128
+// products);
 // the factor L and the M sum_x c(x) term, the same for every step, join when a state's
 // sums are written out (write_sums).
+static_assert((uint64_t(3 * 65535) << 32) * kBatchMaxL / kBatchMaxL == uint64_t(3 * 65535) << 32 &&
+                  (uint64_t(3 * 65535) << 32) * kBatchMaxL < uint64_t(1) << 63,
+              "a ring's sums of low parts");
 struct ModeSums {
   long long v[4];  // cos low, cos high, sin low, sin high
   __device__ __forceinline__ void clear() { v[0] = v[1] = v[2] = v[3] = 0; }
@@ -986,7 +990,7 @@ __global__ void __launch_bounds__(256) batch_obs_kernel(const ReplicaDesc* __res
 }
 
 // ring r's trig[state_off_r / 3 + x] = fixed-point (cos, sin) of 2 pi ((m_r x) mod L_r) / L_r,
-// m_r the mode reduced modulo L_r: the values ring_partials would compute per node
+// m_r the mode reduced modulo L_r
 __global__ void batch_trig_rings_kernel(const ReplicaDesc* __restrict__ desc, uint32_t n, int32_t mode,
                                         longlong2* __restrict__ trig) {
   for (uint32_t r = blockIdx.x; r < n; r += gridDim.x) {
