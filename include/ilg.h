@@ -266,12 +266,15 @@ ilg_status ilg_batch_autotune(ilg_batch* b, uint32_t trial_steps, ilg_tuning* ou
  * Serving loop for D2Q5 lattice requests (continuous batching).  A worker thread
  * admits requests in arrival order while a free slot and room in a device arena
  * of hbm_bytes (allocated once, here) allow, keeps admitted lattices resident, and
- * advances all of them together: one launch per time step, `quantum` steps per
- * round (fewer when a request needs fewer), so newcomers join the next round.  A
+ * advances all of them together: one launch per round of `quantum` steps (32 at
+ * most, fewer when a request needs fewer), so newcomers join the next round.  A
  * finished request's observables go to the result queue and, if final_state was
  * given, its state (5*Lx*Ly uint16) is copied there; its memory returns to the
  * arena.  Results equal those of the request run alone (ilg_create ...), bit for
- * bit.  All requests share the server's seed.  Host waits only (no device spin).
+ * bit.  All requests share the server's seed.  A round's blocks, all resident, wait
+ * for one another between its steps, a bounded time: should a wait give up, the
+ * server ends and its calls return ILG_E_TIMEOUT, and ilg_server_last_error says so
+ * (after wait_idle's own time limit it does not).
  *   ilg_server_create    seed, arena bytes, slots, quantum, stream (NULL: private)
  *   ilg_server_submit    thread-safe, returns at once; final_state must stay valid
  *                        until the request's result has been polled
