@@ -959,7 +959,8 @@ cudaError_t launch_sums(int Q, const uint16_t* in, uint32_t Lx, uint32_t Ly, uns
 // double instructions, are all that is left.  Against compensated double sums (DoubleSums,
 // still taken where 128 bits might not do), whose trees took most of a short mode's time:
 // mass and one mode of a ring of 256 nodes 27 / 35 us, of 1024^2 31 / 39, 64 modes of 16384^2
-// 482 / 556, two modes of 2^22 nodes 707 / 1011; the results are the same to the last bit.
+// 482 / 556, two modes of 2^22 nodes 707 / 1011; on the states tried the results are the same to the
+// last bit (sines below 2^-9 have fewer than 53 bits here: see FixedSums).
 // --------------------------------------------------------------------------
 __device__ __forceinline__ void two_sum(double a, double b, double& s, double& e) {
   s = a + b;
